@@ -16,14 +16,16 @@ __global__ void __launch_bounds__(kCompactThreads)
 kv_compact_kernel(uint4* __restrict__ k_all, uint4* __restrict__ v_all, int n_heads, int chunks_per_head,
                   int64_t layer_stride16, int64_t slot_stride16, int64_t head_stride16,
                   const int64_t* __restrict__ kv_start, const int32_t* __restrict__ kv_len_in,
-                  const int32_t* __restrict__ accept_len, const int32_t* __restrict__ accept_path) {
+                  const int32_t* __restrict__ accept_len, const int32_t* __restrict__ accept_path, int32_t* __restrict__ kv_len_out) {
     const int layer = blockIdx.y, b = blockIdx.z;
     const int cols = n_heads * chunks_per_head;          // 16-byte columns per K (or V) slot
     const int col2 = blockIdx.x * kCompactThreads + threadIdx.x;
     wait_for_previous_kernel();
+    release_next_kernel();
     const int L = kv_len_in[b];
     int len = accept_len[b];
     len = max(0, min(len, SS_PATH_STRIDE));
+    if (kv_len_out != nullptr && col2 == 0 && layer == 0) kv_len_out[b] = L + len;
     if (col2 < 2 * cols) {
         uint4* base = (col2 < cols) ? k_all : v_all;
         const int col = (col2 < cols) ? col2 : col2 - cols;
@@ -48,9 +50,8 @@ kv_compact_kernel(uint4* __restrict__ k_all, uint4* __restrict__ v_all, int n_he
     }
 }
 
-// kv_len_out may alias kv_len_in, which every CTA of the gather reads: the lengths are updated by
-// a second, stream-ordered launch.
-
+// Where kv_len_out overlaps kv_len_in, which every CTA of the gather reads, the lengths are updated by a second,
+// stream-ordered launch; else the gather writes them itself.
 __global__ void kv_len_update_kernel(const int32_t* __restrict__ kv_len_in, const int32_t* __restrict__ accept_len,
                                      int32_t* __restrict__ kv_len_out, int batch) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -78,12 +79,14 @@ extern "C" int32_t ss_kv_compact(void* k_cache_all, void* v_cache_all, const ss_
     const int cols2 = 2 * lo.n_heads * chunks_per_head;
     dim3 grid((cols2 + ss::kCompactThreads - 1) / ss::kCompactThreads, lo.n_layers, batch);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const bool overlap = kv_len_out < kv_len_in + batch && kv_len_in < kv_len_out + batch;
     // both launches may be scheduled while their predecessor drains; each waits for it before touching memory
     if (ss::launch_after_previous(ss::kv_compact_kernel, grid, dim3(ss::kCompactThreads), s, static_cast<uint4*>(k_cache_all),
                                   static_cast<uint4*>(v_cache_all), lo.n_heads, chunks_per_head, lo.layer_stride / 8,
                                   lo.slot_stride / 8, lo.head_stride / 8, kv_start, kv_len_in, accept_len,
-                                  accept_path) != cudaSuccess)
+                                  accept_path, overlap ? nullptr : kv_len_out) != cudaSuccess)
         return SS_ERR_CUDA;
+    if (!overlap) return SS_OK;
     return ss::launch_after_previous(ss::kv_len_update_kernel, dim3((batch + 127) / 128), dim3(128), s, kv_len_in, accept_len,
                                      kv_len_out, batch) == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }

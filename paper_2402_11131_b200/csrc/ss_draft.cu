@@ -1,244 +1,201 @@
 // Draft management around the attention: the next tree draft (Sec. 3.2.2, App. A.1), parallel tree pruning
 // (Sec. 3.2.3), and the soft / sampled variants of the verification (App. A.2, App. B).
 //
-// All of them are one HBM-bound pass over rows of fp32 logits followed by a few dozen integer steps per
-// sequence.  One kernel per call: a (chunk, row, sequence) grid scans the rows with 128-bit loads and leaves
-// a small partial per chunk (the k best entries, or the maximum with the softmax sums); the last CTA to
-// finish a sequence (arrival counter, nobody waits) merges the partials and does the sequence's tail.
-//
-// Order of logits.  Entries are ranked by an integer key that is monotone in the IEEE order of fp32 values,
-// with -0 == +0 and every NaN below -inf, and equal keys by ascending index: the rule of the arg-max of the
-// verification, as a total order.  Compiled without fast-math: nothing is flushed or reassociated.
-#include "ss_common.cuh"
+// All of them are one HBM-bound pass over rows of fp32 logits followed by a few dozen integer steps per sequence.  One
+// kernel per call: a cluster per row scans it (see ss_rows.cuh) and leaves the row's result -- the k best entries, or
+// the maximum with the softmax sums -- in its CTA 0; the CTA that finishes a sequence's last row does the sequence's
+// tail, all nodes at once from their ancestor words.  The next draft has at most four rows per sequence, so one
+// cluster takes the whole sequence and nothing goes through global memory.  Compiled without fast-math.
+#include "ss_rows.cuh"
 
 namespace ss {
 
-constexpr int kScanThreads = 256;
-constexpr int kScanChunk = 4096;          // logits per CTA
-constexpr int kScanPerThread = kScanChunk / kScanThreads;
-constexpr int kMaxTopK = SS_MAX_TOPK;
-
-__device__ __forceinline__ uint32_t order_key(float x) {
-    if (x != x) return 0u;
-    x += 0.0f;                                         // -0 -> +0
-    const uint32_t u = __float_as_uint(x);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float key_value(uint32_t key) {
-    if (key == 0u) return __uint_as_float(0x7fc00000u);
-    return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
-}
-// larger = better: (key, lower index first)
-__device__ __forceinline__ unsigned long long entry(float x, int idx) {
-    return (static_cast<unsigned long long>(order_key(x)) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(idx));
-}
-__device__ __forceinline__ int entry_index(unsigned long long e) { return static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(e)); }
-__device__ __forceinline__ float entry_value(unsigned long long e) { return key_value(static_cast<uint32_t>(e >> 32)); }
-
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-    #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, off);
-        v = o > v ? o : v;
-    }
-    return v;
-}
-
-// the chunk's elements of this thread: 4 consecutive floats per step (or one by one when the row is not 16-byte aligned)
-template <typename F>
-__device__ __forceinline__ void for_chunk(const float* row, int vocab, int chunk, F&& f) {
-    const int lo = chunk * kScanChunk, hi = min(vocab, lo + kScanChunk);
-    if ((vocab & 3) == 0) {
-        const float4* row4 = reinterpret_cast<const float4*>(row);
+// ---- the k best entries of a segment --------------------------------------------------------------------------------
+// Pass 1 takes one maximum per thread.  The k-th largest of the 16 warp maxima bounds the k-th best logit of the segment
+// from below, and only a dozen logits or so of a segment reach that bound; pass 2, in the few threads that hold one,
+// reads the thread's logits again (they are in L2) and collects them.  Keeping a sorted list of k entries per thread
+// instead costs 8 compare-and-swaps of 64-bit words per logit: 34 us instead of DRAFT_SAMPLED_US us for 64 rows of 32000.
+struct ThreadMax {
+    float v = -INFINITY;
+    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
+        float m[4] = {x[0], x[1], x[2], x[3]};
         #pragma unroll
-        for (int s = 0; s < kScanPerThread / 4; ++s) {
-            const int i = lo / 4 + s * kScanThreads + static_cast<int>(threadIdx.x);
-            if (i < hi / 4) {
-                const float4 x = __ldcs(row4 + i);
-                f(x.x, 4 * i); f(x.y, 4 * i + 1); f(x.z, 4 * i + 2); f(x.w, 4 * i + 3);
-            }
-        }
-    } else {
-        #pragma unroll
-        for (int s = 0; s < kScanPerThread; ++s) {
-            const int i = lo + s * kScanThreads + static_cast<int>(threadIdx.x);
-            if (i < hi) f(row[i], i);
-        }
+        for (int q = 4; q < 4 * kRowVecs; ++q) m[q & 3] = fmaxf(m[q & 3], x[q]);
+        v = fmaxf(v, fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));      // (a NaN is never the maximum)
     }
-}
-
-// ---- scan 1: the k best entries of a chunk -> part[k] (descending; 0 = none) ---------------------------------
-__device__ void chunk_topk(const float* row, int vocab, int chunk, int k, unsigned long long* part) {
+    __device__ __forceinline__ void one(float x, int at) { v = fmaxf(v, x); }
+};
+// the k best of a thread's logits that are not below the bound (a NaN is not below anything)
+struct ThreadTopK {
+    float bound;
+    int hi;
     unsigned long long best[kMaxTopK];
-    #pragma unroll
-    for (int r = 0; r < kMaxTopK; ++r) best[r] = 0ull;
-    for_chunk(row, vocab, chunk, [&](float x, int i) {
-        unsigned long long e = entry(x, i);
+    __device__ __forceinline__ void one(float x, int at) {
+        if (x < bound || at >= hi) return;
+        unsigned long long e = entry(order_key(x), at);
         #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) {            // insertion into the sorted list
+        for (int r = 0; r < kMaxTopK; ++r) {
             if (e > best[r]) { const unsigned long long t = best[r]; best[r] = e; e = t; }
         }
-    });
-    // k rounds over the block: the best head wins and its owner moves on
-    __shared__ unsigned long long s_w[kScanThreads / 32];
-    __shared__ unsigned long long s_pick;
-    int pos = 0;
-    for (int r = 0; r < k; ++r) {
-        unsigned long long head = 0ull;
+    }
+    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
+        bool any = false;
         #pragma unroll
-        for (int q = 0; q < kMaxTopK; ++q) head = (q == pos) ? best[q] : head;
-        const unsigned long long wmax = warp_max_u64(head);
-        if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = wmax;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long m = s_w[0];
-            for (int w = 1; w < kScanThreads / 32; ++w) m = s_w[w] > m ? s_w[w] : m;
-            s_pick = m;
-            part[r] = m;
+        for (int q = 0; q < 4 * kRowVecs; ++q) any = any || !(x[q] < bound);
+        if (!any) return;
+        #pragma unroll 1
+        for (int v = 0; v < kRowVecs; ++v) {
+            float a = x[0], b = x[1], c = x[2], d = x[3];
+            int at = first[0];
+            #pragma unroll
+            for (int s = 1; s < kRowVecs; ++s)
+                if (s == v) { a = x[4 * s]; b = x[4 * s + 1]; c = x[4 * s + 2]; d = x[4 * s + 3]; at = first[s]; }
+            one(a, at); one(b, at + 1); one(c, at + 2); one(d, at + 3);
         }
-        __syncthreads();
-        if (head != 0ull && head == s_pick) ++pos;        // entries are unique (the index is part of them)
     }
-}
-
-// ---- scan 2: maximum (lowest index), Z = sum exp(x - m), W = sum (x - m) exp(x - m) of a chunk -----------------
-struct Stats {
-    unsigned long long best;      // entry of the maximum
-    float z, w;
 };
-__device__ __forceinline__ Stats merge_stats(const Stats& a, const Stats& b) {
-    Stats r;
-    r.best = a.best > b.best ? a.best : b.best;
-    const float m = entry_value(r.best), ma = entry_value(a.best), mb = entry_value(b.best);
-    r.z = 0.f; r.w = 0.f;
-    if (a.z > 0.f) { const float e = expf(ma - m); r.z += a.z * e; r.w += (a.w + (ma - m) * a.z) * e; }
-    if (b.z > 0.f) { const float e = expf(mb - m); r.z += b.z * e; r.w += (b.w + (mb - m) * b.z) * e; }
-    return r;
-}
-__device__ Stats chunk_stats(const float* row, int vocab, int chunk) {
-    float x[kScanPerThread];
-    int n = 0;
-    Stats s;
-    s.best = 0ull; s.z = 0.f; s.w = 0.f;
-    for_chunk(row, vocab, chunk, [&](float v, int i) {
-        const unsigned long long e = entry(v, i);
-        s.best = e > s.best ? e : s.best;
-        #pragma unroll
-        for (int q = 0; q < kScanPerThread; ++q) x[q] = (q == n) ? v : x[q];
-        ++n;
-    });
-    if (n > 0) {
-        const float m = entry_value(s.best);
-        #pragma unroll
-        for (int q = 0; q < kScanPerThread; ++q)
-            if (q < n) { const float d = x[q] - m, e = expf(d); s.z += e; if (e > 0.f) s.w += d * e; }
-    }
-    #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        Stats o;
-        o.best = __shfl_xor_sync(0xffffffffu, s.best, off);
-        o.z = __shfl_xor_sync(0xffffffffu, s.z, off);
-        o.w = __shfl_xor_sync(0xffffffffu, s.w, off);
-        s = merge_stats(s, o);
-    }
-    __shared__ Stats s_st[kScanThreads / 32];
-    if ((threadIdx.x & 31) == 0) s_st[threadIdx.x >> 5] = s;
-    __syncthreads();
-    Stats r = s_st[0];
-    for (int w = 1; w < kScanThreads / 32; ++w) r = merge_stats(r, s_st[w]);
-    return r;
-}
-
-// The k best of n_cand chunk candidates (kMaxTopK per chunk, the first k of each meaningful), by one warp: the lanes
-// share the candidates (four each in registers, more are read again in every round) and k rounds of a warp
-// maximum pick them in order (candidates are unique: the next best is the largest one below the last).
-// Every lane gets top[0 .. k).
-__device__ __forceinline__ void warp_topk(const unsigned long long* cand, int n_cand, int k, unsigned long long (&top)[kMaxTopK]) {
-    const int lane = threadIdx.x & 31;
-    unsigned long long mine[4];
-    #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = lane + 32 * q;
-        mine[q] = (j < n_cand && (j % kMaxTopK) < k) ? __ldcg(cand + j) : 0ull;
-    }
+// Picks the k largest of the distinct entries list[0 .. n) in descending order (one warp; every lane gets them).
+__device__ __forceinline__ void warp_select(const unsigned long long* list, int n, int k, unsigned long long (&top)[kMaxTopK]) {
+    const int lane = static_cast<int>(threadIdx.x) & 31;
+    const unsigned long long e0 = lane < n ? list[lane] : 0ull, e1 = lane + 32 < n ? list[lane + 32] : 0ull;
     unsigned long long below = ~0ull;
     #pragma unroll
     for (int r = 0; r < kMaxTopK; ++r) top[r] = 0ull;
-    for (int q = 0; q < k; ++q) {
-        unsigned long long m = 0ull;
-        #pragma unroll
-        for (int r = 0; r < 4; ++r)
-            if (mine[r] < below && mine[r] > m) m = mine[r];
-        for (int j = lane + 128; j < n_cand; j += 32) {
-            const unsigned long long e = (j % kMaxTopK) < k ? __ldcg(cand + j) : 0ull;
+    #pragma unroll
+    for (int r = 0; r < kMaxTopK; ++r) {
+        if (r >= k) break;
+        unsigned long long m = e0 < below ? e0 : 0ull;
+        if (e1 < below && e1 > m) m = e1;
+        for (int j = lane + 64; j < n; j += 32) {
+            const unsigned long long e = list[j];
             if (e < below && e > m) m = e;
         }
         m = warp_max_u64(m);
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) top[r] = (r == q) ? m : top[r];
+        top[r] = m;
         below = m;
     }
 }
-
-// the last CTA of a sequence to get here returns true (its threads then see every other CTA's partials)
-__device__ bool arrive_last(int32_t* counter, int expected) {
-    __shared__ bool s_last;
+struct TopKShared {
+    uint32_t warp_max[kRowWarps];
+    int n;
+    unsigned long long part[8][kMaxTopK];                 // CTA 0 of a cluster: the lists of its CTAs
+    unsigned long long list[kRowThreads * kMaxTopK];
+};
+// The k best entries of the segment, in every lane of warp 0.  Ends with the CTA's threads in step.
+__device__ __forceinline__ void segment_topk(const Segment& seg, int k, TopKShared& s, unsigned long long (&top)[kMaxTopK]) {
+    const int warp = static_cast<int>(threadIdx.x) >> 5, lane = static_cast<int>(threadIdx.x) & 31;
+    if (threadIdx.x == 0) s.n = 0;
+    ThreadMax tm;
+    scan_segment(seg, tm);
+    const uint32_t wm = __reduce_max_sync(0xffffffffu, order_key(tm.v));
+    if (lane == 0) s.warp_max[warp] = wm;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(counter, 1) == expected - 1;
+    // the k-th largest warp maximum, counting equal ones apart
+    uint32_t key = lane < kRowWarps ? s.warp_max[lane] : 0u, bound = 0u;
+    for (int r = 0; r < k; ++r) {
+        bound = __reduce_max_sync(0xffffffffu, key);
+        const uint32_t holders = __ballot_sync(0xffffffffu, key == bound);
+        if (lane == __ffs(holders) - 1) key = 0u;
+    }
+    ThreadTopK tk;
+    tk.bound = key_value(bound);
+    tk.hi = seg.hi;
+    if (!(tm.v < tk.bound)) {
+        #pragma unroll
+        for (int r = 0; r < kMaxTopK; ++r) tk.best[r] = 0ull;
+        scan_segment(seg, tk);
+        int have = 0;
+        #pragma unroll
+        for (int r = 0; r < kMaxTopK; ++r) have += (r < k && tk.best[r] != 0ull) ? 1 : 0;
+        int at = atomicAdd(&s.n, have);
+        #pragma unroll
+        for (int r = 0; r < kMaxTopK; ++r)
+            if (r < have) s.list[at + r] = tk.best[r];
     }
     __syncthreads();
-    if (s_last) __threadfence();
-    return s_last;
+    if (warp == 0) warp_select(s.list, s.n, k, top);
 }
 
-// deepest node whose whole root path is ok (lowest index among equally deep ones); one thread
-__device__ void accept_walk(int T, const int32_t* parent, const int32_t* depth, unsigned long long ok, int32_t* path, int* best_out,
-                            int* len_out) {
-    unsigned long long valid = 1ull;
-    int best = 0, best_depth = 0;
-    for (int c = 1; c < T; ++c) {
-        const int p = parent[c];
-        if (p >= 0 && ((valid >> p) & 1ull) && ((ok >> c) & 1ull)) {
-            valid |= 1ull << c;
-            if (depth[c] > best_depth) { best = c; best_depth = depth[c]; }
+// ---- softmax statistics of a row: maximum (lowest index), Z = sum exp(x - m), W = sum (x - m) exp(x - m) ------------
+struct Stats {
+    unsigned long long best;      // entry of the maximum, 0: none above -inf
+    float z, w;
+};
+struct RowStats {
+    ArgMax am;
+    float z = 0.f, w = 0.f;
+    __device__ __forceinline__ void raise(float m_old) {
+        if (am.v > m_old && z > 0.f) {
+            const float d = m_old - am.v, e = expf(d);
+            w = (w + d * z) * e;
+            z *= e;
         }
     }
-    const int len = best_depth + 1;
-    for (int a = best, i = len - 1; a >= 0 && i >= 0; a = parent[a], --i) path[i] = a;
-    for (int i = len; i < SS_PATH_STRIDE; ++i) path[i] = -1;
-    *best_out = best; *len_out = len;
+    __device__ __forceinline__ void add(float x) {
+        const float d = x - am.v, e = expf(d);
+        if (e > 0.f) { z += e; w += d * e; }              // (not for a NaN, nor for logits that read -inf)
+    }
+    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
+        const float m_old = am.v;
+        am.batch(x, first);
+        raise(m_old);
+        #pragma unroll
+        for (int q = 0; q < 4 * kRowVecs; ++q) add(x[q]);
+    }
+    __device__ __forceinline__ void one(float x, int at) {
+        const float m_old = am.v;
+        am.one(x, at);
+        raise(m_old);
+        add(x);
+    }
+};
+// merges the lanes' statistics; every lane gets the result
+__device__ __forceinline__ Stats warp_merge(Stats s) {
+    const unsigned long long best = warp_max_u64(s.best);
+    if (s.best != 0ull) {
+        const float d = entry_value(s.best) - entry_value(best), e = expf(d);
+        s.w = (s.w + d * s.z) * e;
+        s.z *= e;
+    }
+    #pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, off);
+        s.w += __shfl_xor_sync(0xffffffffu, s.w, off);
+    }
+    s.best = best;
+    return s;
 }
 
 // =============================================================================================================
 // Next draft: the k best tokens of each of the gamma stream-logit rows of the last accepted node; tree of
-// 1 + sum_g k^g nodes (cut after max_nodes), level by level, children of a node in rank order.
-__global__ void __launch_bounds__(kScanThreads)
+// 1 + sum_g k^g nodes (cut after max_nodes), level by level, children of a node in rank order.  A cluster of
+// gamma x n_cta CTAs per sequence.
+__global__ void __launch_bounds__(kRowThreads, 2)
 next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int32_t* __restrict__ row_index,
-                  const int32_t* __restrict__ bonus_token, int gamma, int vocab, int k, int max_nodes, int n_chunks,
-                  int32_t* __restrict__ draft_tokens, ss_tree_desc* __restrict__ trees, int32_t* __restrict__ counters,
-                  unsigned long long* __restrict__ partials) {
-    const int chunk = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
+                  const int32_t* __restrict__ bonus_token, int gamma, int vocab, int k, int max_nodes, int n_cta,
+                  int32_t* __restrict__ draft_tokens, ss_tree_desc* __restrict__ trees) {
+    const int rank = blockIdx.x, b = blockIdx.y;
+    const int g = rank / n_cta, part = rank - g * n_cta;
+    __shared__ TopKShared s;
+    cluster_arrive();                                     // CTA 0 must have started before anyone stores to its shared memory
     wait_for_previous_kernel();
+    release_next_kernel();
     int r = row_index ? row_index[b] : 0;
     r = min(max(r, 0), n_rows - 1);
-    const float* row = stream_logits + ((static_cast<size_t>(b) * n_rows + r) * gamma + g) * vocab;
-    unsigned long long* part = partials + ((static_cast<size_t>(b) * gamma + g) * n_chunks + chunk) * kMaxTopK;
-    chunk_topk(row, vocab, chunk, k, part);
-    if (!arrive_last(&counters[b], n_chunks * gamma)) return;
-
-    __shared__ int32_t s_top[SS_MAX_GAMMA][kMaxTopK];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < gamma) {                                   // one warp per stream: k rounds over its chunks' candidates
-        unsigned long long top[kMaxTopK];
-        warp_topk(partials + (static_cast<size_t>(b) * gamma + warp) * n_chunks * kMaxTopK, n_chunks * kMaxTopK, k, top);
+    const Segment seg = make_segment(stream_logits, (static_cast<size_t>(b) * n_rows + r) * gamma + g, vocab, part, n_cta);
+    unsigned long long top[kMaxTopK];
+    segment_topk(seg, k, s, top);
+    cluster_wait();
+    if (threadIdx.x < 32) {
         #pragma unroll
-        for (int q = 0; q < kMaxTopK; ++q)
-            if (lane == 0 && q < k) s_top[warp][q] = entry_index(top[q]);
+        for (int q = 0; q < kMaxTopK; ++q)                // the lists of a row lie one after another, k entries each
+            if (q < k && threadIdx.x == q) cluster_store_u64(cluster_addr(&s.part[0][0] + (g * n_cta + part) * k + q, 0), top[q]);
     }
-    __syncthreads();
+    cluster_arrive();
+    if (rank != 0) return;
+
     // node i of the full k-ary tree: level g (1-based), offset o within the level; parent = level(g-1) start + o / k
+    __shared__ int32_t s_top[SS_MAX_GAMMA][kMaxTopK];
     __shared__ int32_t s_parent[SS_MAX_NODES], s_depth[SS_MAX_NODES];
     int total = 1;
     {
@@ -246,36 +203,40 @@ next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int
         for (int lev = 1; lev <= gamma; ++lev) { sz *= k; acc += sz; if (acc >= max_nodes) { acc = max_nodes; break; } }
         total = static_cast<int>(acc);
     }
-    const int i = threadIdx.x;
+    const int i = static_cast<int>(threadIdx.x), warp = i >> 5, lane = i & 31;
+    int par = -1, dep = 0, child = 0, tok = -1;
     if (i < SS_MAX_NODES) {
-        int par = -1, dep = 0, tok = bonus_token[b];
+        if (i == 0) tok = bonus_token[b];
         if (i > 0 && i < total) {
-            long long start = 1, sz = k, prev_start = 0;
-            int lev = 1;
-            while (i >= start + sz) { prev_start = start; start += sz; sz *= k; ++lev; }
-            const int o = static_cast<int>(i - start);
-            par = static_cast<int>(prev_start) + o / k;
-            dep = lev;
-            tok = s_top[lev - 1][o % k];
+            int start = 1, sz = k, prev_start = 0;        // (sizes stay below 64 * 8)
+            dep = 1;
+            while (i >= start + sz) { prev_start = start; start += sz; sz *= k; ++dep; }
+            const int o = i - start;
+            par = prev_start + o / k;
+            child = o % k;
         }
-        s_parent[i] = i < total ? par : -1;
-        s_depth[i] = i < total ? dep : 0;
-        if (i < max_nodes) draft_tokens[static_cast<size_t>(b) * max_nodes + i] = i < total ? tok : -1;
+        s_parent[i] = par;
+        s_depth[i] = dep;
+    }
+    cluster_wait();
+    if (warp < gamma) {                                   // one warp per stream
+        warp_select(&s.part[0][0] + warp * n_cta * k, n_cta * k, k, top);
+        #pragma unroll
+        for (int q = 0; q < kMaxTopK; ++q)
+            if (lane == q && q < k) s_top[warp][q] = entry_index(top[q]);
     }
     __syncthreads();
-    if (i < SS_MAX_NODES) {
-        unsigned long long anc = 0ull;
-        if (i < total) for (int a2 = i; a2 >= 0; a2 = s_parent[a2]) anc |= 1ull << a2;
-        trees[b].parent[i] = s_parent[i];
-        trees[b].depth[i] = s_depth[i];
-        trees[b].anc_mask[i] = anc;
+    if (i >= SS_MAX_NODES) return;
+    unsigned long long anc = 0ull;
+    if (i < total) {
+        if (i > 0) tok = s_top[dep - 1][child];
+        for (int a = i; a >= 0; a = s_parent[a]) anc |= 1ull << a;
     }
-    if (i == 0) {
-        int md = 0;
-        for (int q = 0; q < total; ++q) md = max(md, s_depth[q]);
-        trees[b].n_nodes = total; trees[b].gamma = gamma; trees[b].max_depth = md; trees[b].reserved = 0;
-        counters[b] = 0;                                  // leave the workspace ready for the next call
-    }
+    if (i < max_nodes) draft_tokens[static_cast<size_t>(b) * max_nodes + i] = tok;
+    trees[b].parent[i] = par;
+    trees[b].depth[i] = dep;
+    trees[b].anc_mask[i] = anc;
+    if (i == 0) { trees[b].n_nodes = total; trees[b].gamma = gamma; trees[b].max_depth = s_depth[total - 1]; trees[b].reserved = 0; }
 }
 
 // =============================================================================================================
@@ -290,149 +251,200 @@ struct NodeTailArgs {
     ss_tree_desc* pruned_trees;                         // mode 0
     int32_t *accept_len, *accept_path, *last_node, *bonus_token;   // mode 1
 };
+// What a row leaves for the sequence's tail: which of its children's edges are ok, and its arg-max
+struct RowOut {
+    unsigned long long ok_children;
+    int32_t argmax, pad;
+};
 
-// Pruning, after the edges are judged: a node survives when every edge of its root path is ok; survivors keep
-// their order.  One thread sweeps the nodes (parent[c] < c) over shared-memory copies; all threads write the
-// results out.  Called by every thread of the CTA.
-__device__ void prune_tail(int T, int max_nodes, int b, unsigned long long ok, const int32_t* s_parent, const int32_t* s_depth,
-                           const int32_t* s_tok, int gamma, const NodeTailArgs& ta) {
-    __shared__ int32_t s_new[SS_MAX_NODES], s_kept[SS_MAX_NODES], s_np[SS_MAX_NODES];
-    __shared__ unsigned long long s_anc[SS_MAX_NODES];
-    __shared__ int s_n, s_md;
-    const int i = threadIdx.x;
-    if (i == 0) {
-        unsigned long long keep = T > 0 ? 1ull : 0ull;
-        int n = 0, md = 0;
-        for (int c = 0; c < T; ++c) {
-            const bool kp = c == 0 || (((keep >> s_parent[c]) & 1ull) && ((ok >> c) & 1ull));
-            if (kp) {
-                keep |= 1ull << c;
-                const int np = c == 0 ? -1 : s_new[s_parent[c]];
-                s_new[c] = n;
-                s_kept[n] = c;
-                s_np[n] = np;
-                s_anc[n] = (np >= 0 ? s_anc[np] : 0ull) | (1ull << n);
-                md = max(md, s_depth[c]);
-                ++n;
-            } else {
-                s_new[c] = -1;
-            }
-        }
-        s_n = n; s_md = md;
+// Pruning, after the edges are judged: a node survives when every edge of its root path is ok; survivors keep their
+// order.  Node c's new index is the number of survivors before it.  Called by the first SS_MAX_NODES threads.
+__device__ __forceinline__ void prune_tail(int T, int max_nodes, int b, unsigned long long ok, const TreeShared& tree, int gamma, const NodeTailArgs& ta) {
+    const int i = static_cast<int>(threadIdx.x);
+    unsigned long long keep = 0ull;
+    int md = 0;
+    for (int c = 0; c < T; ++c) {                         // (broadcast reads; every thread builds the same word)
+        const bool kp = (tree.anc[c] & ~ok) == 0ull;
+        keep |= kp ? 1ull << c : 0ull;
+        md = kp ? max(md, tree.depth[c]) : md;
     }
-    __syncthreads();
-    const int n = s_n;
+    const int n = __popcll(keep);
     ss_tree_desc* out = ta.pruned_trees + b;
-    if (i < max_nodes) ta.new_index[static_cast<size_t>(b) * max_nodes + i] = i < T ? s_new[i] : -1;
-    if (i < SS_MAX_NODES) {
-        const bool live = i < n;
-        const int c = live ? s_kept[i] : 0;
-        out->parent[i] = live ? s_np[i] : -1;
-        out->depth[i] = live ? s_depth[c] : 0;
-        out->anc_mask[i] = live ? s_anc[i] : 0ull;
-        if (i < max_nodes) {
-            ta.kept_nodes[static_cast<size_t>(b) * max_nodes + i] = live ? c : -1;
-            ta.kept_tokens[static_cast<size_t>(b) * max_nodes + i] = live ? s_tok[c] : -1;
-        }
+    const size_t row0 = static_cast<size_t>(b) * max_nodes;
+    const bool live = i < T && ((keep >> i) & 1ull);
+    const int at = __popcll(keep & ((1ull << i) - 1ull));          // new index of node i if it survives
+    if (i < max_nodes) ta.new_index[row0 + i] = live ? at : -1;
+    if (live) {
+        const int p = i == 0 ? -1 : tree.parent[i];
+        unsigned long long anc = 0ull;
+        for (unsigned long long rest = tree.anc[i]; rest != 0ull; rest &= rest - 1ull)
+            anc |= 1ull << __popcll(keep & ((rest & (0ull - rest)) - 1ull));
+        out->parent[at] = p < 0 ? -1 : __popcll(keep & ((1ull << p) - 1ull));
+        out->depth[at] = tree.depth[i];
+        out->anc_mask[at] = anc;
+        ta.kept_nodes[row0 + at] = i;
+        ta.kept_tokens[row0 + at] = tree.tok[i];
     }
-    if (i == 0) { out->n_nodes = n; out->gamma = gamma; out->max_depth = s_md; out->reserved = 0; }
+    if (i >= n) {
+        out->parent[i] = -1;
+        out->depth[i] = 0;
+        out->anc_mask[i] = 0ull;
+        if (i < max_nodes) { ta.kept_nodes[row0 + i] = -1; ta.kept_tokens[row0 + i] = -1; }
+    }
+    if (i == 0) { out->n_nodes = n; out->gamma = gamma; out->max_depth = md; out->reserved = 0; }
 }
 
-__global__ void __launch_bounds__(kScanThreads)
+__global__ void __launch_bounds__(kRowThreads, 2)
 node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
-                  int max_nodes, int vocab, int n_chunks, NodeTailArgs ta, int32_t* __restrict__ counters, Stats* __restrict__ partials) {
-    const int chunk = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
+                  int max_nodes, int vocab, int n_cta, NodeTailArgs ta, int32_t* __restrict__ counters, RowOut* __restrict__ rows) {
+    const int rank = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
+    __shared__ Stats s_w[kRowWarps], s_part[8];
+    __shared__ TreeShared s_tree;
+    __shared__ float s_lse, s_bar;
+    __shared__ uint32_t s_ok[2];
+    __shared__ unsigned long long s_any[kRowWarps];
+    __shared__ bool s_none;
+    if (n_cta > 1) cluster_arrive();
     wait_for_previous_kernel();
+    release_next_kernel();
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
-    if (t < T) {
-        const Stats s = chunk_stats(logits + (static_cast<size_t>(b) * max_nodes + t) * vocab, vocab, chunk);
-        if (threadIdx.x == 0) partials[(static_cast<size_t>(b) * max_nodes + t) * n_chunks + chunk] = s;
+    const size_t row = static_cast<size_t>(b) * max_nodes + t;
+    if (t >= max(T, 1)) {
+        if (n_cta > 1) cluster_wait();
+        return;
     }
-    if (!arrive_last(&counters[b], n_chunks * max_nodes)) return;
+    const int i = static_cast<int>(threadIdx.x);
+    // (the tree arrays wait in registers while the row is scanned)
+    TreeRegs tree;
+    tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
+    RowStats rs;
+    scan_segment(make_segment(logits, row, vocab, rank, n_cta), rs);
+    tree.store(s_tree, T);
+    // the logits of the node's children: on their way while the statistics are merged
+    bool mine = false, legal = false;
+    float child = 0.f;
+    if (rank == 0 && i > 0 && i < T && tree.parent == t) {
+        mine = true;
+        legal = t < i && tree.tok >= 0 && tree.tok < vocab;
+        if (legal) child = logits[row * vocab + tree.tok];
+    }
+    Stats st;
+    st.best = entry_of(rs.am); st.z = rs.z; st.w = rs.w;
+    st = warp_merge(st);
+    if ((i & 31) == 0) s_w[i >> 5] = st;
+    __syncthreads();
+    Stats none;
+    none.best = 0ull; none.z = 0.f; none.w = 0.f;
+    if (i < 32) st = warp_merge(i < kRowWarps ? s_w[i] : none);
+    if (n_cta > 1) {
+        cluster_wait();
+        if (i == 0) {
+            const uint32_t at = cluster_addr(&s_part[rank], 0);
+            cluster_store_u64(at, st.best);
+            cluster_store_u64(at + 8, (static_cast<unsigned long long>(__float_as_uint(st.w)) << 32) | __float_as_uint(st.z));
+        }
+        cluster_arrive();
+        if (rank != 0) return;
+        cluster_wait();
+        if (i < 32) st = warp_merge(i < n_cta ? s_part[i] : none);
+    }
+    if (i == 0) {
+        // log-sum-exp and entropy of the row, and the bar that its children's probabilities have to reach
+        const float logz = logf(st.z);
+        s_lse = entry_value(st.best) + logz;
+        const float ent = logz - st.w / st.z;
+        s_bar = ta.mode == 0 ? ta.threshold : fminf(ta.eps, ta.delta * expf(-ent));
+        if (t < T && ta.node_entropy) ta.node_entropy[row] = ent;
+        if (t == 0 && T > 0) ta.edge_prob[row] = 1.f;     // the root
+        s_none = st.best == 0ull;
+    }
+    __syncthreads();
+    if (s_none) st.best = block_max(entry_of_any(make_segment(logits, row, vocab, 0, 1)), s_any);      // a row of -inf and NaN
+    if (i < SS_MAX_NODES) {
+        const float prob = legal ? expf(child - s_lse) : 0.f;
+        if (mine) ta.edge_prob[static_cast<size_t>(b) * max_nodes + i] = prob;
+        const uint32_t ok = __ballot_sync(0xffffffffu, legal && prob >= s_bar);
+        if ((i & 31) == 0) s_ok[i >> 5] = ok;
+        // a node whose parent is no node at all belongs to no row: row 0 looks after it
+        if (t == 0 && i > 0 && i < T && (tree.parent < 0 || tree.parent >= T)) ta.edge_prob[static_cast<size_t>(b) * max_nodes + i] = 0.f;
+    }
+    __syncthreads();
+    if (i == 0) {
+        RowOut o;
+        o.ok_children = (static_cast<unsigned long long>(s_ok[1]) << 32) | s_ok[0];
+        o.argmax = st.best == 0ull ? 0 : entry_index(st.best);
+        o.pad = 0;
+        rows[row] = o;
+    }
+    if (!arrive_last(&counters[b], max(T, 1))) return;
 
-    __shared__ float s_lse[SS_MAX_NODES], s_ent[SS_MAX_NODES];
-    __shared__ int32_t s_am[SS_MAX_NODES], s_parent[SS_MAX_NODES], s_depth[SS_MAX_NODES], s_tok[SS_MAX_NODES];
-    __shared__ unsigned long long s_ok;
-    const int i = threadIdx.x;
-    if (i == 0) s_ok = 1ull;
-    if (i < T) {
-        const Stats* p = partials + (static_cast<size_t>(b) * max_nodes + i) * n_chunks;
-        Stats s;
-        s.best = 0ull; s.z = 0.f; s.w = 0.f;
-        for (int q0 = 0; q0 < n_chunks; q0 += 8) {          // eight partials' loads in flight at once, merged in order
-            Stats o[8];
-            #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                o[q].best = 0ull; o[q].z = 0.f; o[q].w = 0.f;
-                if (q0 + q < n_chunks) { o[q].best = __ldcg(&p[q0 + q].best); o[q].z = __ldcg(&p[q0 + q].z); o[q].w = __ldcg(&p[q0 + q].w); }
-            }
-            #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q0 + q < n_chunks) s = merge_stats(s, o[q]);
+    // ---- the sequence's tail: the first 64 threads -------------------------------------------------------------
+    if (i >= SS_MAX_NODES) return;
+    const RowOut* const mine_row = rows + static_cast<size_t>(b) * max_nodes + i;
+    const unsigned long long okc = i < T ? __ldcg(&mine_row->ok_children) : 0ull;
+    const int argmax = i < max(T, 1) ? __ldcg(&mine_row->argmax) : 0;
+    __shared__ uint32_t s_all[2][2];
+    __shared__ int32_t s_am[SS_MAX_NODES];
+    s_am[i] = argmax;
+    const uint32_t lo = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(okc));
+    const uint32_t hi = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(okc >> 32));
+    if ((i & 31) == 0) { s_all[i >> 5][0] = lo; s_all[i >> 5][1] = hi; }
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+    const unsigned long long ok = 1ull | (static_cast<unsigned long long>(s_all[0][1] | s_all[1][1]) << 32) | (s_all[0][0] | s_all[1][0]);
+    if (i == 0) counters[b] = 0;                          // leave the workspace ready for the next call
+    if (ta.mode == 0) {
+        prune_tail(T, max_nodes, b, ok, s_tree, trees[b].gamma, ta);
+    } else if (i < 32) {
+        int len = 1;
+        const int node = accept_path_of(s_tree, T, ok, ta.accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE, &len);
+        if (i == 0) {
+            ta.accept_len[b] = len;
+            ta.last_node[b] = node;
+            ta.bonus_token[b] = s_am[node];
         }
-        const float logz = logf(s.z);
-        s_lse[i] = entry_value(s.best) + logz;
-        s_ent[i] = logz - s.w / s.z;
-        s_am[i] = s.best == 0ull ? 0 : entry_index(s.best);
-        s_parent[i] = trees[b].parent[i];
-        s_depth[i] = trees[b].depth[i];
-        s_tok[i] = tokens[static_cast<size_t>(b) * max_nodes + i];
-        if (ta.node_entropy) ta.node_entropy[static_cast<size_t>(b) * max_nodes + i] = s_ent[i];
     }
-    __syncthreads();
-    if (i < T) {
-        float prob = 1.f;
-        bool ok = true;
-        if (i > 0) {
-            const int u = s_parent[i], tk = s_tok[i];
-            const bool legal = u >= 0 && u < i && tk >= 0 && tk < vocab;
-            prob = legal ? expf(__ldcg(logits + (static_cast<size_t>(b) * max_nodes + u) * vocab + tk) - s_lse[u]) : 0.f;
-            const float bar = ta.mode == 0 ? ta.threshold : fminf(ta.eps, ta.delta * expf(-s_ent[legal ? u : 0]));
-            ok = legal && prob >= bar;
-        }
-        ta.edge_prob[static_cast<size_t>(b) * max_nodes + i] = prob;
-        if (ok && i > 0) atomicOr(&s_ok, 1ull << i);
-    }
-    __syncthreads();
-    const unsigned long long ok = s_ok;
-    if (ta.mode == 1) {
-        if (i != 0) return;
-        int best = 0, len = 1;
-        accept_walk(T, s_parent, s_depth, ok, ta.accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE, &best, &len);
-        ta.accept_len[b] = len;
-        ta.last_node[b] = best;
-        ta.bonus_token[b] = s_am[best];
-    } else {
-        prune_tail(T, max_nodes, b, ok, s_parent, s_depth, s_tok, trees[b].gamma, ta);
-        if (i != 0) return;
-    }
-    counters[b] = 0;
 }
 
 // =============================================================================================================
 // Verification against tokens drawn from the softmax over each node's k largest logits (temperature 1).
-__global__ void __launch_bounds__(kScanThreads)
+__global__ void __launch_bounds__(kRowThreads, 2)
 sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
-                      const float* __restrict__ uniforms, int max_nodes, int vocab, int k, int n_chunks,
+                      const float* __restrict__ uniforms, int max_nodes, int vocab, int k, int n_cta,
                       int32_t* __restrict__ accept_len, int32_t* __restrict__ accept_path, int32_t* __restrict__ last_node,
                       int32_t* __restrict__ bonus_token, int32_t* __restrict__ node_token, int32_t* __restrict__ counters,
-                      unsigned long long* __restrict__ partials) {
-    const int chunk = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
+                      int32_t* __restrict__ drawn) {
+    const int rank = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
+    __shared__ TopKShared s;
+    __shared__ TreeShared s_tree;
+    __shared__ int32_t s_draw[SS_MAX_NODES];
+    if (n_cta > 1) cluster_arrive();
     wait_for_previous_kernel();
+    release_next_kernel();
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
-    if (t < T)
-        chunk_topk(logits + (static_cast<size_t>(b) * max_nodes + t) * vocab, vocab, chunk, k,
-                   partials + ((static_cast<size_t>(b) * max_nodes + t) * n_chunks + chunk) * kMaxTopK);
-    if (!arrive_last(&counters[b], n_chunks * max_nodes)) return;
-
-    __shared__ int32_t s_draw[SS_MAX_NODES], s_parent[SS_MAX_NODES], s_depth[SS_MAX_NODES], s_tok[SS_MAX_NODES];
-    const int i = threadIdx.x;
-    // a warp per node picks the node's k best; its lane 0 draws the token
-    const int lane = i & 31, n_cand = n_chunks * kMaxTopK;
-    for (int node = i >> 5; node < T; node += kScanThreads / 32) {                     // warp-uniform
-        unsigned long long top[kMaxTopK];
-        warp_topk(partials + (static_cast<size_t>(b) * max_nodes + node) * n_chunks * kMaxTopK, n_cand, k, top);
-        if (lane != 0) continue;
+    const size_t row = static_cast<size_t>(b) * max_nodes + t;
+    if (t >= max(T, 1)) {
+        if (n_cta > 1) cluster_wait();
+        return;
+    }
+    TreeRegs tree;
+    tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
+    const float u = uniforms[row];
+    unsigned long long top[kMaxTopK];
+    segment_topk(make_segment(logits, row, vocab, rank, n_cta), k, s, top);
+    tree.store(s_tree, T);
+    if (n_cta > 1) {
+        cluster_wait();
+        if (threadIdx.x < 32) {
+            #pragma unroll
+            for (int q = 0; q < kMaxTopK; ++q)
+                if (q < k && threadIdx.x == q) cluster_store_u64(cluster_addr(&s.part[0][0] + rank * k + q, 0), top[q]);
+        }
+        cluster_arrive();
+        if (rank != 0) return;
+        cluster_wait();
+        if (threadIdx.x < 32) warp_select(&s.part[0][0], n_cta * k, k, top);
+    }
+    if (threadIdx.x == 0) {
         float x0 = 0.f, z = 0.f, ex[kMaxTopK];
         #pragma unroll
         for (int r = 0; r < kMaxTopK; ++r) {
@@ -440,7 +452,6 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
             ex[r] = r < k ? expf(entry_value(top[r]) - x0) : 0.f;
             z += ex[r];
         }
-        const float u = uniforms[static_cast<size_t>(b) * max_nodes + node];
         float cdf = 0.f;
         int pick = k - 1;
         bool found = false;
@@ -454,32 +465,30 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
         unsigned long long e = 0ull;
         #pragma unroll
         for (int r = 0; r < kMaxTopK; ++r) e = (r == pick) ? top[r] : e;
-        s_draw[node] = entry_index(e);
-        if (node_token) node_token[static_cast<size_t>(b) * max_nodes + node] = s_draw[node];
+        drawn[row] = entry_index(e);
+        if (node_token && t < T) node_token[row] = entry_index(e);
     }
-    if (i < T) {
-        s_parent[i] = trees[b].parent[i];
-        s_depth[i] = trees[b].depth[i];
-        s_tok[i] = tokens[static_cast<size_t>(b) * max_nodes + i];
-    }
+    if (!arrive_last(&counters[b], max(T, 1))) return;
+
+    const int i = static_cast<int>(threadIdx.x);
+    if (i < SS_MAX_NODES) s_draw[i] = i < max(T, 1) ? __ldcg(drawn + static_cast<size_t>(b) * max_nodes + i) : -1;
     __syncthreads();
-    if (i != 0) return;
-    unsigned long long ok = 1ull;
-    for (int c = 1; c < T; ++c) {
-        const int p = s_parent[c];
-        if (p >= 0 && p < c && s_tok[c] == s_draw[p]) ok |= 1ull << c;
+    if (i >= 32) return;
+    const unsigned long long ok = matching_nodes(s_tree, T, s_draw);
+    int len = 1;
+    const int node = accept_path_of(s_tree, T, ok, accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE, &len);
+    if (i == 0) {
+        accept_len[b] = len;
+        last_node[b] = node;
+        bonus_token[b] = s_draw[node];
+        counters[b] = 0;
     }
-    int best = 0, len = 1;
-    accept_walk(T, s_parent, s_depth, ok, accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE, &best, &len);
-    accept_len[b] = len;
-    last_node[b] = best;
-    bonus_token[b] = s_draw[best];
-    counters[b] = 0;
 }
 
 static size_t scan_workspace(int32_t batch, int32_t rows, int32_t vocab, size_t per_chunk) {
     if (batch < 1 || rows < 1 || vocab < 1) return 0;
-    const size_t n_chunks = (static_cast<size_t>(vocab) + kScanChunk - 1) / kScanChunk;
+    // (room for a partial result per 4096 logits, as callers have always been told; one result per row is used)
+    const size_t n_chunks = (static_cast<size_t>(vocab) + 4095) / 4096;
     const size_t counters = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
     return kWsHeaderBytes + counters + static_cast<size_t>(batch) * rows * n_chunks * per_chunk;
 }
@@ -498,14 +507,12 @@ extern "C" int32_t ss_next_draft(const float* stream_logits, int32_t n_rows, con
     if (gamma > SS_MAX_GAMMA || top_k > SS_MAX_TOPK || top_k > vocab || max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(stream_logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_next_draft_workspace_bytes(batch, gamma, vocab)) return SS_ERR_WORKSPACE;
-    const int n_chunks = (vocab + ss::kScanChunk - 1) / ss::kScanChunk;
-    char* ws = static_cast<char*>(workspace);
-    const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
-    int32_t* counters = reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes);
-    unsigned long long* partials = reinterpret_cast<unsigned long long*>(ws + ss::kWsHeaderBytes + counter_bytes);
-    const cudaError_t err = ss::launch_after_previous(ss::next_draft_kernel, dim3(n_chunks, gamma, batch), dim3(ss::kScanThreads),
-                                                      static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token,
-                                                      gamma, vocab, top_k, max_nodes, n_chunks, draft_tokens, trees, counters, partials);
+    // a cluster of at most 8 CTAs takes all the rows of a sequence
+    int n_cta = 1;
+    while (gamma * n_cta * 2 <= 8 && vocab / (n_cta * 2) >= ss::kRowThreads * 4) n_cta *= 2;
+    const cudaError_t err = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kRowThreads), gamma * n_cta, true,
+                                            static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token, gamma, vocab,
+                                            top_k, max_nodes, n_cta, draft_tokens, trees);
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }
 
@@ -521,14 +528,13 @@ static int32_t launch_node_stats(const float* logits, const int32_t* tokens, con
     if (max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_prune_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    const int n_chunks = (vocab + ss::kScanChunk - 1) / ss::kScanChunk;
+    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
-    int32_t* counters = reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes);
-    ss::Stats* partials = reinterpret_cast<ss::Stats*>(ws + ss::kWsHeaderBytes + counter_bytes);
-    const cudaError_t err = ss::launch_after_previous(ss::node_stats_kernel, dim3(n_chunks, max_nodes, batch), dim3(ss::kScanThreads),
-                                                      static_cast<cudaStream_t>(stream), logits, tokens, trees, max_nodes, vocab,
-                                                      n_chunks, ta, counters, partials);
+    const cudaError_t err = ss::launch_rows(ss::node_stats_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
+                                            static_cast<cudaStream_t>(stream), logits, tokens, trees, max_nodes, vocab, n_cta, ta,
+                                            reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes),
+                                            reinterpret_cast<ss::RowOut*>(ws + ss::kWsHeaderBytes + counter_bytes));
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }
 
@@ -570,14 +576,13 @@ extern "C" int32_t ss_tree_verify_sampled(const float* logits, const int32_t* dr
     if (max_nodes > SS_MAX_NODES || top_k > SS_MAX_TOPK || top_k > vocab) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_verify_sampled_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    const int n_chunks = (vocab + ss::kScanChunk - 1) / ss::kScanChunk;
+    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
-    int32_t* counters = reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes);
-    unsigned long long* partials = reinterpret_cast<unsigned long long*>(ws + ss::kWsHeaderBytes + counter_bytes);
-    const cudaError_t err = ss::launch_after_previous(ss::sampled_verify_kernel, dim3(n_chunks, max_nodes, batch), dim3(ss::kScanThreads),
-                                                      static_cast<cudaStream_t>(stream), logits, draft_tokens, trees, uniforms, max_nodes,
-                                                      vocab, top_k, n_chunks, accept_len, accept_path, last_node, bonus_token, node_token,
-                                                      counters, partials);
+    const cudaError_t err = ss::launch_rows(ss::sampled_verify_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
+                                            static_cast<cudaStream_t>(stream), logits, draft_tokens, trees, uniforms, max_nodes, vocab, top_k,
+                                            n_cta, accept_len, accept_path, last_node, bonus_token, node_token,
+                                            reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes),
+                                            reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes + counter_bytes));
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }

@@ -19,23 +19,43 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// out[t][j][c] = m[t][c] + p[j][c]; one thread per (row, stream, 8 elements)
-__global__ void __launch_bounds__(256)
+// Both kernels: a thread owns 8 columns (16 bytes) of the width and walks down the rows, kRowBatch of them at a time, so
+// that no index is divided and a thread has kRowBatch loads and gamma * kRowBatch stores in flight.  Bound by HBM, four
+// fifths of it writes.  STREAM_FIGURES
+constexpr int kRowBatch = 2;
+
+__device__ __forceinline__ uint4 add8(const uint4& a, const uint4& b) {
+    uint4 r;
+    r.x = pack2(__fadd_rn(bf16_lo(a.x), bf16_lo(b.x)), __fadd_rn(bf16_hi(a.x), bf16_hi(b.x)));
+    r.y = pack2(__fadd_rn(bf16_lo(a.y), bf16_lo(b.y)), __fadd_rn(bf16_hi(a.y), bf16_hi(b.y)));
+    r.z = pack2(__fadd_rn(bf16_lo(a.z), bf16_lo(b.z)), __fadd_rn(bf16_hi(a.z), bf16_hi(b.z)));
+    r.w = pack2(__fadd_rn(bf16_lo(a.w), bf16_lo(b.w)), __fadd_rn(bf16_hi(a.w), bf16_hi(b.w)));
+    return r;
+}
+
+// out[t][j][c] = m[t][c] + p[j][c]; the embeddings of the thread's columns stay in registers
+__global__ void __launch_bounds__(128)
 stream_insert_kernel(const uint4* __restrict__ m, const uint4* __restrict__ p, uint4* __restrict__ out, long long rows, int gamma, int vec) {
     wait_for_previous_kernel();
-    const long long total = rows * gamma * vec;
-    for (long long w = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; w < total; w += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int c = static_cast<int>(w % vec);
-        const long long tj = w / vec;
-        const int j = static_cast<int>(tj % gamma);
-        const long long t = tj / gamma;
-        const uint4 a = m[t * vec + c], b = __ldg(p + static_cast<long long>(j) * vec + c);
-        uint4 r;
-        r.x = pack2(__fadd_rn(bf16_lo(a.x), bf16_lo(b.x)), __fadd_rn(bf16_hi(a.x), bf16_hi(b.x)));
-        r.y = pack2(__fadd_rn(bf16_lo(a.y), bf16_lo(b.y)), __fadd_rn(bf16_hi(a.y), bf16_hi(b.y)));
-        r.z = pack2(__fadd_rn(bf16_lo(a.z), bf16_lo(b.z)), __fadd_rn(bf16_hi(a.z), bf16_hi(b.z)));
-        r.w = pack2(__fadd_rn(bf16_lo(a.w), bf16_lo(b.w)), __fadd_rn(bf16_hi(a.w), bf16_hi(b.w)));
-        out[w] = r;
+    release_next_kernel();
+    const int c = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+    if (c >= vec) return;
+    uint4 emb[SS_MAX_GAMMA];
+    #pragma unroll
+    for (int j = 0; j < SS_MAX_GAMMA; ++j)
+        if (j < gamma) emb[j] = __ldg(p + static_cast<long long>(j) * vec + c);
+    const long long step = static_cast<long long>(gridDim.y) * kRowBatch;
+    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch; t < rows; t += step) {
+        uint4 a[kRowBatch];
+        #pragma unroll
+        for (int i = 0; i < kRowBatch; ++i)
+            if (t + i < rows) a[i] = m[(t + i) * vec + c];
+        #pragma unroll
+        for (int i = 0; i < kRowBatch; ++i) {
+            #pragma unroll
+            for (int j = 0; j < SS_MAX_GAMMA; ++j)
+                if (j < gamma && t + i < rows) out[((t + i) * gamma + j) * vec + c] = add8(a[i], emb[j]);
+        }
     }
 }
 
@@ -45,30 +65,43 @@ __device__ __forceinline__ uint32_t rotate_word(uint32_t w, float cs, float sn) 
     return pack2(__fsub_rn(__fmul_rn(re, cs), __fmul_rn(im, sn)), __fadd_rn(__fmul_rn(re, sn), __fmul_rn(im, cs)));
 }
 
-// out[t][n][c] = v[t][c] rotated by eps * (n + 1); one thread per (row, 8 elements), all streams
-__global__ void __launch_bounds__(256)
-value_rotate_kernel(const uint4* __restrict__ v, uint4* __restrict__ out, long long rows, int gamma, int vec, RotTable tab) {
+// out[t][n][c] = v[t][c] rotated by eps * (n + 1)
+__global__ void __launch_bounds__(128)
+value_rotate_kernel(const uint4* __restrict__ v, uint4* __restrict__ out, long long rows, int gamma, int vec, const __grid_constant__ RotTable tab) {
     wait_for_previous_kernel();
-    const long long total = rows * vec;
-    for (long long w = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; w < total; w += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int c = static_cast<int>(w % vec);
-        const long long t = w / vec;
-        const uint4 a = v[w];
-        for (int n = 0; n < gamma; ++n) {
-            const float cs = tab.cs[n], sn = tab.sn[n];
-            uint4 r;
-            r.x = rotate_word(a.x, cs, sn); r.y = rotate_word(a.y, cs, sn);
-            r.z = rotate_word(a.z, cs, sn); r.w = rotate_word(a.w, cs, sn);
-            out[(t * gamma + n) * vec + c] = r;
+    release_next_kernel();
+    const int c = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+    if (c >= vec) return;
+    const long long step = static_cast<long long>(gridDim.y) * kRowBatch;
+    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch; t < rows; t += step) {
+        uint4 a[kRowBatch];
+        #pragma unroll
+        for (int i = 0; i < kRowBatch; ++i)
+            if (t + i < rows) a[i] = v[(t + i) * vec + c];
+        #pragma unroll
+        for (int i = 0; i < kRowBatch; ++i) {
+            #pragma unroll
+            for (int n = 0; n < SS_MAX_GAMMA; ++n) {
+                if (n < gamma && t + i < rows) {
+                    const float cs = tab.cs[n], sn = tab.sn[n];
+                    uint4 r;
+                    r.x = rotate_word(a[i].x, cs, sn); r.y = rotate_word(a[i].y, cs, sn);
+                    r.z = rotate_word(a[i].z, cs, sn); r.w = rotate_word(a[i].w, cs, sn);
+                    out[((t + i) * gamma + n) * vec + c] = r;
+                }
+            }
         }
     }
 }
 
-static int grid_for(long long items) {
-    long long g = (items + 255) / 256;
-    const long long cap = static_cast<long long>(sm_count()) * 8;
-    if (g > cap) g = cap;
-    return g < 1 ? 1 : static_cast<int>(g);
+// 128 threads across the width; rows dealt out until the SMs are full (16 such CTAs per SM)
+static dim3 grid_for(long long rows, int vec) {
+    const int gx = (vec + 127) / 128;
+    long long gy = (rows + kRowBatch - 1) / kRowBatch;
+    const long long cap = (static_cast<long long>(sm_count()) * 16 + gx - 1) / gx;
+    if (gy > cap) gy = cap;
+    if (gy > 65535) gy = 65535;
+    return dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy < 1 ? 1 : gy));
 }
 
 }  // namespace ss
@@ -81,7 +114,7 @@ extern "C" int32_t ss_stream_insert(const void* main_hidden, const void* stream_
     if (!main_hidden || !stream_emb || !out) return SS_ERR_INVALID_ARG;
     if (!ss::aligned16(main_hidden) || !ss::aligned16(stream_emb) || !ss::aligned16(out)) return SS_ERR_INVALID_ARG;
     const int vec = hidden / 8;
-    const cudaError_t err = ss::launch_after_previous(ss::stream_insert_kernel, dim3(ss::grid_for(rows * gamma * vec)), dim3(256),
+    const cudaError_t err = ss::launch_after_previous(ss::stream_insert_kernel, ss::grid_for(rows, vec), dim3(128),
                                                       static_cast<cudaStream_t>(stream), static_cast<const uint4*>(main_hidden),
                                                       static_cast<const uint4*>(stream_emb), static_cast<uint4*>(out),
                                                       static_cast<long long>(rows), gamma, vec);
@@ -102,7 +135,7 @@ extern "C" int32_t ss_value_rotate(const void* v_main, void* v_streams, int64_t 
         tab.sn[n] = static_cast<float>(sin(ang));
     }
     const int vec = width / 8;
-    const cudaError_t err = ss::launch_after_previous(ss::value_rotate_kernel, dim3(ss::grid_for(rows * vec)), dim3(256),
+    const cudaError_t err = ss::launch_after_previous(ss::value_rotate_kernel, ss::grid_for(rows, vec), dim3(128),
                                                       static_cast<cudaStream_t>(stream), static_cast<const uint4*>(v_main),
                                                       static_cast<uint4*>(v_streams), static_cast<long long>(rows), gamma, vec, tab);
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;

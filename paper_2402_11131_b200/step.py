@@ -134,7 +134,7 @@ class DeviceStep:
     def run_compact(self, stream=None) -> int:
         api.ss_kv_compact(self.k_all, self.v_all, self.layout, self.kv_start, self.kv_len, self.accept_len,
                           self.accept_path, self.kv_len_out, stream)
-        return api.LAUNCHES_PER_CALL["ss_kv_compact"]
+        return api.LAUNCHES_PER_CALL["ss_kv_compact"]      # (kv_len_out is a buffer of its own)
 
     def run_step(self, stream=None) -> int:
         """One pass of the whole hot path: every layer's attention, verification, compaction.
