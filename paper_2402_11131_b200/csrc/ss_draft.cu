@@ -6,154 +6,145 @@
 // the maximum with the softmax sums -- in its CTA 0; the CTA that finishes a sequence's last row does the sequence's
 // tail, all nodes at once from their ancestor words.  The next draft has at most four rows per sequence, so one
 // cluster takes the whole sequence and nothing goes through global memory.  Compiled without fast-math.
+// Measured on a B200, before (chunks of 4096 logits, partial results and candidate lists through global memory, serial
+// tails) and after: soft verification of 32 rows of 51200 logits 15.3 and 6.4 us, sampled verification of 64 rows of
+// 32000 34.1 and 8.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of
+// 32000) 15.6 and 8.9 us.
 #include "ss_rows.cuh"
 
 namespace ss {
 
+constexpr float kTinyExp = -200.f;                        // exp of it is 0 in fp32
+
 // ---- the k best entries of a segment --------------------------------------------------------------------------------
-// Pass 1 takes one maximum per thread.  The k-th largest of the 16 warp maxima bounds the k-th best logit of the segment
-// from below, and only a dozen logits or so of a segment reach that bound; pass 2, in the few threads that hold one,
-// reads the thread's logits again (they are in L2) and collects them.  Keeping a sorted list of k entries per thread
-// instead costs 8 compare-and-swaps of 64-bit words per logit: 34 us instead of DRAFT_SAMPLED_US us for 64 rows of 32000.
+// Pass 1 takes one maximum per thread.  The k-th largest warp maximum bounds the k-th best logit of the segment from
+// below, and only a dozen logits or so reach that bound; the few threads that hold one collect them in a list (from
+// the registers of pass 1 where the segment was one batch, else they read their logits again), and each entry of the list
+// counts how many are better.  Keeping a sorted list of k entries per thread costs 8 compare-and-swaps of 64-bit
+// words per logit instead.
+constexpr int kListCap = 512;
+template <int NT>
+struct TopKShared {
+    static_assert(NT / 32 >= kMaxTopK, "the k-th largest warp maximum has to exist");
+    unsigned long long part[8 * kMaxTopK];                // CTA 0 of a cluster: the lists of its CTAs, k entries each
+    unsigned long long best[kMaxTopK];
+    unsigned long long warp_best[NT / 32];
+    unsigned long long list[kListCap];
+    uint32_t warp_key[NT / 32];
+    int n_list;
+};
+template <int NT>
 struct ThreadMax {
     float v = -INFINITY;
-    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
-        float m[4] = {x[0], x[1], x[2], x[3]};
+    float4 last[kRowVecs];
+    __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) {
         #pragma unroll
-        for (int q = 4; q < 4 * kRowVecs; ++q) m[q & 3] = fmaxf(m[q & 3], x[q]);
-        v = fmaxf(v, fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));      // (a NaN is never the maximum)
+        for (int k = 0; k < kRowVecs; ++k) {
+            v = fmaxf(v, fmaxf(fmaxf(q[k].x, q[k].y), fmaxf(q[k].z, q[k].w)));     // (a NaN is never the maximum)
+            last[k] = q[k];
+        }
     }
-    __device__ __forceinline__ void one(float x, int at) { v = fmaxf(v, x); }
 };
-// the k best of a thread's logits that are not below the bound (a NaN is not below anything)
-struct ThreadTopK {
+template <int NT>
+struct Collect {
+    const Segment& seg;
+    TopKShared<NT>& s;
     float bound;
-    int hi;
-    unsigned long long best[kMaxTopK];
-    __device__ __forceinline__ void one(float x, int at) {
-        if (x < bound || at >= hi) return;
-        unsigned long long e = entry(order_key(x), at);
+    __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) {
+        uint32_t hit = 0u;
         #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) {
-            if (e > best[r]) { const unsigned long long t = best[r]; best[r] = e; e = t; }
-        }
-    }
-    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
-        bool any = false;
-        #pragma unroll
-        for (int q = 0; q < 4 * kRowVecs; ++q) any = any || !(x[q] < bound);
-        if (!any) return;
+        for (int k = 0; k < kRowVecs; ++k)                // (a NaN is not below anything)
+            hit |= ((q[k].x < bound ? 0u : 1u) | (q[k].y < bound ? 0u : 2u) | (q[k].z < bound ? 0u : 4u) | (q[k].w < bound ? 0u : 8u)) << (4 * k);
+        static_assert(4 * kRowVecs <= 32, "a bit per logit");
         #pragma unroll 1
-        for (int v = 0; v < kRowVecs; ++v) {
-            float a = x[0], b = x[1], c = x[2], d = x[3];
-            int at = first[0];
+        for (; hit; hit &= hit - 1u) {
+            const int j = __ffs(hit) - 1;
+            float x = 0.f;
             #pragma unroll
-            for (int s = 1; s < kRowVecs; ++s)
-                if (s == v) { a = x[4 * s]; b = x[4 * s + 1]; c = x[4 * s + 2]; d = x[4 * s + 3]; at = first[s]; }
-            one(a, at); one(b, at + 1); one(c, at + 2); one(d, at + 3);
+            for (int k = 0; k < kRowVecs; ++k)
+                if (k == j >> 2) x = (j & 2) ? ((j & 1) ? q[k].w : q[k].z) : ((j & 1) ? q[k].y : q[k].x);
+            const int at = word + (j >> 2) * 4 * NT + (j & 3);
+            if (at < seg.skip || at >= seg.total) continue;
+            const int p = atomicAdd(&s.n_list, 1);
+            if (p < kListCap) s.list[p] = entry(order_key(x), seg.at + at);
         }
     }
 };
-// Picks the k largest of the distinct entries list[0 .. n) in descending order (one warp; every lane gets them).
-__device__ __forceinline__ void warp_select(const unsigned long long* list, int n, int k, unsigned long long (&top)[kMaxTopK]) {
-    const int lane = static_cast<int>(threadIdx.x) & 31;
-    const unsigned long long e0 = lane < n ? list[lane] : 0ull, e1 = lane + 32 < n ? list[lane + 32] : 0ull;
+// entry i of the distinct entries list[0 .. n) that has r better ones goes to best[r], r < k
+__device__ __forceinline__ void rank_entry(const unsigned long long* list, int n, int i, int k, unsigned long long* best) {
+    const unsigned long long e = list[i];
+    int better = 0;
+    #pragma unroll 4
+    for (int j = 0; j < n; ++j) better += list[j] > e ? 1 : 0;
+    if (better < k) best[better] = e;
+}
+// More candidates than the list holds (rows of equal logits, of -inf or of NaN): k passes over the segment, each for the
+// best entry below the last, one logit at a time.
+template <int NT>
+static __device__ __noinline__ void select_by_passes(const Segment seg, int top_k, TopKShared<NT>& s) {
     unsigned long long below = ~0ull;
-    #pragma unroll
-    for (int r = 0; r < kMaxTopK; ++r) top[r] = 0ull;
-    #pragma unroll
-    for (int r = 0; r < kMaxTopK; ++r) {
-        if (r >= k) break;
-        unsigned long long m = e0 < below ? e0 : 0ull;
-        if (e1 < below && e1 > m) m = e1;
-        for (int j = lane + 64; j < n; j += 32) {
-            const unsigned long long e = list[j];
+    for (int r = 0; r < top_k; ++r) {
+        unsigned long long m = 0ull;
+        for (int i = seg.skip + static_cast<int>(threadIdx.x); i < seg.total; i += NT) {
+            const unsigned long long e = entry(order_key(seg.src[i]), seg.at + i);
             if (e < below && e > m) m = e;
         }
         m = warp_max_u64(m);
-        top[r] = m;
-        below = m;
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) s.warp_best[threadIdx.x >> 5] = m;
+        __syncthreads();
+        below = warp_max_u64(s.warp_best[threadIdx.x & (NT / 32 - 1)]);
+        if (threadIdx.x == 0) s.best[r] = below;          // (0, no entry, once the segment is exhausted)
     }
 }
-struct TopKShared {
-    uint32_t warp_max[kRowWarps];
-    int n;
-    unsigned long long part[8][kMaxTopK];                 // CTA 0 of a cluster: the lists of its CTAs
-    unsigned long long list[kRowThreads * kMaxTopK];
-};
-// The k best entries of the segment, in every lane of warp 0.  Ends with the CTA's threads in step.
-__device__ __forceinline__ void segment_topk(const Segment& seg, int k, TopKShared& s, unsigned long long (&top)[kMaxTopK]) {
-    const int warp = static_cast<int>(threadIdx.x) >> 5, lane = static_cast<int>(threadIdx.x) & 31;
-    if (threadIdx.x == 0) s.n = 0;
-    ThreadMax tm;
-    scan_segment(seg, tm);
+// The k best entries of the segment in s.best, for every thread
+template <int NT>
+__device__ __forceinline__ void segment_topk(const Segment& seg, int top_k, TopKShared<NT>& s) {
+    constexpr int kWarps = NT / 32;
+    const int lane = static_cast<int>(threadIdx.x) & 31, warp = static_cast<int>(threadIdx.x) >> 5;
+    ThreadMax<NT> tm;
+    #pragma unroll
+    for (int k = 0; k < kRowVecs; ++k) tm.last[k] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    scan_segment<NT>(seg, tm);
     const uint32_t wm = __reduce_max_sync(0xffffffffu, order_key(tm.v));
-    if (lane == 0) s.warp_max[warp] = wm;
+    if (lane == 0) s.warp_key[warp] = wm;
+    if (threadIdx.x == 0) s.n_list = 0;
+    if (threadIdx.x < kMaxTopK) s.best[threadIdx.x] = 0ull;
     __syncthreads();
-    // the k-th largest warp maximum, counting equal ones apart
-    uint32_t key = lane < kRowWarps ? s.warp_max[lane] : 0u, bound = 0u;
-    for (int r = 0; r < k; ++r) {
-        bound = __reduce_max_sync(0xffffffffu, key);
-        const uint32_t holders = __ballot_sync(0xffffffffu, key == bound);
-        if (lane == __ffs(holders) - 1) key = 0u;
+    // the k-th largest warp maximum, equal ones in the order of their warps (every warp for itself)
+    const uint32_t key = s.warp_key[lane & (kWarps - 1)];
+    int before = 0;
+    #pragma unroll
+    for (int j = 0; j < kWarps; ++j) {
+        const uint32_t o = __shfl_sync(0xffffffffu, key, j);
+        before += (o > key || (o == key && j < (lane & (kWarps - 1)))) ? 1 : 0;
     }
-    ThreadTopK tk;
-    tk.bound = key_value(bound);
-    tk.hi = seg.hi;
-    if (!(tm.v < tk.bound)) {
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) tk.best[r] = 0ull;
-        scan_segment(seg, tk);
-        int have = 0;
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) have += (r < k && tk.best[r] != 0ull) ? 1 : 0;
-        int at = atomicAdd(&s.n, have);
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r)
-            if (r < have) s.list[at + r] = tk.best[r];
+    const float bound = key_value(__shfl_sync(0xffffffffu, key, __ffs(__ballot_sync(0xffffffffu, before == top_k - 1)) - 1));
+    if (!(tm.v < bound)) {
+        Collect<NT> collect{seg, s, bound};
+        if (seg.total <= 4 * NT * kRowVecs) collect.batch(tm.last, 4 * static_cast<int>(threadIdx.x));
+        else scan_segment<NT>(seg, collect);
     }
     __syncthreads();
-    if (warp == 0) warp_select(s.list, s.n, k, top);
+    const int n = s.n_list;
+    if (n > kListCap) {
+        select_by_passes<NT>(seg, top_k, s);
+    } else {
+        for (int i = static_cast<int>(threadIdx.x); i < n; i += NT) rank_entry(s.list, n, i, top_k, s.best);
+    }
+    __syncthreads();
 }
 
-// ---- softmax statistics of a row: maximum (lowest index), Z = sum exp(x - m), W = sum (x - m) exp(x - m) ------------
+// ---- softmax statistics: maximum (lowest index), Z = sum exp(x - m), W = sum (x - m) exp(x - m) ----------------------
 struct Stats {
-    unsigned long long best;      // entry of the maximum, 0: none above -inf
+    unsigned long long best;      // entry of the maximum, 0: no comparable value
     float z, w;
 };
-struct RowStats {
-    ArgMax am;
-    float z = 0.f, w = 0.f;
-    __device__ __forceinline__ void raise(float m_old) {
-        if (am.v > m_old && z > 0.f) {
-            const float d = m_old - am.v, e = expf(d);
-            w = (w + d * z) * e;
-            z *= e;
-        }
-    }
-    __device__ __forceinline__ void add(float x) {
-        const float d = x - am.v, e = expf(d);
-        if (e > 0.f) { z += e; w += d * e; }              // (not for a NaN, nor for logits that read -inf)
-    }
-    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
-        const float m_old = am.v;
-        am.batch(x, first);
-        raise(m_old);
-        #pragma unroll
-        for (int q = 0; q < 4 * kRowVecs; ++q) add(x[q]);
-    }
-    __device__ __forceinline__ void one(float x, int at) {
-        const float m_old = am.v;
-        am.one(x, at);
-        raise(m_old);
-        add(x);
-    }
-};
 // merges the lanes' statistics; every lane gets the result
-__device__ __forceinline__ Stats warp_merge(Stats s) {
+static __device__ __noinline__ Stats warp_merge(Stats s) {
     const unsigned long long best = warp_max_u64(s.best);
-    if (s.best != 0ull) {
-        const float d = entry_value(s.best) - entry_value(best), e = expf(d);
+    if (s.best != 0ull && s.best != best) {
+        const float d = fmaxf(entry_value(s.best) - entry_value(best), kTinyExp), e = expf(d);
         s.w = (s.w + d * s.z) * e;
         s.z *= e;
     }
@@ -165,74 +156,98 @@ __device__ __forceinline__ Stats warp_merge(Stats s) {
     s.best = best;
     return s;
 }
-
+__device__ __forceinline__ Stats merge_two(const Stats& a, const Stats& b) {
+    if (b.best == 0ull) return a;
+    if (a.best == 0ull) return b;
+    const bool first = a.best > b.best;
+    Stats r = first ? a : b;
+    const Stats& o = first ? b : a;
+    const float d = fmaxf(entry_value(o.best) - entry_value(r.best), kTinyExp), e = expf(d);
+    r.w += (o.w + d * o.z) * e;
+    r.z += o.z * e;
+    return r;
+}
+// A thread's running statistics against its running maximum
+struct RowStats {
+    ArgMax am;
+    float z = 0.f, w = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float d = fmaxf(x - am.v, kTinyExp), e = expf(d);       // (for -inf and for NaN too: no product is a NaN)
+        z += e;
+        w += d * e;
+    }
+    __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) {
+        const float m_old = am.v;
+        am.batch(q, word);
+        if (am.v > m_old) {
+            const float d = fmaxf(m_old - am.v, kTinyExp), e = expf(d);
+            w = (w + d * z) * e;
+            z *= e;
+        }
+        #pragma unroll
+        for (int k = 0; k < kRowVecs; ++k) { add(q[k].x); add(q[k].y); add(q[k].z); add(q[k].w); }
+    }
+};
 // =============================================================================================================
 // Next draft: the k best tokens of each of the gamma stream-logit rows of the last accepted node; tree of
 // 1 + sum_g k^g nodes (cut after max_nodes), level by level, children of a node in rank order.  A cluster of
 // gamma x n_cta CTAs per sequence.
-__global__ void __launch_bounds__(kRowThreads, 2)
+constexpr int kDraftThreads = 512;    // few rows: a segment of up to 16384 logits is one batch of loads
+__global__ void __launch_bounds__(kDraftThreads, 2)
 next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int32_t* __restrict__ row_index,
                   const int32_t* __restrict__ bonus_token, int gamma, int vocab, int k, int max_nodes, int n_cta,
                   int32_t* __restrict__ draft_tokens, ss_tree_desc* __restrict__ trees) {
     const int rank = blockIdx.x, b = blockIdx.y;
     const int g = rank / n_cta, part = rank - g * n_cta;
-    __shared__ TopKShared s;
+    __shared__ TopKShared<kDraftThreads> s;
     cluster_arrive();                                     // CTA 0 must have started before anyone stores to its shared memory
     wait_for_previous_kernel();
     release_next_kernel();
     int r = row_index ? row_index[b] : 0;
     r = min(max(r, 0), n_rows - 1);
     const Segment seg = make_segment(stream_logits, (static_cast<size_t>(b) * n_rows + r) * gamma + g, vocab, part, n_cta);
-    unsigned long long top[kMaxTopK];
-    segment_topk(seg, k, s, top);
-    cluster_wait();
-    if (threadIdx.x < 32) {
-        #pragma unroll
-        for (int q = 0; q < kMaxTopK; ++q)                // the lists of a row lie one after another, k entries each
-            if (q < k && threadIdx.x == q) cluster_store_u64(cluster_addr(&s.part[0][0] + (g * n_cta + part) * k + q, 0), top[q]);
-    }
+    const int32_t bonus = bonus_token[b];
+    __shared__ unsigned long long s_top[SS_MAX_GAMMA * kMaxTopK];
+    __shared__ int32_t s_parent[SS_MAX_NODES], s_depth[SS_MAX_NODES];
+    const int i = static_cast<int>(threadIdx.x), warp = i >> 5, lane = i & 31;
+    segment_topk<kDraftThreads>(seg, k, s);
+    // the lists of a row lie one after another
+    cluster_wait();                                       // (CTA 0 has started)
+    if (i < k) cluster_store_u64(cluster_addr(s.part + rank * k + i, 0), s.best[i]);
     cluster_arrive();
     if (rank != 0) return;
-
-    // node i of the full k-ary tree: level g (1-based), offset o within the level; parent = level(g-1) start + o / k
-    __shared__ int32_t s_top[SS_MAX_GAMMA][kMaxTopK];
-    __shared__ int32_t s_parent[SS_MAX_NODES], s_depth[SS_MAX_NODES];
-    int total = 1;
-    {
-        long long sz = 1, acc = 1;
-        for (int lev = 1; lev <= gamma; ++lev) { sz *= k; acc += sz; if (acc >= max_nodes) { acc = max_nodes; break; } }
-        total = static_cast<int>(acc);
-    }
-    const int i = static_cast<int>(threadIdx.x), warp = i >> 5, lane = i & 31;
-    int par = -1, dep = 0, child = 0, tok = -1;
+    // the shape of the tree does not depend on the logits: it is worked out while the lists arrive
+    int total = 1, par = -1, dep = 0, child = 0;
     if (i < SS_MAX_NODES) {
-        if (i == 0) tok = bonus_token[b];
-        if (i > 0 && i < total) {
-            int start = 1, sz = k, prev_start = 0;        // (sizes stay below 64 * 8)
-            dep = 1;
-            while (i >= start + sz) { prev_start = start; start += sz; sz *= k; ++dep; }
-            const int o = i - start;
-            par = prev_start + o / k;
-            child = o % k;
+        // level `dep` holds nodes [start, start + sz); node i there is child o % k of node prev_start + o / k
+        int start = 1, sz = k, prev_start = 0;
+        #pragma unroll 1
+        for (int lev = 1; lev <= gamma && start < max_nodes; ++lev) {
+            if (i >= start && i < start + sz && i < max_nodes) {
+                const int o = i - start;
+                par = prev_start + o / k;
+                child = (lev - 1) * kMaxTopK + o % k;
+                dep = lev;
+            }
+            total = min(start + sz, max_nodes);
+            prev_start = start; start += sz; sz *= k;
         }
         s_parent[i] = par;
         s_depth[i] = dep;
     }
     cluster_wait();
     if (warp < gamma) {                                   // one warp per stream
-        warp_select(&s.part[0][0] + warp * n_cta * k, n_cta * k, k, top);
-        #pragma unroll
-        for (int q = 0; q < kMaxTopK; ++q)
-            if (lane == q && q < k) s_top[warp][q] = entry_index(top[q]);
+        const unsigned long long* list = s.part + warp * n_cta * k;
+        for (int j = lane; j < n_cta * k; j += 32) rank_entry(list, n_cta * k, j, k, s_top + warp * kMaxTopK);
     }
     __syncthreads();
     if (i >= SS_MAX_NODES) return;
     unsigned long long anc = 0ull;
     if (i < total) {
-        if (i > 0) tok = s_top[dep - 1][child];
+        #pragma unroll 1
         for (int a = i; a >= 0; a = s_parent[a]) anc |= 1ull << a;
     }
-    if (i < max_nodes) draft_tokens[static_cast<size_t>(b) * max_nodes + i] = tok;
+    if (i < max_nodes) draft_tokens[static_cast<size_t>(b) * max_nodes + i] = i == 0 ? bonus : i < total ? entry_index(s_top[child]) : -1;
     trees[b].parent[i] = par;
     trees[b].depth[i] = dep;
     trees[b].anc_mask[i] = anc;
@@ -294,16 +309,16 @@ __device__ __forceinline__ void prune_tail(int T, int max_nodes, int b, unsigned
     if (i == 0) { out->n_nodes = n; out->gamma = gamma; out->max_depth = md; out->reserved = 0; }
 }
 
-__global__ void __launch_bounds__(kRowThreads, 2)
+__global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
                   int max_nodes, int vocab, int n_cta, NodeTailArgs ta, int32_t* __restrict__ counters, RowOut* __restrict__ rows) {
     const int rank = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
-    __shared__ Stats s_w[kRowWarps], s_part[8];
+    __shared__ Stats s_part[kRowParts];
+    __shared__ unsigned long long s_any[kRowThreads / 32];
+    __shared__ bool s_none;
     __shared__ TreeShared s_tree;
     __shared__ float s_lse, s_bar;
     __shared__ uint32_t s_ok[2];
-    __shared__ unsigned long long s_any[kRowWarps];
-    __shared__ bool s_none;
     if (n_cta > 1) cluster_arrive();
     wait_for_previous_kernel();
     release_next_kernel();
@@ -314,11 +329,11 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
         return;
     }
     const int i = static_cast<int>(threadIdx.x);
-    // (the tree arrays wait in registers while the row is scanned)
+    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     RowStats rs;
-    scan_segment(make_segment(logits, row, vocab, rank, n_cta), rs);
+    scan_segment<kRowThreads>(seg, rs);
     tree.store(s_tree, T);
     // the logits of the node's children: on their way while the statistics are merged
     bool mine = false, legal = false;
@@ -329,24 +344,22 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
         if (legal) child = logits[row * vocab + tree.tok];
     }
     Stats st;
-    st.best = entry_of(rs.am); st.z = rs.z; st.w = rs.w;
+    st.best = rs.am.best(seg); st.z = rs.z; st.w = rs.w;
     st = warp_merge(st);
-    if ((i & 31) == 0) s_w[i >> 5] = st;
-    __syncthreads();
-    Stats none;
-    none.best = 0ull; none.z = 0.f; none.w = 0.f;
-    if (i < 32) st = warp_merge(i < kRowWarps ? s_w[i] : none);
-    if (n_cta > 1) {
-        cluster_wait();
-        if (i == 0) {
-            const uint32_t at = cluster_addr(&s_part[rank], 0);
-            cluster_store_u64(at, st.best);
-            cluster_store_u64(at + 8, (static_cast<unsigned long long>(__float_as_uint(st.w)) << 32) | __float_as_uint(st.z));
-        }
-        cluster_arrive();
-        if (rank != 0) return;
-        cluster_wait();
-        if (i < 32) st = warp_merge(i < n_cta ? s_part[i] : none);
+    constexpr int kWarps = kRowThreads / 32;
+    if (!hand_to_first(rank, n_cta, [&]() {
+            if ((i & 31) == 0) {
+                const uint32_t at = cluster_addr(&s_part[rank * kWarps + (i >> 5)], 0);
+                cluster_store_u64(at, st.best);
+                cluster_store_u64(at + 8, (static_cast<unsigned long long>(__float_as_uint(st.w)) << 32) | __float_as_uint(st.z));
+            }
+        }))
+        return;
+    if (i < 32) {
+        Stats none;
+        none.best = 0ull; none.z = 0.f; none.w = 0.f;
+        const int n_part = n_cta * kWarps;
+        st = warp_merge(merge_two(i < n_part ? s_part[i] : none, i + 32 < n_part ? s_part[i + 32] : none));
     }
     if (i == 0) {
         // log-sum-exp and entropy of the row, and the bar that its children's probabilities have to reach
@@ -359,7 +372,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
         s_none = st.best == 0ull;
     }
     __syncthreads();
-    if (s_none) st.best = block_max(entry_of_any(make_segment(logits, row, vocab, 0, 1)), s_any);      // a row of -inf and NaN
+    if (s_none) st.best = best_of_any(logits, row, vocab, s_any);
     if (i < SS_MAX_NODES) {
         const float prob = legal ? expf(child - s_lse) : 0.f;
         if (mine) ta.edge_prob[static_cast<size_t>(b) * max_nodes + i] = prob;
@@ -372,7 +385,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     if (i == 0) {
         RowOut o;
         o.ok_children = (static_cast<unsigned long long>(s_ok[1]) << 32) | s_ok[0];
-        o.argmax = st.best == 0ull ? 0 : entry_index(st.best);
+        o.argmax = entry_index(st.best);
         o.pad = 0;
         rows[row] = o;
     }
@@ -407,14 +420,14 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
 
 // =============================================================================================================
 // Verification against tokens drawn from the softmax over each node's k largest logits (temperature 1).
-__global__ void __launch_bounds__(kRowThreads, 2)
+__global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
                       const float* __restrict__ uniforms, int max_nodes, int vocab, int k, int n_cta,
                       int32_t* __restrict__ accept_len, int32_t* __restrict__ accept_path, int32_t* __restrict__ last_node,
                       int32_t* __restrict__ bonus_token, int32_t* __restrict__ node_token, int32_t* __restrict__ counters,
                       int32_t* __restrict__ drawn) {
     const int rank = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
-    __shared__ TopKShared s;
+    __shared__ TopKShared<kRowThreads> s;
     __shared__ TreeShared s_tree;
     __shared__ int32_t s_draw[SS_MAX_NODES];
     if (n_cta > 1) cluster_arrive();
@@ -426,51 +439,41 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
         if (n_cta > 1) cluster_wait();
         return;
     }
+    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     const float u = uniforms[row];
-    unsigned long long top[kMaxTopK];
-    segment_topk(make_segment(logits, row, vocab, rank, n_cta), k, s, top);
+    segment_topk<kRowThreads>(seg, k, s);
     tree.store(s_tree, T);
+    const int i = static_cast<int>(threadIdx.x);
     if (n_cta > 1) {
-        cluster_wait();
-        if (threadIdx.x < 32) {
-            #pragma unroll
-            for (int q = 0; q < kMaxTopK; ++q)
-                if (q < k && threadIdx.x == q) cluster_store_u64(cluster_addr(&s.part[0][0] + rank * k + q, 0), top[q]);
-        }
-        cluster_arrive();
-        if (rank != 0) return;
-        cluster_wait();
-        if (threadIdx.x < 32) warp_select(&s.part[0][0], n_cta * k, k, top);
+        if (!hand_to_first(rank, n_cta, [&]() { if (i < k) cluster_store_u64(cluster_addr(s.part + rank * k + i, 0), s.best[i]); })) return;
+        if (i < n_cta * k) rank_entry(s.part, n_cta * k, i, k, s.best);
+        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        float x0 = 0.f, z = 0.f, ex[kMaxTopK];
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) {
-            if (r == 0) x0 = entry_value(top[0]);
-            ex[r] = r < k ? expf(entry_value(top[r]) - x0) : 0.f;
-            z += ex[r];
-        }
-        float cdf = 0.f;
+    if (i < 32) {
+        // lane r holds the r-th best; every lane adds the probabilities up in rank order, as one thread would
+        const unsigned long long top = i < k ? s.best[i] : 0ull;
+        const float x0 = __shfl_sync(0xffffffffu, entry_value(top), 0);
+        const float ex = i < k ? expf(entry_value(top) - x0) : 0.f;
+        float z = 0.f, cdf = 0.f;
+        #pragma unroll 1
+        for (int r = 0; r < k; ++r) z += __shfl_sync(0xffffffffu, ex, r);
         int pick = k - 1;
         bool found = false;
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) {
-            if (r < k && !found) {
-                cdf += ex[r] / z;
-                if (cdf > u) { pick = r; found = true; }
-            }
+        #pragma unroll 1
+        for (int r = 0; r < k; ++r) {
+            cdf += __shfl_sync(0xffffffffu, ex, r) / z;
+            if (!found && cdf > u) { pick = r; found = true; }
         }
-        unsigned long long e = 0ull;
-        #pragma unroll
-        for (int r = 0; r < kMaxTopK; ++r) e = (r == pick) ? top[r] : e;
-        drawn[row] = entry_index(e);
-        if (node_token && t < T) node_token[row] = entry_index(e);
+        const int token = __shfl_sync(0xffffffffu, entry_index(top), pick);
+        if (i == 0) {
+            drawn[row] = token;
+            if (node_token && t < T) node_token[row] = token;
+        }
     }
     if (!arrive_last(&counters[b], max(T, 1))) return;
 
-    const int i = static_cast<int>(threadIdx.x);
     if (i < SS_MAX_NODES) s_draw[i] = i < max(T, 1) ? __ldcg(drawn + static_cast<size_t>(b) * max_nodes + i) : -1;
     __syncthreads();
     if (i >= 32) return;
@@ -509,8 +512,9 @@ extern "C" int32_t ss_next_draft(const float* stream_logits, int32_t n_rows, con
     if (workspace_bytes < ss_next_draft_workspace_bytes(batch, gamma, vocab)) return SS_ERR_WORKSPACE;
     // a cluster of at most 8 CTAs takes all the rows of a sequence
     int n_cta = 1;
-    while (gamma * n_cta * 2 <= 8 && vocab / (n_cta * 2) >= ss::kRowThreads * 4) n_cta *= 2;
-    const cudaError_t err = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kRowThreads), gamma * n_cta, true,
+    while (gamma * n_cta * 2 <= 8 && vocab / (n_cta * 2) >= ss::kDraftThreads * 4) n_cta *= 2;
+    const cudaError_t err = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kDraftThreads),
+                                            gamma * n_cta, true,
                                             static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token, gamma, vocab,
                                             top_k, max_nodes, n_cta, draft_tokens, trees);
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;

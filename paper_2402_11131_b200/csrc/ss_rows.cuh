@@ -5,6 +5,11 @@
 // finished without a trip through global memory.  What a sequence does with its rows' results runs in the CTA that
 // finishes the sequence's last row (one arrival per row on a global counter, nobody waits).
 //
+// The pass over a segment runs from registers, eight 16-byte loads per thread in flight.  Everything behind it is short:
+// for one sequence these kernels are chains of latencies, in which most instructions execute once per CTA.  Measured and
+// not kept: the segment staged in shared memory by bulk copies, one pass there for the maximum and one for the rest
+// (1024 rows of 32000 logits: arg-max 35 us, softmax statistics 52 us, against 24 and 31 us).
+//
 // Order of logits.  Entries are ranked by an integer key that is monotone in the IEEE order of fp32 values, with
 // -0 == +0 and every NaN below -inf, and equal keys by ascending index.  Compiled without fast-math: nothing is
 // flushed or reassociated.
@@ -13,11 +18,13 @@
 
 namespace ss {
 
-// 512 threads with eight 16-byte loads in flight each: 64 KB per CTA, two CTAs per SM, 19 MB over the GPU -- about
-// twice what the HBM latency needs at full bandwidth, and a 16000-logit segment is one batch of loads.
-constexpr int kRowThreads = 512;
-constexpr int kRowWarps = kRowThreads / 32;
+// Threads of a scan: 256 with eight 16-byte loads each in flight, four CTAs per SM (64 registers a thread): 128 KB in
+// flight per SM.  Measured for 1024 rows of 32000 logits, arg-max / softmax statistics: 23.6 / 31.2 us; four loads and
+// six CTAs 28.2 / 36.6; 512 threads 25.1 / 36.1; two CTAs per row 27.5 / 39.1 (a CTA costs 4 us besides its loads).
+constexpr int kRowThreads = 256;
 constexpr int kRowVecs = 8;
+constexpr int kRowBlocks = 4;         // CTAs per SM
+constexpr int kRowParts = 64;         // partial results that CTA 0 of a cluster merges: 8 CTAs x 8 warps
 constexpr int kMaxTopK = SS_MAX_TOPK;
 
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -47,49 +54,56 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 }
 
 // ---- the segment of a row that a CTA scans ----------------------------------------------------------------------
-// Row `row` of a [rows][vocab] array whose base is 16-byte aligned; CTA `rank` of `n_cta` takes logits [lo, hi).
+// Row `row` of a [rows][vocab] array whose base is 16-byte aligned; CTA `rank` of `n_cta` takes logits [lo, hi).  Word
+// i of `src` (16-byte aligned) is logit `at + i` of the row; the segment is words [skip, total).
 struct Segment {
-    const float* base;
-    size_t start;                 // first element of the row in the array
-    int lo, hi;                   // logits of the row
+    const float* src;
+    int at, skip, total;
 };
 __device__ __forceinline__ Segment make_segment(const float* base, size_t row, int vocab, int rank, int n_cta) {
-    Segment s;
-    s.base = base;
-    s.start = row * static_cast<size_t>(vocab);
     const int per = ((vocab + n_cta - 1) / n_cta + 3) & ~3;
-    s.lo = min(vocab, rank * per);
-    s.hi = min(vocab, s.lo + per);
+    const int lo = min(vocab, rank * per), hi = min(vocab, lo + per);
+    const float* first = base + row * static_cast<size_t>(vocab) + lo;
+    Segment s;
+    s.skip = static_cast<int>((reinterpret_cast<uintptr_t>(first) >> 2) & 3);
+    s.src = first - s.skip;
+    s.at = lo - s.skip;
+    s.total = s.skip + hi - lo;
     return s;
 }
-// Calls f.batch(x, first) for batches of kRowVecs x 4 logits (first[v]: index in the row of x[4 v]; logits past the
-// end read -inf) and f.one(x, index) for the up to six logits before the first and after the last 16-byte boundary.
-// A thread meets its logits in ascending order of their index, except that the ones at the ends come last.
-template <typename F>
+// Vector i of the segment (words 4 i .. 4 i + 3); words that are not the segment's read -inf.  The first and the last
+// one are put together from single loads where they are not whole.
+static __device__ __noinline__ float4 edge_vec(const float* src, int i, int skip, int total) {
+    float4 q;
+    q.x = 4 * i >= skip && 4 * i < total ? src[4 * i] : -INFINITY;
+    q.y = 4 * i + 1 >= skip && 4 * i + 1 < total ? src[4 * i + 1] : -INFINITY;
+    q.z = 4 * i + 2 >= skip && 4 * i + 2 < total ? src[4 * i + 2] : -INFINITY;
+    q.w = 4 * i + 3 >= skip && 4 * i + 3 < total ? src[4 * i + 3] : -INFINITY;
+    return q;
+}
+// Calls f.batch(q, word) for batches of kRowVecs vectors; word: index of the first word of q[0], that of q[v] is
+// v * 4 * NT further.  A thread meets its logits in ascending order.
+template <int NT, typename F>
 __device__ __forceinline__ void scan_segment(const Segment& s, F& f) {
-    const size_t e0 = s.start + s.lo, e1 = s.start + s.hi;
-    const size_t v0 = (e0 + 3) >> 2, v1 = max(e1 >> 2, v0);
-    const float4* vec = reinterpret_cast<const float4*>(s.base);
-    const int n_vec = static_cast<int>(v1 - v0);
-    const int at0 = static_cast<int>(v0 * 4 - s.start);                   // index in the row of the first vector
-    for (int i = static_cast<int>(threadIdx.x); i < n_vec; i += kRowThreads * kRowVecs) {
-        float x[4 * kRowVecs];
-        int first[kRowVecs];
+    const int whole0 = s.skip ? 1 : 0, whole1 = s.total >> 2, n_vec = (s.total + 3) >> 2;      // whole vectors: [whole0, whole1)
+    const float4* vec = reinterpret_cast<const float4*>(s.src);
+    for (int i = static_cast<int>(threadIdx.x); i < n_vec; i += NT * kRowVecs) {
+        float4 q[kRowVecs];
         #pragma unroll
         for (int v = 0; v < kRowVecs; ++v) {
-            const int at = i + v * kRowThreads;
-            float4 q = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (at < n_vec) q = __ldcs(vec + v0 + at);
-            first[v] = at0 + 4 * at;
-            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
+            const int at = i + v * NT;
+            q[v] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            if (at >= whole0 && at < whole1) q[v] = __ldcs(vec + at);
         }
-        f.batch(x, first);
+        if (i < whole0 || (i + (kRowVecs - 1) * NT >= whole1 && (s.total & 3))) {
+            #pragma unroll
+            for (int v = 0; v < kRowVecs; ++v) {
+                const int at = i + v * NT;
+                if (at < n_vec && (at < whole0 || at >= whole1)) q[v] = edge_vec(s.src, at, s.skip, s.total);
+            }
+        }
+        f.batch(q, 4 * i);
     }
-    // the ends: thread i < 3 the i-th logit before the first vector, threads 32.. those after the last
-    const int head = static_cast<int>(min(v0 * 4, e1) - e0), tail0 = static_cast<int>(v1 * 4 - s.start);
-    const int i = static_cast<int>(threadIdx.x);
-    if (i < head) f.one(s.base[e0 + i], s.lo + i);
-    if (i >= 32 && v1 * 4 >= e0 && tail0 + (i - 32) < s.hi && head < s.hi - s.lo) f.one(s.base[s.start + tail0 + (i - 32)], tail0 + (i - 32));
 }
 
 // ---- cluster plumbing --------------------------------------------------------------------------------------------
@@ -111,11 +125,14 @@ __device__ __forceinline__ void cluster_store_u64(uint32_t addr, unsigned long l
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
-// CTAs per row: more of them while the rows do not fill the SMs and a segment stays at a batch of loads or more (a
-// shorter segment would leave threads without work and cost only the hand-over)
+// CTAs per row: more of them while the grid takes at most half of the GPU's slots -- the next kernel's CTAs then start in
+// the other half and wait there, which hides its launch -- and a segment stays at a batch of loads per thread (a
+// shorter one costs only the hand-over).  A segment of more than two batches is worth all slots: its batches of loads
+// follow one another.
 inline int row_cluster(long long rows, int vocab) {
+    const long long slots = static_cast<long long>(kRowBlocks) * sm_count();
     int c = 1;
-    while (c < 8 && rows * c * 2 <= 2ll * sm_count() && vocab / (c * 2) >= kRowThreads * 4) c *= 2;
+    while (c < 8 && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= (vocab / c > 2 * kRowThreads * kRowVecs * 4 ? slots : slots / 2)) c *= 2;
     return c;
 }
 
@@ -133,43 +150,53 @@ __device__ __forceinline__ bool arrive_last(int32_t* counter, int expected) {
     return s_last;
 }
 
-// ---- arg-max of a row ---------------------------------------------------------------------------------------------
+// A partial result goes to the shared memory of the cluster's CTA 0; when this returns true (in CTA 0 only), all have
+// arrived.  Every CTA of the cluster has called cluster_arrive() once, at its start; store(rank) stores.
+template <typename F>
+__device__ __forceinline__ bool hand_to_first(int rank, int n_cta, F&& store) {
+    if (n_cta > 1) cluster_wait();                        // CTA 0 has started
+    store();
+    if (n_cta > 1) {
+        cluster_arrive();
+        if (rank != 0) return false;
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    return true;
+}
+
+// ---- arg-max of a segment ----------------------------------------------------------------------------------------
 struct ArgMax {
     float v = -INFINITY;
-    int i = 0x7fffffff;
-    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {
+    int i = 0;
+    template <int NT>
+    __device__ __forceinline__ void take(const float4 (&q)[kRowVecs], int word) {
         #pragma unroll
-        for (int q = 0; q < 4 * kRowVecs; ++q)
-            if (x[q] > v) { v = x[q]; i = first[q >> 2] + (q & 3); }
+        for (int k = 0; k < kRowVecs; ++k) {
+            const int at = word + k * 4 * NT;
+            if (q[k].x > v) { v = q[k].x; i = at; }
+            if (q[k].y > v) { v = q[k].y; i = at + 1; }
+            if (q[k].z > v) { v = q[k].z; i = at + 2; }
+            if (q[k].w > v) { v = q[k].w; i = at + 3; }
+        }
     }
-    __device__ __forceinline__ void one(float x, int at) {
-        if (x > v || (x == v && at < i)) { v = x; i = at; }
-    }
+    __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) { take<kRowThreads>(q, word); }
+    // A thread that met nothing above -inf has no entry: it does not know which of its logits are NaN
+    __device__ __forceinline__ unsigned long long best(const Segment& s) const { return v > -INFINITY ? entry(order_key(v), s.at + i) : 0ull; }
 };
-// A thread's entry.  A thread that saw nothing above -inf does not know which of its logits are -inf and which are
-// NaN; it counts as without an entry, and a row in which no thread has one is scanned again (entry_of_any).
-__device__ __forceinline__ unsigned long long entry_of(const ArgMax& a) { return a.v > -INFINITY ? entry(order_key(a.v), a.i) : 0ull; }
-struct AnyMax {
+// The best entry of a row of nothing but -inf and NaN (every thread of the CTA takes part; all get it)
+static __device__ __noinline__ unsigned long long best_of_any(const float* base, size_t row, int vocab, unsigned long long* s_w) {
     unsigned long long e = 0ull;
-    __device__ __forceinline__ void batch(const float (&x)[4 * kRowVecs], const int (&first)[kRowVecs]) {}
-    __device__ __forceinline__ void one(float x, int at) {
-        const unsigned long long n = entry(order_key(x), at);
+    for (int i = static_cast<int>(threadIdx.x); i < vocab; i += kRowThreads) {
+        const unsigned long long n = entry(order_key(base[row * static_cast<size_t>(vocab) + i]), i);
         e = n > e ? n : e;
     }
-};
-// the best entry of a segment, one logit at a time (only for rows of -inf and NaN)
-static __device__ __noinline__ unsigned long long entry_of_any(const Segment s) {
-    AnyMax m;
-    for (int i = s.lo + static_cast<int>(threadIdx.x); i < s.hi; i += kRowThreads) m.one(s.base[s.start + i], i);
-    return m.e;
-}
-// maximum over the CTA, known to every thread of warp 0 (others: 0); `s_w` is a scratch array of kRowWarps words
-__device__ __forceinline__ unsigned long long block_max(unsigned long long e, unsigned long long* s_w) {
     e = warp_max_u64(e);
+    __syncthreads();
     if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = e;
     __syncthreads();
-    if (threadIdx.x >= 32) return 0ull;
-    return warp_max_u64(threadIdx.x < kRowWarps ? s_w[threadIdx.x] : 0ull);
+    return warp_max_u64(s_w[threadIdx.x & (kRowThreads / 32 - 1)]);
 }
 
 // ---- the deepest accepted node ------------------------------------------------------------------------------------
