@@ -117,7 +117,7 @@ int32_t ss_tree_build(const int32_t* parent, int32_t n_nodes, int32_t gamma, ss_
  * started over: such a block first takes every row's exponentials against the maximum of the row's first
  * 128 keys, and if a later tile exceeds that reference by more than about 2^57 it runs its tiles again
  * with a running maximum (same result, about twice the time for that block).  Diagnostics only.
- * Precondition of a split (batch * n_heads * row blocks below the SM count): the CTAs that share a block's
+ * Precondition of a split (batch * n_heads * row blocks below the SM count, twice that for at most 32 rows): the CTAs that share a block's
  * keys wait for one another's partial rows at the end, so they must all be resident at once.  The call sizes the split from
  * the device's SM count; if other work holds SMs for the whole duration of the call (another stream, another
  * process, a partition of the GPU) the wait can run out: the CTAs then give up, the status word reads

@@ -103,6 +103,8 @@ struct alignas(64) AttnArgs {
     int gamma_magic;                 // ceil(65536 / gamma): x / gamma == (x * gamma_magic) >> 16 for x < 256
     int prefix_stable;               // the caller's SS_ATTN_PREFIX_STABLE promise
     float scale_log2;                // sm_scale * log2(e)
+    const __nv_bfloat16* q_main;
+    const __nv_bfloat16* q_spec;
     __nv_bfloat16* o_main;
     __nv_bfloat16* o_spec;
     float* lse_main;
@@ -477,11 +479,12 @@ __device__ __forceinline__ float chunk_exp_pack(const uint32_t (&v)[64], float s
     return (s0 + s1) + (s2 + s3);
 }
 
-// Which kernel a call takes: kCols, heads of at most 64 rows (msa_attention_small_kernel); kPair, blocks of up to
+// Which kernel a call takes: kFew, heads of at most 64 rows with few rows or few keys (msa_attention_few_rows_kernel, see
+// few_rows_better); kCols, the other heads of at most 64 rows (msa_attention_small_kernel); kPair, blocks of up to
 // 128 rows of larger heads (msa_attention_kernel: warpgroup w takes keys 64w .. 64w+63 of every tile, with its own
 // running maximum and accumulator; the two partials a row then has inside the CTA are combined before the merge
 // across CTAs).
-enum Mode { kPair = 0, kCols = 1 };
+enum Mode { kPair = 0, kCols = 1, kFew = 2 };
 
 template <int HD>
 struct Geo {
@@ -1435,6 +1438,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
 
 }  // namespace ss
 
+#include "ss_attention_few.cuh"
 #include "ss_attention_small.cuh"
 
 namespace ss {
@@ -1480,6 +1484,29 @@ struct AttnPlan {
     size_t partial_bytes;                      // workspace after its header
 };
 
+// Heads of at most 64 rows: which of the two kernels.  The few-rows kernel has little fixed cost (4 us a layer where the
+// tcgen05 one takes 8) but pays more per key, the more the more rows and dimensions.  The lengths are on the device; the
+// slab says how many slots a sequence has on average, which bounds them, so a cache much larger than its contents
+// gets the tcgen05 kernel.  Up to 32 rows of at most 80 dimensions it wins at every length measured (128 to 4096 keys);
+// else up to `keys` per CTA of a grid of one wave, `batch_keys` where the grid takes several (there the CTAs that share
+// an SM hide each other's fixed cost, and up to 32 rows always win).  The lines lie where the two kernels met, us per plain layer of 32 heads, tcgen05 and few rows:
+// 27 rows of 128, 800 keys over 4 CTAs 9.7 and 9.4, 1500 keys 10.7 and 11.6; 64 rows of 64, 1024 keys 9.0 and 8.4, 2048 keys
+// 10.9 and 11.2; 64 rows of 80, 1024 keys 10.2 and 10.0, 2048 keys 12.0 and 13.6; 64 rows of 128, 512 keys 10.7 and 9.4,
+// 1024 keys 11.9 and 12.6; sixteen sequences of 512 keys, 64 rows of 64, 41.9 and 29.8, of 2300 keys 75.9 and 82.6.
+static bool few_rows_better(const ss_attn_params& p, int q_rows, long long groups, int split) {
+    const long long slots = p.kv_total_slots / p.batch;
+    long long keys, batch_keys;
+    if (q_rows <= 32) {
+        if (p.head_dim <= 80) return true;
+        keys = q_rows <= 16 ? 1100 : 240;
+        batch_keys = 1ll << 40;
+    } else {
+        keys = p.head_dim == 64 ? 400 : p.head_dim == 80 ? 290 : 180;
+        batch_keys = p.head_dim == 64 ? 1700 : p.head_dim == 80 ? 1500 : 700;
+    }
+    return groups > sm_count() ? slots <= batch_keys : slots / split <= keys;
+}
+
 static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     if (p.batch < 1 || p.n_heads < 1 || p.max_nodes < 1 || p.gamma < 0) return false;
     if (p.head_dim != 64 && p.head_dim != 80 && p.head_dim != 128) return false;
@@ -1488,15 +1515,32 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     plan->tmax8 = (p.max_nodes + 7) / 8 * 8;
     plan->spec_rows = p.gamma > 0 ? (p.max_nodes * p.gamma + 7) / 8 * 8 : 0;
     const int q_rows = plan->tmax8 + plan->spec_rows;
-    plan->mode = q_rows <= kSmRows ? kCols : kPair;
-    plan->n_blocks = plan->mode != kPair ? 1 : (q_rows + kBlockRows - 1) / kBlockRows;
+    plan->n_blocks = q_rows > kSmRows ? (q_rows + kBlockRows - 1) / kBlockRows : 1;
     // stream rows that share block 0 with the main rows
     plan->s0rows = plan->spec_rows < kBlockRows - plan->tmax8 ? plan->spec_rows : kBlockRows - plan->tmax8;
     // CTAs per (sequence, head, row block): the largest power of two that still fits the grid on the SMs in one wave
     plan->groups = static_cast<long long>(p.batch) * p.n_heads * plan->n_blocks;
-    int c = 1;
-    while (c < 8 && plan->groups * (c * 2) <= sm_count()) c *= 2;
+    const auto split = [&](long long ctas) {
+        int c = 1;
+        while (c < 8 && plan->groups * (c * 2) <= ctas) c *= 2;
+        return c;
+    };
+    const int c = split(sm_count());
     plan->cluster = c;
+    plan->mode = q_rows > kSmRows ? kPair : few_rows_better(p, q_rows, plan->groups, c) ? kFew : kCols;
+    if (plan->mode != kPair) {
+        // the few-rows kernel takes half an SM per CTA (and splits a head no further than its length asks for); with 64 rows
+        // two CTAs on an SM get in each other's way (12 us instead of 9 at 512 keys of 128)
+        const int c2 = q_rows <= 32 ? split(2ll * sm_count()) : c;
+        if (plan->mode == kFew) plan->cluster = c2;
+        // a split head leaves the partial rows (O, m, l) of each of its CTAs in the workspace
+        plan->partial_bytes = c2 > 1 ? static_cast<size_t>(plan->groups) * c2 * kSmRows * (p.head_dim + 4) * 4 : 0;
+    }
+    if (plan->mode == kFew) {
+        plan->n_kslots = plan->n_vslots = 0;       // (its ring and shared memory follow from head_dim and rows)
+        plan->smem = 0;
+        return true;
+    }
     if (plan->mode == kCols) {
         // the query tile (its 64 rows twice), then the K and V rings (at the end they stage 64 partial rows)
         const size_t q_bytes = static_cast<size_t>(halves) * 2 * kSmRows * 128, slot = static_cast<size_t>(halves) * kTileKeys * 128;
@@ -1507,8 +1551,6 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
         plan->n_kslots = slots;
         plan->n_vslots = 0;
         plan->smem = q_bytes + static_cast<size_t>(slots) * slot;
-        // a split head leaves the partial rows (O, m, l) of each of its CTAs in the workspace
-        plan->partial_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * kSmRows * (p.head_dim + 4) * 4 : 0;
         return true;
     }
     // row blocks: the query tile, then the K ring and the V ring (P lives in TMEM)
@@ -1561,6 +1603,37 @@ static int32_t launch(const AttnArgs& args, const AttnPlan& plan, cudaStream_t s
     const cudaError_t err = plan.cluster == 1 ? cudaLaunchKernelEx(&cfg, msa_attention_kernel<HD, true>, args)
                                               : cudaLaunchKernelEx(&cfg, msa_attention_kernel<HD, false>, args);
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
+}
+
+template <int HD, int RG>
+static int32_t launch_few(const AttnArgs& args, const AttnPlan& plan, cudaStream_t stream) {
+    static bool configured[64] = {false};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;
+    if (dev >= 0 && dev < 64 && !configured[dev]) {
+        if (cudaFuncSetAttribute(msa_attention_few_rows_kernel<HD, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 GeoF<HD, RG>::kDynSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(msa_attention_few_rows_kernel<HD, RG>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            return SS_ERR_CUDA;
+        configured[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(plan.groups * plan.cluster), 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(kFwThreads), 1, 1);
+    cfg.dynamicSmemBytes = GeoF<HD, RG>::kDynSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, msa_attention_few_rows_kernel<HD, RG>, args) == cudaSuccess ? SS_OK : SS_ERR_CUDA;
+}
+
+template <int HD>
+static int32_t launch_few_rows(int rows, const AttnArgs& args, const AttnPlan& plan, cudaStream_t stream) {
+    return rows <= 16 ? launch_few<HD, 1>(args, plan, stream) : rows <= 32 ? launch_few<HD, 2>(args, plan, stream) : launch_few<HD, 4>(args, plan, stream);
 }
 
 template <int HD>
@@ -1623,7 +1696,7 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     if (p->workspace_bytes < ss_msa_attention_workspace_bytes(p)) return SS_ERR_WORKSPACE;
 
     ss::AttnArgs a;
-    const int d = p->head_dim, H = p->n_heads, tk = ss::kTileKeys;
+    const int d = p->head_dim, H = p->n_heads, tk = plan.mode == ss::kFew ? ss::kFwKeys : ss::kTileKeys;
     const bool shared_heads = (p->kv_head_stride == 0);
     const long long kv_heads = shared_heads ? 1 : H;
     const long long kv_hstride = shared_heads ? d : p->kv_head_stride;
@@ -1651,6 +1724,8 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     a.gamma_magic = p->gamma > 0 ? (65536 + p->gamma - 1) / p->gamma : 0;
     a.prefix_stable = (p->flags & SS_ATTN_PREFIX_STABLE) ? 1 : 0;
     a.scale_log2 = p->sm_scale * 1.4426950408889634f;
+    a.q_main = static_cast<const __nv_bfloat16*>(p->q_main);
+    a.q_spec = static_cast<const __nv_bfloat16*>(p->q_spec);
     a.o_main = static_cast<__nv_bfloat16*>(p->o_main);
     a.o_spec = static_cast<__nv_bfloat16*>(p->o_spec);
     a.lse_main = p->lse_main; a.lse_spec = p->lse_spec;
@@ -1659,6 +1734,14 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     a.status = reinterpret_cast<int*>(p->workspace);
     a.partials = reinterpret_cast<float*>(static_cast<char*>(p->workspace) + ss::kWsHeaderBytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (plan.mode == ss::kFew) {
+        const int rows = plan.tmax8 + plan.spec_rows;
+        switch (d) {
+            case 64: return ss::launch_few_rows<64>(rows, a, plan, s);
+            case 80: return ss::launch_few_rows<80>(rows, a, plan, s);
+            default: return ss::launch_few_rows<128>(rows, a, plan, s);
+        }
+    }
     if (plan.mode == ss::kCols) {
         switch (d) {
             case 64: return ss::launch_cols<64>(a, plan, s);

@@ -266,6 +266,34 @@ def test_attention_every_split_factor(cuda, oracle, n_heads, expect_split):
             assert_attention_close(oracle, st, st.layer(i), dev, i, check_lse=True)
 
 
+@pytest.mark.parametrize("head_dim", [64, 80, 128])
+@pytest.mark.parametrize("T,gamma,n_heads,lengths", [
+    (16, 0, 5, (31, 32, 33)),            # 16 rows; a tile's edge in the prefix, 8 CTAs per head
+    (1, 3, 300, (0, 415, 900)),          # one node with streams; unsplit heads whose ring wraps under several teams
+    (17, 0, 150, (15, 400, 450)),        # 32 rows, the last rows without a node; two CTAs per head or none
+    (8, 3, 40, (160, 200, 1000)),        # 32 rows with streams, split four ways from 7 tiles on
+    (33, 0, 20, (60, 130, 290)),         # 64 rows, split from 9 tiles on
+    (12, 4, 170, (1, 90, 640)),          # 60 rows with streams, unsplit
+])
+def test_attention_few_rows(cuda, oracle, head_dim, T, gamma, n_heads, lengths):
+    """Heads of at most 64 rows over short prefixes: row groups of 16, 32 and 64, prefixes around the edges of the 32-key
+    tiles, of the ring of tiles (6 or 12) and of the rule that splits a head; a negative scale with the last length."""
+    api, DeviceStep = cuda
+    for k, L in enumerate(lengths):
+        cfg = W.custom_config("few", n_layers=2, n_msa_layers=1, prefix_len=L, n_nodes=T, gamma=max(gamma, 1), max_depth=6,
+                              n_heads=n_heads, head_dim=head_dim, config_id=900 + k)
+        st = W.make_step(cfg)
+        if k == 2:
+            st.sm_scale = -st.sm_scale
+        dev = DeviceStep(st, layers=[1 if gamma else 0], with_lse=True)
+        for _ in range(2):
+            dev.run_attention()
+        assert api.ss_status(dev.attn_ws) == 0
+        assert int(dev.attn_ws.view(torch.int32)[2:].abs().max()) == 0
+        assert_attention_close(oracle, st, st.layer(1 if gamma else 0), dev, 0, check_lse=True,
+                               heads=(max(n_heads - 3, 0), n_heads))
+
+
 # ---- verification ---------------------------------------------------------------------------------
 def _verify_and_compare(api, dev, st, oracle):
     dev.run_verify()
