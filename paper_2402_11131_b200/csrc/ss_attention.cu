@@ -479,8 +479,8 @@ __device__ __forceinline__ float chunk_exp_pack(const uint32_t (&v)[64], float s
     return (s0 + s1) + (s2 + s3);
 }
 
-// Which kernel a call takes: kFew, heads of at most 64 rows with few rows or few keys (msa_attention_few_rows_kernel, see
-// few_rows_better); kCols, the other heads of at most 64 rows (msa_attention_small_kernel); kPair, blocks of up to
+// Which kernel a call takes: kFew, layers with few rows or few keys (msa_attention_few_rows_kernel, see few_rows_block); kCols,
+// the other heads of at most 64 rows (msa_attention_small_kernel); kPair, blocks of up to
 // 128 rows of larger heads (msa_attention_kernel: warpgroup w takes keys 64w .. 64w+63 of every tile, with its own
 // running maximum and accumulator; the two partials a row then has inside the CTA are combined before the merge
 // across CTAs).
@@ -1479,32 +1479,42 @@ static bool make_map(CUtensorMap* out, const void* basep, int d, long long n1, l
 
 struct AttnPlan {
     int tmax8, spec_rows, s0rows, n_blocks, mode, n_kslots, n_vslots, cluster;
+    int few_rows;                              // rows of a block of the few-rows kernel (16, 32, 64), 0: another kernel
     long long groups;                          // (sequence, head, row block) triples
     size_t smem;
     size_t partial_bytes;                      // workspace after its header
 };
 
-// Heads of at most 64 rows: which of the two kernels.  The few-rows kernel has little fixed cost (4 us a layer where the
-// tcgen05 one takes 8) but pays more per key, the more the more rows and dimensions.  The lengths are on the device; the
-// slab says how many slots a sequence has on average, which bounds them, so a cache much larger than its contents
-// gets the tcgen05 kernel.  Up to 32 rows of at most 80 dimensions it wins at every length measured (128 to 4096 keys);
-// else up to `keys` per CTA of a grid of one wave, `batch_keys` where the grid takes several (there the CTAs that share
-// an SM hide each other's fixed cost, and up to 32 rows always win).  The lines lie where the two kernels met, us per plain layer of 32 heads, tcgen05 and few rows:
-// 27 rows of 128, 800 keys over 4 CTAs 9.7 and 9.4, 1500 keys 10.7 and 11.6; 64 rows of 64, 1024 keys 9.0 and 8.4, 2048 keys
-// 10.9 and 11.2; 64 rows of 80, 1024 keys 10.2 and 10.0, 2048 keys 12.0 and 13.6; 64 rows of 128, 512 keys 10.7 and 9.4,
-// 1024 keys 11.9 and 12.6; sixteen sequences of 512 keys, 64 rows of 64, 41.9 and 29.8, of 2300 keys 75.9 and 82.6.
-static bool few_rows_better(const ss_attn_params& p, int q_rows, long long groups, int split) {
-    const long long slots = p.kv_total_slots / p.batch;
-    long long keys, batch_keys;
+// Rows of a block of the few-rows kernel (16, 32 or 64), 0 where a tcgen05 kernel is the better one.  The few-rows kernel
+// has little fixed cost (4 us a layer where the tcgen05 ones take 8) but pays more per key, the more the more rows and
+// dimensions.  The lengths are on the device; the slab says how many slots a sequence has on average, which bounds them, so a
+// cache much larger than its contents gets the tcgen05 kernels.  The lines lie where the kernels met (us per layer of 32
+// heads, one sequence unless said otherwise, tcgen05 / few rows).
+static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups, int split) {
+    const long long slots = p.kv_total_slots / p.batch, keys = slots / split;        // keys per CTA of a grid of one wave
+    const bool d64 = p.head_dim == 64, d80 = p.head_dim == 80;
+    // what the grid in blocks of 32 rows would read per SM
+    const int blocks = (q_rows + 31) / 32;
+    const long long load = static_cast<long long>(p.batch) * p.n_heads * blocks * slots / sm_count();
     if (q_rows <= 32) {
-        if (p.head_dim <= 80) return true;
-        keys = q_rows <= 16 ? 1100 : 240;
-        batch_keys = 1ll << 40;
-    } else {
-        keys = p.head_dim == 64 ? 400 : p.head_dim == 80 ? 290 : 180;
-        batch_keys = p.head_dim == 64 ? 1700 : p.head_dim == 80 ? 1500 : 700;
+        // up to 80 dimensions at every length measured (128 to 4096 keys), and where the grid takes several waves (the CTAs that
+        // share an SM hide each other's fixed cost); 27 rows of 128, 800 keys 9.7 / 9.4, 1500 keys 10.7 / 11.6
+        const int rows = q_rows <= 16 ? 16 : 32;
+        return p.head_dim <= 80 || groups > sm_count() || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
     }
-    return groups > sm_count() ? slots <= batch_keys : slots / split <= keys;
+    if (q_rows <= kSmRows) {
+        // 64 rows of 64, sixteen sequences of 512 keys 41.9 / 29.8, of 2300 keys 76 / 83; of 128, 512 keys 50.9 / 47.7, 2300 keys 115 / 136
+        if (groups > sm_count()) return slots <= (d64 ? 1700 : d80 ? 1500 : 700) ? 64 : 0;
+        // 64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
+        // keys 11.0 / 12.8
+        if (keys <= (d64 ? 280 : d80 ? 290 : 180)) return 64;
+        // two blocks of 32 rows, two CTAs per SM: 64 rows of 64, eight heads and 4096 keys 9.7 / 7.8 (64-row blocks 10.4)
+        return d64 && load <= 950 ? 32 : 0;
+    }
+    // multi-stream layers.  128 rows of 64, 1024 keys 11.7 / 11.5, 2048 keys 15.1 / 16.0, eight heads and 4096 keys 13.3 / 10.7; of
+    // 80, 200 keys 10.9 / 9.6, 1024 keys 14.1 / 14.5; of 128, 200 keys 11.6 / 11.0, 80 rows and 1024 keys 14.8 / 16.5.  320 rows of
+    // 64, eight heads and 512 keys 10.4 / 8.3, 32 heads and 200 keys 10.6 / 11.8
+    return load <= (d64 ? 900 : d80 ? 700 : 320) && (blocks <= 4 || load <= 400) ? 32 : 0;
 }
 
 static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
@@ -1515,26 +1525,32 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     plan->tmax8 = (p.max_nodes + 7) / 8 * 8;
     plan->spec_rows = p.gamma > 0 ? (p.max_nodes * p.gamma + 7) / 8 * 8 : 0;
     const int q_rows = plan->tmax8 + plan->spec_rows;
-    plan->n_blocks = q_rows > kSmRows ? (q_rows + kBlockRows - 1) / kBlockRows : 1;
     // stream rows that share block 0 with the main rows
     plan->s0rows = plan->spec_rows < kBlockRows - plan->tmax8 ? plan->spec_rows : kBlockRows - plan->tmax8;
+    const long long heads = static_cast<long long>(p.batch) * p.n_heads;
     // CTAs per (sequence, head, row block): the largest power of two that still fits the grid on the SMs in one wave
-    plan->groups = static_cast<long long>(p.batch) * p.n_heads * plan->n_blocks;
-    const auto split = [&](long long ctas) {
+    const auto split = [](long long groups, long long ctas) {
         int c = 1;
-        while (c < 8 && plan->groups * (c * 2) <= ctas) c *= 2;
+        while (c < 8 && groups * (c * 2) <= ctas) c *= 2;
         return c;
     };
-    const int c = split(sm_count());
+    plan->n_blocks = q_rows > kSmRows ? (q_rows + kBlockRows - 1) / kBlockRows : 1;
+    plan->groups = heads * plan->n_blocks;
+    const int c = split(plan->groups, sm_count());
     plan->cluster = c;
-    plan->mode = q_rows > kSmRows ? kPair : few_rows_better(p, q_rows, plan->groups, c) ? kFew : kCols;
-    if (plan->mode != kPair) {
+    plan->few_rows = few_rows_block(p, q_rows, plan->groups, c);
+    plan->mode = plan->few_rows ? kFew : q_rows <= kSmRows ? kCols : kPair;
+    // a split block leaves the partial rows (O, m, l) of each of its CTAs in the workspace
+    const size_t row_bytes = static_cast<size_t>(p.head_dim + 4) * 4;
+    plan->partial_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * (q_rows > kSmRows ? kBlockRows : kSmRows) * row_bytes : 0;
+    if (plan->few_rows) {
         // the few-rows kernel takes half an SM per CTA (and splits a head no further than its length asks for); with 64 rows
         // two CTAs on an SM get in each other's way (12 us instead of 9 at 512 keys of 128)
-        const int c2 = q_rows <= 32 ? split(2ll * sm_count()) : c;
-        if (plan->mode == kFew) plan->cluster = c2;
-        // a split head leaves the partial rows (O, m, l) of each of its CTAs in the workspace
-        plan->partial_bytes = c2 > 1 ? static_cast<size_t>(plan->groups) * c2 * kSmRows * (p.head_dim + 4) * 4 : 0;
+        plan->n_blocks = (q_rows + plan->few_rows - 1) / plan->few_rows;
+        plan->groups = heads * plan->n_blocks;
+        plan->cluster = split(plan->groups, plan->few_rows <= 32 ? 2ll * sm_count() : sm_count());
+        const size_t few_bytes = plan->cluster > 1 ? static_cast<size_t>(plan->groups) * plan->cluster * kSmRows * row_bytes : 0;
+        if (few_bytes > plan->partial_bytes) plan->partial_bytes = few_bytes;
     }
     if (plan->mode == kFew) {
         plan->n_kslots = plan->n_vslots = 0;       // (its ring and shared memory follow from head_dim and rows)
@@ -1565,12 +1581,9 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     size_t bytes = qp + static_cast<size_t>(plan->n_kslots + plan->n_vslots) * slot;
     // after the pipeline the same memory stages partial rows ((head_dim + 4) floats each): 2 KB, then the 128
     // outgoing rows
-    const size_t row_bytes = static_cast<size_t>(p.head_dim + 4) * 4;
     const size_t stage = 2048 + kBlockRows * row_bytes;
     if (stage > bytes) bytes = stage;
     plan->smem = bytes + 1024;
-    // workspace: one partial row per (group, CTA of the group, row)
-    plan->partial_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * kBlockRows * row_bytes : 0;
     return plan->smem <= static_cast<size_t>(kPairMaxDynSmem);
 }
 
@@ -1633,7 +1646,7 @@ static int32_t launch_few(const AttnArgs& args, const AttnPlan& plan, cudaStream
 
 template <int HD>
 static int32_t launch_few_rows(int rows, const AttnArgs& args, const AttnPlan& plan, cudaStream_t stream) {
-    return rows <= 16 ? launch_few<HD, 1>(args, plan, stream) : rows <= 32 ? launch_few<HD, 2>(args, plan, stream) : launch_few<HD, 4>(args, plan, stream);
+    return rows == 16 ? launch_few<HD, 1>(args, plan, stream) : rows == 32 ? launch_few<HD, 2>(args, plan, stream) : launch_few<HD, 4>(args, plan, stream);
 }
 
 template <int HD>
@@ -1735,7 +1748,7 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     a.partials = reinterpret_cast<float*>(static_cast<char*>(p->workspace) + ss::kWsHeaderBytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (plan.mode == ss::kFew) {
-        const int rows = plan.tmax8 + plan.spec_rows;
+        const int rows = plan.few_rows;
         switch (d) {
             case 64: return ss::launch_few_rows<64>(rows, a, plan, s);
             case 80: return ss::launch_few_rows<80>(rows, a, plan, s);

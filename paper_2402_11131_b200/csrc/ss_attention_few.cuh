@@ -1,5 +1,5 @@
-// Tree-masked multi-stream attention on register-level MMAs, for heads of at most 64 query rows (Eq. 1, Eq. 2).  Included
-// by ss_attention.cu after its helpers.
+// Tree-masked multi-stream attention on register-level MMAs, for layers with few rows or few keys (Eq. 1, Eq. 2; the rule
+// is few_rows_block).  Included by ss_attention.cu after its helpers.
 //
 // What bounds such a layer.  16 rows against 528 keys of 64 dimensions are 4 MB for 32 heads: 0.7 us of HBM, and less of
 // any other unit.  The layer is a chain of latencies -- the end of the previous kernel, the query rows, S, softmax and
@@ -14,6 +14,8 @@
 // sit beside those of this one with their first K/V tiles loaded, and what they may not read yet (query rows, this
 // step's keys) on its way to L2.
 //
+// The rows of a head -- its main rows, then its stream rows -- are one block, or blocks of 32 or 64 that go to CTAs of their
+// own; a block reads the cached slots and the stream keys of its own nodes.
 // Eight warps: warp (team, g) takes rows 16 g .. 16 g + 15 and every (8 / RG)-th tile of 32 keys, RG = 1, 2, 4 groups of
 // rows.  Every warp runs an online softmax of its own over its tiles (a reference per row, raised when a score exceeds it
 // by more than 2^8; O is in registers, so raising costs a multiplication), so no two warps meet before the end, where
@@ -131,10 +133,10 @@ __device__ __noinline__ bool wait_requested(CtrlF* c, int slot, int t, int* stat
 
 // The CTA's share of its head's tiles: the cached slots [0, L+T) in tiles of kFwKeys, then the stream keys.
 struct SpanF {
-    int L, T, n_stream;
-    int cache_tiles, j0, n;                       // tiles [j0, j0 + n) of the head
+    int L, T, n_stream, slo;                      // the block's stream keys begin at slo
+    int cache_tiles, j0, n;                       // tiles [j0, j0 + n) of the block
     __device__ __forceinline__ bool is_cache(int t) const { return j0 + t < cache_tiles; }
-    __device__ __forceinline__ int first_key(int t) const { return (j0 + t < cache_tiles ? j0 + t : j0 + t - cache_tiles) * kFwKeys; }
+    __device__ __forceinline__ int first_key(int t) const { return j0 + t < cache_tiles ? (j0 + t) * kFwKeys : slo + (j0 + t - cache_tiles) * kFwKeys; }
     __device__ __forceinline__ int region(int t) const { return is_cache(t) ? L + T : n_stream; }
     __device__ __forceinline__ bool prefix_only(int t) const { return is_cache(t) && first_key(t) + kFwKeys <= L; }
 };
@@ -159,9 +161,10 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     const int C = a.cluster;
     const int blk = static_cast<int>(blockIdx.x);
     const int rank = blk & (C - 1);
-    const int group = blk >> a.cluster_shift;              // (sequence, head)
-    int b = group / a.n_heads;
-    const int h = group - b * a.n_heads;
+    const int group = blk >> a.cluster_shift;              // (sequence, head, row block)
+    const int pair = group / a.n_blocks, row0 = (group - pair * a.n_blocks) * G::kRows;
+    int b = pair / a.n_heads;
+    const int h = pair - b * a.n_heads;
     int* const status = a.status;
     const uint32_t q_base = smem_u32(smem_raw);            // [half][rows][128 B], 1024-byte aligned (checked below)
     const uint32_t ring = q_base + G::kQBytes;             // [slot][K, V][half][32 keys][128 B]
@@ -219,8 +222,13 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     const bool skip = over || bad_smem || T == 0;          // nothing read or written; the same in all CTAs of the head
     SpanF sp;
     sp.L = L; sp.T = T; sp.n_stream = T * a.gamma;
+    // stream rows [r0, r1) of the block, numbered from the first stream row; they see stream keys from their first node's on
+    const int r0 = max(row0 - a.tmax8, 0), r1 = min(row0 + G::kRows - a.tmax8, sp.n_stream);
+    sp.slo = r1 > r0 ? ((r0 * a.gamma_magic) >> 16) * a.gamma : 0;
+    const int own_streams = r1 > r0 ? r1 - sp.slo : 0;
+    const bool any_row = row0 < T || r1 > r0;              // (a block without a row reads and writes nothing)
     sp.cache_tiles = (L + T + kFwKeys - 1) / kFwKeys;
-    const int all_tiles = skip ? 0 : sp.cache_tiles + (sp.n_stream + kFwKeys - 1) / kFwKeys;
+    const int all_tiles = skip || !any_row ? 0 : sp.cache_tiles + (own_streams + kFwKeys - 1) / kFwKeys;
     // the CTAs that get tiles; the first ones take the odd tiles, so that the last has the masked ones
     int shift = 0;
     if (all_tiles > few_whole_tiles<HD, RG>())
@@ -228,7 +236,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     const int ce = 1 << shift;
     // The others leave at once: the next layer's CTAs can have their place.  (CTA 0 of a head always waits for the previous
     // kernel, so this kernel never ends before that one.)
-    if (rank > 0 && (rank >= ce || skip)) return;
+    if (rank > 0 && (rank >= ce || all_tiles == 0)) return;
     sp.j0 = (all_tiles * rank + ce - 1) >> shift;
     sp.n = ((all_tiles * (rank + 1) + ce - 1) >> shift) - sp.j0;
 
@@ -252,7 +260,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     // 16-byte piece i of the query rows: row i / (HD / 8); rows that no node owns have none
     constexpr int kPieces = HD / 8;
     auto q_piece = [&](int i) -> const __nv_bfloat16* {
-        const int row = i / kPieces, at = (i - row * kPieces) * 8;
+        const int lrow = i / kPieces, at = (i - lrow * kPieces) * 8, row = row0 + lrow;
         if (row < a.tmax8) return row < T ? a.q_main + ((main_row0 + row) * a.n_heads + h) * HD + at : nullptr;
         const int x = row - a.tmax8;
         return x < sp.n_stream ? a.q_spec + ((spec_row0 + x) * a.n_heads + h) * HD + at : nullptr;
@@ -284,7 +292,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     unsigned long long anc[2] = {0ull, 0ull};
     #pragma unroll
     for (int e = 0; e < 2; ++e) {
-        const int row = 16 * rg + (lane >> 2) + 8 * e;
+        const int row = row0 + 16 * rg + (lane >> 2) + 8 * e;
         ri[e].stream = 0;
         if (row < a.tmax8) {
             ri[e].valid = row < T; ri[e].node = row;
@@ -500,17 +508,18 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     __syncthreads();
     if (!live) return;
     constexpr int kItems = HD / 4;
-    const int n_rows = T + sp.n_stream;
+    // the block's rows that nodes own: main rows [row0, row0 + n_main), then stream rows [r0, r1)
+    const int n_main = max(min(T - row0, G::kRows), 0), n_rows = n_main + max(r1 - r0, 0);
     for (int i = tid; i < n_rows * kItems; i += kFwThreads) {
         const int rr = i / kItems, g4 = i - rr * kItems;
         RowInfo r;
-        r.valid = true; r.node = rr; r.stream = 0;
-        int row = rr;
-        if (rr >= T) {
-            const int xr = rr - T;
+        r.valid = true; r.node = row0 + rr; r.stream = 0;
+        int row = rr;                                                         // in the block
+        if (rr >= n_main) {
+            const int xr = r0 + rr - n_main;
             r.node = (xr * a.gamma_magic) >> 16;
             r.stream = xr - r.node * a.gamma + 1;
-            row = a.tmax8 + xr;
+            row = a.tmax8 + xr - row0;
         }
         // its row group's warp of every team holds the row
         const uint32_t at = w_base + static_cast<uint32_t>(row) * RB;
@@ -549,10 +558,10 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     rows.T = T; rows.gamma = a.gamma; rows.tmax8 = a.tmax8; rows.n_stream = sp.n_stream; rows.spec_end = a.tmax8 + sp.n_stream;
     float* const part_group = a.partials + static_cast<size_t>(group) * C * G::kCtaFloats;
     const int share = G::kRows >> shift, first = rank * share;
-    if (tid == 0) publish_partial_rows<HD>(rows, 0, G::kRows, y_base, part_group + static_cast<size_t>(rank) * G::kCtaFloats, first, share);
+    if (tid == 0) publish_partial_rows<HD>(rows, row0, G::kRows, y_base, part_group + static_cast<size_t>(rank) * G::kCtaFloats, first, share);
     // the other CTAs of the head were launched with this one and need nothing from it: the (bounded) wait is short
     const long long limit = static_cast<long long>(*reinterpret_cast<volatile int*>(&c.wait_limit)) << 10;
-    if (!merge_partial_rows<HD>(a, rows, 0, b, h, spec_row0, ce, rank, y_base, part_group, G::kCtaFloats, first, share, tid, kFwThreads, limit, &c.abort)) {
+    if (!merge_partial_rows<HD>(a, rows, row0, b, h, spec_row0, ce, rank, y_base, part_group, G::kCtaFloats, first, share, tid, kFwThreads, limit, &c.abort)) {
         c.abort = 1;
         set_status(status, SS_ERR_DEVICE_TIMEOUT);
     }

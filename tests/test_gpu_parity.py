@@ -274,9 +274,13 @@ def test_attention_every_split_factor(cuda, oracle, n_heads, expect_split):
     (8, 3, 40, (160, 200, 1000)),        # 32 rows with streams, split four ways from 7 tiles on
     (33, 0, 20, (60, 130, 290)),         # 64 rows, split from 9 tiles on
     (12, 4, 170, (1, 90, 640)),          # 60 rows with streams, unsplit
+    (10, 4, 6, (0, 33, 300)),            # 56 rows; several blocks of 32 rows where a head has more than 64:
+    (16, 4, 3, (1, 64, 500)),            # 80 rows: blocks that begin among the stream rows of a node
+    (41, 1, 5, (31, 200, 400)),          # 96 rows, padding between main and stream rows at a block's edge
+    (64, 4, 2, (5, 96, 700)),            # 320 rows
 ])
 def test_attention_few_rows(cuda, oracle, head_dim, T, gamma, n_heads, lengths):
-    """Heads of at most 64 rows over short prefixes: row groups of 16, 32 and 64, prefixes around the edges of the 32-key
+    """Layers with few rows or few keys: row blocks of 16, 32 and 64, prefixes around the edges of the 32-key
     tiles, of the ring of tiles (6 or 12) and of the rule that splits a head; a negative scale with the last length."""
     api, DeviceStep = cuda
     for k, L in enumerate(lengths):
