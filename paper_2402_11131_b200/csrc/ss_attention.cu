@@ -1514,7 +1514,7 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
     // multi-stream layers.  128 rows of 64, 1024 keys 11.7 / 11.5, 2048 keys 15.1 / 16.0, eight heads and 4096 keys 13.3 / 10.7; of
     // 80, 200 keys 10.9 / 9.6, 1024 keys 14.1 / 14.5; of 128, 200 keys 11.6 / 11.0, 80 rows and 1024 keys 14.8 / 16.5.  320 rows of
     // 64, eight heads and 512 keys 10.4 / 8.3, 32 heads and 200 keys 10.6 / 11.8
-    return load <= (d64 ? 900 : d80 ? 700 : 320) && (blocks <= 4 || load <= 400) ? 32 : 0;
+    return load <= (d64 ? 1300 : d80 ? 700 : 320) && (blocks <= 4 || load <= 400) ? 32 : 0;
 }
 
 static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
@@ -1549,6 +1549,12 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
         plan->n_blocks = (q_rows + plan->few_rows - 1) / plan->few_rows;
         plan->groups = heads * plan->n_blocks;
         plan->cluster = split(plan->groups, plan->few_rows <= 32 ? 2ll * sm_count() : sm_count());
+        // no more CTAs than the slab's slots can ask for (a sequence of a batch: twice the mean); one that finds nothing to
+        // do still costs its launch: 128 or 256 CTAs for 32 whole heads of 528 keys 5.0 and 5.7 us
+        const long long most = (p.batch > 1 ? 2 : 1) * (p.kv_total_slots / p.batch) + static_cast<long long>(p.max_nodes) * p.gamma;
+        const long long tiles = (most + kFwKeys - 1) / kFwKeys + 1;
+        const int whole = few_whole(p.head_dim, plan->few_rows);
+        while (plan->cluster > 1 && (tiles <= whole || plan->cluster / 2 * kFwSplitTiles >= tiles)) plan->cluster /= 2;
         const size_t few_bytes = plan->cluster > 1 ? static_cast<size_t>(plan->groups) * plan->cluster * kSmRows * row_bytes : 0;
         if (few_bytes > plan->partial_bytes) plan->partial_bytes = few_bytes;
     }
@@ -1632,7 +1638,7 @@ static int32_t launch_few(const AttnArgs& args, const AttnPlan& plan, cudaStream
         configured[dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(plan.groups * plan.cluster), 1, 1);
+    cfg.gridDim = dim3(static_cast<unsigned>(plan.groups / plan.n_blocks * plan.cluster), static_cast<unsigned>(plan.n_blocks), 1);
     cfg.blockDim = dim3(static_cast<unsigned>(kFwThreads), 1, 1);
     cfg.dynamicSmemBytes = GeoF<HD, RG>::kDynSmem;
     cfg.stream = stream;

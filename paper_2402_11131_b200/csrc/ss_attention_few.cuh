@@ -145,9 +145,8 @@ struct SpanF {
 // rows, about 2 us), and tiles per CTA that a split aims at.  Measured on plain layers of 32 heads, us: 12 rows of 64,
 // 300 keys whole 4.4, split 5.2; 512 keys 5.0 and 5.8; 800 keys 6.5 and 5.5.  27 rows of 80, 512 keys: 4 tiles per CTA 7.0,
 // 8 tiles 8.6.
-template <int HD, int RG>
-__host__ __device__ constexpr int few_whole_tiles() {
-    return RG == 1 ? (HD > 64 ? 8 : 20) : RG == 2 ? 6 : 8;
+__host__ __device__ constexpr int few_whole(int head_dim, int rows) {
+    return rows == 16 ? (head_dim > 64 ? 8 : 20) : rows == 32 ? 6 : 8;
 }
 constexpr int kFwSplitTiles = 4;
 
@@ -161,8 +160,8 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     const int C = a.cluster;
     const int blk = static_cast<int>(blockIdx.x);
     const int rank = blk & (C - 1);
-    const int group = blk >> a.cluster_shift;              // (sequence, head, row block)
-    const int pair = group / a.n_blocks, row0 = (group - pair * a.n_blocks) * G::kRows;
+    const int pair = blk >> a.cluster_shift;               // (sequence, head); the row block is the grid's second index
+    const int row0 = static_cast<int>(blockIdx.y) * G::kRows;
     int b = pair / a.n_heads;
     const int h = pair - b * a.n_heads;
     int* const status = a.status;
@@ -231,7 +230,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     const int all_tiles = skip || !any_row ? 0 : sp.cache_tiles + (own_streams + kFwKeys - 1) / kFwKeys;
     // the CTAs that get tiles; the first ones take the odd tiles, so that the last has the masked ones
     int shift = 0;
-    if (all_tiles > few_whole_tiles<HD, RG>())
+    if (all_tiles > few_whole(HD, G::kRows))
         while (shift < a.cluster_shift && (all_tiles >> shift) > kFwSplitTiles) ++shift;
     const int ce = 1 << shift;
     // The others leave at once: the next layer's CTAs can have their place.  (CTA 0 of a head always waits for the previous
@@ -556,7 +555,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     __syncthreads();
     Span rows;
     rows.T = T; rows.gamma = a.gamma; rows.tmax8 = a.tmax8; rows.n_stream = sp.n_stream; rows.spec_end = a.tmax8 + sp.n_stream;
-    float* const part_group = a.partials + static_cast<size_t>(group) * C * G::kCtaFloats;
+    float* const part_group = a.partials + (static_cast<size_t>(blockIdx.y) * (gridDim.x >> a.cluster_shift) + pair) * C * G::kCtaFloats;
     const int share = G::kRows >> shift, first = rank * share;
     if (tid == 0) publish_partial_rows<HD>(rows, row0, G::kRows, y_base, part_group + static_cast<size_t>(rank) * G::kCtaFloats, first, share);
     // the other CTAs of the head were launched with this one and need nothing from it: the (bounded) wait is short
