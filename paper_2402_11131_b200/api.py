@@ -30,6 +30,7 @@ SS_ATTN_PREFIX_STABLE = 1
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libss_msa.so")
 _lib = None
+_native = None          # the _pycall module: takes the tensors of the per-step calls apart (see native())
 
 # number of kernels each entry point enqueues per call (for launch accounting in the benchmark); ss_kv_compact enqueues a
 # second one where kv_len_out overlaps kv_len_in
@@ -130,6 +131,22 @@ def lib() -> C.CDLL:
     return _lib
 
 
+def native():
+    """The CPython side of the binding, for the calls of a decode step: pointers, sizes and the current stream are collected
+    in C (1 us of a call that costs 3 us through ctypes).  Raises like lib() if it has not been built."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _pycall
+        except ImportError as e:
+            raise RuntimeError("the binding's native part is missing: run `python -m paper_2402_11131_b200.build`") from e
+        torch.cuda.current_stream()                       # initialises CUDA if nothing has yet
+        _pycall.setup(SsError, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _native = _pycall
+    return _native
+
+
 def _check(status: int, what: str) -> None:
     if status != SS_OK:
         raise SsError(what, status)
@@ -139,20 +156,9 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
-_cuda_up = False
-
-
 def _stream(stream: Optional[torch.cuda.Stream]) -> Optional[int]:
-    """The raw stream of a call: the one given, or the current stream of the current device.  Asking torch for the raw
-    handle takes 0.2 us where building a torch.cuda.Stream object takes 3.4 us, half of a call's host time."""
-    global _cuda_up
-    if stream is not None:
-        return stream.cuda_stream or None
-    if not _cuda_up:
-        s = torch.cuda.current_stream()                # initialises CUDA if nothing has yet
-        _cuda_up = True
-        return s.cuda_stream or None
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
+    s = torch.cuda.current_stream() if stream is None else stream
+    return s.cuda_stream or None
 
 
 # ---- host ---------------------------------------------------------------------------------------
@@ -207,7 +213,7 @@ def ss_msa_attention_workspace_bytes(p: AttnParams) -> int:
 
 def ss_msa_attention(p: AttnParams, stream: Optional[torch.cuda.Stream] = None) -> None:
     """One layer of tree-masked multi-stream attention (asynchronous on `stream`)."""
-    _check(lib().ss_msa_attention(C.byref(p), _stream(stream)), "ss_msa_attention")
+    (_native or native()).msa_attention(p, stream)
 
 
 def ss_tree_verify_workspace_bytes(batch: int, max_nodes: int, vocab: int) -> int:
@@ -217,11 +223,8 @@ def ss_tree_verify_workspace_bytes(batch: int, max_nodes: int, vocab: int) -> in
 def ss_tree_verify(logits, draft_tokens, trees, accept_len, accept_path, last_node, bonus_token,
                    node_argmax, workspace, stream=None) -> None:
     """Greedy verification.  logits f32 [B][Tmax][V]; the int32 outputs are written on the device."""
-    B, Tmax, V = logits.shape
-    _check(lib().ss_tree_verify(_ptr(logits), _ptr(draft_tokens), _ptr(trees), B, Tmax, V, _ptr(accept_len),
-                                _ptr(accept_path), _ptr(last_node), _ptr(bonus_token), _ptr(node_argmax),
-                                _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ss_tree_verify")
+    (_native or native()).tree_verify(logits, draft_tokens, trees, accept_len, accept_path, last_node, bonus_token, node_argmax,
+                                      workspace, stream)
 
 
 def ss_tree_verify_static(logits, draft_tokens, trees, accept_len, accept_path, last_node, bonus_token,
@@ -235,10 +238,6 @@ def ss_tree_verify_static(logits, draft_tokens, trees, accept_len, accept_path, 
     _check(lib().ss_tree_verify_static(_ptr(logits), _ptr(draft_tokens), _ptr(trees), B, Tmax, V,
                                        _ptr(accept_len), _ptr(accept_path), _ptr(last_node), _ptr(bonus_token),
                                        _ptr(node_argmax), _stream(stream)), "ss_tree_verify_static")
-
-
-def _ws_bytes(t: torch.Tensor) -> int:
-    return t.numel() * t.element_size()
 
 
 def empty_trees(batch: int, device="cuda") -> torch.Tensor:
@@ -261,10 +260,8 @@ def ss_next_draft(stream_logits, row_index, bonus_token, top_k: int, max_nodes: 
                   stream=None) -> None:
     """Next tree draft.  stream_logits f32 [B][n_rows][gamma][V]; row_index int32 [B] or None; bonus_token int32 [B];
     draft_tokens int32 [B][max_nodes] and trees (empty_trees(B)) are written on the device."""
-    B, n_rows, gamma, V = stream_logits.shape
-    _check(lib().ss_next_draft(_ptr(stream_logits), n_rows, _ptr(row_index), _ptr(bonus_token), B, gamma, V, int(top_k),
-                               int(max_nodes), _ptr(draft_tokens), _ptr(trees), _ptr(workspace), _ws_bytes(workspace),
-                               _stream(stream)), "ss_next_draft")
+    (_native or native()).next_draft(stream_logits, row_index, bonus_token, int(top_k), int(max_nodes), draft_tokens, trees,
+                                     workspace, stream)
 
 
 def ss_tree_prune_workspace_bytes(batch: int, max_nodes: int, vocab: int) -> int:
@@ -274,20 +271,15 @@ def ss_tree_prune_workspace_bytes(batch: int, max_nodes: int, vocab: int) -> int
 def ss_tree_prune(exit_logits, draft_tokens, trees, threshold: float, edge_prob, new_index, kept_nodes, kept_tokens,
                   pruned_trees, workspace, stream=None) -> None:
     """Parallel tree pruning.  exit_logits f32 [B][Tmax][V]; outputs are written on the device."""
-    B, Tmax, V = exit_logits.shape
-    _check(lib().ss_tree_prune(_ptr(exit_logits), _ptr(draft_tokens), _ptr(trees), B, Tmax, V, float(threshold),
-                               _ptr(edge_prob), _ptr(new_index), _ptr(kept_nodes), _ptr(kept_tokens), _ptr(pruned_trees),
-                               _ptr(workspace), _ws_bytes(workspace), _stream(stream)), "ss_tree_prune")
+    (_native or native()).tree_prune(exit_logits, draft_tokens, trees, threshold, edge_prob, new_index, kept_nodes, kept_tokens,
+                                     pruned_trees, workspace, stream)
 
 
 def ss_tree_verify_soft(logits, draft_tokens, trees, eps: float, delta: float, accept_len, accept_path, last_node,
                         bonus_token, edge_prob, node_entropy, workspace, stream=None) -> None:
     """Verification with the soft (typical-acceptance) criterion; workspace of ss_tree_prune_workspace_bytes."""
-    B, Tmax, V = logits.shape
-    _check(lib().ss_tree_verify_soft(_ptr(logits), _ptr(draft_tokens), _ptr(trees), B, Tmax, V, float(eps), float(delta),
-                                     _ptr(accept_len), _ptr(accept_path), _ptr(last_node), _ptr(bonus_token),
-                                     _ptr(edge_prob), _ptr(node_entropy), _ptr(workspace), _ws_bytes(workspace),
-                                     _stream(stream)), "ss_tree_verify_soft")
+    (_native or native()).tree_verify_soft(logits, draft_tokens, trees, eps, delta, accept_len, accept_path, last_node,
+                                           bonus_token, edge_prob, node_entropy, workspace, stream)
 
 
 def ss_tree_verify_sampled_workspace_bytes(batch: int, max_nodes: int, vocab: int) -> int:
@@ -297,27 +289,18 @@ def ss_tree_verify_sampled_workspace_bytes(batch: int, max_nodes: int, vocab: in
 def ss_tree_verify_sampled(logits, draft_tokens, trees, uniforms, top_k: int, accept_len, accept_path, last_node,
                            bonus_token, node_token, workspace, stream=None) -> None:
     """Verification against tokens drawn from the top-k softmax (temperature 1) with the caller's uniforms f32 [B][Tmax]."""
-    B, Tmax, V = logits.shape
-    _check(lib().ss_tree_verify_sampled(_ptr(logits), _ptr(draft_tokens), _ptr(trees), _ptr(uniforms), B, Tmax, V,
-                                        int(top_k), _ptr(accept_len), _ptr(accept_path), _ptr(last_node),
-                                        _ptr(bonus_token), _ptr(node_token), _ptr(workspace), _ws_bytes(workspace),
-                                        _stream(stream)), "ss_tree_verify_sampled")
+    (_native or native()).tree_verify_sampled(logits, draft_tokens, trees, uniforms, int(top_k), accept_len, accept_path,
+                                              last_node, bonus_token, node_token, workspace, stream)
 
 
 def ss_stream_insert(main_hidden, stream_emb, out, stream=None) -> None:
     """out[t][j] = main_hidden[t] + stream_emb[j] (Eq. 3, identity transformation); bf16 [rows][hidden], [gamma][hidden]."""
-    rows, hidden = main_hidden.shape
-    gamma = stream_emb.shape[0]
-    _check(lib().ss_stream_insert(_ptr(main_hidden), _ptr(stream_emb), _ptr(out), rows, gamma, hidden, _stream(stream)),
-           "ss_stream_insert")
+    (_native or native()).stream_insert(main_hidden, stream_emb, out, stream)
 
 
 def ss_value_rotate(v_main, v_streams, epsilon: float, stream=None) -> None:
     """v_streams[t][n-1] = v_main[t] rotated by epsilon * n on (re, im) pairs (Eq. 7); bf16 [rows][width], [rows][gamma][width]."""
-    rows, width = v_main.shape
-    gamma = v_streams.shape[1]
-    _check(lib().ss_value_rotate(_ptr(v_main), _ptr(v_streams), rows, gamma, width, float(epsilon), _stream(stream)),
-           "ss_value_rotate")
+    (_native or native()).value_rotate(v_main, v_streams, epsilon, stream)
 
 
 def make_cache_layout(k_all: torch.Tensor) -> CacheLayout:
@@ -333,9 +316,7 @@ def make_cache_layout(k_all: torch.Tensor) -> CacheLayout:
 def ss_kv_compact(k_all, v_all, layout: CacheLayout, kv_start, kv_len_in, accept_len, accept_path, kv_len_out,
                   stream=None) -> None:
     """In-place gather of the accepted path's K/V in every layer (asynchronous on `stream`)."""
-    _check(lib().ss_kv_compact(_ptr(k_all), _ptr(v_all), C.byref(layout), kv_start.shape[0], _ptr(kv_start),
-                               _ptr(kv_len_in), _ptr(accept_len), _ptr(accept_path), _ptr(kv_len_out),
-                               _stream(stream)), "ss_kv_compact")
+    (_native or native()).kv_compact(k_all, v_all, layout, kv_start, kv_len_in, accept_len, accept_path, kv_len_out, stream)
 
 
 def ss_wait_selftest(workspace: torch.Tensor, stream=None) -> None:

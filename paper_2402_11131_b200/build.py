@@ -1,4 +1,4 @@
-"""Builds libss_msa.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libss_msa.so (the C-ABI CUDA library, nvcc for sm_100a) and _pycall (the CPython side of the binding) in-tree."""
 from __future__ import annotations
 
 import glob
@@ -6,12 +6,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 TRACE = bool(os.environ.get("SS_TRACE"))       # developer build with in-kernel timestamps
 LIB = os.path.join(PKG, "libss_msa_trace.so" if TRACE else "libss_msa.so")
+PYCALL = os.path.join(PKG, "_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))
 OBJ = os.path.join(PKG, "_build_trace" if TRACE else "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -66,6 +68,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + ".tmp%d" % os.getpid()
         subprocess.check_call([nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp, *objs])
         os.replace(tmp, LIB)
+    pycall = os.path.join(CSRC, "ss_pycall.cpp")
+    if not TRACE and (force or _stale(PYCALL, [pycall, os.path.join(ROOT, "include", "ss_msa.h")])):
+        tmp = PYCALL + ".tmp%d" % os.getpid()
+        subprocess.check_call([shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-I",
+                               os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], pycall, "-o", tmp, "-L", PKG,
+                               "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, PYCALL)
     return LIB
 
 

@@ -1720,18 +1720,14 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     const long long kv_heads = shared_heads ? 1 : H;
     const long long kv_hstride = shared_heads ? d : p->kv_head_stride;
     bool ok = ss::make_map(&a.tm_k, p->k_cache, d, kv_heads, kv_hstride, p->kv_total_slots, p->kv_slot_stride, tk) &&
-              ss::make_map(&a.tm_v, p->v_cache, d, kv_heads, kv_hstride, p->kv_total_slots, p->kv_slot_stride, tk) &&
-              ss::make_map(&a.tm_qm, p->q_main, d, H, d, rows_main, static_cast<long long>(H) * d, plan.tmax8);
-    if (ok && p->gamma > 0) {
-        const long long rows_spec = rows_main * p->gamma;
-        const long long hd = static_cast<long long>(H) * d;
-        ok = ss::make_map(&a.tm_qs, p->q_spec, d, H, d, rows_spec, hd, plan.s0rows > 0 ? plan.s0rows : 8) &&
-             ss::make_map(&a.tm_qs1, p->q_spec, d, H, d, rows_spec, hd, ss::kBlockRows) &&
-             ss::make_map(&a.tm_ks, p->k_spec, d, H, d, rows_spec, hd, tk) &&
-             ss::make_map(&a.tm_vs, p->v_spec, d, H, d, rows_spec, hd, tk);
-    } else if (ok) {
-        a.tm_qs = a.tm_qm; a.tm_qs1 = a.tm_qm; a.tm_ks = a.tm_k; a.tm_vs = a.tm_v;     // never used when gamma == 0
-    }
+              ss::make_map(&a.tm_v, p->v_cache, d, kv_heads, kv_hstride, p->kv_total_slots, p->kv_slot_stride, tk);
+    const long long rows_spec = rows_main * p->gamma, hd = static_cast<long long>(H) * d;
+    if (ok && p->gamma > 0)
+        ok = ss::make_map(&a.tm_ks, p->k_spec, d, H, d, rows_spec, hd, tk) && ss::make_map(&a.tm_vs, p->v_spec, d, H, d, rows_spec, hd, tk);
+    // the query rows: the few-rows kernel reads them itself, and only the row blocks have a second box of stream rows
+    if (ok && plan.mode != ss::kFew) ok = ss::make_map(&a.tm_qm, p->q_main, d, H, d, rows_main, hd, plan.tmax8);
+    if (ok && plan.mode != ss::kFew && p->gamma > 0) ok = ss::make_map(&a.tm_qs, p->q_spec, d, H, d, rows_spec, hd, plan.s0rows > 0 ? plan.s0rows : 8);
+    if (ok && plan.mode == ss::kPair && p->gamma > 0) ok = ss::make_map(&a.tm_qs1, p->q_spec, d, H, d, rows_spec, hd, ss::kBlockRows);
     if (!ok) return SS_ERR_CUDA;
     a.batch = p->batch; a.n_heads = H; a.gamma = p->gamma; a.max_nodes = p->max_nodes;
     a.tmax8 = plan.tmax8; a.s0rows = plan.s0rows; a.n_blocks = plan.n_blocks;
