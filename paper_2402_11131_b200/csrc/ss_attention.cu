@@ -1,6 +1,10 @@
 // Tree-masked multi-stream attention, one layer (Eq. 1, Eq. 2): flash-decode for sm_100a.
 //
-// Work decomposition.  The query rows of a (sequence, head) pair -- T main rows, then the T*gamma
+// Four kernels.  Layers with few rows or few keys run on register-level MMAs (msa_attention_few_rows_kernel, in
+// ss_attention_few.cuh), the others on tcgen05: grids of more heads or row blocks than SMs with two CTAs per SM
+// (msa_attention_half_kernel, in ss_attention_half.cuh), smaller grids with one.  make_plan has the rules.
+//
+// Work decomposition of the last.  The query rows of a (sequence, head) pair -- T main rows, then the T*gamma
 // stream rows -- form one tile when there are at most 64 of them (msa_attention_small_kernel, in
 // ss_attention_small.cuh), else blocks of 128 rows that go to separate CTAs (msa_attention_kernel, here;
 // a block streams the keys it can see: the cached slots, and the stream keys of its own nodes).  C CTAs
@@ -237,6 +241,28 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// The same, issued by the one lane of the warp whose `lead` is set (elect_lane(), taken once: a commit stands for the
+// products of its own thread).  All lanes come here with the same operands, so these are computed and kept in uniform
+// registers; from inside a branch that a single thread takes every operand is moved there by an instruction chain of its
+// own, and an MMA takes 76 to 98 cycles to issue where its execution takes 32 (M = 64, N = 64) to 64 (N = 128).
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ void tc_commit_w(uint32_t lead, uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(bar), "r"(lead) : "memory");
+}
+__device__ __forceinline__ void tc_mma_w(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead) : "memory");
+}
+__device__ __forceinline__ void tc_mma_ts_w(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -479,12 +505,12 @@ __device__ __forceinline__ float chunk_exp_pack(const uint32_t (&v)[64], float s
     return (s0 + s1) + (s2 + s3);
 }
 
-// Which kernel a call takes: kFew, layers with few rows or few keys (msa_attention_few_rows_kernel, see few_rows_block); kCols,
-// the other heads of at most 64 rows (msa_attention_small_kernel); kPair, blocks of up to
-// 128 rows of larger heads (msa_attention_kernel: warpgroup w takes keys 64w .. 64w+63 of every tile, with its own
+// Which kernel a call takes: kFew, layers with few rows or few keys (msa_attention_few_rows_kernel, see few_rows_block); kHalf, other grids
+// of more blocks than SMs (msa_attention_half_kernel); kCols, the other heads of at most 64 rows
+// (msa_attention_small_kernel); kPair, blocks of up to 128 rows of larger heads (msa_attention_kernel: warpgroup w takes keys 64w .. 64w+63 of every tile, with its own
 // running maximum and accumulator; the two partials a row then has inside the CTA are combined before the merge
 // across CTAs).
-enum Mode { kPair = 0, kCols = 1, kFew = 2 };
+enum Mode { kPair = 0, kCols = 1, kFew = 2, kHalf = 3 };
 
 template <int HD>
 struct Geo {
@@ -1440,6 +1466,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
 
 #include "ss_attention_few.cuh"
 #include "ss_attention_small.cuh"
+#include "ss_attention_half.cuh"
 
 namespace ss {
 
@@ -1539,7 +1566,9 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     const int c = split(plan->groups, sm_count());
     plan->cluster = c;
     plan->few_rows = few_rows_block(p, q_rows, plan->groups, c);
-    plan->mode = plan->few_rows ? kFew : q_rows <= kSmRows ? kCols : kPair;
+    // more blocks than SMs: two CTAs per SM.  (us per layer, one CTA per SM / two: five sequences x 32 heads of 2048 x 128, 64
+    // rows 46.6 / 36.9; with fewer blocks than SMs the second half stays empty: three sequences 22.4 / 32)
+    plan->mode = plan->few_rows ? kFew : plan->groups > sm_count() ? kHalf : q_rows <= kSmRows ? kCols : kPair;
     // a split block leaves the partial rows (O, m, l) of each of its CTAs in the workspace
     const size_t row_bytes = static_cast<size_t>(p.head_dim + 4) * 4;
     plan->partial_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * (q_rows > kSmRows ? kBlockRows : kSmRows) * row_bytes : 0;
@@ -1558,8 +1587,8 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
         const size_t few_bytes = plan->cluster > 1 ? static_cast<size_t>(plan->groups) * plan->cluster * kSmRows * row_bytes : 0;
         if (few_bytes > plan->partial_bytes) plan->partial_bytes = few_bytes;
     }
-    if (plan->mode == kFew) {
-        plan->n_kslots = plan->n_vslots = 0;       // (its ring and shared memory follow from head_dim and rows)
+    if (plan->mode == kFew || plan->mode == kHalf) {
+        plan->n_kslots = plan->n_vslots = 0;       // (rings and shared memory follow from head_dim and rows)
         plan->smem = 0;
         return true;
     }
@@ -1681,6 +1710,31 @@ static int32_t launch_cols(const AttnArgs& args, const AttnPlan& plan, cudaStrea
     return cudaLaunchKernelEx(&cfg, msa_attention_small_kernel<HD>, args) == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }
 
+template <int HD, int M>
+static int32_t launch_half(const AttnArgs& args, const AttnPlan& plan, cudaStream_t stream) {
+    static bool configured[64] = {false};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;
+    if (dev >= 0 && dev < 64 && !configured[dev]) {
+        if (cudaFuncSetAttribute(msa_attention_half_kernel<HD, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, GeoH<HD, M>::kDynSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(msa_attention_half_kernel<HD, M>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            return SS_ERR_CUDA;
+        configured[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(plan.groups), 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(kHfThreads), 1, 1);
+    cfg.dynamicSmemBytes = GeoH<HD, M>::kDynSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, msa_attention_half_kernel<HD, M>, args) == cudaSuccess ? SS_OK : SS_ERR_CUDA;
+}
+
 }  // namespace ss
 
 extern "C" size_t ss_msa_attention_workspace_bytes(const ss_attn_params* p) {
@@ -1715,7 +1769,7 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     if (p->workspace_bytes < ss_msa_attention_workspace_bytes(p)) return SS_ERR_WORKSPACE;
 
     ss::AttnArgs a;
-    const int d = p->head_dim, H = p->n_heads, tk = plan.mode == ss::kFew ? ss::kFwKeys : ss::kTileKeys;
+    const int d = p->head_dim, H = p->n_heads, tk = plan.mode == ss::kFew ? ss::kFwKeys : plan.mode == ss::kHalf ? ss::kHfKeys : ss::kTileKeys;
     const bool shared_heads = (p->kv_head_stride == 0);
     const long long kv_heads = shared_heads ? 1 : H;
     const long long kv_hstride = shared_heads ? d : p->kv_head_stride;
@@ -1727,7 +1781,7 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     // the query rows: the few-rows kernel reads them itself, and only the row blocks have a second box of stream rows
     if (ok && plan.mode != ss::kFew) ok = ss::make_map(&a.tm_qm, p->q_main, d, H, d, rows_main, hd, plan.tmax8);
     if (ok && plan.mode != ss::kFew && p->gamma > 0) ok = ss::make_map(&a.tm_qs, p->q_spec, d, H, d, rows_spec, hd, plan.s0rows > 0 ? plan.s0rows : 8);
-    if (ok && plan.mode == ss::kPair && p->gamma > 0) ok = ss::make_map(&a.tm_qs1, p->q_spec, d, H, d, rows_spec, hd, ss::kBlockRows);
+    if (ok && (plan.mode == ss::kPair || plan.n_blocks > 1) && plan.mode != ss::kFew && p->gamma > 0) ok = ss::make_map(&a.tm_qs1, p->q_spec, d, H, d, rows_spec, hd, ss::kBlockRows);
     if (!ok) return SS_ERR_CUDA;
     a.batch = p->batch; a.n_heads = H; a.gamma = p->gamma; a.max_nodes = p->max_nodes;
     a.tmax8 = plan.tmax8; a.s0rows = plan.s0rows; a.n_blocks = plan.n_blocks;
@@ -1755,6 +1809,14 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
             case 64: return ss::launch_few_rows<64>(rows, a, plan, s);
             case 80: return ss::launch_few_rows<80>(rows, a, plan, s);
             default: return ss::launch_few_rows<128>(rows, a, plan, s);
+        }
+    }
+    if (plan.mode == ss::kHalf) {
+        const bool few = plan.tmax8 + plan.spec_rows <= ss::kSmRows;
+        switch (d) {
+            case 64: return few ? ss::launch_half<64, 64>(a, plan, s) : ss::launch_half<64, 128>(a, plan, s);
+            case 80: return few ? ss::launch_half<80, 64>(a, plan, s) : ss::launch_half<80, 128>(a, plan, s);
+            default: return few ? ss::launch_half<128, 64>(a, plan, s) : ss::launch_half<128, 128>(a, plan, s);
         }
     }
     if (plan.mode == ss::kCols) {
