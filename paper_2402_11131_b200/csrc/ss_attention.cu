@@ -196,6 +196,22 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, status));
 }
 // after giving up: a short bounded wait that lets a copy already in flight land
+// the whole warp, without a branch that its lanes could take differently
+__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
+        const bool late = clock64() - t0 > kWaitCycles;
+        if (__any_sync(0xffffffffu, late || *abort != 0)) {
+            if (late && *abort == 0) {
+                *abort = 1;
+                set_status(status, SS_ERR_DEVICE_TIMEOUT);
+            }
+            return false;
+        }
+    }
+    return true;
+}
 __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
     while (!mbar_try(bar, parity) && clock64() - t0 < kWaitCycles / 16) {}

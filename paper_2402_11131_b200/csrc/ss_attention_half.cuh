@@ -84,22 +84,6 @@ __device__ __forceinline__ void tmem_st_p64(uint32_t taddr, const uint32_t (&r)[
     asm volatile("tcgen05.st.sync.aligned.16x128b.x8.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};"
                  ::SS_W16(r, 0), "r"(taddr) : "memory");
 }
-// the whole warp, without a branch that its lanes could take differently
-__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
-    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-    const long long t0 = clock64();
-    while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
-        const bool late = clock64() - t0 > kWaitCycles;
-        if (__any_sync(0xffffffffu, late || *abort != 0)) {
-            if (late && *abort == 0) {
-                *abort = 1;
-                set_status(status, SS_ERR_DEVICE_TIMEOUT);
-            }
-            return false;
-        }
-    }
-    return true;
-}
 // order keys: unsigned integers in the order of the floats
 __device__ __forceinline__ uint32_t max_key(float x) {
     const uint32_t u = __float_as_uint(x);
