@@ -1546,15 +1546,19 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
         return p.head_dim <= 80 || groups > sm_count() || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
     }
     if (q_rows <= kSmRows) {
-        // 64 rows of 64, sixteen sequences of 512 keys 41.9 / 29.8, of 2300 keys 76 / 83; of 128, 512 keys 50.9 / 47.7, 2300 keys 115 / 136
-        if (groups > sm_count()) return slots <= (d64 ? 1700 : d80 ? 1500 : 700) ? 64 : 0;
+        // more heads than SMs.  Sixteen sequences, 64 rows of 64, 130 keys 20.0 / 18.3, 330 keys 25.8 / 25.7, 1024 keys 40.3 / 47.0; of
+        // 80, 30 keys 18.5 / 17.2, 130 keys 22.4 / 22.5, 1024 keys 45.0 / 57.3; of 128, 30 keys 20.5 / 21.6, 512 keys 36.2 / 48.6
+        if (groups > sm_count()) return slots <= (d64 ? 390 : d80 ? 180 : 0) ? 64 : 0;
         // 64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
         // keys 11.0 / 12.8
         if (keys <= (d64 ? 280 : d80 ? 290 : 180)) return 64;
         // two blocks of 32 rows, two CTAs per SM: 64 rows of 64, eight heads and 4096 keys 9.7 / 7.8 (64-row blocks 10.4)
         return d64 && load <= 950 ? 32 : 0;
     }
-    // multi-stream layers.  128 rows of 64, 1024 keys 11.7 / 11.5, 2048 keys 15.1 / 16.0, eight heads and 4096 keys 13.3 / 10.7; of
+    // multi-stream layers; more row blocks than SMs: sixteen sequences, 80 rows of 64, 30 keys 17.4 / 33.9, 1024 keys 42.9 / 49.5, five
+    // sequences, 96 rows, 200 keys 9.2 / 13.8
+    if (groups > sm_count()) return 0;
+    // 128 rows of 64, 1024 keys 11.7 / 11.5, 2048 keys 15.1 / 16.0, eight heads and 4096 keys 13.3 / 10.7; of
     // 80, 200 keys 10.9 / 9.6, 1024 keys 14.1 / 14.5; of 128, 200 keys 11.6 / 11.0, 80 rows and 1024 keys 14.8 / 16.5.  320 rows of
     // 64, eight heads and 512 keys 10.4 / 8.3, 32 heads and 200 keys 10.6 / 11.8
     return load <= (d64 ? 1300 : d80 ? 700 : 320) && (blocks <= 4 || load <= 400) ? 32 : 0;

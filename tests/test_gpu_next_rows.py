@@ -83,6 +83,23 @@ def test_next_draft_special_values_follow_the_order_of_the_verification(cuda, or
     assert list(want_tok[1:4]) == [5, 17, 0] and list(want_tok[4:7]) == [250, 0, 1] and list(want_tok[13:16]) == [100, 0, 1]
 
 
+@pytest.mark.parametrize("V,k", [(4095, 8), (4097, 4), (16383, 3), (32771, 8)])       # 1, 2, 4 and 8 CTAs per row, odd rows unaligned
+def test_next_draft_of_rows_with_more_ties_than_the_candidate_list(cuda, oracle, V, k):
+    """A row's candidates are listed against a bound; rows of equal entries (one value, -inf, NaN) outgrow the list and
+    are selected by passes over the row instead."""
+    api = cuda
+    lg = np.random.default_rng(V).standard_normal((2, 1, 4, V)).astype(np.float32)
+    lg[0, 0, 1], lg[0, 0, 2], lg[0, 0, 3] = 0.5, -np.inf, np.nan
+    lg[1, 0, 0], lg[1, 0, 0, V - 1] = 0.5, 0.75
+    d_tokens = torch.zeros((2, 64), dtype=torch.int32, device="cuda")
+    ws = api.workspace(api.ss_next_draft_workspace_bytes(2, 4, V))
+    api.ss_next_draft(torch.from_numpy(lg).cuda(), None, _i32([4, 5]), k, 64, d_tokens, api.empty_trees(2), ws)
+    assert api.ss_status(ws) == 0
+    for b in range(2):
+        want, _ = oracle.next_draft(lg[b, 0], k, 4 + b, 64)
+        np.testing.assert_array_equal(d_tokens.cpu().numpy()[b, :len(want)], want)
+
+
 # ---- pruning -----------------------------------------------------------------------------------------
 @pytest.mark.parametrize("name", ["1.3b", "7b", "7b_ragged16"])
 def test_tree_prune_matches_the_oracle(cuda, oracle, name):

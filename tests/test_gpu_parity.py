@@ -298,6 +298,29 @@ def test_attention_few_rows(cuda, oracle, head_dim, T, gamma, n_heads, lengths):
                                heads=(max(n_heads - 3, 0), n_heads))
 
 
+@pytest.mark.parametrize("head_dim", [64, 80, 128])
+@pytest.mark.parametrize("T,gamma,n_heads,lengths,ramp", [
+    (64, 0, 60, (385, 448), 0.0),        # 64 rows; a tile's edge in the prefix and in the tree, rings that wrap
+    (33, 0, 53, (400, 900), 0.3),        # rows past the tree; blocks that start over
+    (12, 3, 60, (1, 70), 0.0),           # 64 rows with streams; a prefix shorter than a tile
+    (64, 4, 20, (5, 330), 0.0),          # 320 rows: three blocks, the last of 64 rows
+    (40, 4, 30, (63, 1500), 0.3),        # 200 rows, starting over
+    (21, 3, 60, (127, 129), 0.0),        # 88 rows: one block
+])
+def test_attention_more_blocks_than_sms(cuda, oracle, head_dim, T, gamma, n_heads, lengths, ramp):
+    """Ragged batches whose heads (or blocks of 128 rows) outnumber the SMs: two CTAs per SM, tiles of 64 keys."""
+    api, DeviceStep = cuda
+    cfg = W.custom_config("half", batch=3, n_layers=2, n_msa_layers=1, prefix_len_range=lengths, n_nodes=T, gamma=max(gamma, 1),
+                          max_depth=6, n_heads=n_heads, head_dim=head_dim, k_ramp=ramp, config_id=940 + T)
+    st = W.make_step(cfg)
+    dev = DeviceStep(st, layers=[1 if gamma else 0], with_lse=True)
+    for _ in range(2):
+        dev.run_attention()
+    assert api.ss_status(dev.attn_ws) == 0
+    assert (int(dev.attn_ws.view(torch.int32)[2]) > 0) == (ramp > 0)
+    assert_attention_close(oracle, st, st.layer(1 if gamma else 0), dev, 0, check_lse=True, heads=(n_heads - 2, n_heads))
+
+
 # ---- verification ---------------------------------------------------------------------------------
 def _verify_and_compare(api, dev, st, oracle):
     dev.run_verify()
@@ -338,6 +361,21 @@ def test_verify_odd_vocab_sizes_and_ties(cuda, oracle, vocab):
     st.draft_tokens = np.minimum(st.draft_tokens, vocab - 1).astype(np.int32)
     dev = DeviceStep(st, layers=[])
     _verify_and_compare(api, dev, st, oracle)
+
+
+@pytest.mark.parametrize("vocab", [4095, 4097, 8191, 16385, 32771])          # 1, 2, 2, 4 and 8 CTAs per row
+def test_verify_rows_split_over_a_cluster(cuda, oracle, vocab):
+    """The maximum at either end of a CTA's segment of a row, and rows of one value only (the lowest index wins)."""
+    api, DeviceStep = cuda
+    cfg = W.custom_config("vc%d" % vocab, batch=2, n_layers=1, prefix_len=4, n_nodes=12, gamma=0, max_depth=4, vocab=vocab,
+                          p_accept=0.8, config_id=720)
+    st = W.make_step(cfg)
+    lg = st.logits().copy()
+    for t in range(1, 12):
+        lg[0, t, (vocab * t // 8 + (t & 1) - 1) % vocab] = 50.0
+    lg[1, 3], lg[1, 4], lg[1, 5, :vocab - 1] = 0.25, -np.inf, -np.inf
+    st._logits = lg
+    _verify_and_compare(api, DeviceStep(st, layers=[]), st, oracle)
 
 
 def test_verify_duplicate_siblings_and_all_correct(cuda, oracle):
