@@ -321,6 +321,25 @@ def test_attention_more_blocks_than_sms(cuda, oracle, head_dim, T, gamma, n_head
     assert_attention_close(oracle, st, st.layer(1 if gamma else 0), dev, 0, check_lse=True, heads=(n_heads - 2, n_heads))
 
 
+@pytest.mark.parametrize("scale", [0.0, 1e-40])              # 1e-40 is subnormal: products with it may be flushed
+@pytest.mark.parametrize("kw", [
+    dict(prefix_len=100, n_nodes=12, gamma=3, n_heads=8, head_dim=64),                                  # register-level MMAs
+    dict(prefix_len=1500, n_nodes=16, gamma=3, n_heads=32, head_dim=128),                               # one tile of 64 rows
+    dict(prefix_len=1500, n_nodes=40, gamma=4, n_heads=20, head_dim=128),                               # blocks of 128 rows
+    dict(batch=3, prefix_len_range=(100, 500), n_nodes=16, gamma=3, n_heads=60, head_dim=128),          # two CTAs per SM
+    dict(batch=3, prefix_len_range=(100, 500), n_nodes=40, gamma=4, n_heads=30, head_dim=80),
+], ids=["few", "small", "blocks", "half64", "half128"])
+def test_attention_of_a_scale_of_zero_is_the_mean_of_the_visible_values(cuda, oracle, kw, scale):
+    api, DeviceStep = cuda
+    st = W.make_step(W.custom_config("scale0", n_layers=2, n_msa_layers=1, max_depth=4, config_id=980, **kw))
+    st.sm_scale = scale
+    dev = DeviceStep(st, with_lse=True)
+    dev.run_attention()
+    assert api.ss_status(dev.attn_ws) == 0
+    for i in range(2):
+        assert_attention_close(oracle, st, st.layer(i), dev, i, check_lse=True, heads=(0, 2))
+
+
 # ---- verification ---------------------------------------------------------------------------------
 def _verify_and_compare(api, dev, st, oracle):
     dev.run_verify()
