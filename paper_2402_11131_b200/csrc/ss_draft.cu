@@ -201,8 +201,7 @@ next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int
     const int g = rank / n_cta, part = rank - g * n_cta;
     __shared__ TopKShared<kDraftThreads> s;
     cluster_arrive();                                     // CTA 0 must have started before anyone stores to its shared memory
-    wait_for_previous_kernel();
-    release_next_kernel();
+    wait_for_previous_kernel();                           // (no early release of the next kernel: this one writes descriptors)
     int r = row_index ? row_index[b] : 0;
     r = min(max(r, 0), n_rows - 1);
     const Segment seg = make_segment(stream_logits, (static_cast<size_t>(b) * n_rows + r) * gamma + g, vocab, part, n_cta);
@@ -321,7 +320,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     __shared__ uint32_t s_ok[2];
     if (n_cta > 1) cluster_arrive();
     wait_for_previous_kernel();
-    release_next_kernel();
+    if (ta.mode != 0) release_next_kernel();              // (pruning writes descriptors)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
     const size_t row = static_cast<size_t>(b) * max_nodes + t;
     if (t >= max(T, 1)) {

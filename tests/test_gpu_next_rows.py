@@ -143,6 +143,60 @@ def test_tree_prune_matches_the_oracle(cuda, oracle, name):
         assert 0 < n_dropped < B * T
 
 
+# ---- attention directly behind the calls that write its trees ---------------------------------------------
+@pytest.mark.parametrize("batch,heads", [(1, 8), (6, 30)])               # both kernels that read the trees before their wait
+@pytest.mark.parametrize("writer", ["draft", "prune"])
+def test_attention_sees_the_trees_that_the_call_before_it_wrote(cuda, writer, batch, heads):
+    """compaction -> next draft (or pruning) -> attention on the new trees, which promises a stable prefix and so reads the
+    descriptors before it waits for the kernel before it.  The trees alternate between two sizes, nothing
+    synchronises; every output has to be that of its own tree."""
+    api = cuda
+    from paper_2402_11131_b200.step import DeviceStep
+    T, g, V = 31, 4, 20000
+    cfg = W.custom_config("order", batch=batch, n_layers=1, n_msa_layers=1, prefix_len=200, n_nodes=T, gamma=g, max_depth=4, vocab=V,
+                          n_heads=heads, head_dim=128, tree_kind="topk_growth", config_id=990)
+    st = W.make_step(cfg)
+    dev = DeviceStep(st)
+    dev.run_verify()
+    dev.accept_len.fill_(1)                                              # (a path of the root alone moves nothing)
+    full = dev.trees.clone()
+    rng = np.random.default_rng(991)
+    logits = torch.from_numpy(rng.standard_normal((batch, 1, g, V)).astype(np.float32)).cuda()
+    exits = torch.from_numpy(rng.standard_normal((batch, T, V)).astype(np.float32)).cuda()
+    new_tokens, index, kept, kept_tokens = (torch.zeros((batch, T), dtype=torch.int32, device="cuda") for _ in range(4))
+    prob = torch.zeros((batch, T), device="cuda")
+    ws = api.workspace(max(api.ss_next_draft_workspace_bytes(batch, g, V), api.ss_tree_prune_workspace_bytes(batch, T, V)))
+
+    def write(kind):
+        if writer == "draft":                                            # 31 nodes, or a chain of 5
+            api.ss_next_draft(logits, None, dev.bonus_token, 2 - kind, T, new_tokens, dev.trees, ws)
+        else:                                                            # all nodes, or the root alone
+            api.ss_tree_prune(exits, dev.tokens, full, (0.0, 2.0)[kind], prob, index, kept, kept_tokens, dev.trees, ws)
+
+    def outputs():
+        return dev.o_main[0].clone(), dev.o_spec[0].clone()
+
+    want = []
+    for kind in (0, 1):
+        write(kind)
+        torch.cuda.synchronize()
+        dev.o_main[0].fill_(7.0), dev.o_spec[0].fill_(7.0)
+        dev.run_attention()
+        torch.cuda.synchronize()
+        want.append(outputs())
+    assert not torch.equal(want[0][0], want[1][0])
+    got = []
+    for i in range(40):
+        dev.o_main[0].fill_(7.0), dev.o_spec[0].fill_(7.0)
+        dev.run_compact()
+        write(i & 1)
+        dev.run_attention()
+        got.append(outputs())
+    assert api.ss_status(dev.attn_ws) == 0 and api.ss_status(ws) == 0
+    for i, out in enumerate(got):
+        assert all(torch.equal(x, y) for x, y in zip(out, want[i & 1])), i
+
+
 # ---- soft and sampled verification ----------------------------------------------------------------------
 def _verify_outputs(B):
     return dict(accept_len=torch.full((B,), -7, dtype=torch.int32, device="cuda"),
