@@ -397,6 +397,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     const int argmax = i < max(T, 1) ? __ldcg(&mine_row->argmax) : 0;
     __shared__ uint32_t s_all[2][2];
     __shared__ int32_t s_am[SS_MAX_NODES];
+    if (i < T) s_tree.anc[i] = root_path(s_tree, i);      // (while the rows' results are on their way)
     s_am[i] = argmax;
     const uint32_t lo = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(okc));
     const uint32_t hi = __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(okc >> 32));
@@ -473,7 +474,11 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
     }
     if (!arrive_last(&counters[b], max(T, 1))) return;
 
-    if (i < SS_MAX_NODES) s_draw[i] = i < max(T, 1) ? __ldcg(drawn + static_cast<size_t>(b) * max_nodes + i) : -1;
+    if (i < SS_MAX_NODES) {
+        const int32_t token_i = i < max(T, 1) ? __ldcg(drawn + static_cast<size_t>(b) * max_nodes + i) : -1;
+        if (i < T) s_tree.anc[i] = root_path(s_tree, i);
+        s_draw[i] = token_i;
+    }
     __syncthreads();
     if (i >= 32) return;
     const unsigned long long ok = matching_nodes(s_tree, T, s_draw);

@@ -200,7 +200,8 @@ static __device__ __noinline__ unsigned long long best_of_any(const float* base,
 }
 
 // ---- the deepest accepted node ------------------------------------------------------------------------------------
-// Tree arrays of a sequence in shared memory, loaded by the first SS_MAX_NODES threads
+// Tree arrays of a sequence in shared memory, loaded by the first SS_MAX_NODES threads (the ancestor words come last, from
+// root_path, in the CTA that needs them)
 struct TreeShared {
     int32_t parent[SS_MAX_NODES], depth[SS_MAX_NODES], tok[SS_MAX_NODES];
     unsigned long long anc[SS_MAX_NODES];
@@ -209,17 +210,24 @@ struct TreeShared {
 // after the load would hold up the thread's scan by a round trip to L2)
 struct TreeRegs {
     int32_t parent, depth, tok;
-    unsigned long long anc;
     __device__ __forceinline__ void load(const ss_tree_desc& tree, const int32_t* tokens, int T) {
         const int i = static_cast<int>(threadIdx.x);
-        parent = -1; depth = 0; tok = -1; anc = 0ull;
-        if (i < T) { parent = tree.parent[i]; depth = tree.depth[i]; anc = tree.anc_mask[i]; tok = tokens[i]; }
+        parent = -1; depth = 0; tok = -1;
+        if (i < T) { parent = tree.parent[i]; depth = tree.depth[i]; tok = tokens[i]; }
     }
     __device__ __forceinline__ void store(TreeShared& s, int T) const {
         const int i = static_cast<int>(threadIdx.x);
-        if (i < T) { s.parent[i] = parent; s.depth[i] = depth; s.anc[i] = anc; s.tok[i] = tok; }
+        if (i < T) { s.parent[i] = parent; s.depth[i] = depth; s.tok[i] = tok; }
     }
 };
+// Ancestor word of node i from the parents (a verification needs no ancestor words in its descriptors).  The walk ends at a
+// node whose parent is not below it: such a node is never ok, nor is anything behind it.
+__device__ __forceinline__ unsigned long long root_path(const TreeShared& s, int i) {
+    unsigned long long anc = 1ull << i;
+    #pragma unroll 1
+    for (int a = i, p = s.parent[i]; p >= 0 && p < a; a = p, p = s.parent[a]) anc |= 1ull << p;
+    return anc;
+}
 // Bit c: node c's token is the one that `chosen` names for its parent (and bit 0, the root); one warp
 __device__ __forceinline__ unsigned long long matching_nodes(const TreeShared& s, int T, const int32_t* chosen) {
     unsigned long long ok = 1ull;

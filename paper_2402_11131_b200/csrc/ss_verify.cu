@@ -51,7 +51,11 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     if (!arrive_last(&counters[b], max(T, 1))) return;
 
     const int i = static_cast<int>(threadIdx.x);
-    if (i < SS_MAX_NODES) s_am[i] = i < max(T, 1) ? __ldcg(row_argmax + static_cast<size_t>(b) * max_nodes + i) : -1;
+    if (i < SS_MAX_NODES) {
+        const int32_t am_i = i < max(T, 1) ? __ldcg(row_argmax + static_cast<size_t>(b) * max_nodes + i) : -1;
+        if (i < T) s_tree.anc[i] = root_path(s_tree, i);  // (while the arg-max is on its way)
+        s_am[i] = am_i;
+    }
     __syncthreads();
     if (i >= 32) return;
     const unsigned long long ok = matching_nodes(s_tree, T, s_am);

@@ -292,6 +292,45 @@ def test_sampled_verification_matches_the_oracle(cuda, oracle, name, k):
         assert int(o["accept_len"].max()) >= 2
 
 
+def test_verification_and_pruning_need_no_ancestor_words(cuda):
+    """Descriptors that carry parents and depths only give what complete ones give: the ancestor words are the
+    attention's."""
+    api = cuda
+    st = W.make_step(W.custom_config("noanc", batch=3, n_layers=1, prefix_len=4, n_nodes=40, gamma=2, max_depth=5, vocab=500, p_accept=0.8,
+                                     tree_kind="topk_growth", config_id=992))
+    B, T, V = 3, 40, 500
+    logits, tok = torch.from_numpy(st.logits()).cuda(), _i32(st.draft_tokens)
+    u = torch.rand((B, T), generator=torch.Generator().manual_seed(5)).cuda()
+    ws = api.workspace(max(api.ss_tree_verify_workspace_bytes(B, T, V), api.ss_tree_prune_workspace_bytes(B, T, V),
+                           api.ss_tree_verify_sampled_workspace_bytes(B, T, V)))
+    results = []
+    for with_words in (True, False):
+        descs = [api.ss_tree_build(st.parent[b], 2) for b in range(B)]
+        if not with_words:
+            for d in descs:
+                C.memset(C.addressof(d) + api.TreeDesc.anc_mask.offset, 0, 8 * 64)
+        trees = api.trees_to_device(descs)
+        for call in ("greedy", "soft", "sampled", "prune"):
+            o = list(_verify_outputs(B).values())
+            node = torch.zeros((B, T), dtype=torch.int32, device="cuda")
+            prob, ent = torch.zeros((B, T), device="cuda"), torch.zeros((B, T), device="cuda")
+            extra = [torch.zeros((B, T), dtype=torch.int32, device="cuda") for _ in range(3)]
+            pruned = api.empty_trees(B)
+            if call == "greedy":
+                api.ss_tree_verify(logits, tok, trees, *o, node, ws)
+            elif call == "soft":
+                api.ss_tree_verify_soft(logits, tok, trees, 0.05, 0.3, *o, prob, ent, ws)
+            elif call == "sampled":
+                api.ss_tree_verify_sampled(logits, tok, trees, u, 2, *o, node, ws)
+            else:
+                api.ss_tree_prune(logits, tok, trees, 0.05, prob, *extra, pruned, ws)
+            assert api.ss_status(ws) == 0
+            results.append([t.cpu().clone() for t in (*o, node, prob, ent, *extra, pruned)])
+    assert int(results[0][0].max()) >= 3                                 # (accept_len: there is a path to get wrong)
+    for full, bare in zip(results[:4], results[4:]):
+        assert all(torch.equal(x, y) for x, y in zip(full, bare))
+
+
 # ---- stream insertion and value rotation ------------------------------------------------------------------
 @pytest.mark.parametrize("rows,gamma,hidden", [(64, 4, 4096), (1, 1, 8), (37, 3, 2560), (1024, 4, 4096), (0, 2, 64)])
 def test_stream_insert_is_bit_exact(cuda, oracle, rows, gamma, hidden):
