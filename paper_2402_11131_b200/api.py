@@ -33,7 +33,7 @@ _lib = None
 _native = None          # the _pycall module: takes the tensors of the per-step calls apart (see native())
 
 # number of kernels each entry point enqueues per call (for launch accounting in the benchmark); ss_kv_compact enqueues a
-# second one where kv_len_out overlaps kv_len_in
+# second one where kv_len_out overlaps one of its inputs
 LAUNCHES_PER_CALL = {"ss_msa_attention": 1, "ss_tree_verify": 1, "ss_kv_compact": 1, "ss_next_draft": 1,
                      "ss_tree_prune": 1, "ss_tree_verify_soft": 1, "ss_tree_verify_sampled": 1, "ss_stream_insert": 1,
                      "ss_value_rotate": 1}

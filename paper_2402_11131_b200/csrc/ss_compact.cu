@@ -50,8 +50,8 @@ kv_compact_kernel(uint4* __restrict__ k_all, uint4* __restrict__ v_all, int n_he
     }
 }
 
-// Where kv_len_out overlaps kv_len_in, which every CTA of the gather reads, the lengths are updated by a second,
-// stream-ordered launch; else the gather writes them itself.
+// Where kv_len_out overlaps an array that every CTA of the gather reads (the lengths, the accepted lengths or paths, the
+// starts), the lengths are updated by a second, stream-ordered launch; else the gather writes them itself.
 __global__ void kv_len_update_kernel(const int32_t* __restrict__ kv_len_in, const int32_t* __restrict__ accept_len,
                                      int32_t* __restrict__ kv_len_out, int batch) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -79,7 +79,13 @@ extern "C" int32_t ss_kv_compact(void* k_cache_all, void* v_cache_all, const ss_
     const int cols2 = 2 * lo.n_heads * chunks_per_head;
     dim3 grid((cols2 + ss::kCompactThreads - 1) / ss::kCompactThreads, lo.n_layers, batch);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool overlap = kv_len_out < kv_len_in + batch && kv_len_in < kv_len_out + batch;
+    const size_t n = static_cast<size_t>(batch);
+    const auto overlaps_out = [&](const void* p, size_t bytes) {
+        const uintptr_t out = reinterpret_cast<uintptr_t>(kv_len_out), in = reinterpret_cast<uintptr_t>(p);
+        return out < in + bytes && in < out + 4 * n;
+    };
+    const bool overlap = overlaps_out(kv_len_in, 4 * n) || overlaps_out(accept_len, 4 * n) || overlaps_out(accept_path, 4 * n * SS_PATH_STRIDE) ||
+                         overlaps_out(kv_start, 8 * n);
     // both launches may be scheduled while their predecessor drains; each waits for it before touching memory
     if (ss::launch_after_previous(ss::kv_compact_kernel, grid, dim3(ss::kCompactThreads), s, static_cast<uint4*>(k_cache_all),
                                   static_cast<uint4*>(v_cache_all), lo.n_heads, chunks_per_head, lo.layer_stride / 8,

@@ -461,6 +461,26 @@ def test_compaction_long_path_and_aliased_lengths(cuda, oracle):
     assert list(dev.accept_path[0, :4].cpu().numpy()) == [0, 1, 3, 5]
 
 
+@pytest.mark.parametrize("array", ["kv_len", "accept_len", "accept_path", "kv_start"])
+def test_compaction_writes_the_lengths_over_any_of_its_inputs(cuda, oracle, array):
+    """kv_len_out in the memory of an array that the gather reads: the gather sees the old words throughout."""
+    api, DeviceStep = cuda
+    cfg = W.custom_config("overlap", batch=3, n_layers=3, n_msa_layers=1, prefix_len=37, n_nodes=12, gamma=1, max_depth=4, vocab=97,
+                          p_accept=0.9, n_heads=8, head_dim=64, config_id=735)
+    st = W.make_step(cfg)
+    want, dev = DeviceStep(st), DeviceStep(st)
+    for d in (want, dev):
+        d.run_verify()
+    want.run_compact()
+    words = getattr(dev, array).view(torch.int32)
+    dev.kv_len_out = words.reshape(-1)[:3]
+    dev.run_compact()
+    torch.cuda.synchronize()
+    assert torch.equal(dev.kv_len_out, want.kv_len_out) and int(want.accept_len.max()) >= 2
+    assert torch.equal(dev.k_all.view(torch.int16), want.k_all.view(torch.int16))
+    assert torch.equal(dev.v_all.view(torch.int16), want.v_all.view(torch.int16))
+
+
 def test_two_steps_in_a_row_with_aliased_lengths(cuda, oracle):
     """A second step on the cache that the first step's compaction left behind: the lengths are updated in
     place (kv_len_out aliases kv_len), the accepted nodes have become prefix, new tree nodes are appended
