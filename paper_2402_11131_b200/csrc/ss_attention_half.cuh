@@ -310,9 +310,6 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             bool ok = request(false, n_k);
             while (ok && (n_k < sp.n || n_v < sp.n)) ok = request(false, n_k) && request(true, n_v);
             if (kMax) n_v = 0;
-            // gave up: let the copies already in flight land before the CTA leaves (a CTA that starts over waits below)
-            if (!ok && *reinterpret_cast<volatile int*>(&c.abort) == 1)
-                land();
         }
     } else if (warp == 9) {
         bool ok = sp.n == 0 || mbar_wait_uniform(smem_u32(&c.q_full), 0, &c.abort, status);
@@ -498,6 +495,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     __syncwarp();     // the single-lane roles rejoin their warps
     };   // run_tiles
 
+    int n_drains = 0;                                      // phases of the drain barrier so far
     run_tiles(std::false_type{}, early_k, early_v);
     if (__syncthreads_or(*reinterpret_cast<volatile int*>(&c.abort) == 2)) {
         // A reference did not hold.  Twice: what is in flight lands, the barriers are set up anew, the tiles run again --
@@ -509,8 +507,9 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
                 mbar_drain(smem_u32(&c.q_full), 0);
             } else if (warp == 9) {
                 tc_commit_w(lead, smem_u32(&c.drain));
-                mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(pass));
+                mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(n_drains & 1));
             }
+            ++n_drains;
             __syncwarp();
             if (is_softmax) { tmem_wait_ld(); tmem_wait_st(); }
             tc_fence_before();
@@ -549,6 +548,19 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     // The rings are idle: every copy has landed and every MMA is complete.  The two threads that hold the same rows, one per
     // team, exchange their sums; then each finishes its team's columns of the rows.
     const bool aborted = __syncthreads_or(*reinterpret_cast<volatile int*>(&c.abort) != 0);
+    if (aborted) {
+        // A wait ran out.  Shared memory and TMEM are not given up before what is in flight has landed: copies (the producer may
+        // have requested its last one long before another role gave up), MMAs with their commits, the softmax threads' stores.
+        if (producer) {
+            land();
+            mbar_drain(smem_u32(&c.q_full), 0);
+        } else if (warp == 9) {
+            tc_commit_w(lead, smem_u32(&c.drain));
+            mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(n_drains & 1));
+        }
+        __syncwarp();
+        if (is_softmax) { tmem_wait_ld(); tmem_wait_st(); }
+    }
     if (is_softmax && sp.n > 0 && !aborted) {
         const uint32_t x_base = k_base;                                       // [team][M rows] sums
         #pragma unroll

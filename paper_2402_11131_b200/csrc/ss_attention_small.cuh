@@ -80,10 +80,13 @@ struct CtrlS {
     // neither two phases ahead of the wait nor behind it.  With one barrier per copy a copy could find the other
     // copy's barrier two phases ahead (tiles j - 3 and j - 1 both complete), and its parity wait then never ends.
     unsigned long long pv_done[4];
+    unsigned long long drain[2];               // a CTA that gives up: the last MMAs of the S and of the P V issuer complete
     unsigned long long anc[SS_MAX_NODES];
     alignas(16) float xch[4][2 * kSmRows];     // exchange between the four threads of a lane (maxima, row sums)
     uint32_t tmem_base;
     int abort;
+    int requested[2];                          // K tiles, V tiles requested so far
+    int gave_up[2];                            // a softmax thread of the copy has given up (set before the copy's reducing barrier)
     int wait_limit;                            // bound of every wait, in units of 1024 cycles
 };
 
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     if (tid == 0) {
         mbar_init(smem_u32(&c.q_full), 1);
         for (int s = 0; s < kSmMaxSlots / 2; ++s) { mbar_init(smem_u32(&c.slot_full[0][s]), 1); mbar_init(smem_u32(&c.slot_full[1][s]), 1); }
-        c.abort = 0;
+        c.abort = c.gave_up[0] = c.gave_up[1] = 0;
         c.wait_limit = static_cast<int>(kWaitCycles >> 10);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&a.tm_qm); tma_prefetch_desc(&a.tm_k); tma_prefetch_desc(&a.tm_v);
@@ -199,6 +202,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             mbar_init(smem_u32(&c.p_full[s]), 8);
         }
         for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&c.pv_done[s]), 1);
+        for (int s = 0; s < 2; ++s) mbar_init(smem_u32(&c.drain[s]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     auto dependency_wait = [&]() {
@@ -279,6 +283,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
         }
         for (int j = n_pre; j < n_early_k; ++j) load_tile(0, j, j);
         for (int j = 0; j < n_early; ++j) load_tile(1, j, j);
+        c.requested[0] = n_early_k; c.requested[1] = n_early;
         SS_TRC(0, 5);
     }
     if (tid >= kAuxThreads && tid < kAuxThreads + SS_MAX_NODES) c.anc[tid - kAuxThreads] = __ldcg(&a.trees[b].anc_mask[tid - kAuxThreads]);
@@ -295,8 +300,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     auto wait_tile_full = [&](int kind, const Ring& r) {
         return mbar_wait_s(smem_u32(&c.slot_full[kind][r.slot]), static_cast<uint32_t>(r.round & 1), &c, status);
     };
-    // the tiles after the early ones, each as soon as its slot is free; a producer that gives up lets the
-    // copies already in flight land before the CTA leaves
+    // the tiles after the early ones, each as soon as its slot is free
     auto produce = [&](int kind) {
         Ring r;
         r.start();
@@ -309,13 +313,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             if (kind == 0) SS_TRC(0, 8 + j);
             if (ok) { load_tile(kind, j, r.slot); r.advance(n_ring); }
         }
-        if (!ok) {
-            const int issued = r.slot + r.round * n_ring;
-            Ring d;
-            d.start();
-            for (int i = 0; i < issued; ++i, d.advance(n_ring))
-                if (i >= issued - n_ring) mbar_drain(smem_u32(&c.slot_full[kind][d.slot]), static_cast<uint32_t>(d.round & 1));
-        }
+        c.requested[kind] = r.slot + r.round * n_ring;
     };
 
     // =============================== warps 0 and 3: tile requests ================================
@@ -512,10 +510,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
                 // one reducing barrier per tile: did a score outgrow its reference, or did a wait run out
                 // (a thread's 32 exponentials sum to at most 32 unless a score is above the reference; past
                 // 32 * 2^8 one of them is more than 2^8 above it)
+                if (!ok) *reinterpret_cast<volatile int*>(&c.gave_up[copy]) = 1;
                 const uint32_t any = bar_red_or(4 + copy, 256, !ok || lsum > 32.f * 256.f);
                 if (leader) SS_TRC(3, 10 + 6 * j);
                 if (!any) { l_part += lsum; break; }
-                if (*reinterpret_cast<volatile int*>(&c.abort)) { leave = true; break; }
+                // (all of the copy's threads leave, or none: what follows has barriers.  The abort flag could be set by another role
+                // while they read it.)
+                if (*reinterpret_cast<volatile int*>(&c.gave_up[copy])) { leave = true; break; }
                 ok = raise() && ok;
                 if (attempt == 2) l_part += lsum;
             }
@@ -677,6 +678,23 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     if (tid == kAuxThreads) SS_TRC(5, 5);
     tc_fence_before();
     __syncthreads();
+    if (*reinterpret_cast<volatile int*>(&c.abort) != 0) {                    // (CTA-uniform: every role has left its loop)
+        // A wait ran out.  Shared memory and TMEM are not given up before what is in flight has landed: copies (a producer may
+        // have requested its last one long before another role gave up), MMAs with their commits, the softmax threads' stores.
+        if (tid == 0 || tid == 96) {
+            const int kind = tid == 0 ? 0 : 1, n = c.requested[kind];
+            for (int s = 0; s < n_ring; ++s)
+                if (n > s) mbar_drain(smem_u32(&c.slot_full[kind][s]), static_cast<uint32_t>(((n - 1 - s) / n_ring) & 1));
+            if (tid == 0) mbar_drain(smem_u32(&c.q_full), 0);
+        } else if (warp == 1 || warp == 2) {
+            tc_commit_w(elect_lane(), smem_u32(&c.drain[warp - 1]));          // (the lane that issued the MMAs: the election is deterministic)
+            mbar_drain(smem_u32(&c.drain[warp - 1]), 0);
+        }
+        __syncwarp();
+        if (warp >= 4) { tmem_wait_ld(); tmem_wait_st(); }
+        tc_fence_before();
+        __syncthreads();
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();

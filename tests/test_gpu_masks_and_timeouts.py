@@ -143,6 +143,40 @@ def test_a_wait_that_runs_out_reports_a_timeout_and_the_stream_stays_usable(cuda
     assert int(words[2:].abs().max()) == 0                     # a call leaves the partial rows' area zero again
 
 
+SHORT_BOUND = {                    # heads of at most 64 rows
+    "split": dict(prefix_len=3000, n_nodes=64, gamma=0, n_heads=32),
+    "whole": dict(prefix_len=3000, n_nodes=64, gamma=0, n_heads=100),
+}
+
+
+@pytest.mark.parametrize("name", list(SHORT_BOUND))
+def test_a_call_whose_waits_run_out_ends_and_leaves_the_stream_usable(cuda, oracle, name):
+    """With a bound of 1024 cycles the waits for the first tiles, all of which the grid requests at once, run out in the
+    middle of the pipeline, in any of its roles.  The call ends, with whatever it had in flight, and the same call with
+    the default bound on a cleared workspace matches the oracle."""
+    api, DeviceStep = cuda
+    cfg = W.custom_config("short", n_layers=1, n_msa_layers=0, max_depth=4, head_dim=128, tree_kind="topk_growth", config_id=811,
+                          **SHORT_BOUND[name])
+    st = W.make_step(cfg)
+    dev = DeviceStep(st)
+    words = dev.attn_ws.view(torch.int32)
+    flush = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    seen = set()
+    for _ in range(10):
+        flush.zero_()                                          # the tiles come from HBM
+        words.zero_()
+        words[1] = 1
+        dev.run_attention()
+        seen.add(api.ss_status(dev.attn_ws))
+    assert seen <= {0, api.SS_ERR_DEVICE_TIMEOUT}
+    print(name, seen)
+    words.zero_()
+    for _ in range(2):
+        dev.run_attention()
+    assert api.ss_status(dev.attn_ws) == 0
+    assert_attention_close(oracle, st, st.layer(0), dev, 0, heads=(0, 2), **({} if cfg.batch == 1 else dict(seqs=[0])))
+
+
 def test_no_wait_runs_out_over_many_replays(cuda):
     """The attention kernels' roles meet on phase-parity barriers; a waiter that falls two phases behind one of
     them would wait until its bound runs out (a one-second stall and SS_ERR_DEVICE_TIMEOUT).  Whether that can
