@@ -50,6 +50,7 @@
 // kernel is bounded and reports SS_ERR_DEVICE_TIMEOUT.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cfloat>
 #include <type_traits>
 
 #include "ss_common.cuh"
@@ -106,7 +107,7 @@ struct alignas(64) AttnArgs {
     int head_coord;                  // 1, or 0 when all heads share one K/V (head stride 0)
     int gamma_magic;                 // ceil(65536 / gamma): x / gamma == (x * gamma_magic) >> 16 for x < 256
     int prefix_stable;               // the caller's SS_ATTN_PREFIX_STABLE promise
-    float scale_log2;                // sm_scale * log2(e)
+    float scale_log2;                // sm_scale * log2(e), never zero: a score that is hidden by -inf stays so when it is scaled
     const __nv_bfloat16* q_main;
     const __nv_bfloat16* q_spec;
     __nv_bfloat16* o_main;
@@ -1813,6 +1814,8 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     a.gamma_magic = p->gamma > 0 ? (65536 + p->gamma - 1) / p->gamma : 0;
     a.prefix_stable = (p->flags & SS_ATTN_PREFIX_STABLE) ? 1 : 0;
     a.scale_log2 = p->sm_scale * 1.4426950408889634f;
+    // (1e-37 makes every score zero just as well; below the smallest normal number products may be flushed)
+    if (fabsf(a.scale_log2) < FLT_MIN) a.scale_log2 = 1e-37f;
     a.q_main = static_cast<const __nv_bfloat16*>(p->q_main);
     a.q_spec = static_cast<const __nv_bfloat16*>(p->q_spec);
     a.o_main = static_cast<__nv_bfloat16*>(p->o_main);

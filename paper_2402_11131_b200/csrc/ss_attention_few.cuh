@@ -350,8 +350,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
             off_k[j] = static_cast<uint32_t>(mrow + 8 * upper) * 128u + (static_cast<uint32_t>((2 * j + odd) ^ mrow) << 4);
             off_v[j] = static_cast<uint32_t>(mrow + 8 * odd) * 128u + (static_cast<uint32_t>((2 * j + upper) ^ mrow) << 4);
         }
-        // (a scale of zero is as good as one that makes every score zero: a hidden score is -inf before and after scaling)
-        const float scale = a.scale_log2 == 0.f ? 1e-37f : fabsf(a.scale_log2);
+        const float scale = fabsf(a.scale_log2);
         const unsigned long long scale2 = pack_f32x2(scale, scale);
         auto load_q = [&](int ks, uint32_t (&f)[4]) { ldsm_x4(q_base + static_cast<uint32_t>(rg * 16 * 128) + off_v[ks & 3] + (ks >> 2) * G::kQHalf, f); };
         uint32_t qf[G::kQInRegs ? G::kKSteps : 1][4];

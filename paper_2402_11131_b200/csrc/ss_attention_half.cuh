@@ -262,8 +262,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     const int team = warp >> 2, quad = lane & 3, row_a = M == 64 ? 16 * (warp & 3) + (lane >> 2) : 32 * (warp & 3) + lane;
     RowInfo ri[G::kRows];
     unsigned long long anc[G::kRows];
-    // (a scale of zero is as good as one that makes every score zero; a hidden score is -inf after scaling, whatever its sign)
-    const float scale = a.scale_log2 == 0.f ? 1e-37f : a.scale_log2;
+    const float scale = a.scale_log2;                      // (a hidden score is -inf after scaling, whatever the sign)
     const uint32_t hidden = scale < 0.f ? 0x7f800000u : 0xff800000u;
     // reference; sums of the weights as rounded to bf16, and before
     float m_ref[G::kRows], l_part[G::kRows], l_exact[G::kRows];
