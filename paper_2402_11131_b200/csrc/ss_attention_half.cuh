@@ -43,6 +43,7 @@ struct CtrlH {
     unsigned long long drain;                      // start over: the issuer's last MMAs complete
     uint32_t row_ref[128];                         // the rows' references; start over: their exact maxima, as order keys
     uint32_t tmem_base;
+    int n_drains;                                  // completed phases of the drain barrier
     int abort;                                     // 1: a wait ran out of time; 2: a reference did not hold, start over
 };
 
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         tma_prefetch_desc(&a.tm_k); tma_prefetch_desc(&a.tm_v); tma_prefetch_desc(&a.tm_qm);
         if (a.gamma > 0) { tma_prefetch_desc(M == 128 && rb > 0 ? &a.tm_qs1 : &a.tm_qs); tma_prefetch_desc(&a.tm_ks); tma_prefetch_desc(&a.tm_vs); }
     } else if (tid == 0) {
-        c.abort = 0;
+        c.abort = c.n_drains = 0;
         for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&c.m_full[s]), 1);
         mbar_init(smem_u32(&c.drain), 1);
         init_tiles();
@@ -494,7 +495,6 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     __syncwarp();     // the single-lane roles rejoin their warps
     };   // run_tiles
 
-    int n_drains = 0;                                      // phases of the drain barrier so far
     run_tiles(std::false_type{}, early_k, early_v);
     if (__syncthreads_or(*reinterpret_cast<volatile int*>(&c.abort) == 2)) {
         // A reference did not hold.  Twice: what is in flight lands, the barriers are set up anew, the tiles run again --
@@ -506,9 +506,8 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
                 mbar_drain(smem_u32(&c.q_full), 0);
             } else if (warp == 9) {
                 tc_commit_w(lead, smem_u32(&c.drain));
-                mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(n_drains & 1));
+                mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(pass));
             }
-            ++n_drains;
             __syncwarp();
             if (is_softmax) { tmem_wait_ld(); tmem_wait_st(); }
             tc_fence_before();
@@ -522,6 +521,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
                 init_rings();
                 init_tiles();
                 c.abort = 0;
+                c.n_drains = pass + 1;
                 if (pass == 0) atomicAdd(a.status + 2, 1);            // diagnostics: blocks that started over
             }
             if (pass == 0 && tid < 128) c.row_ref[tid] = kNoMax;
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             mbar_drain(smem_u32(&c.q_full), 0);
         } else if (warp == 9) {
             tc_commit_w(lead, smem_u32(&c.drain));
-            mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(n_drains & 1));
+            mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(*reinterpret_cast<volatile int*>(&c.n_drains) & 1));
         }
         __syncwarp();
         if (is_softmax) { tmem_wait_ld(); tmem_wait_st(); }
