@@ -196,13 +196,42 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, status));
 }
-// after giving up: a short bounded wait that lets a copy already in flight land
+// Waits whose bound is in the kernel's control block (abort; wait_limit, in units of 1024 cycles): the caller may shorten it
+// through the workspace header.
+__device__ __forceinline__ long long limit_cycles(const int& wait_limit) {
+    return static_cast<long long>(*const_cast<const volatile int*>(&wait_limit)) << 10;
+}
+__device__ __noinline__ bool mbar_wait_limit_slow(uint32_t bar, uint32_t parity, volatile int* abort, const int* wait_limit, int* status) {
+    const long long t0 = clock64(), limit = limit_cycles(*wait_limit);
+    for (;;) {
+        for (int i = 0; i < 256; ++i) {
+            if (mbar_try(bar, parity)) return true;
+            if (*abort) return false;
+        }
+        if (clock64() - t0 > limit) {
+            *abort = 1;
+            set_status(status, SS_ERR_DEVICE_TIMEOUT);
+            return false;
+        }
+    }
+}
+template <typename Control>
+__device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, Control* c, int* status) {
+    if (mbar_try(bar, parity)) return true;
+    return mbar_wait_limit_slow(bar, parity, &c->abort, &c->wait_limit, status);
+}
+template <typename Control>
+__device__ __forceinline__ bool mbar_wait_limit_warp(uint32_t bar, uint32_t parity, Control* c, int* status) {
+    return __all_sync(0xffffffffu, mbar_wait_limit(bar, parity, c, status));
+}
 // the whole warp, without a branch that its lanes could take differently
-__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+template <typename Control>
+__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, Control* c, int* status) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    volatile int* const abort = &c->abort;
     const long long t0 = clock64();
     while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
-        const bool late = clock64() - t0 > kWaitCycles;
+        const bool late = clock64() - t0 > limit_cycles(c->wait_limit);
         if (__any_sync(0xffffffffu, late || *abort != 0)) {
             if (late && *abort == 0) {
                 *abort = 1;
@@ -213,6 +242,7 @@ __device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity,
     }
     return true;
 }
+// after giving up: a short bounded wait that lets a copy already in flight land
 __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
     while (!mbar_try(bar, parity) && clock64() - t0 < kWaitCycles / 16) {}

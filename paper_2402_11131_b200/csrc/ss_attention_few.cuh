@@ -80,26 +80,9 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, 
     asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-// bounded wait whose limit comes from the control block (the caller may shorten it through the workspace header)
-__device__ __noinline__ bool mbar_wait_slow_f(uint32_t bar, uint32_t parity, CtrlF* c, int* status) {
-    const long long t0 = clock64();
-    volatile int* abort = &c->abort;
-    const long long limit = static_cast<long long>(*reinterpret_cast<volatile int*>(&c->wait_limit)) << 10;
-    for (;;) {
-        for (int i = 0; i < 256; ++i) {
-            if (mbar_try(bar, parity)) return true;
-            if (*abort) return false;
-        }
-        if (clock64() - t0 > limit) {
-            *abort = 1;
-            set_status(status, SS_ERR_DEVICE_TIMEOUT);
-            return false;
-        }
-    }
-}
 __device__ __forceinline__ bool mbar_wait_warp_f(uint32_t bar, uint32_t parity, CtrlF* c, int* status) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait_slow_f(bar, parity, c, status));
+    return __all_sync(0xffffffffu, mbar_wait_limit_slow(bar, parity, &c->abort, &c->wait_limit, status));
 }
 
 // Visible keys x .. x + 31 of a row (Eq. 1 / Eq. 2 with the tree mask of App. A): the prefix and the node's root path, or
@@ -326,10 +309,10 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
                 st_shared_v4(q_base + (pc >> 3) * G::kQHalf + row * 128u + (static_cast<uint32_t>((pc ^ row) & 7) << 4), q[k].x, q[k].y, q[k].z, q[k].w);
         }
         if (tid == 0) {
-            // the caller may shorten the bound of the device-side waits (workspace word 1, units of 1024 cycles)
+            // the caller may shorten the bound of the waits of a head of at most 64 rows (workspace word 1, units of 1024 cycles)
             int lim;
             asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(lim) : "l"(a.status + 1) : "memory");
-            if (lim > 0) *reinterpret_cast<volatile int*>(&c.wait_limit) = lim;
+            if (lim > 0 && gridDim.y * G::kRows <= 64) *reinterpret_cast<volatile int*>(&c.wait_limit) = lim;
         }
     }
     if (tid == 0 && (over || bad_smem)) set_status(status, bad_smem ? SS_ERR_CUDA : SS_ERR_CAPACITY);

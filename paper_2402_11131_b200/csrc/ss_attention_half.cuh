@@ -43,6 +43,7 @@ struct CtrlH {
     unsigned long long drain;                      // start over: the issuer's last MMAs complete
     uint32_t row_ref[128];                         // the rows' references; start over: their exact maxima, as order keys
     uint32_t tmem_base;
+    int wait_limit;                                // bound of every wait, in units of 1024 cycles
     int n_drains;                                  // completed phases of the drain barrier
     int abort;                                     // 1: a wait ran out of time; 2: a reference did not hold, start over
 };
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         if (a.gamma > 0) { tma_prefetch_desc(M == 128 && rb > 0 ? &a.tm_qs1 : &a.tm_qs); tma_prefetch_desc(&a.tm_ks); tma_prefetch_desc(&a.tm_vs); }
     } else if (tid == 0) {
         c.abort = c.n_drains = 0;
+        c.wait_limit = static_cast<int>(kWaitCycles >> 10);
         for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&c.m_full[s]), 1);
         mbar_init(smem_u32(&c.drain), 1);
         init_tiles();
@@ -247,6 +249,12 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             if (t < early_k) load_tile(false, t, t);
             load_tile(true, t, t);
         }
+        if (M == 64) {
+            // the caller may shorten the bound of the waits of a head of at most 64 rows (workspace word 1, units of 1024 cycles)
+            int lim;
+            asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(lim) : "l"(a.status + 1) : "memory");
+            if (lim > 0) *reinterpret_cast<volatile int*>(&c.wait_limit) = lim;
+        }
     }
     int n_k = early_k, n_v = early_v;                      // tiles requested so far (producer)
     // (producer) waits until every copy requested so far has landed
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             auto request = [&](bool is_v, int& t) {
                 if (t >= sp.n) return true;
                 const int ring = is_v ? G::kRingV : G::kRingK, st = t % ring;
-                if (t >= ring && !mbar_wait(smem_u32(is_v ? &c.v_empty[st] : &c.k_empty[st]), (t / ring - 1) & 1, &c.abort, status)) return false;
+                if (t >= ring && !mbar_wait_limit(smem_u32(is_v ? &c.v_empty[st] : &c.k_empty[st]), (t / ring - 1) & 1, &c, status)) return false;
                 load_tile(is_v, t, st);
                 ++t;
                 return true;
@@ -312,7 +320,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             if (kMax) n_v = 0;
         }
     } else if (warp == 9) {
-        bool ok = sp.n == 0 || mbar_wait_uniform(smem_u32(&c.q_full), 0, &c.abort, status);
+        bool ok = sp.n == 0 || mbar_wait_uniform(smem_u32(&c.q_full), 0, &c, status);
         if (!ok && lane == 0) mbar_drain(smem_u32(&c.q_full), 0);
         const uint64_t dq = desc_k_major(uniform(q_base));
         const uint32_t ut_o = uniform(tmem_o), ut_s = uniform(tmem_s);
@@ -320,7 +328,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         rk.start(); rv.start();
         int ts = 0;                                       // next tile of S
         auto issue_s = [&]() {
-            if (!mbar_wait_uniform(smem_u32(&c.k_full[rk.slot]), rk.round & 1, &c.abort, status)) return false;
+            if (!mbar_wait_uniform(smem_u32(&c.k_full[rk.slot]), rk.round & 1, &c, status)) return false;
             tc_fence_after();
             const uint64_t dk = desc_k_major(uniform(k_base + rk.slot * G::kSlotBytes));
             const uint32_t sd = uniform(ut_s + (ts & 1) * kHfKeys);
@@ -339,8 +347,8 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         if (ok && sp.n > 1) ok = issue_s();
         for (int t = 0; ok && t < sp.n; ++t, rv.advance(G::kRingV)) {
             const int buf = t & 1;
-            if (!kMax && !mbar_wait_uniform(smem_u32(&c.v_full[rv.slot]), rv.round & 1, &c.abort, status)) break;
-            if (!mbar_wait_uniform(smem_u32(&c.p_full[buf]), (t >> 1) & 1, &c.abort, status)) break;
+            if (!kMax && !mbar_wait_uniform(smem_u32(&c.v_full[rv.slot]), rv.round & 1, &c, status)) break;
+            if (!mbar_wait_uniform(smem_u32(&c.p_full[buf]), (t >> 1) & 1, &c, status)) break;
             tc_fence_after();
             if (!kMax) {
                 const uint64_t dv = desc_mn_major(uniform(v_base + rv.slot * G::kSlotBytes), G::kBoxBytes);
@@ -356,13 +364,13 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     } else {
         bool ok = true;
         if (!kMax && !exact && team == 1 && sp.n > 1) {
-            ok = mbar_wait_warp(smem_u32(&c.m_full[warp & 3]), 0, &c.abort, status);
+            ok = mbar_wait_limit_warp(smem_u32(&c.m_full[warp & 3]), 0, &c, status);
             #pragma unroll
             for (int e = 0; e < G::kRows; ++e) m_ref[e] = __uint_as_float(c.row_ref[row_a + 8 * e]);
         }
         #pragma unroll 1
         for (int t = team; ok && t < sp.n; t += 2) {
-            if (!mbar_wait_warp(smem_u32(&c.s_full[team]), (t >> 1) & 1, &c.abort, status)) break;
+            if (!mbar_wait_limit_warp(smem_u32(&c.s_full[team]), (t >> 1) & 1, &c, status)) break;
             tc_fence_after();
             const int x0 = sp.first_key(t);
             const bool cache = sp.is_cache(t);
@@ -473,7 +481,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             // is NaN, so they are cleared before P V reads them
             if (!kMax && nvk < kHfKeys) {
                 const int vs = t % G::kRingV;
-                if (!mbar_wait_warp(smem_u32(&c.v_full[vs]), static_cast<uint32_t>((t / G::kRingV) & 1), &c.abort, status)) break;
+                if (!mbar_wait_limit_warp(smem_u32(&c.v_full[vs]), static_cast<uint32_t>((t / G::kRingV) & 1), &c, status)) break;
                 constexpr int kRowPieces = G::kHalves * 8;            // 16-byte pieces of a V row
                 for (int i = tid & 127; i < (kHfKeys - nvk) * kRowPieces; i += 128) {
                     const int vr = nvk + i / kRowPieces, pc = i % kRowPieces;
@@ -488,7 +496,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         }
         // the last P V must be complete before the accumulator is read; products complete in issue order
         if (!kMax && sp.n > 0 && *reinterpret_cast<volatile int*>(&c.abort) == 0) {
-            mbar_wait_warp(smem_u32(&c.o_done), 0, &c.abort, status);
+            mbar_wait_limit_warp(smem_u32(&c.o_done), 0, &c, status);
             tc_fence_after();
         }
     }

@@ -100,31 +100,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
                  ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
 }
-// waits whose limit comes from the control block (the caller may shorten it through the workspace header)
-__device__ __noinline__ bool mbar_wait_slow_s(uint32_t bar, uint32_t parity, CtrlS* c, int* status) {
-    const long long t0 = clock64();
-    volatile int* abort = &c->abort;
-    const long long limit = static_cast<long long>(*reinterpret_cast<volatile int*>(&c->wait_limit)) << 10;
-    for (;;) {
-        for (int i = 0; i < 256; ++i) {
-            if (mbar_try(bar, parity)) return true;
-            if (*abort) return false;
-        }
-        if (clock64() - t0 > limit) {
-            *abort = 1;
-            set_status(status, SS_ERR_DEVICE_TIMEOUT);
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ bool mbar_wait_s(uint32_t bar, uint32_t parity, CtrlS* c, int* status) {
-    if (mbar_try(bar, parity)) return true;
-    return mbar_wait_slow_s(bar, parity, c, status);
-}
-__device__ __forceinline__ bool mbar_wait_warp_s(uint32_t bar, uint32_t parity, CtrlS* c, int* status) {
-    return __all_sync(0xffffffffu, mbar_wait_s(bar, parity, c, status));
-}
-
 template <int HD>
 __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(const __grid_constant__ AttnArgs a) {
     using G = GeoS<HD>;
@@ -296,20 +271,16 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     const uint32_t tmem_s = tmem + 128;                    // two score buffers of 128 columns, one per copy
     const uint32_t tmem_p = tmem + 384;                    // two P buffers of 64 columns (128 keys as bf16), one per copy
     int* const status = a.status;
-    // tile j of a kind: slot j mod depth, filled for the (j / depth)-th time
-    auto wait_tile_full = [&](int kind, const Ring& r) {
-        return mbar_wait_s(smem_u32(&c.slot_full[kind][r.slot]), static_cast<uint32_t>(r.round & 1), &c, status);
-    };
     // the tiles after the early ones, each as soon as its slot is free
     auto produce = [&](int kind) {
         Ring r;
         r.start();
         const int first = kind ? n_early : n_early_k;
         for (int j = 0; j < first; ++j) r.advance(n_ring);
-        bool ok = mbar_wait_s(smem_u32(&c.q_full), 0, &c, status);
+        bool ok = mbar_wait_limit(smem_u32(&c.q_full), 0, &c, status);
         int j = first;
         for (; ok && j < sp.n_tiles; ++j) {
-            if (r.round > 0) ok = mbar_wait_s(smem_u32(&c.slot_empty[kind][r.slot]), (r.round - 1) & 1, &c, status);
+            if (r.round > 0) ok = mbar_wait_limit(smem_u32(&c.slot_empty[kind][r.slot]), (r.round - 1) & 1, &c, status);
             if (kind == 0) SS_TRC(0, 8 + j);
             if (ok) { load_tile(kind, j, r.slot); r.advance(n_ring); }
         }
@@ -335,7 +306,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     else if (warp == 1) {
         {
             const uint32_t lead = elect_lane();
-            bool ok = mbar_wait_uniform(smem_u32(&c.q_full), 0, &c.abort, status);
+            bool ok = mbar_wait_uniform(smem_u32(&c.q_full), 0, &c, status);
             if (!ok) mbar_drain(smem_u32(&c.q_full), 0);
             SS_TRC(1, 0);
             const uint64_t dq = desc_k_major(uniform(q_base));
@@ -343,10 +314,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             r.start();
             for (int j = 0; ok && j < sp.n_tiles; ++j) {
                 const int buf = j & 1;
-                if (!mbar_wait_uniform(smem_u32(&c.slot_full[0][r.slot]), static_cast<uint32_t>(r.round & 1), &c.abort, status)) break;
+                if (!mbar_wait_uniform(smem_u32(&c.slot_full[0][r.slot]), static_cast<uint32_t>(r.round & 1), &c, status)) break;
                 SS_TRC(1, 8 + 4 * j);
                 // the copy's scores of its tile before must be in registers
-                if (j >= 2 && !mbar_wait_uniform(smem_u32(&c.s_free[buf]), ((j >> 1) - 1) & 1, &c.abort, status)) break;
+                if (j >= 2 && !mbar_wait_uniform(smem_u32(&c.s_free[buf]), ((j >> 1) - 1) & 1, &c, status)) break;
                 SS_TRC(1, 9 + 4 * j);
                 tc_fence_after();
                 const uint64_t dk = desc_k_major(uniform(slot_addr(0, r.slot)));
@@ -370,12 +341,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             const uint32_t lead = elect_lane();
             Ring rv;
             rv.start();
-            bool okq = mbar_wait_uniform(smem_u32(&c.q_ready), 0, &c.abort, status);     // the P buffers' constant zeros are in place
+            bool okq = mbar_wait_uniform(smem_u32(&c.q_ready), 0, &c, status);     // the P buffers' constant zeros are in place
             for (int j = 0; okq && j < sp.n_tiles; ++j) {
                 const int buf = j & 1;
-                if (!mbar_wait_uniform(smem_u32(&c.slot_full[1][rv.slot]), static_cast<uint32_t>(rv.round & 1), &c.abort, status)) break;
+                if (!mbar_wait_uniform(smem_u32(&c.slot_full[1][rv.slot]), static_cast<uint32_t>(rv.round & 1), &c, status)) break;
                 SS_TRC(2, 8 + 4 * j);
-                if (!mbar_wait_uniform(smem_u32(&c.p_full[buf]), (j >> 1) & 1, &c.abort, status)) break;
+                if (!mbar_wait_uniform(smem_u32(&c.p_full[buf]), (j >> 1) & 1, &c, status)) break;
                 SS_TRC(2, 9 + 4 * j);
                 tc_fence_after();
                 const uint64_t dv = desc_mn_major(uniform(slot_addr(1, rv.slot)), G::kBoxBytes);
@@ -420,12 +391,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
         const uint32_t p_addr = tmem_p + lane_base + static_cast<uint32_t>(copy * 64 + 16 * w4);   // my 32 keys of a tile as bf16
         const uint32_t o_addr = tmem_o + lane_base + 32u * w4;
         auto wait_pv_tile = [&](int t) {                                       // P V of tile t complete
-            return mbar_wait_warp_s(smem_u32(&c.pv_done[t & 3]), static_cast<uint32_t>((t >> 2) & 1), &c, status);
+            return mbar_wait_limit_warp(smem_u32(&c.pv_done[t & 3]), static_cast<uint32_t>((t >> 2) & 1), &c, status);
         };
         bool failed = false;
         // copy c takes the tiles j = c, c + 2, ..: all 128 keys of the tile for its 64 rows
         for (int j = copy; j < sp.n_tiles; j += 2) {
-            bool ok = mbar_wait_warp_s(smem_u32(&c.s_full[copy]), (j >> 1) & 1, &c, status);
+            bool ok = mbar_wait_limit_warp(smem_u32(&c.s_full[copy]), (j >> 1) & 1, &c, status);
             if (leader) SS_TRC(3, 8 + 6 * j);
             tc_fence_after();
             const int x0 = sp.first_key(j), nvk = sp.valid_keys(j);
@@ -526,7 +497,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             const int region_left = (cache ? sp.L + sp.T : sp.n_stream) - x0;
             if (region_left < TK) {
                 const int vs = j % n_ring;
-                if (mbar_wait_warp_s(smem_u32(&c.slot_full[1][vs]), static_cast<uint32_t>((j / n_ring) & 1), &c, status)) {
+                if (mbar_wait_limit_warp(smem_u32(&c.slot_full[1][vs]), static_cast<uint32_t>((j / n_ring) & 1), &c, status)) {
                     #pragma unroll
                     for (int up = 0; up < 2; ++up) {
                         const int vr = row + 64 * up;

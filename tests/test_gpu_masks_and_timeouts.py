@@ -143,17 +143,19 @@ def test_a_wait_that_runs_out_reports_a_timeout_and_the_stream_stays_usable(cuda
     assert int(words[2:].abs().max()) == 0                     # a call leaves the partial rows' area zero again
 
 
-SHORT_BOUND = {                    # heads of at most 64 rows
+SHORT_BOUND = {                    # heads of at most 64 rows: on one CTA per SM, split and whole, and on two
     "split": dict(prefix_len=3000, n_nodes=64, gamma=0, n_heads=32),
     "whole": dict(prefix_len=3000, n_nodes=64, gamma=0, n_heads=100),
+    "batch": dict(batch=6, prefix_len_range=(300, 600), n_nodes=64, gamma=0, n_heads=64),
 }
 
 
 @pytest.mark.parametrize("name", list(SHORT_BOUND))
 def test_a_call_whose_waits_run_out_ends_and_leaves_the_stream_usable(cuda, oracle, name):
-    """With a bound of 1024 cycles the waits for the first tiles, all of which the grid requests at once, run out in the
-    middle of the pipeline, in any of its roles.  The call ends, with whatever it had in flight, and the same call with
-    the default bound on a cleared workspace matches the oracle."""
+    """With a bound of 1024 cycles the wait for the partial rows of a split head runs out, and any wait of the pipeline may
+    (one on a barrier rarely does: the hardware holds the thread for a while before it looks at the clock).  The call
+    ends, with whatever it had in flight, and the same call with the default bound on a cleared workspace matches the
+    oracle."""
     api, DeviceStep = cuda
     cfg = W.custom_config("short", n_layers=1, n_msa_layers=0, max_depth=4, head_dim=128, tree_kind="topk_growth", config_id=811,
                           **SHORT_BOUND[name])
@@ -168,8 +170,7 @@ def test_a_call_whose_waits_run_out_ends_and_leaves_the_stream_usable(cuda, orac
         words[1] = 1
         dev.run_attention()
         seen.add(api.ss_status(dev.attn_ws))
-    assert seen <= {0, api.SS_ERR_DEVICE_TIMEOUT}
-    print(name, seen)
+    assert seen <= {0, api.SS_ERR_DEVICE_TIMEOUT} and (name != "split" or api.SS_ERR_DEVICE_TIMEOUT in seen)
     words.zero_()
     for _ in range(2):
         dev.run_attention()

@@ -138,3 +138,16 @@ def test_verify_and_compact_reject_bad_arguments_before_any_launch(lib):
 def test_error_strings(lib):
     assert lib.ss_error_string(0) == b"ok"
     assert b"workspace" in lib.ss_error_string(api.SS_ERR_WORKSPACE)
+
+
+@pytest.mark.parametrize("kernel", ["small", "few", "half"])
+def test_waits_of_heads_of_at_most_64_rows_keep_the_bound_of_the_workspace_header(kernel):
+    """Read from the source, since no run can make a barrier's wait last: every wait of the kernels that such heads take
+    goes by the bound in the control block, which is loaded from word 1 of the workspace."""
+    src = open(os.path.join(ROOT, "paper_2402_11131_b200", "csrc", "ss_attention_%s.cuh" % kernel)).read()
+    waits = re.findall(r"\b(mbar_wait\w*)\((.*?status)\)", src)
+    assert len(waits) > 0
+    for name, args in waits:
+        assert name not in ("mbar_wait", "mbar_wait_warp", "mbar_wait_slow"), args       # these have the default bound
+        assert "abort" not in args or "wait_limit" in args, (name, args)
+    assert '"l"(a.status + 1)' in src and "c.wait_limit) = lim" in src
