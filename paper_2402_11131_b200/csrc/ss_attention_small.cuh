@@ -100,6 +100,26 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
                  ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
 }
+// A wait ran out (all threads of the CTA).  Shared memory and TMEM are not given up before what is in flight has landed: copies (a
+// producer may have requested its last one long before another role gave up), MMAs with their commits, the softmax
+// threads' stores.  Out of line: in the kernel itself it costs a 7B step of 28 plain layers 2 us more (495.3, here 493.3, without it 491.5).
+__device__ __noinline__ void land_all_s(CtrlS* c, int n_ring) {
+    const int tid = threadIdx.x, warp = tid >> 5;
+    if (tid == 0 || tid == 96) {
+        const int kind = tid == 0 ? 0 : 1, n = c->requested[kind];
+        for (int s = 0; s < n_ring; ++s)
+            if (n > s) mbar_drain(smem_u32(&c->slot_full[kind][s]), static_cast<uint32_t>(((n - 1 - s) / n_ring) & 1));
+        if (tid == 0) mbar_drain(smem_u32(&c->q_full), 0);
+    } else if (warp == 1 || warp == 2) {
+        tc_commit_w(elect_lane(), smem_u32(&c->drain[warp - 1]));          // (the lane that issued the MMAs: the election is deterministic)
+        mbar_drain(smem_u32(&c->drain[warp - 1]), 0);
+    }
+    __syncwarp();
+    if (warp >= 4) { tmem_wait_ld(); tmem_wait_st(); }
+    tc_fence_before();
+    __syncthreads();
+}
+
 template <int HD>
 __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(const __grid_constant__ AttnArgs a) {
     using G = GeoS<HD>;
@@ -649,23 +669,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     if (tid == kAuxThreads) SS_TRC(5, 5);
     tc_fence_before();
     __syncthreads();
-    if (*reinterpret_cast<volatile int*>(&c.abort) != 0) {                    // (CTA-uniform: every role has left its loop)
-        // A wait ran out.  Shared memory and TMEM are not given up before what is in flight has landed: copies (a producer may
-        // have requested its last one long before another role gave up), MMAs with their commits, the softmax threads' stores.
-        if (tid == 0 || tid == 96) {
-            const int kind = tid == 0 ? 0 : 1, n = c.requested[kind];
-            for (int s = 0; s < n_ring; ++s)
-                if (n > s) mbar_drain(smem_u32(&c.slot_full[kind][s]), static_cast<uint32_t>(((n - 1 - s) / n_ring) & 1));
-            if (tid == 0) mbar_drain(smem_u32(&c.q_full), 0);
-        } else if (warp == 1 || warp == 2) {
-            tc_commit_w(elect_lane(), smem_u32(&c.drain[warp - 1]));          // (the lane that issued the MMAs: the election is deterministic)
-            mbar_drain(smem_u32(&c.drain[warp - 1]), 0);
-        }
-        __syncwarp();
-        if (warp >= 4) { tmem_wait_ld(); tmem_wait_st(); }
-        tc_fence_before();
-        __syncthreads();
-    }
+    if (*reinterpret_cast<volatile int*>(&c.abort) != 0) land_all_s(&c, n_ring);          // (CTA-uniform: every role has left its loop)
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
