@@ -35,7 +35,8 @@ __device__ __forceinline__ uint4 add8(const uint4& a, const uint4& b) {
 }
 
 // out[t][j][c] = m[t][c] + p[j][c]; the embeddings of the thread's columns stay in registers
-__global__ void __launch_bounds__(128)
+template <bool kNarrow>
+__global__ void __launch_bounds__(kNarrow ? 256 : 128)
 stream_insert_kernel(const uint4* __restrict__ m, const uint4* __restrict__ p, uint4* __restrict__ out, long long rows, int gamma, int vec) {
     wait_for_previous_kernel();
     release_next_kernel();
@@ -45,17 +46,18 @@ stream_insert_kernel(const uint4* __restrict__ m, const uint4* __restrict__ p, u
     #pragma unroll
     for (int j = 0; j < SS_MAX_GAMMA; ++j)
         if (j < gamma) emb[j] = __ldg(p + static_cast<long long>(j) * vec + c);
-    const long long step = static_cast<long long>(gridDim.y) * kRowBatch;
-    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch; t < rows; t += step) {
+    const int by = kNarrow ? static_cast<int>(blockDim.y) : 1;
+    const long long step = static_cast<long long>(gridDim.y) * kRowBatch * by;
+    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch * by + (kNarrow ? threadIdx.y : 0u); t < rows; t += step) {
         uint4 a[kRowBatch];
         #pragma unroll
         for (int i = 0; i < kRowBatch; ++i)
-            if (t + i < rows) a[i] = m[(t + i) * vec + c];
+            if (t + i * by < rows) a[i] = m[(t + i * by) * vec + c];
         #pragma unroll
         for (int i = 0; i < kRowBatch; ++i) {
             #pragma unroll
             for (int j = 0; j < SS_MAX_GAMMA; ++j)
-                if (j < gamma && t + i < rows) out[((t + i) * gamma + j) * vec + c] = add8(a[i], emb[j]);
+                if (j < gamma && t + i * by < rows) out[((t + i * by) * gamma + j) * vec + c] = add8(a[i], emb[j]);
         }
     }
 }
@@ -67,38 +69,46 @@ __device__ __forceinline__ uint32_t rotate_word(uint32_t w, float cs, float sn) 
 }
 
 // out[t][n][c] = v[t][c] rotated by eps * (n + 1)
-__global__ void __launch_bounds__(128)
+template <bool kNarrow>
+__global__ void __launch_bounds__(kNarrow ? 256 : 128)
 value_rotate_kernel(const uint4* __restrict__ v, uint4* __restrict__ out, long long rows, int gamma, int vec, const __grid_constant__ RotTable tab) {
     wait_for_previous_kernel();
     release_next_kernel();
     const int c = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
     if (c >= vec) return;
-    const long long step = static_cast<long long>(gridDim.y) * kRowBatch;
-    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch; t < rows; t += step) {
+    const int by = kNarrow ? static_cast<int>(blockDim.y) : 1;
+    const long long step = static_cast<long long>(gridDim.y) * kRowBatch * by;
+    for (long long t = static_cast<long long>(blockIdx.y) * kRowBatch * by + (kNarrow ? threadIdx.y : 0u); t < rows; t += step) {
         uint4 a[kRowBatch];
         #pragma unroll
         for (int i = 0; i < kRowBatch; ++i)
-            if (t + i < rows) a[i] = v[(t + i) * vec + c];
+            if (t + i * by < rows) a[i] = v[(t + i * by) * vec + c];
         #pragma unroll
         for (int i = 0; i < kRowBatch; ++i) {
             #pragma unroll
             for (int n = 0; n < SS_MAX_GAMMA; ++n) {
-                if (n < gamma && t + i < rows) {
+                if (n < gamma && t + i * by < rows) {
                     const float cs = tab.cs[n], sn = tab.sn[n];
                     uint4 r;
                     r.x = rotate_word(a[i].x, cs, sn); r.y = rotate_word(a[i].y, cs, sn);
                     r.z = rotate_word(a[i].z, cs, sn); r.w = rotate_word(a[i].w, cs, sn);
-                    out[((t + i) * gamma + n) * vec + c] = r;
+                    out[((t + i * by) * gamma + n) * vec + c] = r;
                 }
             }
         }
     }
 }
 
-// 128 threads across the width; rows dealt out until the SMs are full (16 such CTAs per SM)
+// 128 threads across the width.  A narrower one (kNarrow) has a thread for each of its vectors and as many rows as fit 256
+// threads (262144 rows of 128, four streams, both calls 202 -> 108 us; 100000 of 8 55 -> 10 us).  Rows are dealt out
+// until the SMs are full (16 such CTAs per SM).
+static dim3 block_for(int vec) {
+    return vec < 128 ? dim3(static_cast<unsigned>(vec), static_cast<unsigned>(256 / vec)) : dim3(128);
+}
 static dim3 grid_for(long long rows, int vec) {
     const int gx = (vec + 127) / 128;
-    long long gy = (rows + kRowBatch - 1) / kRowBatch;
+    const long long per = static_cast<long long>(kRowBatch) * block_for(vec).y;
+    long long gy = (rows + per - 1) / per;
     const long long cap = (static_cast<long long>(sm_count()) * 16 + gx - 1) / gx;
     if (gy > cap) gy = cap;
     if (gy > 65535) gy = 65535;
@@ -115,7 +125,7 @@ extern "C" int32_t ss_stream_insert(const void* main_hidden, const void* stream_
     if (!main_hidden || !stream_emb || !out) return SS_ERR_INVALID_ARG;
     if (!ss::aligned16(main_hidden) || !ss::aligned16(stream_emb) || !ss::aligned16(out)) return SS_ERR_INVALID_ARG;
     const int vec = hidden / 8;
-    const cudaError_t err = ss::launch_after_previous(ss::stream_insert_kernel, ss::grid_for(rows, vec), dim3(128),
+    const cudaError_t err = ss::launch_after_previous(vec < 128 ? ss::stream_insert_kernel<true> : ss::stream_insert_kernel<false>, ss::grid_for(rows, vec), ss::block_for(vec),
                                                       static_cast<cudaStream_t>(stream), static_cast<const uint4*>(main_hidden),
                                                       static_cast<const uint4*>(stream_emb), static_cast<uint4*>(out),
                                                       static_cast<long long>(rows), gamma, vec);
@@ -136,7 +146,7 @@ extern "C" int32_t ss_value_rotate(const void* v_main, void* v_streams, int64_t 
         tab.sn[n] = static_cast<float>(sin(ang));
     }
     const int vec = width / 8;
-    const cudaError_t err = ss::launch_after_previous(ss::value_rotate_kernel, ss::grid_for(rows, vec), dim3(128),
+    const cudaError_t err = ss::launch_after_previous(vec < 128 ? ss::value_rotate_kernel<true> : ss::value_rotate_kernel<false>, ss::grid_for(rows, vec), ss::block_for(vec),
                                                       static_cast<cudaStream_t>(stream), static_cast<const uint4*>(v_main),
                                                       static_cast<uint4*>(v_streams), static_cast<long long>(rows), gamma, vec, tab);
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;

@@ -346,6 +346,25 @@ def test_stream_insert_is_bit_exact(cuda, oracle, rows, gamma, hidden):
         np.testing.assert_array_equal(api.bf16_to_host_bits(out), oracle.stream_insert(m, p))
 
 
+@pytest.mark.parametrize("width", [8, 24, 80, 512, 520, 1016, 1024, 1032])
+def test_streams_of_narrow_widths_with_odd_numbers_of_rows(cuda, oracle, width):
+    """Widths below 8 x 128 put several rows in a CTA: rows that fill no CTA, and one more than a CTA takes at a time."""
+    api = cuda
+    per_cta = 2 * max(256 // (width // 8), 1)
+    for rows in (1, per_cta - 1, per_cta + 1, 7 * per_cta + 3):
+        rng = np.random.default_rng(rows + width)
+        m = W.f32_to_bf16_bits(rng.standard_normal((rows, width)).astype(np.float32))
+        p = W.f32_to_bf16_bits(rng.standard_normal((3, width)).astype(np.float32))
+        out = torch.full((rows + 1, 3, width), 7.0, dtype=torch.bfloat16, device="cuda")
+        rot = out.clone()
+        api.ss_stream_insert(api.bf16_to_device(m), api.bf16_to_device(p), out)
+        api.ss_value_rotate(api.bf16_to_device(m), rot, 0.25)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(api.bf16_to_host_bits(out)[:rows], oracle.stream_insert(m, p))
+        np.testing.assert_array_equal(api.bf16_to_host_bits(rot)[:rows], oracle.value_rotate(m, 3, 0.25))
+        assert bool((out[rows] == 7.0).all()) and bool((rot[rows] == 7.0).all())
+
+
 @pytest.mark.parametrize("rows,gamma,width,eps", [(64 * 32, 4, 128, 0.01), (5, 1, 8, 0.3), (2048, 3, 80, 1.0 / 4100)])
 def test_value_rotation_is_bit_exact(cuda, oracle, rows, gamma, width, eps):
     api = cuda
