@@ -168,7 +168,9 @@ typedef struct ss_attn_params {
     uint32_t flags;                 /* SS_ATTN_* bits, 0 for none */
 } ss_attn_params;
 
-/* Bytes of workspace ss_msa_attention needs for these shapes (pointers in *p are not read). */
+/* Bytes of workspace ss_msa_attention needs for these shapes, whatever the slab's size (kv_total_slots) and the pointers in
+ * *p, which are not read.  (Calls of at most 32 rows per head and more heads than half of the SMs also run with as little
+ * as 256 bytes, unsplit.) */
 size_t ss_msa_attention_workspace_bytes(const ss_attn_params* p);
 int32_t ss_msa_attention(const ss_attn_params* p, void* stream);
 

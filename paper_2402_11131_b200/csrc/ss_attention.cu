@@ -1556,8 +1556,14 @@ struct AttnPlan {
     int few_rows;                              // rows of a block of the few-rows kernel (16, 32, 64), 0: another kernel
     long long groups;                          // (sequence, head, row block) triples
     size_t smem;
-    size_t partial_bytes;                      // workspace after its header
+    // Workspace after its header: what any call of these shapes has to bring, and what the few-rows kernel can use besides, on a
+    // slab of any size.  A call that brings less than that splits its heads less far.
+    size_t base_bytes, partial_bytes;
+    size_t few_bytes() const;                  // what the few-rows kernel takes at `cluster`
+    size_t row_bytes;                          // of a partial row
 };
+
+size_t AttnPlan::few_bytes() const { return cluster > 1 ? static_cast<size_t>(groups) * cluster * few_rows * row_bytes : 0; }
 
 // Rows of a block of the few-rows kernel (16, 32 or 64), 0 where a tcgen05 kernel is the better one.  The few-rows kernel
 // has little fixed cost (4 us a layer where the tcgen05 ones take 8) but pays more per key, the more the more rows and
@@ -1621,22 +1627,32 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     // rows 46.6 / 36.9; with fewer blocks than SMs the second half stays empty: three sequences 22.4 / 32)
     plan->mode = plan->few_rows ? kFew : plan->groups > sm_count() ? kHalf : q_rows <= kSmRows ? kCols : kPair;
     // a split block leaves the partial rows (O, m, l) of each of its CTAs in the workspace
-    const size_t row_bytes = static_cast<size_t>(p.head_dim + 4) * 4;
-    plan->partial_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * (q_rows > kSmRows ? kBlockRows : kSmRows) * row_bytes : 0;
+    plan->row_bytes = static_cast<size_t>(p.head_dim + 4) * 4;
+    plan->base_bytes = c > 1 ? static_cast<size_t>(plan->groups) * c * (q_rows > kSmRows ? kBlockRows : kSmRows) * plan->row_bytes : 0;
+    plan->partial_bytes = plan->base_bytes;
+    // The few-rows kernel takes half an SM per CTA; with 64 rows two CTAs on an SM get in each other's way (12 us instead of 9 at
+    // 512 keys of 128).  It takes 64 rows or blocks of 32 of them according to the slab, so the workspace holds either.
+    AttnPlan few = *plan;
+    const auto few_plan = [&](int rows) {
+        few.few_rows = rows;
+        few.n_blocks = (q_rows + rows - 1) / rows;
+        few.groups = heads * few.n_blocks;
+        few.cluster = split(few.groups, rows <= 32 ? 2ll * sm_count() : sm_count());
+    };
+    for (const int rows : {q_rows <= 16 ? 16 : 32, q_rows > 32 && q_rows <= kSmRows ? 64 : 0}) {
+        if (rows == 0) continue;
+        few_plan(rows);
+        if (few.few_bytes() > plan->partial_bytes) plan->partial_bytes = few.few_bytes();
+    }
     if (plan->few_rows) {
-        // the few-rows kernel takes half an SM per CTA (and splits a head no further than its length asks for); with 64 rows
-        // two CTAs on an SM get in each other's way (12 us instead of 9 at 512 keys of 128)
-        plan->n_blocks = (q_rows + plan->few_rows - 1) / plan->few_rows;
-        plan->groups = heads * plan->n_blocks;
-        plan->cluster = split(plan->groups, plan->few_rows <= 32 ? 2ll * sm_count() : sm_count());
+        few_plan(plan->few_rows);
+        plan->n_blocks = few.n_blocks; plan->groups = few.groups; plan->cluster = few.cluster;
         // no more CTAs than the slab's slots can ask for (a sequence of a batch: twice the mean); one that finds nothing to
         // do still costs its launch: 128 or 256 CTAs for 32 whole heads of 528 keys 5.0 and 5.7 us
         const long long most = (p.batch > 1 ? 2 : 1) * (p.kv_total_slots / p.batch) + static_cast<long long>(p.max_nodes) * p.gamma;
         const long long tiles = (most + kFwKeys - 1) / kFwKeys + 1;
         const int whole = few_whole(p.head_dim, plan->few_rows);
         while (plan->cluster > 1 && (tiles <= whole || plan->cluster / 2 * kFwSplitTiles >= tiles)) plan->cluster /= 2;
-        const size_t few_bytes = plan->cluster > 1 ? static_cast<size_t>(plan->groups) * plan->cluster * kSmRows * row_bytes : 0;
-        if (few_bytes > plan->partial_bytes) plan->partial_bytes = few_bytes;
     }
     if (plan->mode == kFew || plan->mode == kHalf) {
         plan->n_kslots = plan->n_vslots = 0;       // (rings and shared memory follow from head_dim and rows)
@@ -1667,7 +1683,7 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     size_t bytes = qp + static_cast<size_t>(plan->n_kslots + plan->n_vslots) * slot;
     // after the pipeline the same memory stages partial rows ((head_dim + 4) floats each): 2 KB, then the 128
     // outgoing rows
-    const size_t stage = 2048 + kBlockRows * row_bytes;
+    const size_t stage = 2048 + kBlockRows * plan->row_bytes;
     if (stage > bytes) bytes = stage;
     plan->smem = bytes + 1024;
     return plan->smem <= static_cast<size_t>(kPairMaxDynSmem);
@@ -1817,7 +1833,9 @@ extern "C" int32_t ss_msa_attention(const ss_attn_params* p, void* stream) {
     for (const void* q : ptrs)
         if (!ss::aligned16(q)) return SS_ERR_INVALID_ARG;
     if (!(p->sm_scale == p->sm_scale)) return SS_ERR_INVALID_ARG;
-    if (p->workspace_bytes < ss_msa_attention_workspace_bytes(p)) return SS_ERR_WORKSPACE;
+    if (p->workspace_bytes < ss::kWsHeaderBytes + plan.base_bytes) return SS_ERR_WORKSPACE;
+    if (plan.few_rows)
+        while (plan.few_bytes() > p->workspace_bytes - ss::kWsHeaderBytes) plan.cluster /= 2;
 
     ss::AttnArgs a;
     const int d = p->head_dim, H = p->n_heads, tk = plan.mode == ss::kFew ? ss::kFwKeys : plan.mode == ss::kHalf ? ss::kHfKeys : ss::kTileKeys;

@@ -46,7 +46,7 @@ struct GeoF {
     static constexpr int kDynSmem = kQBytes + 2 * kRing * kTileBytes;
     static constexpr int kKSteps = HD / 16;
     static constexpr int kPitch = HD + 4;                         // floats of a partial row: O, m, l, pad
-    static constexpr size_t kCtaFloats = static_cast<size_t>(64) * kPitch;        // workspace of one CTA of a split head
+    static constexpr size_t kCtaFloats = static_cast<size_t>(kRows) * kPitch;     // workspace of one CTA of a split block
     // teams of RG warps on different tiles = partials per row (16 rows at head_dim > 64: as many as there are slots)
     static constexpr int kTeams = RG == 1 && HD > 64 ? 6 : kFwWarps / RG;
     // A tile's slot held the tile kRing before it.  Where that was another team's, the team does not know that it has landed,

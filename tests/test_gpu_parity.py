@@ -298,6 +298,23 @@ def test_attention_few_rows(cuda, oracle, head_dim, T, gamma, n_heads, lengths):
                                heads=(max(n_heads - 3, 0), n_heads))
 
 
+def test_attention_with_less_workspace_than_a_further_split_could_use(cuda, oracle):
+    """100 heads of at most 32 rows: without a workspace for partial rows the heads are not split, and nothing behind the
+    header is touched."""
+    api, DeviceStep = cuda
+    for k, (T, gamma) in enumerate([(12, 1), (27, 0)]):
+        cfg = W.custom_config("lessws", n_layers=2, n_msa_layers=1, prefix_len=900, n_nodes=T, gamma=max(gamma, 1), max_depth=4, n_heads=100,
+                              head_dim=64, config_id=930 + k)
+        st = W.make_step(cfg)
+        dev = DeviceStep(st, layers=[1 if gamma else 0])
+        assert dev.attn_ws.numel() > 256
+        dev.attn_ws[256:] = 1
+        dev.params[0].workspace_bytes = 256
+        dev.run_attention()
+        assert api.ss_status(dev.attn_ws) == 0 and bool((dev.attn_ws[256:] == 1).all())
+        assert_attention_close(oracle, st, st.layer(1 if gamma else 0), dev, 0, heads=(98, 100))
+
+
 @pytest.mark.parametrize("head_dim", [64, 80, 128])
 @pytest.mark.parametrize("T,gamma,n_heads,lengths,ramp", [
     (64, 0, 60, (385, 448), 0.0),        # 64 rows; a tile's edge in the prefix and in the tree, rings that wrap

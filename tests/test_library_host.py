@@ -118,6 +118,17 @@ def test_attention_rejects_bad_arguments_before_any_launch(lib):
     assert lib.ss_msa_attention(None, None) == api.SS_ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("head_dim", [64, 80, 128])
+def test_attention_workspace_follows_from_the_shapes_not_from_the_slab(lib, head_dim):
+    """One answer for every slab a cache may grow to, also while there is none yet."""
+    for T, gamma in ((1, 0), (12, 0), (12, 1), (16, 3), (33, 0), (64, 0), (40, 2), (64, 4)):
+        for batch, heads in ((1, 2), (1, 32), (5, 13), (3, 32), (16, 32)):
+            answers = {lib.ss_msa_attention_workspace_bytes(C.byref(_fake_params(
+                batch=batch, n_heads=heads, head_dim=head_dim, gamma=gamma, max_nodes=T, kv_total_slots=slots)))
+                for slots in (0, 1, 100, 512, 1024, 2048, 4096, 1 << 20, 1 << 30)}
+            assert len(answers) == 1 and min(answers) >= 256, (T, gamma, batch, heads, answers)
+
+
 def test_verify_and_compact_reject_bad_arguments_before_any_launch(lib):
     need = lib.ss_tree_verify_workspace_bytes(2, 6, 512)
     assert need >= 256 + 2 * 6 * 8
