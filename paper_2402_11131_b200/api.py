@@ -141,8 +141,10 @@ def native():
             from . import _pycall
         except ImportError as e:
             raise RuntimeError("the binding's native part is missing: run `python -m paper_2402_11131_b200.build`") from e
-        torch.cuda.current_stream()                       # initialises CUDA if nothing has yet
-        _pycall.setup(SsError, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        if torch.cuda.is_available():
+            torch.cuda.current_stream()                   # initialises CUDA if nothing has yet
+        _pycall.setup(SsError, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, AttnParams, CacheLayout, C.byref,
+                      C.ArgumentError)
         _native = _pycall
     return _native
 

@@ -13,6 +13,8 @@ namespace {
 
 PyObject *s_data_ptr, *s_shape, *s_nbytes, *s_cuda_stream;      // interned attribute names
 PyObject *g_error, *g_raw_stream, *g_device;                    // SsError; torch's raw current stream and current device
+PyObject *g_attn_params, *g_cache_layout;                       // the ctypes structures of ss_attn_params and ss_cache_layout
+PyObject *g_byref, *g_argument_error;                           // ctypes.byref and ctypes.ArgumentError
 
 // One call's arguments.  After the first Python error everything reads as zero and `ok` stays false.
 struct Args {
@@ -75,16 +77,27 @@ struct Args {
         Py_XDECREF(r);
         return p;
     }
-    // the memory of a ctypes structure
+    // The memory of a ctypes structure of class `type`.  Anything else is refused as ctypes refuses it: a TypeError for what is
+    // no ctypes object, an ArgumentError for another one.
     template <typename T>
-    const T* structure(int i, Py_buffer* view) {
+    const T* structure(int i, PyObject* type, Py_buffer* view) {
         view->obj = nullptr;
         if (!ok) return nullptr;
-        if (PyObject_GetBuffer(a[i], view, PyBUF_SIMPLE) != 0) {
-            ok = false;
+        ok = false;
+        const int is = PyObject_IsInstance(a[i], type);
+        if (is < 0) return nullptr;
+        if (!is) {
+            PyObject* r = PyObject_CallOneArg(g_byref, a[i]);
+            if (r) PyErr_Format(g_argument_error, "expected an instance of %R instead of %R", type, reinterpret_cast<PyObject*>(Py_TYPE(a[i])));
+            Py_XDECREF(r);
             return nullptr;
         }
-        return static_cast<const T*>(view->buf);
+        if (PyObject_GetBuffer(a[i], view, PyBUF_SIMPLE) != 0) return nullptr;
+        ok = view->len >= static_cast<Py_ssize_t>(sizeof(T));
+        if (ok) return static_cast<const T*>(view->buf);
+        PyBuffer_Release(view);
+        PyErr_Format(g_argument_error, "%R is smaller than the structure", type);
+        return nullptr;
     }
 };
 
@@ -110,7 +123,7 @@ PyObject* done(const char* what, int32_t status) {
 SS_ENTRY(msa_attention, 2)
     Py_buffer view;
     void* const s = a.stream(1);
-    const ss_attn_params* const p = a.structure<ss_attn_params>(0, &view);
+    const ss_attn_params* const p = a.structure<ss_attn_params>(0, g_attn_params, &view);
     SS_CALL(ss_msa_attention(p, s))
     PyBuffer_Release(&view);
     return done("ss_msa_attention", st);
@@ -206,7 +219,7 @@ SS_ENTRY(kv_compact, 9)
     const int32_t *kl = a.as<int32_t>(4), *al = a.as<int32_t>(5), *ap = a.as<int32_t>(6);
     int32_t* ko = a.as<int32_t>(7);
     void* const s = a.stream(8);
-    const ss_cache_layout* const lo = a.structure<ss_cache_layout>(2, &view);
+    const ss_cache_layout* const lo = a.structure<ss_cache_layout>(2, g_cache_layout, &view);
     SS_CALL(ss_kv_compact(k, v, lo, static_cast<int32_t>(n[0]), ks, kl, al, ap, ko, s))
     PyBuffer_Release(&view);
     return done("ss_kv_compact", st);
@@ -233,12 +246,11 @@ SS_ENTRY(value_rotate, 4)
     return done("ss_value_rotate", st);
 }
 
-// setup(SsError, raw_stream(device) -> int, device() -> int)
-SS_ENTRY(setup, 3)
+// setup(SsError, raw_stream(device) -> int, device() -> int, AttnParams, CacheLayout, ctypes.byref, ctypes.ArgumentError)
+SS_ENTRY(setup, 7)
     (void)a; (void)st;
-    Py_XSETREF(g_error, Py_NewRef(argv[0]));
-    Py_XSETREF(g_raw_stream, Py_NewRef(argv[1]));
-    Py_XSETREF(g_device, Py_NewRef(argv[2]));
+    PyObject** const kept[7] = {&g_error, &g_raw_stream, &g_device, &g_attn_params, &g_cache_layout, &g_byref, &g_argument_error};
+    for (int i = 0; i < 7; ++i) Py_XSETREF(*kept[i], Py_NewRef(argv[i]));
     Py_RETURN_NONE;
 }
 

@@ -9,6 +9,8 @@ import pytest
 
 from paper_2402_11131_b200 import api, build
 
+torch = pytest.importorskip("torch")
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 GOLDEN = os.path.join(os.path.dirname(__file__), "golden")
 
@@ -162,3 +164,27 @@ def test_waits_of_heads_of_at_most_64_rows_keep_the_bound_of_the_workspace_heade
         assert name not in ("mbar_wait", "mbar_wait_warp", "mbar_wait_slow"), args       # these have the default bound
         assert "abort" not in args or "wait_limit" in args, (name, args)
     assert '"l"(a.status + 1)' in src and "c.wait_limit) = lim" in src
+
+
+class _Stream:
+    cuda_stream = 0                          # stands for a torch.cuda.Stream where there is no GPU
+
+
+def test_binding_refuses_what_is_not_the_call_s_structure(lib):
+    """As ctypes does: another structure is an ArgumentError, what is no ctypes object a TypeError; nothing is read."""
+    class Derived(api.AttnParams):
+        pass
+
+    for call, own in ((lambda p: api.ss_msa_attention(p, _Stream()), api.AttnParams),
+                      (lambda p: api.ss_kv_compact(None, None, p, torch.zeros(1), None, None, None, None, _Stream()), api.CacheLayout)):
+        for other in (api.TreeDesc(), api.CacheLayout() if own is api.AttnParams else api.AttnParams(), C.c_int32(), C.pointer(own())):
+            with pytest.raises(C.ArgumentError):
+                call(other)
+        for other in (None, b"\0" * 512, bytearray(512), np.zeros(64), 0):
+            with pytest.raises(TypeError):
+                call(other)
+        with pytest.raises(api.SsError) as e:                # an empty structure reaches the library
+            call(own())
+        assert e.value.status == api.SS_ERR_INVALID_ARG
+    with pytest.raises(api.SsError):
+        api.ss_msa_attention(Derived(), _Stream())
