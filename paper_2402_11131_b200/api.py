@@ -31,6 +31,8 @@ SS_ATTN_PREFIX_STABLE = 1
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libss_msa.so")
 _lib = None
 _native = None          # the _pycall module: takes the tensors of the per-step calls apart (see native())
+_NATIVE_CALLS = ("ss_msa_attention", "ss_tree_verify", "ss_tree_verify_soft", "ss_tree_verify_sampled", "ss_tree_prune", "ss_next_draft",
+                 "ss_kv_compact", "ss_stream_insert", "ss_value_rotate")        # in the order of _pycall.setup
 
 # number of kernels each entry point enqueues per call (for launch accounting in the benchmark); ss_kv_compact enqueues a
 # second one where kv_len_out overlaps one of its inputs
@@ -80,7 +82,7 @@ SS_VERIFY_STATIC_SCRATCH_BYTES = 1 << 20
 
 def lib() -> C.CDLL:
     """Loads libss_msa.so (built in-tree by paper_2402_11131_b200.build).  Raises if it is missing."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise RuntimeError("CUDA library %s is missing: run `python -m paper_2402_11131_b200.build` "
@@ -127,7 +129,7 @@ def lib() -> C.CDLL:
         l.ss_version.restype = C.c_int32
         l.ss_error_string.restype = C.c_char_p
         l.ss_error_string.argtypes = [C.c_int32]
-        _lib = l
+        _lib, _native = l, None                           # (the native part takes the new library's addresses)
     return _lib
 
 
@@ -143,8 +145,9 @@ def native():
             raise RuntimeError("the binding's native part is missing: run `python -m paper_2402_11131_b200.build`") from e
         if torch.cuda.is_available():
             torch.cuda.current_stream()                   # initialises CUDA if nothing has yet
+        addresses = tuple(C.cast(getattr(lib(), name), C.c_void_p).value for name in _NATIVE_CALLS)
         _pycall.setup(SsError, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, AttnParams, CacheLayout, C.byref,
-                      C.ArgumentError)
+                      C.ArgumentError, addresses)
         _native = _pycall
     return _native
 

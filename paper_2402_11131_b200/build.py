@@ -69,11 +69,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp, *objs])
         os.replace(tmp, LIB)
     pycall = os.path.join(CSRC, "ss_pycall.cpp")
-    if not TRACE and (force or _stale(PYCALL, [pycall, os.path.join(ROOT, "include", "ss_msa.h")])):
+    if force or _stale(PYCALL, [pycall, os.path.join(ROOT, "include", "ss_msa.h")]):
         tmp = PYCALL + ".tmp%d" % os.getpid()
         subprocess.check_call([shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-I",
-                               os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], pycall, "-o", tmp, "-L", PKG,
-                               "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
+                               os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], pycall, "-o", tmp])
         os.replace(tmp, PYCALL)
     return LIB
 

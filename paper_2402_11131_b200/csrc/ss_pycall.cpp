@@ -1,4 +1,5 @@
-// CPython side of the binding: takes tensors apart and calls the C entry points (ss_msa.h).
+// CPython side of the binding: takes tensors apart and calls the C entry points (ss_msa.h) of the library that api.py has
+// loaded, whose addresses it is given: it is not linked to one.
 //
 // A decode step of a small model is a handful of calls of 3 to 8 us of GPU time each, so the host has to spend less than that
 // on a call.  Through ctypes, with the pointers collected in Python, a verification call took 5.6 us, of which the launch is
@@ -14,6 +15,14 @@ namespace {
 PyObject *s_data_ptr, *s_shape, *s_nbytes, *s_cuda_stream;      // interned attribute names
 PyObject *g_error, *g_raw_stream, *g_device;                    // SsError; torch's raw current stream and current device
 PyObject *g_attn_params, *g_cache_layout;                       // the ctypes structures of ss_attn_params and ss_cache_layout
+// the entry points, in the order in which setup() takes them
+#define SS_FUNCTIONS(F)                                                                                                 \
+    F(ss_msa_attention) F(ss_tree_verify) F(ss_tree_verify_soft) F(ss_tree_verify_sampled) F(ss_tree_prune)             \
+    F(ss_next_draft) F(ss_kv_compact) F(ss_stream_insert) F(ss_value_rotate)
+struct Functions {
+#define SS_MEMBER(name) decltype(&::name) name;
+    SS_FUNCTIONS(SS_MEMBER)
+} g_lib;
 PyObject *g_byref, *g_argument_error;                           // ctypes.byref and ctypes.ArgumentError
 
 // One call's arguments.  After the first Python error everything reads as zero and `ok` stays false.
@@ -124,7 +133,7 @@ SS_ENTRY(msa_attention, 2)
     Py_buffer view;
     void* const s = a.stream(1);
     const ss_attn_params* const p = a.structure<ss_attn_params>(0, g_attn_params, &view);
-    SS_CALL(ss_msa_attention(p, s))
+    SS_CALL(g_lib.ss_msa_attention(p, s))
     PyBuffer_Release(&view);
     return done("ss_msa_attention", st);
 }
@@ -139,7 +148,7 @@ SS_ENTRY(tree_verify, 10)
     void* const ws = a.ptr(8);
     const size_t wb = a.nbytes(8);
     void* const s = a.stream(9);
-    SS_CALL(ss_tree_verify(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), al, ap, ln, bt, am, ws, wb, s))
+    SS_CALL(g_lib.ss_tree_verify(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), al, ap, ln, bt, am, ws, wb, s))
     return done("ss_tree_verify", st);
 }
 
@@ -155,7 +164,7 @@ SS_ENTRY(tree_verify_soft, 13)
     void* const ws = a.ptr(11);
     const size_t wb = a.nbytes(11);
     void* const s = a.stream(12);
-    SS_CALL(ss_tree_verify_soft(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), eps, delta, al, ap, ln, bt,
+    SS_CALL(g_lib.ss_tree_verify_soft(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), eps, delta, al, ap, ln, bt,
                                 ep, en, ws, wb, s))
     return done("ss_tree_verify_soft", st);
 }
@@ -172,7 +181,7 @@ SS_ENTRY(tree_verify_sampled, 12)
     void* const ws = a.ptr(10);
     const size_t wb = a.nbytes(10);
     void* const s = a.stream(11);
-    SS_CALL(ss_tree_verify_sampled(lg, tok, tr, un, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), k, al, ap, ln, bt, nt,
+    SS_CALL(g_lib.ss_tree_verify_sampled(lg, tok, tr, un, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), k, al, ap, ln, bt, nt,
                                    ws, wb, s))
     return done("ss_tree_verify_sampled", st);
 }
@@ -190,7 +199,7 @@ SS_ENTRY(tree_prune, 11)
     void* const ws = a.ptr(9);
     const size_t wb = a.nbytes(9);
     void* const s = a.stream(10);
-    SS_CALL(ss_tree_prune(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), threshold, ep, ni, kn, kt, pt, ws, wb, s))
+    SS_CALL(g_lib.ss_tree_prune(lg, tok, tr, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[1]), static_cast<int32_t>(n[2]), threshold, ep, ni, kn, kt, pt, ws, wb, s))
     return done("ss_tree_prune", st);
 }
 
@@ -205,7 +214,7 @@ SS_ENTRY(next_draft, 9)
     void* const ws = a.ptr(7);
     const size_t wb = a.nbytes(7);
     void* const s = a.stream(8);
-    SS_CALL(ss_next_draft(lg, static_cast<int32_t>(n[1]), ri, bt, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[2]), static_cast<int32_t>(n[3]), k, nodes, tok,
+    SS_CALL(g_lib.ss_next_draft(lg, static_cast<int32_t>(n[1]), ri, bt, static_cast<int32_t>(n[0]), static_cast<int32_t>(n[2]), static_cast<int32_t>(n[3]), k, nodes, tok,
                           tr, ws, wb, s))
     return done("ss_next_draft", st);
 }
@@ -220,7 +229,7 @@ SS_ENTRY(kv_compact, 9)
     int32_t* ko = a.as<int32_t>(7);
     void* const s = a.stream(8);
     const ss_cache_layout* const lo = a.structure<ss_cache_layout>(2, g_cache_layout, &view);
-    SS_CALL(ss_kv_compact(k, v, lo, static_cast<int32_t>(n[0]), ks, kl, al, ap, ko, s))
+    SS_CALL(g_lib.ss_kv_compact(k, v, lo, static_cast<int32_t>(n[0]), ks, kl, al, ap, ko, s))
     PyBuffer_Release(&view);
     return done("ss_kv_compact", st);
 }
@@ -231,7 +240,7 @@ SS_ENTRY(stream_insert, 4)
     a.sizes(1, 1, g, false);
     void *m = a.ptr(0), *e = a.ptr(1), *o = a.ptr(2);
     void* const s = a.stream(3);
-    SS_CALL(ss_stream_insert(m, e, o, n[0], static_cast<int32_t>(g[0]), static_cast<int32_t>(n[1]), s))
+    SS_CALL(g_lib.ss_stream_insert(m, e, o, n[0], static_cast<int32_t>(g[0]), static_cast<int32_t>(n[1]), s))
     return done("ss_stream_insert", st);
 }
 
@@ -242,13 +251,23 @@ SS_ENTRY(value_rotate, 4)
     void *v = a.ptr(0), *o = a.ptr(1);
     const float epsilon = a.f32(2);
     void* const s = a.stream(3);
-    SS_CALL(ss_value_rotate(v, o, n[0], static_cast<int32_t>(g[1]), static_cast<int32_t>(n[1]), epsilon, s))
+    SS_CALL(g_lib.ss_value_rotate(v, o, n[0], static_cast<int32_t>(g[1]), static_cast<int32_t>(n[1]), epsilon, s))
     return done("ss_value_rotate", st);
 }
 
-// setup(SsError, raw_stream(device) -> int, device() -> int, AttnParams, CacheLayout, ctypes.byref, ctypes.ArgumentError)
-SS_ENTRY(setup, 7)
+// setup(SsError, raw_stream(device) -> int, device() -> int, AttnParams, CacheLayout, ctypes.byref, ctypes.ArgumentError,
+//       addresses of SS_FUNCTIONS: a tuple of int)
+SS_ENTRY(setup, 8)
     (void)a; (void)st;
+    PyObject* const at = argv[7];
+    Py_ssize_t n = 0;
+    Functions lib = {};
+#define SS_TAKE(name)                                                                                                   \
+    if (PyTuple_Check(at) && n < PyTuple_GET_SIZE(at)) lib.name = reinterpret_cast<decltype(lib.name)>(PyLong_AsVoidPtr(PyTuple_GET_ITEM(at, n))); \
+    if (!lib.name) return PyErr_Occurred() ? nullptr : PyErr_Format(PyExc_ValueError, "setup: no address of %s", #name);  \
+    ++n;
+    SS_FUNCTIONS(SS_TAKE)
+    g_lib = lib;
     PyObject** const kept[7] = {&g_error, &g_raw_stream, &g_device, &g_attn_params, &g_cache_layout, &g_byref, &g_argument_error};
     for (int i = 0; i < 7; ++i) Py_XSETREF(*kept[i], Py_NewRef(argv[i]));
     Py_RETURN_NONE;

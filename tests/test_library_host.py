@@ -3,6 +3,7 @@ header declares, builds tree descriptors, and rejects bad arguments before launc
 import ctypes as C
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -188,3 +189,35 @@ def test_binding_refuses_what_is_not_the_call_s_structure(lib):
         assert e.value.status == api.SS_ERR_INVALID_ARG
     with pytest.raises(api.SsError):
         api.ss_msa_attention(Derived(), _Stream())
+
+
+def test_per_step_calls_go_to_the_library_that_was_loaded(lib, tmp_path):
+    """A library under another path (a tracing build, say) gets every call, those that the binding's native part makes too."""
+    names = [n for n in api.EXPORTS if n != "ss_error_string"]
+    src = "".join("int %s() { return -77; }\n" % n for n in names) + 'const char* ss_error_string() { return "other"; }\n'
+    (tmp_path / "other.c").write_text(src)
+    other = str(tmp_path / "libother.so")
+    subprocess.check_call(["gcc", "-w", "-shared", "-fPIC", "-o", other, str(tmp_path / "other.c")])
+    with pytest.raises(api.SsError) as e:                    # (the native part is set up with the library as it is)
+        api.ss_msa_attention(api.AttnParams(), _Stream())
+    assert e.value.status == api.SS_ERR_INVALID_ARG
+    x, own = torch.zeros((1, 1, 1, 1)), api._lib
+    try:
+        api._LIB_PATH, api._lib, api._native, path = other, None, None, api._LIB_PATH
+        for call in (lambda: api.ss_msa_attention(api.AttnParams(), _Stream()),
+                     lambda: api.ss_tree_verify(x[0], x, x, x, x, x, x, x, x, _Stream()),
+                     lambda: api.ss_tree_verify_soft(x[0], x, x, 0.1, 0.1, x, x, x, x, x, x, x, _Stream()),
+                     lambda: api.ss_tree_verify_sampled(x[0], x, x, x, 1, x, x, x, x, x, x, _Stream()),
+                     lambda: api.ss_tree_prune(x[0], x, x, 0.1, x, x, x, x, x, x, _Stream()),
+                     lambda: api.ss_next_draft(x, x, x, 1, 1, x, x, x, _Stream()),
+                     lambda: api.ss_kv_compact(x, x, api.CacheLayout(), x, x, x, x, x, _Stream()),
+                     lambda: api.ss_stream_insert(x[0, 0], x, x, _Stream()), lambda: api.ss_value_rotate(x[0, 0], x, 0.1, _Stream()),
+                     lambda: api.ss_tree_build([-1], 0)):
+            with pytest.raises(api.SsError) as e:
+                call()
+            assert e.value.status == -77
+    finally:
+        api._LIB_PATH, api._lib, api._native = path, own, None
+    with pytest.raises(api.SsError) as e:
+        api.ss_msa_attention(api.AttnParams(), _Stream())
+    assert e.value.status == api.SS_ERR_INVALID_ARG
