@@ -1598,6 +1598,9 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
     // 128 rows of 64, 1024 keys 11.7 / 11.5, 2048 keys 15.1 / 16.0, eight heads and 4096 keys 13.3 / 10.7; of
     // 80, 200 keys 10.9 / 9.6, 1024 keys 14.1 / 14.5; of 128, 200 keys 11.6 / 11.0, 80 rows and 1024 keys 14.8 / 16.5.  320 rows of
     // 64, eight heads and 512 keys 10.4 / 8.3, 32 heads and 200 keys 10.6 / 11.8
+    // (one wave of two CTAs per SM: past that they are slower, sixteen sequences of eight heads, 128 rows, 30 keys of 64 9.7 / 11.7, 200
+    // keys 10.4 / 15.0, of 128, 30 keys 11.8 / 16.7; 40 heads of 320 rows, 60 keys of 80 10.4 / 13.9)
+    if (static_cast<long long>(p.batch) * p.n_heads * blocks > 2ll * sm_count()) return 0;
     return load <= (d64 ? 1300 : d80 ? 700 : 320) && (blocks <= 4 || load <= 400) ? 32 : 0;
 }
 
