@@ -140,8 +140,8 @@ int32_t ss_tree_build(const int32_t* parent, int32_t n_nodes, int32_t gamma, ss_
  * the kv_len array the attention reads (kv_len_out == kv_len) or when the attention's lengths already
  * include the compacted slots: compaction turns tree slots into prefix and writes the lengths.  Pass
  * flags = 0 to the first attention call after such a compaction, or put any other kernel between them.
- * ss_next_draft and ss_tree_prune let the next kernel of the stream be scheduled only once they have ended, so an
- * attention call directly behind one of them may make the promise for the descriptors that it wrote. */
+ * ss_next_draft and ss_tree_prune let the next kernel of the stream be scheduled only once their descriptors are in
+ * memory, so an attention call directly behind one of them may make the promise for these. */
 #define SS_ATTN_PREFIX_STABLE 1u
 
 typedef struct ss_attn_params {

@@ -35,7 +35,8 @@ __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("gridd
 
 // The other half: lets the next kernel of the stream be scheduled from here on.  Called after the wait only, so at most
 // two kernels of a stream are ever on the GPU: what ran before the previous kernel is complete.  A kernel that writes tree
-// descriptors does not call it: an attention call behind it may promise that they are stable and reads them before its wait.
+// descriptors calls it only once they are in memory, or not at all: an attention call behind it may promise that they are
+// stable and reads them before its wait.
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // `cluster` CTAs along x form a cluster; early: may be scheduled while the previous kernel of the stream drains
