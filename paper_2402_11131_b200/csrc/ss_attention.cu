@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
     const int group = blockIdx.x >> a.cluster_shift;       // (pair, row block): the CTAs that share its keys
     const int rb = group % a.n_blocks;
     const int pair = group / a.n_blocks;
-    int b = pair / a.n_heads;                              // the sequence (for a batch: its place in the dispatch order, see below)
+    const int b = pair / a.n_heads;                        // the sequence
     const int h = pair - b * a.n_heads;
     const int nk = a.n_kslots, nv_slots = a.n_vslots;
     volatile int* abort_flag = &c.abort;
@@ -852,21 +852,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
     // their latency passes while the barriers are set up (volatile: the loads stay where they are written).
     int L = 0, T = 0, cap = 0x7fffffff;
     long long slot0 = 0;
-    // A batch whose grid takes several waves is dispatched longest sequence first (CTAs start in the order of
-    // their index), so that the last wave holds the short ones: place s of the order goes to the sequence with
-    // the s-th longest prefix.  Every warp ranks the (at most 32) lengths for itself.
-    const bool by_length = a.batch > 1 && a.batch <= 32 && C == 1;
     auto load_scalars = [&]() {
-        if (by_length) {
-            int len = -1;
-            if (lane < a.batch) asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(len) : "l"(a.kv_len + lane) : "memory");
-            int longer = 0;                                // sequences that come before this lane's in the order
-            for (int o = 0; o < a.batch; ++o) {
-                const int other = __shfl_sync(0xffffffffu, len, o);
-                longer += (other > len || (other == len && o < lane)) ? 1 : 0;
-            }
-            b = __ffs(__ballot_sync(0xffffffffu, lane < a.batch && longer == b)) - 1;
-        }
         asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(L) : "l"(a.kv_len + b) : "memory");
         asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(T) : "l"(&a.trees[b].n_nodes) : "memory");
         asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(slot0) : "l"(a.kv_start + b) : "memory");
@@ -1567,9 +1553,10 @@ size_t AttnPlan::few_bytes() const { return cluster > 1 ? static_cast<size_t>(gr
 
 // Rows of a block of the few-rows kernel (16, 32 or 64), 0 where a tcgen05 kernel is the better one.  The few-rows kernel
 // has little fixed cost (4 us a layer where the tcgen05 ones take 8) but pays more per key, the more the more rows and
-// dimensions.  The lengths are on the device; the slab says how many slots a sequence has on average, which bounds them, so a
-// cache much larger than its contents gets the tcgen05 kernels.  The lines lie where the kernels met (us per layer of 32
-// heads, one sequence unless said otherwise, tcgen05 / few rows).
+// dimensions.  The lengths are on the device; the slab says how many slots a sequence has on average, which bounds the mean
+// length: a cache much larger than its contents gets the tcgen05 kernels, and a batch in which one sequence is far longer
+// than the rest is taken for a short one.  The lines lie where the kernels met (us per layer of 32 heads, one sequence unless said
+// otherwise, tcgen05 / few rows).
 static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups, int split) {
     const long long slots = p.kv_total_slots / p.batch, keys = slots / split;        // keys per CTA of a grid of one wave
     const bool d64 = p.head_dim == 64, d80 = p.head_dim == 80;
@@ -1577,8 +1564,12 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
     const int blocks = (q_rows + 31) / 32;
     const long long load = static_cast<long long>(p.batch) * p.n_heads * blocks * slots / sm_count();
     if (q_rows <= 32) {
-        // up to 80 dimensions at every length measured (128 to 4096 keys), and where the grid takes several waves (the CTAs that
-        // share an SM hide each other's fixed cost); 27 rows of 128, 800 keys 9.7 / 9.4, 1500 keys 10.7 / 11.6
+        // up to 80 dimensions at every length measured (128 to 4096 keys).  One sequence, 12 rows of 128: 4000 keys 15.9 / 15.4, 6000 keys
+        // 20.5 / 20.8, eight heads and 6000 keys 11.6 / 11.5, 9000 keys 13.8 / 16.1; 27 rows of 128: 800 keys 9.9 / 9.0, 2000 keys 11.9 /
+        // 13.0.  And where the grid takes several waves, at any length (the others are then the kernel with two CTAs per SM): sixteen
+        // sequences, 12 rows of 128, 130 keys 19.1 / 14.6, 2048 keys 89.4 / 84.3; 27 rows of 80, 130 keys 18.5 / 15.2, 2048 keys 68.0 / 64.9; of
+        // 128, 130 keys 19.8 / 19.3, 512 keys 33.8 / 36.2, 2048 keys 91.5 / 92.9, but 256 to 4096 keys 92.0 / 90.0 and fifteen of 64 beside one of
+        // 4096 65.6 / 52.8
         const int rows = q_rows <= 16 ? 16 : 32;
         return p.head_dim <= 80 || groups > sm_count() || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
     }
@@ -1586,7 +1577,8 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
         // more heads than SMs.  Sixteen sequences, 64 rows of 64, 130 keys 20.0 / 18.3, 330 keys 25.8 / 25.7, 1024 keys 40.3 / 47.0; of
         // 80, 30 keys 18.5 / 17.2, 130 keys 22.4 / 22.5, 1024 keys 45.0 / 57.3; of 128, 30 keys 20.5 / 21.6, 512 keys 36.2 / 48.6
         if (groups > sm_count()) return slots <= (d64 ? 390 : d80 ? 180 : 0) ? 64 : 0;
-        // 64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
+        // (a batch goes by its mean: sixteen sequences of eight heads, 64 rows of 64, 200 keys 9.7 / 7.8, fifteen of 64 beside one of 2048
+        // 16.6 / 28.6.)  64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
         // keys 11.0 / 12.8
         if (keys <= (d64 ? 280 : d80 ? 290 : 180)) return 64;
         // two blocks of 32 rows, two CTAs per SM: 64 rows of 64, eight heads and 4096 keys 9.7 / 7.8 (64-row blocks 10.4)

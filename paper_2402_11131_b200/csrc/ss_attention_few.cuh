@@ -127,7 +127,8 @@ struct SpanF {
 // Tiles of a head up to which it is not split (what a split saves on the tiles has to outweigh the merge of the partial
 // rows, about 2 us), and tiles per CTA that a split aims at.  Measured on plain layers of 32 heads, us: 12 rows of 64,
 // 300 keys whole 4.4, split 5.2; 512 keys 5.0 and 5.8; 800 keys 6.5 and 5.5.  27 rows of 80, 512 keys: 4 tiles per CTA 7.0,
-// 8 tiles 8.6.
+// 8 tiles 8.6.  12 rows of 128, 130 keys 4.3 and 5.9, 500 keys 8.4 and 6.4; 64 rows of 64, 130 keys 6.2 and 6.5, 400 keys 8.9 and 6.8; of
+// 128, 100 keys 8.0 and 9.0, 200 keys 10.5 and 9.4.
 __host__ __device__ constexpr int few_whole(int head_dim, int rows) {
     return rows == 16 ? (head_dim > 64 ? 8 : 20) : rows == 32 ? 6 : 8;
 }

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     const int blk = static_cast<int>(blockIdx.x);
     const uint32_t rank = blk & (C - 1);
     const int group = blk >> a.cluster_shift;              // (sequence, head)
-    int b = group / a.n_heads;
+    const int b = group / a.n_heads;
     const int h = group - b * a.n_heads;
     const int n_ring = a.n_kslots >> 1;                    // depth of the K ring and of the V ring
     if (tid == 0) SS_TRC(0, 0);
@@ -162,18 +162,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     // ---- prologue (see msa_attention_kernel: the same launch protocol) ------------------------------
     int L = 0, T = 0, cap = 0x7fffffff;
     long long slot0 = 0;
-    const bool by_length = a.batch > 1 && a.batch <= 32 && C == 1;
     auto load_scalars = [&]() {
-        if (by_length) {
-            int len = -1;
-            if (lane < a.batch) asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(len) : "l"(a.kv_len + lane) : "memory");
-            int longer = 0;
-            for (int o = 0; o < a.batch; ++o) {
-                const int other = __shfl_sync(0xffffffffu, len, o);
-                longer += (other > len || (other == len && o < lane)) ? 1 : 0;
-            }
-            b = __ffs(__ballot_sync(0xffffffffu, lane < a.batch && longer == b)) - 1;
-        }
         asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(L) : "l"(a.kv_len + b) : "memory");
         asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(T) : "l"(&a.trees[b].n_nodes) : "memory");
         asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(slot0) : "l"(a.kv_start + b) : "memory");
