@@ -106,18 +106,21 @@ int32_t ss_tree_build(const int32_t* parent, int32_t n_nodes, int32_t gamma, ss_
  *                                  optional natural-log sum-exp of the scaled scores (NULL to skip).
  * Scores are sm_scale * <q, k>; softmax statistics and both products accumulate in fp32.
  * The workspace holds, after its 256-byte header, the partial rows (fp32 O, m, l per query row) of blocks
- * of 128 query rows whose keys are split over several CTAs (ss_msa_attention_workspace_bytes).  The rows are
+ * of query rows whose keys are split over several CTAs (ss_msa_attention_workspace_bytes).  The rows are
  * their own arrival flags: between calls that area is all zero, a partial row is never stored with a +0
  * word (-0 is stored instead), a CTA waits for the words it combines to read non-zero and stores zeros over
  * them afterwards.  So calls of different shapes may share one workspace as long as they are ordered on one
  * stream and it is large enough for each.  Word 1 of the workspace, if positive, shortens the bound of the
  * device-side waits to that many units of 1024 cycles (default: about one second) for calls whose heads
  * have at most 64 query rows and for ss_wait_selftest; the library reads it and never writes it.
- * Word 2 counts, over all calls since the caller last cleared it, the CTAs of unsplit 128-row blocks that
- * started over: such a block first takes every row's exponentials against the maximum of the row's first
- * 128 keys, and if a later tile exceeds that reference by more than about 2^57 it runs its tiles again
- * with a running maximum (same result, about twice the time for that block).  Diagnostics only.
- * Precondition of a split (batch * n_heads * row blocks below the SM count, twice that for at most 32 rows): the CTAs that share a block's
+ * Word 2 counts, over all calls since the caller last cleared it, the CTAs of unsplit blocks that started
+ * over.  Blocks of 64 or 128 rows of grids of more blocks than SMs, and unsplit blocks of 128 rows of smaller
+ * grids, first take every row's exponentials against the maximum of the row's first 64 (128) keys.  If a
+ * later tile exceeds that reference by more than about 2^57, the CTA runs its tiles again: the former after a
+ * further pass over its keys that takes the exact maxima, the latter
+ * with a running maximum (about twice the time for that block).  The result is the same.  Diagnostics only.
+ * Precondition of a split (a grid of less than one CTA per SM; of less than two where the rows go in blocks of
+ * at most 32, which layers with few rows or few keys do whatever their number): the CTAs that share a block's
  * keys wait for one another's partial rows at the end, so they must all be resident at once.  The call sizes the split from
  * the device's SM count; if other work holds SMs for the whole duration of the call (another stream, another
  * process, a partition of the GPU) the wait can run out: the CTAs then give up, the status word reads
