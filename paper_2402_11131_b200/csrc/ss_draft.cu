@@ -8,11 +8,40 @@
 // cluster takes the whole sequence and nothing goes through global memory.  Compiled without fast-math.
 // Measured on a B200, before (chunks of 4096 logits, partial results and candidate lists through global memory, serial
 // tails) and after: soft verification of 32 rows of 51200 logits 15.3 and 6.4 us, sampled verification of 64 rows of
-// 32000 34.1 and 8.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of
+// 32000 34.1 and 8.2 us, pruning over 1024 rows of 32000 126 and 31 us (28 with packed exponentials and without the sums that only
+// the verification uses), the next draft of 16 sequences (64 rows of
 // 32000) 15.6 and 8.9 us.
 #include "ss_rows.cuh"
 
 namespace ss {
+
+// packed pairs of fp32 (one instruction for two values)
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float exp2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 constexpr float kTinyExp = -200.f;                        // exp of it is 0 in fp32
 
@@ -167,25 +196,65 @@ __device__ __forceinline__ Stats merge_two(const Stats& a, const Stats& b) {
     r.z += o.z * e;
     return r;
 }
-// A thread's running statistics against its running maximum
+// exp(x - m) for pairs of logits: 2^t of t = (x - m) log2(e), and what t lost to rounding as a factor 1 + r ln(2).  Six packed
+// operations, two clamps and two exponentials a pair: a third of what expf, the clamp and the sums take.  The clamp is for -inf
+// and for NaN: they add nothing.  (exp(-100) is 0 with what is flushed to zero)
+struct ExpPair {
+    unsigned long long e, d;      // the exponentials; x - m
+};
+__device__ __forceinline__ ExpPair exp_pair(float x0, float x1, unsigned long long minus_m) {
+    const unsigned long long log2e = pack2(1.44269502f, 1.44269502f), log2e_low = pack2(1.92596299e-8f, 1.92596299e-8f);
+    const unsigned long long ln2 = pack2(0.693147182f, 0.693147182f), one = pack2(1.f, 1.f);
+    float d0, d1;
+    unpack2(add2(pack2(x0, x1), minus_m), d0, d1);
+    const unsigned long long d = pack2(fmaxf(d0, -100.f), fmaxf(d1, -100.f));
+    const unsigned long long t = mul2(d, log2e);
+    const unsigned long long r = fma2(d, log2e_low, fma2(d, log2e, t ^ 0x8000000080000000ull));
+    float t0, t1;
+    unpack2(t, t0, t1);
+    return {mul2(pack2(exp2_approx(t0), exp2_approx(t1)), fma2(r, ln2, one)), d};
+}
+// A thread's running statistics against its running maximum.  FULL: with the index of the maximum and W (pruning needs neither).
+template <bool FULL>
 struct RowStats {
     ArgMax am;
-    float z = 0.f, w = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float d = fmaxf(x - am.v, kTinyExp), e = expf(d);       // (for -inf and for NaN too: no product is a NaN)
-        z += e;
-        w += d * e;
-    }
+    unsigned long long z[2] = {0ull, 0ull}, w[2] = {0ull, 0ull};     // two pairs of partial sums each
     __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) {
         const float m_old = am.v;
-        am.batch(q, word);
+        if constexpr (FULL) {
+            am.batch(q, word);
+        } else {
+            #pragma unroll
+            for (int k = 0; k < kRowVecs; ++k) am.v = fmaxf(am.v, fmaxf(fmaxf(q[k].x, q[k].y), fmaxf(q[k].z, q[k].w)));     // (a NaN is never the maximum)
+        }
         if (am.v > m_old) {
             const float d = fmaxf(m_old - am.v, kTinyExp), e = expf(d);
-            w = (w + d * z) * e;
-            z *= e;
+            #pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                if constexpr (FULL) w[j] = mul2(fma2(pack2(d, d), z[j], w[j]), pack2(e, e));
+                z[j] = mul2(z[j], pack2(e, e));
+            }
         }
+        const unsigned long long minus_m = pack2(-am.v, -am.v);
         #pragma unroll
-        for (int k = 0; k < kRowVecs; ++k) { add(q[k].x); add(q[k].y); add(q[k].z); add(q[k].w); }
+        for (int k = 0; k < kRowVecs; ++k) {
+            #pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const ExpPair p = j ? exp_pair(q[k].z, q[k].w, minus_m) : exp_pair(q[k].x, q[k].y, minus_m);
+                z[j] = add2(z[j], p.e);
+                if constexpr (FULL) w[j] = fma2(p.d, p.e, w[j]);
+            }
+        }
+    }
+    __device__ __forceinline__ Stats stats(const Segment& s) const {
+        Stats st;
+        st.best = am.best(s);
+        float a, b;
+        unpack2(add2(z[0], z[1]), a, b);
+        st.z = a + b;
+        unpack2(add2(w[0], w[1]), a, b);
+        st.w = a + b;
+        return st;
     }
 };
 // =============================================================================================================
@@ -270,16 +339,14 @@ next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int
 }
 
 // =============================================================================================================
-// Row statistics of every node's logits, then per sequence either the pruning of the tree (mode 0) or the
-// soft verification (mode 1).
+// Row statistics of every node's logits, then per sequence either the pruning of the tree or the soft verification.
 struct NodeTailArgs {
-    int mode;
     float threshold, eps, delta;
     float* edge_prob;                 // [B][max_nodes]
-    float* node_entropy;              // mode 1, may be null
-    int32_t *new_index, *kept_nodes, *kept_tokens;     // mode 0
-    ss_tree_desc* pruned_trees;                         // mode 0
-    int32_t *accept_len, *accept_path, *last_node, *bonus_token;   // mode 1
+    float* node_entropy;              // verification, may be null
+    int32_t *new_index, *kept_nodes, *kept_tokens;     // pruning
+    ss_tree_desc* pruned_trees;                         // pruning
+    int32_t *accept_len, *accept_path, *last_node, *bonus_token;   // verification
 };
 // What a row leaves for the sequence's tail: which of its children's edges are ok, and its arg-max
 struct RowOut {
@@ -324,6 +391,8 @@ __device__ __forceinline__ void prune_tail(int T, int max_nodes, int b, unsigned
     if (i == 0) { out->n_nodes = n; out->gamma = gamma; out->max_depth = md; out->reserved = 0; }
 }
 
+// SOFT: the verification, else the pruning
+template <bool SOFT>
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
                   int max_nodes, int vocab, int n_cta, NodeTailArgs ta, int32_t* __restrict__ counters, RowOut* __restrict__ rows) {
@@ -336,7 +405,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     __shared__ uint32_t s_ok[2];
     if (n_cta > 1) cluster_arrive();
     wait_for_previous_kernel();
-    if (ta.mode != 0) release_next_kernel();              // (pruning writes descriptors)
+    if (SOFT) release_next_kernel();                      // (pruning writes descriptors)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
     const size_t row = static_cast<size_t>(b) * max_nodes + t;
     if (t >= max(T, 1)) {
@@ -347,7 +416,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
-    RowStats rs;
+    RowStats<SOFT> rs;
     scan_segment<kRowThreads>(seg, rs);
     tree.store(s_tree, T);
     // the logits of the node's children: on their way while the statistics are merged
@@ -358,9 +427,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
         legal = t < i && tree.tok >= 0 && tree.tok < vocab;
         if (legal) child = logits[row * vocab + tree.tok];
     }
-    Stats st;
-    st.best = rs.am.best(seg); st.z = rs.z; st.w = rs.w;
-    st = warp_merge(st);
+    Stats st = warp_merge(rs.stats(seg));
     constexpr int kWarps = kRowThreads / 32;
     if (!hand_to_first(rank, n_cta, [&]() {
             if ((i & 31) == 0) {
@@ -380,14 +447,17 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
         // log-sum-exp and entropy of the row, and the bar that its children's probabilities have to reach
         const float logz = logf(st.z);
         s_lse = entry_value(st.best) + logz;
-        const float ent = logz - st.w / st.z;
-        s_bar = ta.mode == 0 ? ta.threshold : fminf(ta.eps, ta.delta * expf(-ent));
-        if (t < T && ta.node_entropy) ta.node_entropy[row] = ent;
+        s_bar = ta.threshold;
+        if (SOFT) {
+            const float ent = logz - st.w / st.z;
+            s_bar = fminf(ta.eps, ta.delta * expf(-ent));
+            if (t < T && ta.node_entropy) ta.node_entropy[row] = ent;
+        }
         if (t == 0 && T > 0) ta.edge_prob[row] = 1.f;     // the root
         s_none = st.best == 0ull;
     }
     __syncthreads();
-    if (s_none) st.best = best_of_any(logits, row, vocab, s_any);
+    if (SOFT && s_none) st.best = best_of_any(logits, row, vocab, s_any);
     if (i < SS_MAX_NODES) {
         const float prob = legal ? expf(child - s_lse) : 0.f;
         if (mine) ta.edge_prob[static_cast<size_t>(b) * max_nodes + i] = prob;
@@ -421,7 +491,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     asm volatile("bar.sync 1, 64;" ::: "memory");
     const unsigned long long ok = 1ull | (static_cast<unsigned long long>(s_all[0][1] | s_all[1][1]) << 32) | (s_all[0][0] | s_all[1][0]);
     if (i == 0) counters[b] = 0;                          // leave the workspace ready for the next call
-    if (ta.mode == 0) {
+    if constexpr (!SOFT) {
         prune_tail(T, max_nodes, b, ok, s_tree, trees[b].gamma, ta);
     } else if (i < 32) {
         int len = 1;
@@ -544,6 +614,7 @@ extern "C" size_t ss_tree_prune_workspace_bytes(int32_t batch, int32_t max_nodes
     return ss::scan_workspace(batch, max_nodes, vocab, sizeof(ss::Stats));
 }
 
+template <bool SOFT>
 static int32_t launch_node_stats(const float* logits, const int32_t* tokens, const ss_tree_desc* trees, int32_t batch,
                                  int32_t max_nodes, int32_t vocab, const ss::NodeTailArgs& ta, void* workspace, size_t workspace_bytes,
                                  void* stream) {
@@ -555,7 +626,7 @@ static int32_t launch_node_stats(const float* logits, const int32_t* tokens, con
     const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
-    const cudaError_t err = ss::launch_rows(ss::node_stats_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
+    const cudaError_t err = ss::launch_rows(ss::node_stats_kernel<SOFT>, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
                                             static_cast<cudaStream_t>(stream), logits, tokens, trees, max_nodes, vocab, n_cta, ta,
                                             reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes),
                                             reinterpret_cast<ss::RowOut*>(ws + ss::kWsHeaderBytes + counter_bytes));
@@ -569,9 +640,9 @@ extern "C" int32_t ss_tree_prune(const float* exit_logits, const int32_t* draft_
     if (!new_index || !kept_nodes || !kept_tokens || !pruned_trees) return SS_ERR_INVALID_ARG;
     if (!(threshold == threshold)) return SS_ERR_INVALID_ARG;
     ss::NodeTailArgs ta = {};
-    ta.mode = 0; ta.threshold = threshold; ta.edge_prob = edge_prob;
+    ta.threshold = threshold; ta.edge_prob = edge_prob;
     ta.new_index = new_index; ta.kept_nodes = kept_nodes; ta.kept_tokens = kept_tokens; ta.pruned_trees = pruned_trees;
-    return launch_node_stats(exit_logits, draft_tokens, trees, batch, max_nodes, vocab, ta, workspace, workspace_bytes, stream);
+    return launch_node_stats<false>(exit_logits, draft_tokens, trees, batch, max_nodes, vocab, ta, workspace, workspace_bytes, stream);
 }
 
 extern "C" int32_t ss_tree_verify_soft(const float* logits, const int32_t* draft_tokens, const ss_tree_desc* trees, int32_t batch,
@@ -581,9 +652,9 @@ extern "C" int32_t ss_tree_verify_soft(const float* logits, const int32_t* draft
     if (!accept_len || !accept_path || !last_node || !bonus_token) return SS_ERR_INVALID_ARG;
     if (!(eps == eps) || !(delta == delta)) return SS_ERR_INVALID_ARG;
     ss::NodeTailArgs ta = {};
-    ta.mode = 1; ta.eps = eps; ta.delta = delta; ta.edge_prob = edge_prob; ta.node_entropy = node_entropy;
+    ta.eps = eps; ta.delta = delta; ta.edge_prob = edge_prob; ta.node_entropy = node_entropy;
     ta.accept_len = accept_len; ta.accept_path = accept_path; ta.last_node = last_node; ta.bonus_token = bonus_token;
-    return launch_node_stats(logits, draft_tokens, trees, batch, max_nodes, vocab, ta, workspace, workspace_bytes, stream);
+    return launch_node_stats<true>(logits, draft_tokens, trees, batch, max_nodes, vocab, ta, workspace, workspace_bytes, stream);
 }
 
 extern "C" size_t ss_tree_verify_sampled_workspace_bytes(int32_t batch, int32_t max_nodes, int32_t vocab) {
