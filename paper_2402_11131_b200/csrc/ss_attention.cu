@@ -311,6 +311,37 @@ __device__ __forceinline__ void tc_mma_ts_w(uint32_t lead, uint32_t d_tmem, uint
     asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead) : "memory");
 }
+// The same for STEPS (1 to 4) steps of 16 elements of the contraction inside one 64-element box, in one block with an election
+// of its own, for a warp in step whose index and loop bounds the compiler knows to be uniform.  The steps of an operand are
+// additions to the low word of its descriptor (or to its TMEM column).  The first step accumulates if `acc` is not zero.
+#define SS_MMA_STEP(A, B, P) "@e tcgen05.mma.cta_group::1.kind::f16 [%0], " A ", " B ", %5, " P ";\n\t"
+#define SS_MMA_NEXT(SA, SB) "add.u32 x, %1, " SA ";\n\tmov.b64 a, {x, %2};\n\tadd.u32 x, %3, " SB ";\n\tmov.b64 b, {x, %4};\n\t" SS_MMA_STEP("a", "b", "t")
+#define SS_MMA_NEXT_TS(SA, SB) "add.u32 y, %1, " SA ";\n\tadd.u32 x, %2, " SB ";\n\tmov.b64 b, {x, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [y], b, %4, t;\n\t"
+template <int STEPS>
+__device__ __forceinline__ void tc_mma_steps(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    const uint32_t alo = static_cast<uint32_t>(a), ahi = static_cast<uint32_t>(a >> 32), blo = static_cast<uint32_t>(b), bhi = static_cast<uint32_t>(b >> 32);
+    if constexpr (STEPS == 1)
+        asm volatile("{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %6, 0;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+                     SS_MMA_STEP("a", "b", "p") "}" ::"r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p, e, t;\n\t.reg .b32 x;\n\t.reg .b64 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %6, 0;\n\tsetp.eq.u32 t, 0, 0;\n\t"
+                     "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+                     SS_MMA_STEP("a", "b", "p") SS_MMA_NEXT("2", "2") SS_MMA_NEXT("4", "4") SS_MMA_NEXT("6", "6") "}"
+                     ::"r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc) : "memory");
+    static_assert(STEPS == 1 || STEPS == 4, "of a box of 64 elements");
+}
+// four steps with A in TMEM (8 columns a step) and B MN-major (2048 bytes a step)
+__device__ __forceinline__ void tc_mma_ts_steps(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    const uint32_t blo = static_cast<uint32_t>(b), bhi = static_cast<uint32_t>(b >> 32);
+    asm volatile("{\n\t.reg .pred p, e, t;\n\t.reg .b32 x, y;\n\t.reg .b64 b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.u32 t, 0, 0;\n\t"
+                 "mov.b64 b, {%2, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t"
+                 SS_MMA_NEXT_TS("8", "128") SS_MMA_NEXT_TS("16", "256") SS_MMA_NEXT_TS("24", "384") "}"
+                 ::"r"(d), "r"(a), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tc_commit_e(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 

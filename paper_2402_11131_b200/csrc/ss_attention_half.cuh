@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(16) CtrlH c;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = static_cast<int>(uniform(tid >> 5)), lane = tid & 31;
     const int rb = M == 64 ? 0 : static_cast<int>(blockIdx.x) % a.n_blocks;              // row block of the head
     const int pair = M == 64 ? static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x) / a.n_blocks;
     int b = pair / a.n_heads;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
     int* const status = a.status;
     const uint32_t q_base = smem_u32(smem_raw);            // [half][M rows][128 B], 1024-byte aligned (checked below)
     const uint32_t k_base = q_base + G::kQBytes, v_base = k_base + G::kRingK * G::kSlotBytes;   // [slot][half][64 keys][128 B]
-    const bool is_softmax = warp < 8, producer = tid == kHfSoftmax, issuer = warp == 9;
+    const bool is_softmax = warp < 8, producer = tid == kHfSoftmax;
 
     // ---- prologue (see msa_attention_kernel: the same launch protocol) ------------------------------
     int L = 0, T = 0, cap = 0x7fffffff;
@@ -184,6 +184,8 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         dependency_wait();
         load_scalars();
     }
+    L = static_cast<int>(uniform(L));                       // (for the compiler: what follows from them is the same in all lanes)
+    T = static_cast<int>(uniform(T));
     const long long spec_row0 = static_cast<long long>(b) * a.max_nodes * a.gamma;
     T = min(max(T, 0), a.max_nodes);
     const bool over = L < 0 || L + T > cap, bad_smem = (q_base & 1023u) != 0u;       // (the latter never expected)
@@ -262,7 +264,6 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
         for (int s = 0; s < G::kRingK; ++s) if (n_k > s) mbar_drain(smem_u32(&c.k_full[s]), ((n_k - 1 - s) / G::kRingK) & 1);
         for (int s = 0; s < G::kRingV; ++s) if (n_v > s) mbar_drain(smem_u32(&c.v_full[s]), ((n_v - 1 - s) / G::kRingV) & 1);
     };
-    const uint32_t lead = issuer ? elect_lane() : 0u;       // the lane that issues the MMAs
     const uint32_t tmem_o = c.tmem_base, tmem_s = tmem_o + 128;
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
 
@@ -332,13 +333,10 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             tc_fence_after();
             const uint64_t dk = desc_k_major(uniform(k_base + rk.slot * G::kSlotBytes));
             const uint32_t sd = uniform(ut_s + (ts & 1) * kHfKeys);
-            #pragma unroll
-            for (int ks = 0; ks < G::kKSteps; ++ks) {
-                const uint32_t at = (ks & 3) * 32u;
-                tc_mma_w(lead, sd, dq + (((ks >> 2) * G::kQHalfBytes + at) >> 4), dk + (((ks >> 2) * G::kBoxBytes + at) >> 4), G::kIdescS, ks > 0);
-            }
-            tc_commit_w(lead, smem_u32(&c.s_full[ts & 1]));
-            tc_commit_w(lead, smem_u32(&c.k_empty[rk.slot]));
+            tc_mma_steps<4>(sd, dq, dk, G::kIdescS, 0u);
+            if constexpr (G::kHalves == 2) tc_mma_steps<G::kKSteps - 4>(sd, dq + (G::kQHalfBytes >> 4), dk + (G::kBoxBytes >> 4), G::kIdescS, 1u);
+            tc_commit_e(smem_u32(&c.s_full[ts & 1]));
+            tc_commit_e(smem_u32(&c.k_empty[rk.slot]));
             rk.advance(G::kRingK);
             ++ts;
             return true;
@@ -353,11 +351,9 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             if (!kMax) {
                 const uint64_t dv = desc_mn_major(uniform(v_base + rv.slot * G::kSlotBytes), G::kBoxBytes);
                 const uint32_t pa = uniform(ut_s + buf * kHfKeys);
-                #pragma unroll
-                for (int ks = 0; ks < kHfKeys / 16; ++ks)
-                    tc_mma_ts_w(lead, ut_o, pa + 8u * ks, dv + ((ks * 2048u) >> 4), G::kIdescPV, (t > 0 || ks > 0) ? 1u : 0u);
-                tc_commit_w(lead, smem_u32(&c.v_empty[rv.slot]));
-                if (t == sp.n - 1) tc_commit_w(lead, smem_u32(&c.o_done));
+                tc_mma_ts_steps(ut_o, pa, dv, G::kIdescPV, t > 0 ? 1u : 0u);
+                tc_commit_e(smem_u32(&c.v_empty[rv.slot]));
+                if (t == sp.n - 1) tc_commit_e(smem_u32(&c.o_done));
             }
             if (ts < sp.n && !issue_s()) break;           // S of tile t + 2 over the buffer that P V of tile t reads before it
         }
@@ -513,7 +509,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
                 land();
                 mbar_drain(smem_u32(&c.q_full), 0);
             } else if (warp == 9) {
-                tc_commit_w(lead, smem_u32(&c.drain));
+                tc_commit_e(smem_u32(&c.drain));
                 mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(pass));
             }
             __syncwarp();
@@ -562,7 +558,7 @@ __global__ void __launch_bounds__(kHfThreads, 2) msa_attention_half_kernel(const
             land();
             mbar_drain(smem_u32(&c.q_full), 0);
         } else if (warp == 9) {
-            tc_commit_w(lead, smem_u32(&c.drain));
+            tc_commit_e(smem_u32(&c.drain));
             mbar_drain(smem_u32(&c.drain), static_cast<uint32_t>(*reinterpret_cast<volatile int*>(&c.n_drains) & 1));
         }
         __syncwarp();
