@@ -19,7 +19,7 @@
 //   threads 0, 96  TMA producers of the K ring and of the V ring (mbarrier complete_tx); swizzle-128B
 //               boxes straight from the caller's strided tensors.  A K slot is handed back as soon
 //               as S is queued, a V slot after P V.  Thread 0 also requests Q once.
-//   warp 1      tcgen05 issuer of S = Q K^T (128 x 128 keys x d) into one of two TMEM buffers;
+//   warp 1      tcgen05 issuer, all lanes in step, of S = Q K^T (128 x 128 keys x d) into one of two TMEM buffers;
 //   warp 2      tcgen05 issuer of O += P V (A = P in TMEM) into the TMEM accumulator of a warpgroup;
 //               tcgen05.commit arrives on the mbarriers that hand buffers back.
 //   warps 4..11 two softmax warpgroups, one thread per TMEM lane: tcgen05.ld of the row's scores, tree /
@@ -139,6 +139,7 @@ struct Ctrl {
     unsigned long long mref_full[4], drain[2];
     float m_ref[kBlockRows];
     uint32_t tmem_base;
+    int wait_limit;                             // bound of the issuing warps' waits, in units of 1024 cycles
     int abort;                                  // 1: a wait ran out of time; 2: the shared reference did not hold, start over
 #ifdef SS_TRACE
     unsigned int trace_launch;
@@ -274,46 +275,15 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]: A is 128 lanes x 16 bf16, two to a 32-bit column (8 columns per step)
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// The same, issued by the one lane of the warp whose `lead` is set (elect_lane(), taken once: a commit stands for the
-// products of its own thread).  All lanes come here with the same operands, so these are computed and kept in uniform
-// registers; from inside a branch that a single thread takes every operand is moved there by an instruction chain of its
-// own, and an MMA takes 76 to 98 cycles to issue where its execution takes 32 (M = 64, N = 64) to 64 (N = 128).
-__device__ __forceinline__ uint32_t elect_lane() {
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(r));
-    return r;
-}
+// lane 0's value, which the compiler knows to be the same in all lanes
 __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
-__device__ __forceinline__ void tc_commit_w(uint32_t lead, uint32_t bar) {
-    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-                 ::"r"(bar), "r"(lead) : "memory");
-}
-__device__ __forceinline__ void tc_mma_w(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead) : "memory");
-}
-__device__ __forceinline__ void tc_mma_ts_w(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead) : "memory");
-}
-// The same for STEPS (1 to 4) steps of 16 elements of the contraction inside one 64-element box, in one block with an election
-// of its own, for a warp in step whose index and loop bounds the compiler knows to be uniform.  The steps of an operand are
-// additions to the low word of its descriptor (or to its TMEM column).  The first step accumulates if `acc` is not zero.
+// D[tmem] (+)= A * B, bf16 inputs, fp32 accumulate, issued by one elected lane of a warp that comes here in step (a commit stands
+// for the products of its own thread; the election is deterministic).  STEPS (1 or 4) steps of 16 elements of the contraction
+// inside one 64-element box go in one block; a step is an addition to the low word of an operand's descriptor (or to its TMEM
+// column).  The first one accumulates if `acc` is not zero.  With the warp's index and the loop bounds known to be uniform (see
+// uniform()) the operands are kept in uniform registers; where a single thread issues in a branch of its own, or a lane's
+// predicate comes from a register, every MMA takes an instruction chain that competes with the softmax warps for issue slots:
+// 8 + 4 MMAs of a 64-key tile beside them then take some 1.1 k cycles instead of the 512 to 736 that they execute in.
 #define SS_MMA_STEP(A, B, P) "@e tcgen05.mma.cta_group::1.kind::f16 [%0], " A ", " B ", %5, " P ";\n\t"
 #define SS_MMA_NEXT(SA, SB) "add.u32 x, %1, " SA ";\n\tmov.b64 a, {x, %2};\n\tadd.u32 x, %3, " SB ";\n\tmov.b64 b, {x, %4};\n\t" SS_MMA_STEP("a", "b", "t")
 #define SS_MMA_NEXT_TS(SA, SB) "add.u32 y, %1, " SA ";\n\tadd.u32 x, %2, " SB ";\n\tmov.b64 b, {x, %3};\n\t@e tcgen05.mma.cta_group::1.kind::f16 [%0], [y], b, %4, t;\n\t"
@@ -839,7 +809,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
     extern __shared__ unsigned char smem_raw[];
     __shared__ Ctrl c;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = static_cast<int>(uniform(tid >> 5)), lane = tid & 31;
     const int C = a.cluster;
     const uint32_t rank = blockIdx.x & (C - 1);            // C is a power of two
     const int group = blockIdx.x >> a.cluster_shift;       // (pair, row block): the CTAs that share its keys
@@ -896,6 +866,7 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
         mbar_init(smem_u32(&c.q_full), 1);
         for (int s = 0; s < kMaxSlots; ++s) mbar_init(smem_u32(&c.k_full[s]), 1);
         c.abort = 0;
+        c.wait_limit = static_cast<int>(kWaitCycles >> 10);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&a.tm_qm); tma_prefetch_desc(&a.tm_k);
         if (a.gamma > 0) { tma_prefetch_desc(&a.tm_qs); tma_prefetch_desc(&a.tm_qs1); tma_prefetch_desc(&a.tm_ks); }
@@ -945,6 +916,8 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
     }
     if (tid == 0) SS_TR(0, 3);
 
+    L = static_cast<int>(uniform(L));                      // (for the compiler: what follows from them is the same in all lanes)
+    T = static_cast<int>(uniform(T));
     const Span sp = make_span(a, L, T, static_cast<int>(rank), rb, kUnit);
 
     // K tile j / V tile j of the span -> ring slot st (K: thread 0, V: thread 96)
@@ -1064,61 +1037,57 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
     }
     // ============================ warp 1: issues S = Q K^T, one MMA group per tile ================
     else if (warp == 1) {
-        if (lane == 0) {
+        {
             // the query tile is always requested, so it is always awaited (shared memory is reused later)
-            bool ok = mbar_wait(smem_u32(&c.q_full), 0, abort_flag, a.status);
+            bool ok = mbar_wait_uniform(smem_u32(&c.q_full), 0, &c, a.status);
             if (!ok) mbar_drain(smem_u32(&c.q_full), 0);
             SS_TR(1, 0);
             Ring rk;
             rk.start();
             // A descriptor's low word is (address >> 4): a step inside the tile is an addition to the descriptor
-            // (shared memory ends below 2^18, so nothing carries out of the field), and the issuing thread
+            // (shared memory ends below 2^18, so nothing carries out of the field), and the issuing warp
             // spends its cycles on the MMAs, not on rebuilding descriptors
-            const uint64_t dq = desc_k_major(q_base);
+            const uint64_t dq = desc_k_major(uniform(q_base));
             for (int j = 0; ok && j < sp.n_tiles; ++j, rk.advance(nk)) {
                 const int buf = j & 1;
-                if (!mbar_wait(smem_u32(&c.k_full[rk.slot]), rk.round & 1, abort_flag, a.status)) break;
+                if (!mbar_wait_uniform(smem_u32(&c.k_full[rk.slot]), rk.round & 1, &c, a.status)) break;
                 SS_TR(1, 8 + 4 * j);
-                if (j >= 2 && !mbar_wait(smem_u32(&c.s_free[buf]), ((j >> 1) - 1) & 1, abort_flag, a.status)) break;
+                if (j >= 2 && !mbar_wait_uniform(smem_u32(&c.s_free[buf]), ((j >> 1) - 1) & 1, &c, a.status)) break;
                 SS_TR(1, 9 + 4 * j);
                 tc_fence_after();
-                const uint64_t dk = desc_k_major(k_base + rk.slot * G::kSlotBytes);
-                const uint32_t sd = (kShared ? tmem_s1 : tmem_s) + buf * TK;
-                #pragma unroll
-                for (int ks = 0; ks < G::kKSteps; ++ks) {
-                    const uint32_t hh = ks >> 2, off = (ks & 3) * 32u;
-                    tc_mma(sd, dq + ((hh * kQHalfBytes + off) >> 4), dk + ((hh * G::kBoxBytes + off) >> 4), G::kIdescS, ks > 0);
-                }
+                const uint64_t dk = desc_k_major(uniform(k_base + rk.slot * G::kSlotBytes));
+                const uint32_t sd = uniform((kShared ? tmem_s1 : tmem_s) + buf * TK);
+                tc_mma_steps<4>(sd, dq, dk, G::kIdescS, 0u);
+                if constexpr (G::kHalves == 2) tc_mma_steps<G::kKSteps - 4>(sd, dq + (kQHalfBytes >> 4), dk + (G::kBoxBytes >> 4), G::kIdescS, 1u);
                 SS_TR(1, 10 + 4 * j);
-                tc_commit(smem_u32(&c.s_full[0][buf]));
-                if (!kShared) tc_commit(smem_u32(&c.s_full[1][buf]));
-                tc_commit(smem_u32(&c.k_empty[rk.slot]));                // S of tile j is queued: K may go
+                tc_commit_e(smem_u32(&c.s_full[0][buf]));
+                if (!kShared) tc_commit_e(smem_u32(&c.s_full[1][buf]));
+                tc_commit_e(smem_u32(&c.k_empty[rk.slot]));                // S of tile j is queued: K may go
                 SS_TR(1, 11 + 4 * j);
             }
         }
     }
     // ============================ warp 2: issues O += P V ==========================================
     else if (warp == 2) {
-        if (lane == 0) {
+        {
             Ring rv;
             rv.start();
             bool ok = true;
             for (int j = 0; ok && j < sp.n_tiles; ++j, rv.advance(nv_slots)) {
-                if (!mbar_wait(smem_u32(&c.v_full[rv.slot]), rv.round & 1, abort_flag, a.status)) break;
+                if (!mbar_wait_uniform(smem_u32(&c.v_full[rv.slot]), rv.round & 1, &c, a.status)) break;
                 SS_TR(2, 8 + 4 * j);
-                const uint32_t va = v_base + rv.slot * G::kSlotBytes;
+                const uint32_t va = uniform(v_base + rv.slot * G::kSlotBytes);
                 if constexpr (kShared) {
                     // the tile's 128 keys into the one accumulator; P is read from its own TMEM buffer
                     const int buf = j & 1;
                     const uint64_t dv = desc_mn_major(va, G::kBoxBytes);
-                    if (!mbar_wait(smem_u32(&c.p_full[0][buf]), (j >> 1) & 1, abort_flag, a.status)) break;
+                    if (!mbar_wait_uniform(smem_u32(&c.p_full[0][buf]), (j >> 1) & 1, &c, a.status)) break;
                     SS_TR(2, 9 + 4 * j);
                     tc_fence_after();
-                    const uint32_t pa = tmem_p1 + buf * (TK / 2);
-                    #pragma unroll
-                    for (int ks = 0; ks < TK / 16; ++ks)
-                        tc_mma_ts(tmem, pa + ks * 8u, dv + ((ks * 2048u) >> 4), G::kIdescPV, (j > 0 || ks > 0) ? 1u : 0u);
-                    tc_commit(smem_u32(&c.o_done[buf][(j >> 1) & 1]));   // P of the buffer may be overwritten
+                    const uint32_t od = uniform(tmem), pa = uniform(tmem_p1 + buf * (TK / 2));
+                    tc_mma_ts_steps(od, pa, dv, G::kIdescPV, j > 0 ? 1u : 0u);
+                    tc_mma_ts_steps(od, pa + 32u, dv + ((4 * 2048u) >> 4), G::kIdescPV, 1u);
+                    tc_commit_e(smem_u32(&c.o_done[buf][(j >> 1) & 1]));   // P of the buffer may be overwritten
                 } else {
                     // keys 64w .. 64w+63 into the accumulator of warpgroup w; P is read from TMEM, where the
                     // warpgroup left it over the first 32 columns of its half of the S buffer
@@ -1126,20 +1095,17 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
                     const uint64_t dv = desc_mn_major(va, G::kBoxBytes);
                     #pragma unroll
                     for (int w = 0; w < 2; ++w) {
-                        if (!mbar_wait(smem_u32(&c.p_full[w][buf]), (j >> 1) & 1, abort_flag, a.status)) { ok = false; break; }
+                        if (!mbar_wait_uniform(smem_u32(&c.p_full[w][buf]), (j >> 1) & 1, &c, a.status)) { ok = false; break; }
                         if (w == 0) SS_TR(2, 9 + 4 * j);
                         tc_fence_after();
-                        const uint32_t pa = tmem_s + buf * TK + w * 64;
-                        #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            tc_mma_ts(tmem + w * G::kOCols, pa + ks * 8u, dv + (((w * 4 + ks) * 2048u) >> 4), G::kIdescPV, (j > 0 || ks > 0) ? 1u : 0u);
-                        tc_commit(smem_u32(&c.o_done[w][buf]));
+                        tc_mma_ts_steps(uniform(tmem + w * G::kOCols), uniform(tmem_s + buf * TK + w * 64), dv + ((w * 4 * 2048u) >> 4), G::kIdescPV, j > 0 ? 1u : 0u);
+                        tc_commit_e(smem_u32(&c.o_done[w][buf]));
                     }
                     if (!ok) break;
-                    tc_commit(smem_u32(&c.s_free[buf]));                 // both halves of P have been read: S may be overwritten
+                    tc_commit_e(smem_u32(&c.s_free[buf]));               // both halves of P have been read: S may be overwritten
                 }
                 SS_TR(2, 10 + 4 * j);
-                tc_commit(smem_u32(&c.v_empty[rv.slot]));                // P V of tile j is queued: V may go when it completes
+                tc_commit_e(smem_u32(&c.v_empty[rv.slot]));              // P V of tile j is queued: V may go when it completes
                 SS_TR(2, 11 + 4 * j);
             }
         }
@@ -1367,9 +1333,9 @@ __global__ void __launch_bounds__(Geo<HD>::kThreads, 1) msa_attention_kernel(con
                 for (int sl = 0; sl < slots; ++sl)
                     if (n_requested > sl) mbar_drain(smem_u32(&full[sl]), ((n_requested - 1 - sl) / slots) & 1);
                 if (tid == 0) mbar_drain(smem_u32(&c.q_full), 0);
-            } else if (tid == 32 || tid == 64) {
-                const uint32_t bar = smem_u32(&c.drain[tid == 64 ? 1 : 0]);
-                tc_commit(bar);
+            } else if (warp == 1 || warp == 2) {
+                const uint32_t bar = smem_u32(&c.drain[warp - 1]);
+                tc_commit_e(bar);                         // (by the lane that issued the MMAs: the election is deterministic)
                 mbar_drain(bar, 0);
             }
             __syncwarp();

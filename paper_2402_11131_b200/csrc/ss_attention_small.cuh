@@ -111,7 +111,7 @@ __device__ __noinline__ void land_all_s(CtrlS* c, int n_ring) {
             if (n > s) mbar_drain(smem_u32(&c->slot_full[kind][s]), static_cast<uint32_t>(((n - 1 - s) / n_ring) & 1));
         if (tid == 0) mbar_drain(smem_u32(&c->q_full), 0);
     } else if (warp == 1 || warp == 2) {
-        tc_commit_w(elect_lane(), smem_u32(&c->drain[warp - 1]));          // (the lane that issued the MMAs: the election is deterministic)
+        tc_commit_e(smem_u32(&c->drain[warp - 1]));                        // (the lane that issued the MMAs: the election is deterministic)
         mbar_drain(smem_u32(&c->drain[warp - 1]), 0);
     }
     __syncwarp();
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(16) CtrlS c;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = static_cast<int>(uniform(tid >> 5)), lane = tid & 31;
     const int C = a.cluster;
     const int blk = static_cast<int>(blockIdx.x);
     const uint32_t rank = blk & (C - 1);
@@ -217,6 +217,8 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
         skip = true;
         L = 0; T = 0;
     }
+    L = static_cast<int>(uniform(L));                       // (for the compiler: what follows from them is the same in all lanes)
+    T = static_cast<int>(uniform(T));
     // whole tiles are dealt out, the first CTAs of a head taking the odd ones: the last CTA has the masked tiles
     const Span sp = make_span(a, L, T, static_cast<int>(rank), 0, kTileKeys, true);
 
@@ -308,13 +310,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
             if (sp.n_tiles > n_early) produce(1);
         }
     }
-    // Warps 1 and 2 issue the MMAs with all lanes in step (see elect_lane); a layer is 0.2 to 0.5 us shorter than with a single
-    // thread in a branch of its own (64 rows of 128, 1024 keys 10.8 / 10.35, 2048 keys 12.5 / 12.2; of 64, 4096 keys 13.7 / 13.2).
-    // (The row blocks' kernel gains nothing by it.)
+    // Warps 1 and 2 issue the MMAs with all lanes in step (see tc_mma_steps); a layer is 0.2 to 0.5 us shorter than with a single
+    // thread in a branch of its own (64 rows of 128, 1024 keys 10.8 / 10.35, 2048 keys 12.5 / 12.2; of 64, 4096 keys 13.7 / 13.2), and
+    // 0.1 to 0.2 us more with their MMAs in blocks of four (13.02 / 12.91, 14.07 / 13.89; 48 rows of 80, 2048 keys 12.23 / 12.02).
     // =============================== warp 1: S = Q K^T ==============================================
     else if (warp == 1) {
         {
-            const uint32_t lead = elect_lane();
             bool ok = mbar_wait_uniform(smem_u32(&c.q_full), 0, &c, status);
             if (!ok) mbar_drain(smem_u32(&c.q_full), 0);
             SS_TRC(1, 0);
@@ -331,14 +332,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
                 tc_fence_after();
                 const uint64_t dk = desc_k_major(uniform(slot_addr(0, r.slot)));
                 const uint32_t sd = uniform(tmem_s + buf * TK);
-                #pragma unroll
-                for (int ks = 0; ks < G::kKSteps; ++ks) {
-                    const uint32_t hh = ks >> 2, off = (ks & 3) * 32u;
-                    tc_mma_w(lead, sd, dq + ((hh * G::kQHalfBytes + off) >> 4), dk + ((hh * G::kBoxBytes + off) >> 4),
-                           idesc_bf16(TK, false, false), ks > 0);
-                }
-                tc_commit_w(lead, smem_u32(&c.s_full[buf]));
-                tc_commit_w(lead, smem_u32(&c.slot_empty[0][r.slot]));                // K may go when S is complete
+                tc_mma_steps<4>(sd, dq, dk, idesc_bf16(TK, false, false), 0u);
+                if constexpr (G::kHalves == 2) tc_mma_steps<HD / 16 - 4>(sd, dq + (G::kQHalfBytes >> 4), dk + (G::kBoxBytes >> 4), idesc_bf16(TK, false, false), 1u);
+                tc_commit_e(smem_u32(&c.s_full[buf]));
+                tc_commit_e(smem_u32(&c.slot_empty[0][r.slot]));                      // K may go when S is complete
                 SS_TRC(1, 10 + 4 * j);
                 r.advance(n_ring);
             }
@@ -347,7 +344,6 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
     // =============================== warp 2: O += P V, A from TMEM ================================
     else if (warp == 2) {
         {
-            const uint32_t lead = elect_lane();
             Ring rv;
             rv.start();
             bool okq = mbar_wait_uniform(smem_u32(&c.q_ready), 0, &c, status);     // the P buffers' constant zeros are in place
@@ -362,12 +358,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) msa_attention_small_kernel(cons
                 const uint32_t od = uniform(tmem_o), pa = uniform(tmem_p + buf * 64u);
                 // P of the tile: the copy's buffer, keys 16 ks .. 16 ks + 15 in columns 8 ks .. 8 ks + 7 (zero in the
                 // other copy's lanes)
-                #pragma unroll
-                for (int ks = 0; ks < TK / 16; ++ks)
-                    tc_mma_ts_w(lead, od, pa + 8u * ks, dv + ((ks * 2048u) >> 4), idesc_bf16(HD, false, true),
-                              (j > 0 || ks > 0) ? 1u : 0u);
-                tc_commit_w(lead, smem_u32(&c.pv_done[j & 3]));
-                tc_commit_w(lead, smem_u32(&c.slot_empty[1][rv.slot]));
+                tc_mma_ts_steps(od, pa, dv, idesc_bf16(HD, false, true), j > 0 ? 1u : 0u);
+                tc_mma_ts_steps(od, pa + 32u, dv + ((4 * 2048u) >> 4), idesc_bf16(HD, false, true), 1u);
+                tc_commit_e(smem_u32(&c.pv_done[j & 3]));
+                tc_commit_e(smem_u32(&c.slot_empty[1][rv.slot]));
                 SS_TRC(2, 10 + 4 * j);
                 rv.advance(n_ring);
             }
