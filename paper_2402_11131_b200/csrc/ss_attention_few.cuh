@@ -79,7 +79,6 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, int c1, int c2) {
     asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ bool mbar_wait_warp_f(uint32_t bar, uint32_t parity, CtrlF* c, int* status) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait_limit_slow(bar, parity, &c->abort, &c->wait_limit, status));

@@ -39,6 +39,8 @@ __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("gridd
 // stable and reads them before its wait.
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // `cluster` CTAs along x form a cluster; early: may be scheduled while the previous kernel of the stream drains
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, bool early, cudaStream_t stream, Args... args) {

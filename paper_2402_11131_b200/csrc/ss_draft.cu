@@ -404,16 +404,17 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     __shared__ float s_lse, s_bar;
     __shared__ uint32_t s_ok[2];
     if (n_cta > 1) cluster_arrive();
+    const size_t row = static_cast<size_t>(b) * max_nodes + t;
+    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
+    prefetch_batch(seg);
     wait_for_previous_kernel();
     if (SOFT) release_next_kernel();                      // (pruning writes descriptors)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
-    const size_t row = static_cast<size_t>(b) * max_nodes + t;
     if (t >= max(T, 1)) {
         if (n_cta > 1) cluster_wait();
         return;
     }
     const int i = static_cast<int>(threadIdx.x);
-    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     RowStats<SOFT> rs;
@@ -517,15 +518,16 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
     __shared__ TreeShared s_tree;
     __shared__ int32_t s_draw[SS_MAX_NODES];
     if (n_cta > 1) cluster_arrive();
+    const size_t row = static_cast<size_t>(b) * max_nodes + t;
+    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
+    prefetch_batch(seg);
     wait_for_previous_kernel();
     release_next_kernel();
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
-    const size_t row = static_cast<size_t>(b) * max_nodes + t;
     if (t >= max(T, 1)) {
         if (n_cta > 1) cluster_wait();
         return;
     }
-    const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     const float u = uniforms[row];

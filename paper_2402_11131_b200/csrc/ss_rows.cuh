@@ -71,6 +71,13 @@ __device__ __forceinline__ Segment make_segment(const float* base, size_t row, i
     s.total = s.skip + hi - lo;
     return s;
 }
+// The first batch of the segment on its way to L2, a line to a thread: no data reaches the SM, so it may be asked for before the
+// wait for the previous kernel, whoever writes the logits.  Calls behind one another, 1024 rows of 32000: arg-max 23.6 -> 21.6 us, softmax
+// sums 28.4 -> 26.8 us; 32 rows of 51200, softmax statistics 7.1 -> 6.8 us.  (Rows that a smaller tree does not own are asked for too.)
+__device__ __forceinline__ void prefetch_batch(const Segment& s) {
+    static_assert(kRowThreads * 32 == kRowThreads * kRowVecs * 4, "a batch is a line of 32 logits to a thread");
+    if (32 * static_cast<int>(threadIdx.x) < s.total) prefetch_l2(s.src + 32 * threadIdx.x);
+}
 // Vector i of the segment (words 4 i .. 4 i + 3); words that are not the segment's read -inf.  The first and the last
 // one are put together from single loads where they are not whole.
 static __device__ __noinline__ float4 edge_vec(const float* src, int i, int skip, int total) {

@@ -21,6 +21,8 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     __shared__ int32_t s_am[SS_MAX_NODES];
     __shared__ TreeShared s_tree;
     if (n_cta > 1) cluster_arrive();                      // CTA 0 must have started before anyone stores to its shared memory
+    const Segment seg = make_segment(logits, static_cast<size_t>(b) * max_nodes + t, vocab, rank, n_cta);
+    prefetch_batch(seg);
     wait_for_previous_kernel();
     release_next_kernel();
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);     // a descriptor is never trusted beyond the arrays' extent
@@ -30,7 +32,6 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     }
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
-    const Segment seg = make_segment(logits, static_cast<size_t>(b) * max_nodes + t, vocab, rank, n_cta);
     ArgMax am;
     scan_segment<kRowThreads>(seg, am);
     tree.store(s_tree, T);
