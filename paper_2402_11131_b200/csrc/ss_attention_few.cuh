@@ -291,6 +291,10 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     if (sp.n > 0) {
         constexpr int kEach = (G::kRows * kPieces + kFwThreads - 1) / kFwThreads;
         uint4 q[kEach];
+        // the caller may shorten the bound of the waits of a head of at most 64 rows (workspace word 1, units of 1024 cycles); asked for
+        // with the query rows: behind them it would be a second round trip to L2 in every CTA's way
+        int lim = 0;
+        if (tid == 0) asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(lim) : "l"(a.status + 1) : "memory");
         #pragma unroll
         for (int k = 0; k < kEach; ++k) {
             const int i = tid + k * kFwThreads;
@@ -308,12 +312,7 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
             if (i < G::kRows * kPieces)
                 st_shared_v4(q_base + (pc >> 3) * G::kQHalf + row * 128u + (static_cast<uint32_t>((pc ^ row) & 7) << 4), q[k].x, q[k].y, q[k].z, q[k].w);
         }
-        if (tid == 0) {
-            // the caller may shorten the bound of the waits of a head of at most 64 rows (workspace word 1, units of 1024 cycles)
-            int lim;
-            asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(lim) : "l"(a.status + 1) : "memory");
-            if (lim > 0 && gridDim.y * G::kRows <= 64) *reinterpret_cast<volatile int*>(&c.wait_limit) = lim;
-        }
+        if (tid == 0 && lim > 0 && gridDim.y * G::kRows <= 64) *reinterpret_cast<volatile int*>(&c.wait_limit) = lim;
     }
     if (tid == 0 && (over || bad_smem)) set_status(status, bad_smem ? SS_ERR_CUDA : SS_ERR_CAPACITY);
     __syncthreads();                                       // the query rows are in shared memory
@@ -492,6 +491,9 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
     constexpr int kItems = HD / 4;
     // the block's rows that nodes own: main rows [row0, row0 + n_main), then stream rows [r0, r1)
     const int n_main = max(min(T - row0, G::kRows), 0), n_rows = n_main + max(r1 - r0, 0);
+    // (one copy of the code for all of a thread's items, which runs once a layer: with the items of a thread unrolled, their loads in flight
+    // together, layers take up to 0.25 us longer)
+    #pragma unroll 1
     for (int i = tid; i < n_rows * kItems; i += kFwThreads) {
         const int rr = i / kItems, g4 = i - rr * kItems;
         RowInfo r;
@@ -503,19 +505,24 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
             r.stream = xr - r.node * a.gamma + 1;
             row = a.tmax8 + xr - row0;
         }
-        // its row group's warp of every team holds the row
+        // its row group's warp of every team holds the row: everything is asked for at once
         const uint32_t at = w_base + static_cast<uint32_t>(row) * RB;
-        float m = -INFINITY, l = 0.f;
-        #pragma unroll 4
-        for (int p = 0; p < G::kTeams; ++p) m = fmaxf(m, ld_shared_v2(at + static_cast<uint32_t>(G::kRows * p) * RB + HD * 4u).x);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        #pragma unroll 2
+        float2 ml[G::kTeams];
+        float4 v[G::kTeams];
+        #pragma unroll
         for (int p = 0; p < G::kTeams; ++p) {
-            const float2 ml = ld_shared_v2(at + static_cast<uint32_t>(G::kRows * p) * RB + HD * 4u);
-            const float4 v = ld_shared_v4(at + static_cast<uint32_t>(G::kRows * p) * RB + static_cast<uint32_t>(g4) * 16u);
-            const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - m);        // 0: saw no visible key
-            l += w * ml.y;
-            acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
+            ml[p] = ld_shared_v2(at + static_cast<uint32_t>(G::kRows * p) * RB + HD * 4u);
+            v[p] = ld_shared_v4(at + static_cast<uint32_t>(G::kRows * p) * RB + static_cast<uint32_t>(g4) * 16u);
+        }
+        float m = -INFINITY, l = 0.f;
+        #pragma unroll
+        for (int p = 0; p < G::kTeams; ++p) m = fmaxf(m, ml[p].x);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        #pragma unroll
+        for (int p = 0; p < G::kTeams; ++p) {
+            const float w = ml[p].x == -INFINITY ? 0.f : exp2f(ml[p].x - m);        // 0: saw no visible key
+            l += w * ml[p].y;
+            acc.x += w * v[p].x; acc.y += w * v[p].y; acc.z += w * v[p].z; acc.w += w * v[p].w;
         }
         if (!split) {
             const OutPtr dst = out_ptr<HD>(a, b, h, spec_row0, r);
