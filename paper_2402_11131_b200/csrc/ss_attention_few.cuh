@@ -53,6 +53,9 @@ struct GeoF {
     // and a parity wait could take the phase before for the one awaited: such a team first waits for the request.
     static constexpr bool kForeign = kRing % kTeams != 0;
     static constexpr bool kQInRegs = HD <= 80;                    // (at 128 the fragments do not fit beside O)
+    // The fragments of a step are loaded while the step before is multiplied.  32 rows of 80, 1024 keys 8.83 / 8.65 us; 16 heads 6.43 / 6.30;
+    // but 16 rows of 64, 512 keys 4.67 / 4.88, 64 rows of 80, 250 keys 7.26 / 7.38, and at 128 neither way.
+    static constexpr bool kAhead = HD == 80 && RG <= 2;
     static_assert(kQBytes % 1024 == 0, "swizzle atoms");
     static_assert(kDynSmem + 1024 <= (228 * 1024) / 2 - 1024, "two CTAs per SM");
     static_assert((kFwWarps * 16 + kRows) * kPitch * 4 <= kDynSmem, "shared memory holds the warps' partial rows and the CTA's");
@@ -358,17 +361,35 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
                 uint32_t ka[4];
                 #pragma unroll
                 for (int j = 0; j < 4; ++j) ka[j] = kt + off_k[j];
-                #pragma unroll
-                for (int ks = 0; ks < G::kKSteps; ++ks) {
-                    uint32_t kf[2][4];
-                    ldsm_x4(ka[ks & 3] + (ks >> 2) * G::kBoxBytes, kf[0]);
-                    ldsm_x4(ka[ks & 3] + (ks >> 2) * G::kBoxBytes + 16 * 128, kf[1]);
-                    if constexpr (!G::kQInRegs) load_q(ks, qf[0]);
-                    const uint32_t (&qk)[4] = qf[G::kQInRegs ? ks : 0];
-                    mma_bf16(s[0], qk, kf[0][0], kf[0][1]);
-                    mma_bf16(s[1], qk, kf[0][2], kf[0][3]);
-                    mma_bf16(s[2], qk, kf[1][0], kf[1][1]);
-                    mma_bf16(s[3], qk, kf[1][2], kf[1][3]);
+                if constexpr (G::kAhead) {
+                    uint32_t kf[2][2][4];
+                    ldsm_x4(ka[0], kf[0][0]);
+                    ldsm_x4(ka[0] + 16 * 128, kf[0][1]);
+                    #pragma unroll
+                    for (int ks = 0; ks < G::kKSteps; ++ks) {
+                        if (ks + 1 < G::kKSteps) {
+                            ldsm_x4(ka[(ks + 1) & 3] + ((ks + 1) >> 2) * G::kBoxBytes, kf[(ks + 1) & 1][0]);
+                            ldsm_x4(ka[(ks + 1) & 3] + ((ks + 1) >> 2) * G::kBoxBytes + 16 * 128, kf[(ks + 1) & 1][1]);
+                        }
+                        const uint32_t (&f)[2][4] = kf[ks & 1];
+                        mma_bf16(s[0], qf[ks], f[0][0], f[0][1]);
+                        mma_bf16(s[1], qf[ks], f[0][2], f[0][3]);
+                        mma_bf16(s[2], qf[ks], f[1][0], f[1][1]);
+                        mma_bf16(s[3], qf[ks], f[1][2], f[1][3]);
+                    }
+                } else {
+                    #pragma unroll
+                    for (int ks = 0; ks < G::kKSteps; ++ks) {
+                        uint32_t kf[2][4];
+                        ldsm_x4(ka[ks & 3] + (ks >> 2) * G::kBoxBytes, kf[0]);
+                        ldsm_x4(ka[ks & 3] + (ks >> 2) * G::kBoxBytes + 16 * 128, kf[1]);
+                        if constexpr (!G::kQInRegs) load_q(ks, qf[0]);
+                        const uint32_t (&qk)[4] = qf[G::kQInRegs ? ks : 0];
+                        mma_bf16(s[0], qk, kf[0][0], kf[0][1]);
+                        mma_bf16(s[1], qk, kf[0][2], kf[0][3]);
+                        mma_bf16(s[2], qk, kf[1][0], kf[1][1]);
+                        mma_bf16(s[3], qk, kf[1][2], kf[1][3]);
+                    }
                 }
                 // s[n][2 e + i]: row e, key 8 n + 2 quad + i
                 if (masked) {
@@ -434,14 +455,26 @@ __global__ void __launch_bounds__(kFwThreads, 2) msa_attention_few_rows_kernel(c
                 uint32_t va[4];
                 #pragma unroll
                 for (int j = 0; j < 4; ++j) va[j] = vt + off_v[j];
-                #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                if constexpr (G::kAhead) {
+                    uint32_t vf[2][4];
+                    ldsm_x4_t(va[0], vf[0]);
                     #pragma unroll
-                    for (int d = 0; d < HD / 16; ++d) {
-                        uint32_t vf[4];
-                        ldsm_x4_t(va[d & 3] + 16 * 128 * j + (d >> 2) * G::kBoxBytes, vf);
-                        mma_bf16(o[2 * d], pf[j], vf[0], vf[1]);
-                        mma_bf16(o[2 * d + 1], pf[j], vf[2], vf[3]);
+                    for (int i = 0; i < HD / 8; ++i) {                            // keys 16 j .., dimensions 16 d ..
+                        const int j = i / (HD / 16), d = i % (HD / 16), jn = (i + 1) / (HD / 16), dn = (i + 1) % (HD / 16);
+                        if (i + 1 < HD / 8) ldsm_x4_t(va[dn & 3] + 16 * 128 * jn + (dn >> 2) * G::kBoxBytes, vf[(i + 1) & 1]);
+                        mma_bf16(o[2 * d], pf[j], vf[i & 1][0], vf[i & 1][1]);
+                        mma_bf16(o[2 * d + 1], pf[j], vf[i & 1][2], vf[i & 1][3]);
+                    }
+                } else {
+                    #pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        #pragma unroll
+                        for (int d = 0; d < HD / 16; ++d) {
+                            uint32_t vf[4];
+                            ldsm_x4_t(va[d & 3] + 16 * 128 * j + (d >> 2) * G::kBoxBytes, vf);
+                            mma_bf16(o[2 * d], pf[j], vf[0], vf[1]);
+                            mma_bf16(o[2 * d + 1], pf[j], vf[2], vf[3]);
+                        }
                     }
                 }
             }
