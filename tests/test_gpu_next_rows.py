@@ -143,6 +143,48 @@ def test_tree_prune_matches_the_oracle(cuda, oracle, name):
         assert 0 < n_dropped < B * T
 
 
+@pytest.mark.parametrize("soft", [False, True])
+@pytest.mark.parametrize("V", [1, 2, 33, 1023, 8191, 8193, 20001])       # one vector, unaligned rows, a batch of loads and one logit more
+def test_row_statistics_at_the_edges_of_a_scan(cuda, V, soft):
+    """Edge probabilities (and entropies) of short, unaligned and peaked rows with -inf and NaN among the logits, against fp64.  A
+    term is off by at most 2 ulp of the exponential and a row's sum by the roundings of its longest chain of additions (20001
+    logits over 256 threads and 4 partial sums, then 10 merges: 30 roundings), 34 * 2^-24 = 2e-6 in all; the entropy's terms
+    carry a factor |x - m| <= 12 for the logits that count.  PROB_RTOL is ten times the former."""
+    api = cuda
+    B, T = 2, 6
+    rng = np.random.default_rng(77 + V)
+    scale = np.array([1.0, 1.0, 4.0, 30.0, 1.0, 1.0])[None, :, None]
+    lg = (rng.standard_normal((B, T, V)) * scale + np.array([0.0, 300.0, 0.0, 0.0, -80.0, 5.0])[None, :, None]).astype(np.float32)
+    tok = rng.integers(0, V, (B, T)).astype(np.int32)
+    if V > 8:                                                            # (not at the children's tokens)
+        for t, bad in ((0, np.nan), (4, -np.inf), (5, np.nan)):
+            at = np.setdiff1d(rng.integers(0, V, V // 3), tok)
+            lg[:, t, at] = bad
+    parent = [-1, 0, 1, 2, 3, 4]
+    trees = api.trees_to_device([api.ss_tree_build(parent, 2)] * B)
+    edge = torch.zeros((B, T), device="cuda")
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")  # noqa: E731
+    ws = api.workspace(api.ss_tree_prune_workspace_bytes(B, T, V))
+    x = np.where(np.isnan(lg), -np.inf, lg.astype(np.float64))
+    m = x.max(-1, keepdims=True)
+    e = np.exp(x - m)
+    z = e.sum(-1)
+    if soft:
+        ent = torch.zeros((B, T), device="cuda")
+        api.ss_tree_verify_soft(torch.from_numpy(lg).cuda(), _i32(tok), trees, 0.09, 0.3, i32(B), i32(B, api.SS_PATH_STRIDE), i32(B), i32(B), edge, ent, ws)
+        want = np.log(z) - (np.where(e > 0, x - m, 0.0) * e).sum(-1) / z
+        # log z and the mean of x - m may cancel: their sizes bound the error
+        np.testing.assert_allclose(ent.cpu().numpy(), want, rtol=0, atol=PROB_RTOL * (1.0 + np.log(V)))
+    else:
+        api.ss_tree_prune(torch.from_numpy(lg).cuda(), _i32(tok), trees, 0.1, edge, i32(B, T), i32(B, T), i32(B, T), api.empty_trees(B), ws)
+    assert api.ss_status(ws) == 0
+    want = np.ones((B, T))
+    for c in range(1, T):
+        want[:, c] = [np.exp(x[b, c - 1, tok[b, c]] - m[b, c - 1, 0]) / z[b, c - 1] for b in range(B)]
+    # (the exponent child - log-sum-exp is rounded at the size of the logits: 300 * 2^-24 = 1.8e-5 in the second row)
+    np.testing.assert_allclose(edge.cpu().numpy(), want, rtol=PROB_RTOL + 4e-5, atol=1e-30)
+
+
 # ---- attention directly behind the calls that write its trees ---------------------------------------------
 @pytest.mark.parametrize("batch,heads", [(1, 8), (6, 30)])               # both kernels that read the trees before their wait
 @pytest.mark.parametrize("writer", ["draft", "prune"])
