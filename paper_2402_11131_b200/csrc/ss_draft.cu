@@ -52,10 +52,11 @@ constexpr float kTinyExp = -200.f;                        // exp of it is 0 in f
 // counts how many are better.  Keeping a sorted list of k entries per thread costs 8 compare-and-swaps of 64-bit
 // words per logit instead.
 constexpr int kListCap = 512;
+constexpr int kMaxClusterCtas = 16;   // CTAs of a cluster: 8 are portable, sm_100a takes 16
 template <int NT>
 struct TopKShared {
     static_assert(NT / 32 >= kMaxTopK, "the k-th largest warp maximum has to exist");
-    unsigned long long part[8 * kMaxTopK];                // CTA 0 of a cluster: the lists of its CTAs, k entries each
+    unsigned long long part[kMaxClusterCtas * kMaxTopK];  // CTA 0 of a cluster: the lists of its CTAs, k entries each
     unsigned long long best[kMaxTopK];
     unsigned long long warp_best[NT / 32];
     unsigned long long list[kListCap];
@@ -602,9 +603,23 @@ extern "C" int32_t ss_next_draft(const float* stream_logits, int32_t n_rows, con
     if (gamma > SS_MAX_GAMMA || top_k > SS_MAX_TOPK || top_k > vocab || max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(stream_logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_next_draft_workspace_bytes(batch, gamma, vocab)) return SS_ERR_WORKSPACE;
-    // a cluster of at most 8 CTAs takes all the rows of a sequence
+    // A cluster takes all the rows of a sequence: up to 8 CTAs, and up to 16 for a few sequences where a CTA's segment is then one batch of
+    // loads instead of two (whose candidates would be read again).  Three rows of 51200 logits, 8 / 16: one sequence 7.3 / 6.1 us, six
+    // 7.7 / 6.8, four rows of 50257 7.4 / 6.4 and 8.4 / 6.9; but eight sequences 8.1 / 9.1, sixteen 11.7 / 14.3 (the clusters of 12 or 16
+    // CTAs no longer run all at once), and four rows of 32000, one batch already, 6.2 / 6.2.
+    constexpr int kOneBatch = 4 * ss::kDraftThreads * ss::kRowVecs;
     int n_cta = 1;
-    while (gamma * n_cta * 2 <= 8 && vocab / (n_cta * 2) >= ss::kDraftThreads * 4) n_cta *= 2;
+    while (vocab / (n_cta * 2) >= ss::kDraftThreads * 4 &&
+           (gamma * n_cta * 2 <= 8 || (batch <= 6 && vocab / n_cta > kOneBatch && gamma * n_cta * 2 <= ss::kMaxClusterCtas))) n_cta *= 2;
+    if (gamma * n_cta > 8) {
+        static bool configured[64] = {false};
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;
+        if (dev < 0 || dev >= 64 || !configured[dev]) {
+            if (cudaFuncSetAttribute(ss::next_draft_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return SS_ERR_CUDA;
+            if (dev >= 0 && dev < 64) configured[dev] = true;
+        }
+    }
     const cudaError_t err = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kDraftThreads),
                                             gamma * n_cta, true,
                                             static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token, gamma, vocab,

@@ -67,6 +67,13 @@ def test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, max_nodes, ties):
             assert _desc_fields(descs[b]) == _desc_fields(host)
 
 
+# clusters of 12 and 16 CTAs, and the sizes next to them
+@pytest.mark.parametrize("B,gamma,V,k,ties", [(1, 3, 32769, 8, True), (6, 4, 51201, 8, True), (7, 4, 51201, 8, True), (2, 2, 131100, 8, False),
+                                              (1, 4, 32768, 8, False)])
+def test_next_draft_with_clusters_beyond_eight_ctas(cuda, oracle, B, gamma, V, k, ties):
+    test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, 64, ties)
+
+
 def test_next_draft_special_values_follow_the_order_of_the_verification(cuda, oracle):
     api = cuda
     V = 300
