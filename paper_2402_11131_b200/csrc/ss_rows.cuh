@@ -134,14 +134,13 @@ __device__ __forceinline__ void cluster_store_u64(uint32_t addr, unsigned long l
 
 // CTAs per row: more of them while the grid takes at most half of the GPU's slots -- the next kernel's CTAs then start in
 // the other half and wait there, which hides its launch -- and a segment keeps two 16-byte loads per thread, a quarter of a batch.
-// Measured against a line at a whole batch, greedy / soft / sampled: 16 rows of 51200 4.3 / 6.5 / 8.0 and 4.7 / 7.0 / 8.6 us, 32 of 51200 the
-// same, 64 of 9000 4.8 / 7.5 / 9.0 and 4.3 / 6.6 / 7.6.  Half of the slots against all of them for segments of more than two batches: 135 rows
-// of 50257 6.5 / 10.4 / 12.8 and 6.7 / 10.9 / 14.2, 192 of 32000 6.0 / 9.9 / 11.7 and 6.6 / 10.4 / 13.7, 240 of 51200 8.5 / 14.2 / 17.0 and
-// 9.1 / 15.6 / 17.4, 256 of 40000 7.0 / 11.3 / 13.7 and 7.9 / 13.2 / 15.7.
+// A segment of more than two batches is worth all slots: its batches of loads follow one another.  Measured against a
+// line at a whole batch, greedy / soft / sampled: 16 rows of 51200 4.3 / 6.5 / 8.0 and 4.7 / 7.0 / 8.6 us, 32 of 51200 the same, 64 of 9000
+// 4.8 / 7.5 / 9.0 and 4.3 / 6.6 / 7.6.
 inline int row_cluster(long long rows, int vocab) {
     const long long slots = static_cast<long long>(kRowBlocks) * sm_count();
     int c = 1;
-    while (c < 8 && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= slots / 2) c *= 2;
+    while (c < 8 && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= (vocab / c > 2 * kRowThreads * kRowVecs * 4 ? slots : slots / 2)) c *= 2;
     return c;
 }
 
