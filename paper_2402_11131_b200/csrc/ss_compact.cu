@@ -22,6 +22,11 @@ kv_compact_kernel(uint4* __restrict__ k_all, uint4* __restrict__ v_all, int n_he
     const int col2 = blockIdx.x * kCompactThreads + threadIdx.x;
     wait_for_previous_kernel();
     release_next_kernel();
+    // the first entries of the path are asked for with the lengths, not behind them
+    const int32_t* path = accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE;
+    int head[kBatch];
+    #pragma unroll
+    for (int k = 0; k < kBatch; ++k) asm volatile("ld.global.s32 %0, [%1];" : "=r"(head[k]) : "l"(path + k));
     const int L = kv_len_in[b];
     int len = accept_len[b];
     len = max(0, min(len, SS_PATH_STRIDE));
@@ -31,14 +36,13 @@ kv_compact_kernel(uint4* __restrict__ k_all, uint4* __restrict__ v_all, int n_he
         const int col = (col2 < cols) ? col2 : col2 - cols;
         const int h = col / chunks_per_head, c = col - h * chunks_per_head;
         base += layer * layer_stride16 + (kv_start[b] + L) * slot_stride16 + h * head_stride16 + c;
-        const int32_t* path = accept_path + static_cast<size_t>(b) * SS_PATH_STRIDE;
         for (int i0 = 0; i0 < len; i0 += kBatch) {
             uint4 regs[kBatch];
             int src[kBatch];
             #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
                 const int i = i0 + k;
-                src[k] = (i < len) ? path[i] : -1;
+                src[k] = i < len ? (i0 == 0 ? head[k] : path[i]) : -1;
                 if (src[k] >= 0 && src[k] != i) regs[k] = base[src[k] * slot_stride16];
             }
             #pragma unroll

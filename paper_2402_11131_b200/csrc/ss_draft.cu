@@ -66,13 +66,9 @@ struct TopKShared {
 template <int NT>
 struct ThreadMax {
     float v = -INFINITY;
-    float4 last[kRowVecs];
     __device__ __forceinline__ void batch(const float4 (&q)[kRowVecs], int word) {
         #pragma unroll
-        for (int k = 0; k < kRowVecs; ++k) {
-            v = fmaxf(v, fmaxf(fmaxf(q[k].x, q[k].y), fmaxf(q[k].z, q[k].w)));     // (a NaN is never the maximum)
-            last[k] = q[k];
-        }
+        for (int k = 0; k < kRowVecs; ++k) v = fmaxf(v, fmaxf(fmaxf(q[k].x, q[k].y), fmaxf(q[k].z, q[k].w)));     // (a NaN is never the maximum)
     }
 };
 template <int NT>
@@ -127,15 +123,13 @@ static __device__ __noinline__ void select_by_passes(const Segment seg, int top_
         if (threadIdx.x == 0) s.best[r] = below;          // (0, no entry, once the segment is exhausted)
     }
 }
-// The k best entries of the segment in s.best, for every thread
+// The k best entries of the segment in s.best, for every thread; q: the first batch of the segment
 template <int NT>
-__device__ __forceinline__ void segment_topk(const Segment& seg, int top_k, TopKShared<NT>& s) {
+__device__ __forceinline__ void segment_topk(const Segment& seg, int top_k, TopKShared<NT>& s, float4 (&q)[kRowVecs]) {
     constexpr int kWarps = NT / 32;
     const int lane = static_cast<int>(threadIdx.x) & 31, warp = static_cast<int>(threadIdx.x) >> 5;
     ThreadMax<NT> tm;
-    #pragma unroll
-    for (int k = 0; k < kRowVecs; ++k) tm.last[k] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    scan_segment<NT>(seg, tm);
+    scan_segment<NT>(seg, tm, q);
     const uint32_t wm = __reduce_max_sync(0xffffffffu, order_key(tm.v));
     if (lane == 0) s.warp_key[warp] = wm;
     if (threadIdx.x == 0) s.n_list = 0;
@@ -152,8 +146,12 @@ __device__ __forceinline__ void segment_topk(const Segment& seg, int top_k, TopK
     const float bound = key_value(__shfl_sync(0xffffffffu, key, __ffs(__ballot_sync(0xffffffffu, before == top_k - 1)) - 1));
     if (!(tm.v < bound)) {
         Collect<NT> collect{seg, s, bound};
-        if (seg.total <= 4 * NT * kRowVecs) collect.batch(tm.last, 4 * static_cast<int>(threadIdx.x));
-        else scan_segment<NT>(seg, collect);
+        if (seg.total <= 4 * NT * kRowVecs) {
+            collect.batch(q, 4 * static_cast<int>(threadIdx.x));
+        } else {
+            load_batch<NT>(seg, static_cast<int>(threadIdx.x), q);
+            scan_segment<NT>(seg, collect, q);
+        }
     }
     __syncthreads();
     const int n = s.n_list;
@@ -321,7 +319,9 @@ next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int
     int r = row_index ? row_index[b] : 0;
     r = min(max(r, 0), n_rows - 1);
     const Segment seg = make_segment(stream_logits, (static_cast<size_t>(b) * n_rows + r) * gamma + g, vocab, part, n_cta);
-    segment_topk<kDraftThreads>(seg, k, s);
+    float4 q[kRowVecs];
+    load_first<kDraftThreads>(seg, q);
+    segment_topk<kDraftThreads>(seg, k, s, q);
     const int i = static_cast<int>(threadIdx.x), warp = i >> 5, lane = i & 31;
     // the lists of a row lie one after another
     cluster_wait();                                       // (CTA 0 has started)
@@ -410,6 +410,8 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     prefetch_batch(seg);
     wait_for_previous_kernel();
     if (SOFT) release_next_kernel();                      // (pruning writes descriptors)
+    float4 q[kRowVecs];
+    load_first<kRowThreads>(seg, q);                      // (a row that no node owns is within the logits too)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
     if (t >= max(T, 1)) {
         if (n_cta > 1) cluster_wait();
@@ -419,7 +421,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     RowStats<SOFT> rs;
-    scan_segment<kRowThreads>(seg, rs);
+    scan_segment<kRowThreads>(seg, rs, q);
     tree.store(s_tree, T);
     // the logits of the node's children: on their way while the statistics are merged
     bool mine = false, legal = false;
@@ -529,10 +531,12 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
         if (n_cta > 1) cluster_wait();
         return;
     }
+    float4 q[kRowVecs];
+    load_first<kRowThreads>(seg, q);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     const float u = uniforms[row];
-    segment_topk<kRowThreads>(seg, k, s);
+    segment_topk<kRowThreads>(seg, k, s, q);
     tree.store(s_tree, T);
     const int i = static_cast<int>(threadIdx.x);
     if (n_cta > 1) {

@@ -88,20 +88,31 @@ static __device__ __noinline__ float4 edge_vec(const float* src, int i, int skip
     q.w = 4 * i + 3 >= skip && 4 * i + 3 < total ? src[4 * i + 3] : -INFINITY;
     return q;
 }
-// Calls f.batch(q, word) for batches of kRowVecs vectors; word: index of the first word of q[0], that of q[v] is
-// v * 4 * NT further.  A thread meets its logits in ascending order.
-template <int NT, typename F>
-__device__ __forceinline__ void scan_segment(const Segment& s, F& f) {
-    const int whole0 = s.skip ? 1 : 0, whole1 = s.total >> 2, n_vec = (s.total + 3) >> 2;      // whole vectors: [whole0, whole1)
+// A batch of a thread's vectors, from vector i on, those that are whole.  FIRST: the loads stay where they are written, so that they
+// are on their way while what decides whether the row is scanned at all arrives (the length of the tree: a round trip to L2).
+template <int NT, bool FIRST = false>
+__device__ __forceinline__ void load_batch(const Segment& s, int i, float4 (&q)[kRowVecs]) {
+    const int whole0 = s.skip ? 1 : 0, whole1 = s.total >> 2;                     // whole vectors: [whole0, whole1)
     const float4* vec = reinterpret_cast<const float4*>(s.src);
-    for (int i = static_cast<int>(threadIdx.x); i < n_vec; i += NT * kRowVecs) {
-        float4 q[kRowVecs];
-        #pragma unroll
-        for (int v = 0; v < kRowVecs; ++v) {
-            const int at = i + v * NT;
-            q[v] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (at >= whole0 && at < whole1) q[v] = __ldcs(vec + at);
+    #pragma unroll
+    for (int v = 0; v < kRowVecs; ++v) {
+        const int at = i + v * NT;
+        q[v] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        if (at >= whole0 && at < whole1) {
+            if constexpr (FIRST) asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q[v].x), "=f"(q[v].y), "=f"(q[v].z), "=f"(q[v].w) : "l"(vec + at));
+            else q[v] = __ldcs(vec + at);
         }
+    }
+}
+template <int NT>
+__device__ __forceinline__ void load_first(const Segment& s, float4 (&q)[kRowVecs]) { load_batch<NT, true>(s, static_cast<int>(threadIdx.x), q); }
+// Calls f.batch(q, word) for batches of kRowVecs vectors, of which the first has been loaded; word: index of the first word of q[0],
+// that of q[v] is v * 4 * NT further.  A thread meets its logits in ascending order.
+template <int NT, typename F>
+__device__ __forceinline__ void scan_segment(const Segment& s, F& f, float4 (&q)[kRowVecs]) {
+    const int whole0 = s.skip ? 1 : 0, whole1 = s.total >> 2, n_vec = (s.total + 3) >> 2;
+    for (int i = static_cast<int>(threadIdx.x); i < n_vec; i += NT * kRowVecs) {
+        if (i >= NT * kRowVecs) load_batch<NT>(s, i, q);
         if (i < whole0 || (i + (kRowVecs - 1) * NT >= whole1 && (s.total & 3))) {
             #pragma unroll
             for (int v = 0; v < kRowVecs; ++v) {

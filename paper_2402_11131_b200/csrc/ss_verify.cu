@@ -25,6 +25,8 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     prefetch_batch(seg);
     wait_for_previous_kernel();
     release_next_kernel();
+    float4 q[kRowVecs];
+    load_first<kRowThreads>(seg, q);                      // (a row that no node owns is within the logits too)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);     // a descriptor is never trusted beyond the arrays' extent
     if (t >= max(T, 1)) {                                 // (the whole cluster: t is its row)
         if (n_cta > 1) cluster_wait();
@@ -33,7 +35,7 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     ArgMax am;
-    scan_segment<kRowThreads>(seg, am);
+    scan_segment<kRowThreads>(seg, am, q);
     tree.store(s_tree, T);
     unsigned long long best = warp_max_u64(am.best(seg));
     constexpr int kWarps = kRowThreads / 32;
