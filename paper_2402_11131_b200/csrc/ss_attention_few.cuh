@@ -7,8 +7,8 @@
 // committed, scores to registers, P to TMEM, P V issued and committed), about 1.2 us of an 8 us layer for each tile that
 // is waited for.  With this few rows the register-level MMA (mma.sync, 950 FMA per cycle and SM measured) keeps up, and a
 // warp that holds scores, P and O in registers hands nothing over.  Measured, us per plain layer of
-// 32 heads, before (tcgen05) and after: 12 rows of 64, 512 keys 7.9 and 5.0; 27 rows of 80, 800 keys 9.1 and 7.5; sixteen
-// sequences of 512 keys, 27 rows of 64, 40.8 and 21.0.
+// 32 heads, before (tcgen05) and after: 12 rows of 64, 512 keys 7.9 and 4.7; 27 rows of 80, 800 keys 9.1 and 7.4; sixteen
+// sequences of 512 keys, 27 rows of 64, 40.8 and 20.9.
 //
 // A CTA takes half of an SM (113 KB of shared memory): under programmatic dependent launch the CTAs of the next layer
 // sit beside those of this one with their first K/V tiles loaded, and what they may not read yet (query rows, this

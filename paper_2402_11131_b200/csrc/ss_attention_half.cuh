@@ -9,7 +9,8 @@
 // layer wait with the first tiles of their prefix loaded.  Measured, us per
 // layer, one CTA per SM (the kernels of the smaller grids) / this one: 64 rows, 16 sequences x 32 heads of 256 to 4096 keys x 128
 // 112 / 97 (alone, 6.5 TB/s would be 88), of 2304 keys x 64 80 / 70, x 80 95 / 78; 320 rows, of 256 to 4096 keys x 128 322 / 288;
-// 192 rows, of 1024 keys x 64 124 / 92.
+// 192 rows, of 1024 keys x 64 124 / 92.  With its MMAs in blocks of four (tc_mma_steps), of 512 to 4096 keys x 128 64 rows 102.8 -> 96.7, 320
+// rows 288 -> 265.
 //
 //   S = Q K^T     A = the query rows, B = a K tile of 64 keys, both K-major in shared memory, N = 64
 //   O += P V      A = P in TMEM, B = the V tile (MN-major), N = head_dim
