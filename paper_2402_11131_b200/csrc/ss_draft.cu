@@ -692,7 +692,9 @@ extern "C" int32_t ss_tree_verify_sampled(const float* logits, const int32_t* dr
     if (max_nodes > SS_MAX_NODES || top_k > SS_MAX_TOPK || top_k > vocab) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_verify_sampled_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
+    // The k best of two batches are found faster by one CTA than the lists of two CTAs are merged: 64 rows of 32000 9.67 -> 8.82 us with two
+    // CTAs a row instead of four.
+    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab, 2 * 4 * ss::kRowThreads * ss::kRowVecs);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
     const cudaError_t err = ss::launch_rows(ss::sampled_verify_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
