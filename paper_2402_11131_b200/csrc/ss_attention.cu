@@ -1561,19 +1561,22 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
     const int blocks = (q_rows + 31) / 32;
     const long long load = static_cast<long long>(p.batch) * p.n_heads * blocks * slots / sm_count();
     if (q_rows <= 32) {
-        // up to 80 dimensions at every length measured (128 to 4096 keys).  One sequence, 12 rows of 128: 4000 keys 15.9 / 15.4, 6000 keys
-        // 20.5 / 20.8, eight heads and 6000 keys 11.6 / 11.5, 9000 keys 13.8 / 16.1; 27 rows of 128: 800 keys 9.9 / 9.0, 2000 keys 11.9 /
-        // 13.0.  And where the grid takes several waves, at any length (the others are then the kernel with two CTAs per SM): sixteen
-        // sequences, 12 rows of 128, 130 keys 19.1 / 14.6, 2048 keys 89.4 / 84.3; 27 rows of 80, 130 keys 18.5 / 15.2, 2048 keys 68.0 / 64.9; of
-        // 128, 130 keys 19.8 / 19.3, 512 keys 33.8 / 36.2, 2048 keys 91.5 / 92.9, but 256 to 4096 keys 92.0 / 90.0 and fifteen of 64 beside one of
-        // 4096 65.6 / 52.8
+        // One wave: up to 80 dimensions at every length measured (128 to 4096 keys).  One sequence, 12 rows of 128: 4000 keys 15.9 / 15.4, 6000
+        // keys 20.5 / 20.8, eight heads and 6000 keys 11.6 / 11.5, 9000 keys 13.8 / 16.1; 27 rows of 128: 800 keys 9.9 / 9.0, 2000 keys 11.9 /
+        // 13.0.  Several waves (the others are then the kernel with two CTAs per SM), sixteen sequences, tcgen05 / few rows.  12 rows at any
+        // length: of 64, 130 keys 15.5 / 11.3, 4000 keys 86 / 80; of 80, 2048 keys 63.3 / 60.8; of 128, 256 keys 21.4 / 19.8, 400 25.6 / 26.2, 1200
+        // 54.9 / 56.3, 4000 154.2 / 154.4.  27 rows of 64: 130 keys 15.7 / 13.5, 1200 36.4 / 36.3, 4000 86.7 / 87.9; of 80: 256 keys 20.1 / 19.1, 2048
+        // 63.8 / 65.3, but fifteen of 300 beside one of 4096 48.8 / 43.2; of 128: 130 keys 18.2 / 19.6, 700 38.3 / 43.2, 4000 156 / 164, fifteen of
+        // 300 beside one of 4096 51.6 / 60.3, eight sequences of 24 heads, 256 keys 10.0 / 11.8.
         const int rows = q_rows <= 16 ? 16 : 32;
-        return p.head_dim <= 80 || groups > sm_count() || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
+        if (groups > sm_count()) return rows == 16 || p.head_dim <= 80 ? rows : 0;
+        return p.head_dim <= 80 || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
     }
     if (q_rows <= kSmRows) {
-        // more heads than SMs.  Sixteen sequences, 64 rows of 64, 130 keys 20.0 / 18.3, 330 keys 25.8 / 25.7, 1024 keys 40.3 / 47.0; of
-        // 80, 30 keys 18.5 / 17.2, 130 keys 22.4 / 22.5, 1024 keys 45.0 / 57.3; of 128, 30 keys 20.5 / 21.6, 512 keys 36.2 / 48.6
-        if (groups > sm_count()) return slots <= (d64 ? 390 : d80 ? 180 : 0) ? 64 : 0;
+        // more heads than SMs.  Sixteen sequences, 64 rows of 64, 30 keys 15.8 / 14.7, 64 keys 14.5 / 14.9, 130 keys 17.6 / 18.8, 256 keys 18.9 /
+        // 21.9, 1024 keys 40.3 / 47.0; of 80, 30 keys 17.8 / 17.7, 64 keys 15.8 / 18.2, 1024 keys 45.0 / 57.3; of 128, 30 keys 20.5 / 21.6, 512
+        // keys 36.2 / 48.6
+        if (groups > sm_count()) return d64 && slots <= 48 ? 64 : 0;
         // (a batch goes by its mean: sixteen sequences of eight heads, 64 rows of 64, 200 keys 9.7 / 7.8, fifteen of 64 beside one of 2048
         // 16.6 / 28.6.)  64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
         // keys 11.0 / 12.8

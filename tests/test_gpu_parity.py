@@ -331,6 +331,23 @@ def test_attention_few_rows_at_the_steps_of_the_split(cuda, oracle, head_dim, T,
     assert_attention_close(oracle, st, st.layer(0), dev, 0, check_lse=True)
 
 
+@pytest.mark.parametrize("head_dim,T,n_heads,lengths", [
+    (128, 16, 60, (1, 200)), (128, 17, 60, (1, 200)), (128, 32, 50, (63, 900)), (128, 32, 49, (63, 900)),
+    (64, 64, 60, (40, 41)), (64, 64, 60, (49, 50)), (80, 64, 60, (1, 70)),
+])
+def test_attention_batches_on_both_sides_of_the_few_rows(cuda, oracle, head_dim, T, n_heads, lengths):
+    """Batches of three around the rows, heads and lengths at which the few-rows kernel ends."""
+    api, DeviceStep = cuda
+    cfg = W.custom_config("side", batch=3, n_layers=2, n_msa_layers=1, prefix_len_range=lengths, n_nodes=T, gamma=1, max_depth=6,
+                          n_heads=n_heads, head_dim=head_dim, config_id=990 + T)
+    st = W.make_step(cfg)
+    dev = DeviceStep(st, layers=[0], with_lse=True)
+    for _ in range(2):
+        dev.run_attention()
+    assert api.ss_status(dev.attn_ws) == 0
+    assert_attention_close(oracle, st, st.layer(0), dev, 0, check_lse=True)
+
+
 @pytest.mark.parametrize("head_dim", [64, 80, 128])
 @pytest.mark.parametrize("T,gamma,n_heads,lengths,ramp", [
     (64, 0, 60, (385, 448), 0.0),        # 64 rows; a tile's edge in the prefix and in the tree, rings that wrap
