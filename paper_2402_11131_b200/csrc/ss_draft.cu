@@ -8,9 +8,9 @@
 // cluster takes the whole sequence and nothing goes through global memory.  Compiled without fast-math.
 // Measured on a B200, before (chunks of 4096 logits, partial results and candidate lists through global memory, serial
 // tails) and after: soft verification of 32 rows of 51200 logits 15.3 and 6.4 us, sampled verification of 64 rows of
-// 32000 34.1 and 8.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of 32000) 15.6 and
-// 8.9 us.  Pruning then 31.4 -> 28.4 with packed exponentials and without the sums that only the verification uses, 26.8 with the prefetch
-// before the wait; the next draft 9.5 -> 8.55 with one copy of the batch in registers.
+// 32000 34.1 and 7.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of 32000) 15.6 and
+// 5.3 us.  Pruning then 31.4 -> 28.4 with packed exponentials and without the sums that only the verification uses, 26.7 with the prefetch
+// before the wait.
 #include "ss_rows.cuh"
 
 namespace ss {
@@ -47,10 +47,12 @@ constexpr float kTinyExp = -200.f;                        // exp of it is 0 in f
 
 // ---- the k best entries of a segment --------------------------------------------------------------------------------
 // Pass 1 takes one maximum per thread.  The k-th largest warp maximum bounds the k-th best logit of the segment from
-// below, and only a dozen logits or so reach that bound; the few threads that hold one collect them in a list (from
-// the registers of pass 1 where the segment was one batch, else they read their logits again), and each entry of the list
-// counts how many are better.  Keeping a sorted list of k entries per thread costs 8 compare-and-swaps of 64-bit
-// words per logit instead.
+// below, and only a dozen logits or so reach that bound; the few threads that hold one find them (in
+// the registers of pass 1 where the segment was one batch, else they read their logits again) and put them in a list, and each entry of the
+// list counts how many are better.  Keeping a sorted list of k entries per thread costs 8 compare-and-swaps of 64-bit
+// words per logit instead.  A logit for the list is read once more from memory, where it is in L2: picked out of the registers by an
+// index, it takes the whole batch through a stack frame in local memory.  From HBM, before / after: sampled verification of 64 rows of 32000
+// 9.4 / 7.2 us, 135 of 50257 16.3 / 12.0, 1024 of 8000 20.1 / 12.2, 1024 of 32000 40.2 / 30.3; 16 next drafts of four rows of 32000 8.6 / 5.3.
 constexpr int kListCap = 512;
 constexpr int kMaxClusterCtas = 16;   // CTAs of a cluster: 8 are portable, sm_100a takes 16
 template <int NT>
@@ -85,14 +87,10 @@ struct Collect {
         #pragma unroll 1
         for (; hit; hit &= hit - 1u) {
             const int j = __ffs(hit) - 1;
-            float x = 0.f;
-            #pragma unroll
-            for (int k = 0; k < kRowVecs; ++k)
-                if (k == j >> 2) x = (j & 2) ? ((j & 1) ? q[k].w : q[k].z) : ((j & 1) ? q[k].y : q[k].x);
             const int at = word + (j >> 2) * 4 * NT + (j & 3);
             if (at < seg.skip || at >= seg.total) continue;
             const int p = atomicAdd(&s.n_list, 1);
-            if (p < kListCap) s.list[p] = entry(order_key(x), seg.at + at);
+            if (p < kListCap) s.list[p] = entry(order_key(seg.src[at]), seg.at + at);
         }
     }
 };
@@ -692,10 +690,7 @@ extern "C" int32_t ss_tree_verify_sampled(const float* logits, const int32_t* dr
     if (max_nodes > SS_MAX_NODES || top_k > SS_MAX_TOPK || top_k > vocab) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_verify_sampled_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    // The k best of two batches are found faster by one CTA than the lists of two CTAs are merged: 64 rows of 32000 9.67 -> 8.82 us with two
-    // CTAs a row instead of four, of 9000 9.69 -> 7.38 with one, 32 rows of 51200 10.24 -> 8.86; 16 rows of 51200 8.16 / 8.29.
-    const long long rows = static_cast<long long>(batch) * max_nodes;
-    const int n_cta = ss::row_cluster(rows, vocab, rows > 16 ? 2 * 4 * ss::kRowThreads * ss::kRowVecs : 0);
+    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
     const cudaError_t err = ss::launch_rows(ss::sampled_verify_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,

@@ -145,14 +145,14 @@ __device__ __forceinline__ void cluster_store_u64(uint32_t addr, unsigned long l
 
 // CTAs per row: more of them while the grid takes at most half of the GPU's slots -- the next kernel's CTAs then start in
 // the other half and wait there, which hides its launch -- and a segment keeps two 16-byte loads per thread, a quarter of a batch.
-// (`whole`: segments of so many logits are not cut further.)
 // A segment of more than two batches is worth all slots: its batches of loads follow one another.  Measured against a
 // line at a whole batch, greedy / soft / sampled: 16 rows of 51200 4.3 / 6.5 / 8.0 and 4.7 / 7.0 / 8.6 us, 32 of 51200 the same, 64 of 9000
-// 4.8 / 7.5 / 9.0 and 4.3 / 6.6 / 7.6.
-inline int row_cluster(long long rows, int vocab, int whole = 0) {
+// 4.8 / 7.5 / 9.0 and 4.3 / 6.6 / 7.6.  (For sampled verification alone, fewer CTAs per row were faster while its lists went through local
+// memory; since they do not, more are: 64 rows of 32000, two CTAs and four 7.5 / 7.1 us, 32 of 51200 7.35 / 6.9.)
+inline int row_cluster(long long rows, int vocab) {
     const long long slots = static_cast<long long>(kRowBlocks) * sm_count();
     int c = 1;
-    while (c < 8 && vocab / c > whole && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= (vocab / c > 2 * kRowThreads * kRowVecs * 4 ? slots : slots / 2)) c *= 2;
+    while (c < 8 && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= (vocab / c > 2 * kRowThreads * kRowVecs * 4 ? slots : slots / 2)) c *= 2;
     return c;
 }
 

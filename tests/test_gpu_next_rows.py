@@ -9,6 +9,7 @@ import ctypes as C
 import numpy as np
 import pytest
 
+import launch_info
 from paper_2402_11131_b200 import workloads as W
 
 torch = pytest.importorskip("torch")
@@ -72,6 +73,25 @@ def test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, max_nodes, ties):
                                               (1, 4, 32768, 8, False)])
 def test_next_draft_with_clusters_beyond_eight_ctas(cuda, oracle, B, gamma, V, k, ties):
     test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, 64, ties)
+
+
+@pytest.mark.parametrize("call", ["draft", "sampled"])
+def test_selection_keeps_no_logits_in_local_memory(cuda, call):
+    """The batch of logits that a thread scans stays in registers (with an index into it, it would be 128 bytes of stack)."""
+    api = cuda
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")  # noqa: E731
+    B, T, V, g = 2, 8, 20000, 2
+    trees = api.trees_to_device([api.ss_tree_build([-1] + [0] * (T - 1), g)] * B)
+    if call == "draft":
+        ws = api.workspace(api.ss_next_draft_workspace_bytes(B, g, V))
+        lg = torch.randn((B, 1, g, V), device="cuda")
+        run = lambda: api.ss_next_draft(lg, None, i32(B), 2, T, i32(B, T), trees, ws)  # noqa: E731
+    else:
+        ws = api.workspace(api.ss_tree_verify_sampled_workspace_bytes(B, T, V))
+        lg, u = torch.randn((B, T, V), device="cuda"), torch.rand((B, T), device="cuda")
+        run = lambda: api.ss_tree_verify_sampled(lg, i32(B, T), trees, u, 4, i32(B), i32(B, api.SS_PATH_STRIDE), i32(B), i32(B), i32(B, T), ws)  # noqa: E731
+    mine = [k for k in launch_info.kernels(run) if "next_draft" in k["name"] or "sampled_verify" in k["name"]]
+    assert len(mine) == 1 and mine[0]["local_bytes"] <= 16
 
 
 def test_next_draft_special_values_follow_the_order_of_the_verification(cuda, oracle):
