@@ -390,11 +390,11 @@ __device__ __forceinline__ void prune_tail(int T, int max_nodes, int b, unsigned
     if (i == 0) { out->n_nodes = n; out->gamma = gamma; out->max_depth = md; out->reserved = 0; }
 }
 
-// SOFT: the verification, else the pruning
-template <bool SOFT>
+// SOFT: the verification, else the pruning; AHEAD: see RowsAhead
+template <bool SOFT, int AHEAD>
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
-                  int max_nodes, int vocab, int n_cta, NodeTailArgs ta, int32_t* __restrict__ counters, RowOut* __restrict__ rows) {
+                  int max_nodes, int vocab, int n_cta, int slots, NodeTailArgs ta, int32_t* __restrict__ counters, RowOut* __restrict__ rows) {
     const int rank = blockIdx.x, t = blockIdx.y, b = blockIdx.z;
     __shared__ Stats s_part[kRowParts];
     __shared__ unsigned long long s_any[kRowThreads / 32];
@@ -402,20 +402,23 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
     __shared__ TreeShared s_tree;
     __shared__ float s_lse, s_bar;
     __shared__ uint32_t s_ok[2];
+    __shared__ volatile int s_passed;
     if (n_cta > 1) cluster_arrive();
     const size_t row = static_cast<size_t>(b) * max_nodes + t;
     const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
-    prefetch_batch(seg);
+    ask_ahead<AHEAD>(seg, trees[b], t, slots, &s_passed);
     wait_for_previous_kernel();
     if (SOFT) release_next_kernel();                      // (pruning writes descriptors)
+    if (AHEAD == kIfWaiting) wait_passed(&s_passed);
     float4 q[kRowVecs];
-    load_first<kRowThreads>(seg, q);                      // (a row that no node owns is within the logits too)
+    if (AHEAD == kEveryRow) load_first<kRowThreads>(seg, q);    // (a row that no node owns is within the logits too)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
     if (t >= max(T, 1)) {
         if (n_cta > 1) cluster_wait();
         return;
     }
     const int i = static_cast<int>(threadIdx.x);
+    if (AHEAD != kEveryRow) load_first<kRowThreads>(seg, q);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     RowStats<SOFT> rs;
@@ -510,7 +513,7 @@ node_stats_kernel(const float* __restrict__ logits, const int32_t* __restrict__ 
 // Verification against tokens drawn from the softmax over each node's k largest logits (temperature 1).
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens, const ss_tree_desc* __restrict__ trees,
-                      const float* __restrict__ uniforms, int max_nodes, int vocab, int k, int n_cta,
+                      const float* __restrict__ uniforms, int max_nodes, int vocab, int k, int n_cta, int slots,
                       int32_t* __restrict__ accept_len, int32_t* __restrict__ accept_path, int32_t* __restrict__ last_node,
                       int32_t* __restrict__ bonus_token, int32_t* __restrict__ node_token, int32_t* __restrict__ counters,
                       int32_t* __restrict__ drawn) {
@@ -518,12 +521,14 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
     __shared__ TopKShared<kRowThreads> s;
     __shared__ TreeShared s_tree;
     __shared__ int32_t s_draw[SS_MAX_NODES];
+    __shared__ volatile int s_passed;
     if (n_cta > 1) cluster_arrive();
     const size_t row = static_cast<size_t>(b) * max_nodes + t;
     const Segment seg = make_segment(logits, row, vocab, rank, n_cta);
-    prefetch_batch(seg);
+    ask_ahead<kIfWaiting>(seg, trees[b], t, slots, &s_passed);
     wait_for_previous_kernel();
     release_next_kernel();
+    wait_passed(&s_passed);
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);
     if (t >= max(T, 1)) {
         if (n_cta > 1) cluster_wait();
@@ -642,11 +647,16 @@ static int32_t launch_node_stats(const float* logits, const int32_t* tokens, con
     if (max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_prune_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
+    const long long n_rows = static_cast<long long>(batch) * max_nodes;
+    const int n_cta = ss::row_cluster(n_rows, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
-    const cudaError_t err = ss::launch_rows(ss::node_stats_kernel<SOFT>, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
-                                            static_cast<cudaStream_t>(stream), logits, tokens, trees, max_nodes, vocab, n_cta, ta,
+    const ss::RowsAhead ahead = ss::rows_ahead(n_rows, vocab, n_cta);
+    const auto kernel = ahead == ss::kEveryRow    ? ss::node_stats_kernel<SOFT, ss::kEveryRow>
+                        : ahead == ss::kOwnedRows ? ss::node_stats_kernel<SOFT, ss::kOwnedRows>
+                                                  : ss::node_stats_kernel<SOFT, ss::kIfWaiting>;
+    const cudaError_t err = ss::launch_rows(kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
+                                            static_cast<cudaStream_t>(stream), logits, tokens, trees, max_nodes, vocab, n_cta, ss::row_slots(), ta,
                                             reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes),
                                             reinterpret_cast<ss::RowOut*>(ws + ss::kWsHeaderBytes + counter_bytes));
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
@@ -690,12 +700,13 @@ extern "C" int32_t ss_tree_verify_sampled(const float* logits, const int32_t* dr
     if (max_nodes > SS_MAX_NODES || top_k > SS_MAX_TOPK || top_k > vocab) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_tree_verify_sampled_workspace_bytes(batch, max_nodes, vocab)) return SS_ERR_WORKSPACE;
-    const int n_cta = ss::row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
+    const long long n_rows = static_cast<long long>(batch) * max_nodes;
+    const int n_cta = ss::row_cluster(n_rows, vocab);
     char* ws = static_cast<char*>(workspace);
     const size_t counter_bytes = (static_cast<size_t>(batch) * sizeof(int32_t) + 255) / 256 * 256;
     const cudaError_t err = ss::launch_rows(ss::sampled_verify_kernel, dim3(n_cta, max_nodes, batch), dim3(ss::kRowThreads), n_cta, true,
                                             static_cast<cudaStream_t>(stream), logits, draft_tokens, trees, uniforms, max_nodes, vocab, top_k,
-                                            n_cta, accept_len, accept_path, last_node, bonus_token, node_token,
+                                            n_cta, ss::row_slots(), accept_len, accept_path, last_node, bonus_token, node_token,
                                             reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes),
                                             reinterpret_cast<int32_t*>(ws + ss::kWsHeaderBytes + counter_bytes));
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;

@@ -71,12 +71,39 @@ __device__ __forceinline__ Segment make_segment(const float* base, size_t row, i
     s.total = s.skip + hi - lo;
     return s;
 }
-// The first batch of the segment on its way to L2, a line to a thread: no data reaches the SM, so it may be asked for before the
-// wait for the previous kernel, whoever writes the logits.  Calls behind one another, 1024 rows of 32000: arg-max 23.6 -> 21.6 us, softmax
-// sums 28.4 -> 26.8 us; 32 rows of 51200, softmax statistics 7.1 -> 6.8 us.  (Rows that a smaller tree does not own are asked for too.)
-__device__ __forceinline__ void prefetch_batch(const Segment& s) {
-    static_assert(kRowThreads * 32 == kRowThreads * kRowVecs * 4, "a batch is a line of 32 logits to a thread");
-    if (32 * static_cast<int>(threadIdx.x) < s.total) prefetch_l2(s.src + 32 * threadIdx.x);
+// What a CTA asks for before the wait for the previous kernel: the first batch of its segment, on its way to L2.  No data reaches the SM,
+// so it does not matter who writes the logits.  It pays where the previous kernel releases its successor early; behind one that does not,
+// the wait is over at once.  Which CTAs ask (see rows_ahead for the sizes):
+//   kEveryRow   all, whether a node owns their row or not
+//   kOwnedRows  those of a row that a node owns by the tree's length as it stands before the wait.  The previous kernel may still be writing
+//               it: a hint.  (Row t lies within the logits whatever it says.)
+//   kIfWaiting  of those the ones that the GPU holds at once, by one thread and only if thread 32 is still in the wait (wait_passed) when the
+//               length arrives: a prefetch that the loads meet costs 0.8 us (256 rows of 32000 in L2, 7.2 / 8.1)
+// With kEveryRow the batch is also loaded beside the tree's length, with the others behind it.
+enum RowsAhead { kEveryRow, kOwnedRows, kIfWaiting };
+template <int AHEAD>
+__device__ __forceinline__ void ask_ahead(const Segment& s, const ss_tree_desc& tree, int t, int slots, volatile int* passed) {
+    constexpr int kBatchWords = 4 * kRowThreads * kRowVecs;
+    if constexpr (AHEAD == kIfWaiting) {
+        if (threadIdx.x != 0) return;
+        *passed = 0;                                      // (later than thread 32's 1: it asks in vain)
+        if (static_cast<int>((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) >= slots) return;
+    }
+    if constexpr (AHEAD != kEveryRow) {
+        int n;
+        asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(&tree.n_nodes) : "memory");
+        if (t >= max(n, 1)) return;
+    }
+    if constexpr (AHEAD == kIfWaiting) {
+        const uint32_t bytes = static_cast<uint32_t>(min(s.total, kBatchWords)) / 4 * 16;
+        if (*passed == 0 && bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(s.src), "r"(bytes) : "memory");
+    } else {
+        static_assert(kRowThreads * 32 == kBatchWords, "a batch is a line of 32 logits to a thread");
+        if (32 * static_cast<int>(threadIdx.x) < s.total) prefetch_l2(s.src + 32 * threadIdx.x);
+    }
+}
+__device__ __forceinline__ void wait_passed(volatile int* passed) {
+    if (threadIdx.x == 32) *passed = 1;
 }
 // Vector i of the segment (words 4 i .. 4 i + 3); words that are not the segment's read -inf.  The first and the last
 // one are put together from single loads where they are not whole.
@@ -155,6 +182,17 @@ inline int row_cluster(long long rows, int vocab) {
     while (c < 8 && vocab / (c * 2) >= kRowThreads * 8 && rows * c * 2 <= (vocab / c > 2 * kRowThreads * kRowVecs * 4 ? slots : slots / 2)) c *= 2;
     return c;
 }
+// kEveryRow on grids of at most half of the slots: at most a batch each for 296 CTAs, 9.7 MB, which little waits for.  64 rows of 32000,
+// arg-max, loads behind the length / beside it and prefetched 5.2 / 4.5 us, 16 of them owned 4.25 / 4.2; 128 rows of 32000 6.8 / 6.1 and, 32
+// owned, 5.45 / 5.45.  On larger grids it costs smaller trees more than it gives full ones: sixteen trees of 16 of 64 nodes, 32000 logits a row
+// 11.9 us and 9.3 with owned rows only, 8000 logits 8.4 and 5.3.  kOwnedRows where the logits are too many to be in L2 (126 MB), 1024
+// rows of 32000, kOwnedRows / kIfWaiting: 21.1 / 21.6 us, behind a kernel that does not release early 22.0 / 23.5; but 20000 logits (82 MB) that
+// are in L2 10.8 / 9.4.
+inline RowsAhead rows_ahead(long long rows, int vocab, int n_cta) {
+    if (2 * rows * n_cta <= static_cast<long long>(kRowBlocks) * sm_count()) return kEveryRow;
+    return rows * vocab > 25000000ll ? kOwnedRows : kIfWaiting;
+}
+inline int row_slots() { return kRowBlocks * sm_count(); }
 
 // The first CTA of a row's cluster to see all rows of the sequence done returns true (every thread of it; it then sees
 // what every other row's CTA wrote before its own call).  Word `counter` is zero between calls.

@@ -5,14 +5,15 @@
 // launch: a cluster per row (see ss_rows.cuh) finds the row's arg-max; the CTA that finishes a sequence's last row
 // reads the T arg-maxes and picks the path from the ancestor words, all nodes at once.  Measured on a B200, before (a grid of
 // 4096-logit chunks, one arrival per chunk, a serial walk) and after: 64 rows of 32000 logits 8.7 and 5.0 us, 1024 such
-// rows 37.3 and 24.1 us; with the prefetch before the wait 21.6 (6.1 TB/s).
+// rows 37.3 and 24.1 us; with the prefetch 21.4 (6.1 TB/s).
 #include "ss_rows.cuh"
 
 namespace ss {
 
+template <int AHEAD>
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks)
 tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens,
-                   const ss_tree_desc* __restrict__ trees, int max_nodes, int vocab, int n_cta,
+                   const ss_tree_desc* __restrict__ trees, int max_nodes, int vocab, int n_cta, int slots,
                    int32_t* __restrict__ accept_len, int32_t* __restrict__ accept_path,
                    int32_t* __restrict__ last_node, int32_t* __restrict__ bonus_token,
                    int32_t* __restrict__ node_argmax, int32_t* __restrict__ counters, int32_t* __restrict__ row_argmax) {
@@ -20,18 +21,21 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
     __shared__ unsigned long long s_part[kRowParts];
     __shared__ int32_t s_am[SS_MAX_NODES];
     __shared__ TreeShared s_tree;
+    __shared__ volatile int s_passed;
     if (n_cta > 1) cluster_arrive();                      // CTA 0 must have started before anyone stores to its shared memory
     const Segment seg = make_segment(logits, static_cast<size_t>(b) * max_nodes + t, vocab, rank, n_cta);
-    prefetch_batch(seg);
+    ask_ahead<AHEAD>(seg, trees[b], t, slots, &s_passed);
     wait_for_previous_kernel();
     release_next_kernel();
+    if (AHEAD == kIfWaiting) wait_passed(&s_passed);
     float4 q[kRowVecs];
-    load_first<kRowThreads>(seg, q);                      // (a row that no node owns is within the logits too)
+    if (AHEAD == kEveryRow) load_first<kRowThreads>(seg, q);    // (a row that no node owns is within the logits too)
     const int T = min(max(trees[b].n_nodes, 0), max_nodes);     // a descriptor is never trusted beyond the arrays' extent
     if (t >= max(T, 1)) {                                 // (the whole cluster: t is its row)
         if (n_cta > 1) cluster_wait();
         return;
     }
+    if (AHEAD != kEveryRow) load_first<kRowThreads>(seg, q);
     TreeRegs tree;
     tree.load(trees[b], tokens + static_cast<size_t>(b) * max_nodes, T);
     ArgMax am;
@@ -75,10 +79,13 @@ tree_verify_kernel(const float* __restrict__ logits, const int32_t* __restrict__
 static cudaError_t launch_verify(const float* logits, const int32_t* tokens, const ss_tree_desc* trees, int batch, int max_nodes, int vocab,
                                  int32_t* accept_len, int32_t* accept_path, int32_t* last_node, int32_t* bonus_token, int32_t* node_argmax,
                                  char* ws, size_t counter_bytes, cudaStream_t stream, bool early) {
-    const int n_cta = row_cluster(static_cast<long long>(batch) * max_nodes, vocab);
-    return launch_rows(tree_verify_kernel, dim3(n_cta, max_nodes, batch), dim3(kRowThreads), n_cta, early, stream, logits, tokens, trees, max_nodes,
-                       vocab, n_cta, accept_len, accept_path, last_node, bonus_token, node_argmax, reinterpret_cast<int32_t*>(ws + kWsHeaderBytes),
-                       reinterpret_cast<int32_t*>(ws + kWsHeaderBytes + counter_bytes));
+    const long long rows = static_cast<long long>(batch) * max_nodes;
+    const int n_cta = row_cluster(rows, vocab);
+    const RowsAhead ahead = rows_ahead(rows, vocab, n_cta);
+    const auto kernel = ahead == kEveryRow ? tree_verify_kernel<kEveryRow> : ahead == kOwnedRows ? tree_verify_kernel<kOwnedRows> : tree_verify_kernel<kIfWaiting>;
+    return launch_rows(kernel, dim3(n_cta, max_nodes, batch), dim3(kRowThreads), n_cta, early, stream, logits, tokens, trees, max_nodes, vocab,
+                       n_cta, row_slots(), accept_len, accept_path, last_node, bonus_token, node_argmax,
+                       reinterpret_cast<int32_t*>(ws + kWsHeaderBytes), reinterpret_cast<int32_t*>(ws + kWsHeaderBytes + counter_bytes));
 }
 
 }  // namespace ss

@@ -212,6 +212,46 @@ def test_row_statistics_at_the_edges_of_a_scan(cuda, V, soft):
     np.testing.assert_allclose(edge.cpu().numpy(), want, rtol=PROB_RTOL + 4e-5, atol=1e-30)
 
 
+@pytest.mark.parametrize("call", ["greedy", "soft", "prune"])
+def test_rows_that_no_node_owns_cost_no_traffic(cuda, call):
+    """Trees of one node in buffers for 64: of 131 MB of logits (more than L2 holds) only a 64th is needed.  A call that touches the
+    others' 8000 logits, a batch each, takes about as long as with full trees; one that does not is launches and little else."""
+    api = cuda
+    B, N, V = 64, 64, 8000
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")  # noqa: E731
+    f32 = lambda *shape: torch.zeros(shape, dtype=torch.float32, device="cuda")  # noqa: E731
+    lg, tok = torch.randn((B, N, V), device="cuda"), i32(B, N)
+    out = (i32(B), i32(B, api.SS_PATH_STRIDE), i32(B), i32(B))
+    ws = api.workspace((api.ss_tree_verify_workspace_bytes if call == "greedy" else api.ss_tree_prune_workspace_bytes)(B, N, V))
+    edge, ent, node, pruned = f32(B, N), f32(B, N), (i32(B, N), i32(B, N), i32(B, N)), api.empty_trees(B)
+
+    def run(trees):
+        if call == "greedy":
+            api.ss_tree_verify(lg, tok, trees, *out, node[0], ws)
+        elif call == "soft":
+            api.ss_tree_verify_soft(lg, tok, trees, 0.09, 0.3, *out, edge, ent, ws)
+        else:
+            api.ss_tree_prune(lg, tok, trees, 0.1, edge, *node, pruned, ws)
+
+    def us(n_nodes):
+        trees = api.trees_to_device([api.ss_tree_build([-1] + [0] * (n_nodes - 1), 1)] * B)
+        run(trees)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for _ in range(20):
+                run(trees)
+        best = 1e9
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(); g.replay(); b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 50)
+        return best
+
+    small, full = us(1), us(64)
+    assert small < 0.42 * full, (small, full)             # (8 / 23 to 10 / 36 us; 14 / 21 to 16 / 35 with a batch of every row loaded)
+
+
 # ---- attention directly behind the calls that write its trees ---------------------------------------------
 @pytest.mark.parametrize("batch,heads", [(1, 8), (6, 30)])               # both kernels that read the trees before their wait
 @pytest.mark.parametrize("writer", ["draft", "prune"])
