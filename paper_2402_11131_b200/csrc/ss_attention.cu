@@ -1557,6 +1557,10 @@ size_t AttnPlan::few_bytes() const { return cluster > 1 ? static_cast<size_t>(gr
 static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups, int split) {
     const long long slots = p.kv_total_slots / p.batch, keys = slots / split;        // keys per CTA of a grid of one wave
     const bool d64 = p.head_dim == 64, d80 = p.head_dim == 80;
+    // what a head can have keys of, and whether these are so few that a block of the half-SM kernel is mostly its fixed cost (the more of that the
+    // more waves there are): slabs in steps of 64 slots have to fall on the better side with most of the lengths that they stand for
+    const long long all_keys = slots + static_cast<long long>(p.max_nodes) * p.gamma;
+    const bool few_keys = all_keys <= (groups > 2 * sm_count() ? 128 : 96);
     // what the grid in blocks of 32 rows would read per SM
     const int blocks = (q_rows + 31) / 32;
     const long long load = static_cast<long long>(p.batch) * p.n_heads * blocks * slots / sm_count();
@@ -1569,14 +1573,22 @@ static int few_rows_block(const ss_attn_params& p, int q_rows, long long groups,
         // 63.8 / 65.3, but fifteen of 300 beside one of 4096 48.8 / 43.2; of 128: 130 keys 18.2 / 19.6, 700 38.3 / 43.2, 4000 156 / 164, fifteen of
         // 300 beside one of 4096 51.6 / 60.3, eight sequences of 24 heads, 256 keys 10.0 / 11.8.
         const int rows = q_rows <= 16 ? 16 : 32;
-        if (groups > sm_count()) return rows == 16 || p.head_dim <= 80 ? rows : 0;
+        // of 128, keys per head (tree included) 17 to 24 rows, half-SM / few rows: 40 keys 15.2 / 14.6, 70 keys 17.7 / 15.4, 114 keys 15.8 / 16.2, five
+        // sequences 6.1 / 6.25, 7.3 / 6.7, 6.5 / 7.2; 32 rows, 33 keys 15.3 / 15.9, 78 keys 17.8 / 16.6, 122 keys 16.0 / 17.6.
+        if (groups > sm_count()) return rows == 16 || p.head_dim <= 80 || (q_rows <= 24 && few_keys) ? rows : 0;
         return p.head_dim <= 80 || keys <= (q_rows <= 16 ? 1100 : 240) ? rows : 0;
     }
     if (q_rows <= kSmRows) {
-        // more heads than SMs.  Sixteen sequences, 64 rows of 64, 30 keys 15.8 / 14.7, 64 keys 14.5 / 14.9, 130 keys 17.6 / 18.8, 256 keys 18.9 /
-        // 21.9, 1024 keys 40.3 / 47.0; of 80, 30 keys 17.8 / 17.7, 64 keys 15.8 / 18.2, 1024 keys 45.0 / 57.3; of 128, 30 keys 20.5 / 21.6, 512
-        // keys 36.2 / 48.6
-        if (groups > sm_count()) return d64 && slots <= 48 ? 64 : 0;
+        // More heads than SMs, keys per head (tree and stream keys included), half-SM / few rows.  Sixteen sequences, of 64: 64 rows, 65 keys 15.8 /
+        // 14.7, 110 keys 15.8 / 15.1, 128 keys 14.5 / 14.8, 192 keys 16.1 / 17.0; 40 rows, 56 keys 13.75 / 12.1, 104 keys 14.3 / 13.6, 168 keys 15.9 /
+        // 15.7; 9 nodes and 3 streams, 96 keys 17.1 / 14.1, 156 keys 17.4 / 16.1; of 80: 40 rows, 56 keys 15.3 / 13.8, 86 keys 17.3 / 15.3, 130 keys
+        // 17.4 / 18.5, 64 rows, 65 keys 17.7 / 17.8, 110 keys 17.8 / 18.5.  Five sequences, of 64: 64 rows, 65 keys 6.3 / 6.35, 110 keys 6.2 / 6.6; 40 rows,
+        // 86 keys 6.1 / 5.7, 130 keys 6.4 / 6.65; of 80: 40 rows, 86 keys 7.1 / 6.6, 130 keys 7.35 / 8.4.  (The half-SM kernel's tiles have 64 keys.)
+        // Of 128, 64 rows, 94 keys 20.5 / 21.6.
+        if (groups > sm_count()) {
+            if (d64 && q_rows <= 48) return all_keys <= 160 ? 64 : 0;
+            return (d64 || (d80 && q_rows <= 48)) && few_keys ? 64 : 0;
+        }
         // (a batch goes by its mean: sixteen sequences of eight heads, 64 rows of 64, 200 keys 9.7 / 7.8, fifteen of 64 beside one of 2048
         // 16.6 / 28.6.)  64 rows of 64, 1024 keys 9.0 / 8.4; of 80, 1024 keys 10.9 / 10.4, 2048 keys 12.3 / 14.0; of 128, 512 keys 10.6 / 9.6, 1024
         // keys 11.0 / 12.8

@@ -5,6 +5,7 @@ Verification and compaction: bit-exact."""
 import numpy as np
 import pytest
 
+import launch_info
 from paper_2402_11131_b200 import workloads as W
 from parity_util import assert_attention_close, oracle_layer
 
@@ -331,21 +332,28 @@ def test_attention_few_rows_at_the_steps_of_the_split(cuda, oracle, head_dim, T,
     assert_attention_close(oracle, st, st.layer(0), dev, 0, check_lse=True)
 
 
-@pytest.mark.parametrize("head_dim,T,n_heads,lengths", [
-    (128, 16, 60, (1, 200)), (128, 17, 60, (1, 200)), (128, 32, 50, (63, 900)), (128, 32, 49, (63, 900)),
-    (64, 64, 60, (40, 41)), (64, 64, 60, (49, 50)), (80, 64, 60, (1, 70)),
+# (a sequence's slots are its length and its nodes, rounded up to 64)
+@pytest.mark.parametrize("head_dim,T,gamma,n_heads,lengths,kernel", [
+    (128, 16, 0, 60, (1, 200), "few_rows"), (128, 17, 0, 60, (1, 200), "half"), (128, 32, 0, 50, (63, 900), "half"), (128, 32, 0, 49, (63, 900), "small"),
+    (128, 24, 0, 60, (40, 40), "few_rows"), (128, 24, 0, 60, (41, 41), "half"), (128, 25, 0, 60, (1, 1), "half"),
+    (128, 24, 0, 99, (104, 104), "few_rows"), (128, 24, 0, 99, (105, 105), "half"), (128, 24, 0, 98, (104, 104), "half"),
+    (64, 64, 0, 60, (40, 41), "half"), (64, 64, 0, 60, (49, 50), "half"), (64, 64, 0, 99, (64, 64), "few_rows"), (64, 64, 0, 99, (65, 65), "half"),
+    (64, 48, 0, 60, (80, 80), "few_rows"), (64, 48, 0, 60, (81, 81), "half"), (64, 49, 0, 60, (15, 15), "few_rows"), (64, 49, 0, 60, (16, 16), "half"),
+    (64, 9, 3, 60, (119, 119), "few_rows"), (64, 9, 3, 60, (120, 120), "half"),
+    (80, 64, 0, 60, (1, 70), "half"), (80, 48, 0, 60, (16, 16), "few_rows"), (80, 48, 0, 60, (17, 17), "half"), (80, 49, 0, 99, (15, 15), "half"),
 ])
-def test_attention_batches_on_both_sides_of_the_few_rows(cuda, oracle, head_dim, T, n_heads, lengths):
+def test_attention_batches_on_both_sides_of_the_few_rows(cuda, oracle, head_dim, T, gamma, n_heads, lengths, kernel):
     """Batches of three around the rows, heads and lengths at which the few-rows kernel ends."""
     api, DeviceStep = cuda
-    cfg = W.custom_config("side", batch=3, n_layers=2, n_msa_layers=1, prefix_len_range=lengths, n_nodes=T, gamma=1, max_depth=6,
+    cfg = W.custom_config("side", batch=3, n_layers=2, n_msa_layers=1, prefix_len_range=lengths, n_nodes=T, gamma=max(gamma, 1), max_depth=6,
                           n_heads=n_heads, head_dim=head_dim, config_id=990 + T)
     st = W.make_step(cfg)
-    dev = DeviceStep(st, layers=[0], with_lse=True)
-    for _ in range(2):
-        dev.run_attention()
+    layer = 1 if gamma else 0
+    dev = DeviceStep(st, layers=[layer], with_lse=True)
+    assert [kernel in k["name"] for k in launch_info.kernels(dev.run_attention)] == [True]
+    dev.run_attention()
     assert api.ss_status(dev.attn_ws) == 0
-    assert_attention_close(oracle, st, st.layer(0), dev, 0, check_lse=True)
+    assert_attention_close(oracle, st, st.layer(layer), dev, 0, check_lse=True, heads=(n_heads - 8, n_heads))
 
 
 @pytest.mark.parametrize("head_dim", [64, 80, 128])
