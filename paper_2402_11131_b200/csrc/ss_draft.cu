@@ -11,6 +11,7 @@
 // 32000 34.1 and 7.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of 32000) 15.6 and
 // 5.3 us.  Pruning then 31.4 -> 28.4 with packed exponentials and without the sums that only the verification uses, 26.7 with the prefetch
 // before the wait.
+#include "ss_draft_plan.h"
 #include "ss_rows.cuh"
 
 namespace ss {
@@ -54,7 +55,6 @@ constexpr float kTinyExp = -200.f;                        // exp of it is 0 in f
 // index, it takes the whole batch through a stack frame in local memory.  From HBM, before / after: sampled verification of 64 rows of 32000
 // 9.4 / 7.2 us, 135 of 50257 16.3 / 12.0, 1024 of 8000 20.1 / 12.2, 1024 of 32000 40.2 / 30.3; 16 next drafts of four rows of 32000 8.6 / 5.3.
 constexpr int kListCap = 512;
-constexpr int kMaxClusterCtas = 16;   // CTAs of a cluster: 8 are portable, sm_100a takes 16
 template <int NT>
 struct TopKShared {
     static_assert(NT / 32 >= kMaxTopK, "the k-th largest warp maximum has to exist");
@@ -298,7 +298,7 @@ static __device__ __forceinline__ void write_shape(DraftShape& s, int gamma, int
     __threadfence();
     asm volatile("bar.sync 1, 64;" ::: "memory");
 }
-constexpr int kDraftThreads = 512;    // few rows: a segment of up to 16384 logits is one batch of loads
+static_assert(kDraftBatch == 4 * kDraftThreads * kRowVecs, "a batch of loads");
 __global__ void __launch_bounds__(kDraftThreads, 2)
 next_draft_kernel(const float* __restrict__ stream_logits, int n_rows, const int32_t* __restrict__ row_index,
                   const int32_t* __restrict__ bonus_token, int gamma, int vocab, int k, int max_nodes, int n_cta,
@@ -610,15 +610,8 @@ extern "C" int32_t ss_next_draft(const float* stream_logits, int32_t n_rows, con
     if (gamma > SS_MAX_GAMMA || top_k > SS_MAX_TOPK || top_k > vocab || max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(stream_logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_next_draft_workspace_bytes(batch, gamma, vocab)) return SS_ERR_WORKSPACE;
-    // A cluster takes all the rows of a sequence: up to 8 CTAs, and up to 16 for a few sequences where a CTA's segment is then one batch of
-    // loads instead of two (whose candidates would be read again).  Three rows of 51200 logits, 8 / 16: one sequence 7.3 / 6.1 us, six
-    // 7.7 / 6.8, four rows of 50257 7.4 / 6.4 and 8.4 / 6.9; but eight sequences 8.1 / 9.1, sixteen 11.7 / 14.3 (the clusters of 12 or 16
-    // CTAs no longer run all at once), and four rows of 32000, one batch already, 6.2 / 6.2.
-    constexpr int kOneBatch = 4 * ss::kDraftThreads * ss::kRowVecs;
-    int n_cta = 1;
-    while (vocab / (n_cta * 2) >= ss::kDraftThreads * 4 &&
-           (gamma * n_cta * 2 <= 8 || (batch <= 6 && vocab / n_cta > kOneBatch && gamma * n_cta * 2 <= ss::kMaxClusterCtas))) n_cta *= 2;
-    if (gamma * n_cta > 8) {
+    const int n_cta = ss::draft_ctas(batch, gamma, vocab, ss::kMaxClusterCtas);
+    if (gamma * n_cta > ss::kPortableCtas) {
         static bool configured[64] = {false};
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;

@@ -68,10 +68,16 @@ def test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, max_nodes, ties):
             assert _desc_fields(descs[b]) == _desc_fields(host)
 
 
-# clusters of 12 and 16 CTAs, and the sizes next to them
-@pytest.mark.parametrize("B,gamma,V,k,ties", [(1, 3, 32769, 8, True), (6, 4, 51201, 8, True), (7, 4, 51201, 8, True), (2, 2, 131100, 8, False),
-                                              (1, 4, 32768, 8, False)])
-def test_next_draft_with_clusters_beyond_eight_ctas(cuda, oracle, B, gamma, V, k, ties):
+# clusters of 12 and 16 CTAs, and the sizes next to them; the CTAs of a sequence are the grid's first dimension
+@pytest.mark.parametrize("B,gamma,V,k,ties,ctas", [(1, 3, 32768, 8, True, 6), (1, 3, 32769, 8, True, 12), (1, 3, 32773, 8, True, 12), (6, 3, 50257, 8, True, 12),
+                                                   (6, 4, 51201, 8, True, 16), (7, 4, 51201, 8, True, 8), (2, 2, 131100, 8, True, 16),
+                                                   (1, 4, 32768, 8, False, 8), (1, 4, 32766, 8, False, 16), (1, 1, 131100, 8, True, 8)])
+def test_next_draft_with_clusters_beyond_eight_ctas(cuda, oracle, B, gamma, V, k, ties, ctas):
+    api = cuda
+    ws, lg = api.workspace(api.ss_next_draft_workspace_bytes(B, gamma, V)), torch.zeros((B, 1, gamma, V), device="cuda")
+    trees, tokens, bonus = api.empty_trees(B), _i32(np.zeros((B, 64))), _i32(np.zeros(B))
+    launched = launch_info.kernels(lambda: api.ss_next_draft(lg, None, bonus, k, 64, tokens, trees, ws))
+    assert [x["grid"] for x in launched] == [(ctas, B, 1)]
     test_next_draft_is_bit_exact(cuda, oracle, B, gamma, V, k, 64, ties)
 
 

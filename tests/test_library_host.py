@@ -221,3 +221,21 @@ def test_per_step_calls_go_to_the_library_that_was_loaded(lib, tmp_path):
     with pytest.raises(api.SsError) as e:
         api.ss_msa_attention(api.AttnParams(), _Stream())
     assert e.value.status == api.SS_ERR_INVALID_ARG
+
+
+def _draft_plan(tmp_path, body):
+    """The output of a program that includes the next draft's host rules."""
+    src, exe = tmp_path / "plan.cpp", tmp_path / "plan"
+    src.write_text('#include <cstdio>\n#include "ss_draft_plan.h"\nint main() {\n%s\nreturn 0; }\n' % body)
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Werror", "-I", build.CSRC, str(src), "-o", str(exe)])
+    return subprocess.check_output([str(exe)], text=True).split()
+
+
+def test_next_draft_cluster_sizes(tmp_path):
+    """More than 8 CTAs where a segment of 8 spans more than one batch of 16384 words (rows of a vocabulary that is no multiple of four begin up
+    to three words after an aligned address), for at most six sequences of at least two rows."""
+    cases = [((1, 4, 32000), 8), ((1, 4, 32768), 8), ((1, 4, 32769), 16), ((1, 4, 32766), 16), ((1, 4, 32764), 8), ((6, 4, 51201), 16),
+             ((7, 4, 51201), 8), ((1, 3, 32768), 6), ((1, 3, 32769), 12), ((1, 3, 50257), 12), ((6, 3, 51200), 12), ((16, 3, 51200), 6),
+             ((1, 2, 65536), 8), ((1, 2, 65540), 16), ((1, 1, 131072), 8), ((1, 1, 131100), 8), ((1, 1, 262144), 8), ((1, 4, 4095), 4), ((1, 1, 37), 1)]
+    got = _draft_plan(tmp_path, "\n".join('printf("%%d\\n", %d * ss::draft_ctas(%d, %d, %d, ss::kMaxClusterCtas));' % (c[1], *c) for c, _ in cases))
+    assert [int(x) for x in got] == [want for _, want in cases]
