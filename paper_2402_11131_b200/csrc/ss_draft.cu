@@ -11,6 +11,8 @@
 // 32000 34.1 and 7.2 us, pruning over 1024 rows of 32000 126 and 31 us, the next draft of 16 sequences (64 rows of 32000) 15.6 and
 // 5.3 us.  Pruning then 31.4 -> 28.4 with packed exponentials and without the sums that only the verification uses, 26.7 with the prefetch
 // before the wait.
+#include <atomic>
+
 #include "ss_draft_plan.h"
 #include "ss_rows.cuh"
 
@@ -588,6 +590,33 @@ sampled_verify_kernel(const float* __restrict__ logits, const int32_t* __restric
     }
 }
 
+// Whether the current device can hold a cluster of that many CTAs of the next draft (12 or 16): it takes a GPC with as many free places, which
+// a partition of a GPU may not have.  Asked for once per device and size.
+static bool draft_cluster_fits(int ctas) {
+    static std::atomic<signed char> known[64][kMaxClusterCtas + 1];          // 0: not asked for yet
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    signed char k = known[dev][ctas].load(std::memory_order_relaxed);
+    if (k == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ctas, 1);
+        cfg.blockDim = dim3(kDraftThreads);
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim = {static_cast<unsigned>(ctas), 1, 1};
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(next_draft_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, next_draft_kernel, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        known[dev][ctas].store(k = n > 0 ? 1 : -1, std::memory_order_relaxed);
+    }
+    return k > 0;
+}
+
 static size_t scan_workspace(int32_t batch, int32_t rows, int32_t vocab, size_t per_chunk) {
     if (batch < 1 || rows < 1 || vocab < 1) return 0;
     // (room for a partial result per 4096 logits, as callers have always been told; one result per row is used)
@@ -610,20 +639,13 @@ extern "C" int32_t ss_next_draft(const float* stream_logits, int32_t n_rows, con
     if (gamma > SS_MAX_GAMMA || top_k > SS_MAX_TOPK || top_k > vocab || max_nodes > SS_MAX_NODES) return SS_ERR_UNSUPPORTED;
     if (!ss::aligned16(stream_logits) || !ss::aligned16(workspace)) return SS_ERR_INVALID_ARG;
     if (workspace_bytes < ss_next_draft_workspace_bytes(batch, gamma, vocab)) return SS_ERR_WORKSPACE;
-    const int n_cta = ss::draft_ctas(batch, gamma, vocab, ss::kMaxClusterCtas);
-    if (gamma * n_cta > ss::kPortableCtas) {
-        static bool configured[64] = {false};
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_CUDA;
-        if (dev < 0 || dev >= 64 || !configured[dev]) {
-            if (cudaFuncSetAttribute(ss::next_draft_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return SS_ERR_CUDA;
-            if (dev >= 0 && dev < 64) configured[dev] = true;
-        }
-    }
-    const cudaError_t err = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kDraftThreads),
-                                            gamma * n_cta, true,
-                                            static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token, gamma, vocab,
-                                            top_k, max_nodes, n_cta, draft_tokens, trees);
+    const cudaError_t err = ss::launch_draft(batch, gamma, vocab, ss::draft_cluster_fits, [&](int n_cta) {
+        const cudaError_t e = ss::launch_rows(ss::next_draft_kernel, dim3(gamma * n_cta, batch), dim3(ss::kDraftThreads), gamma * n_cta, true,
+                                              static_cast<cudaStream_t>(stream), stream_logits, n_rows, row_index, bonus_token, gamma, vocab,
+                                              top_k, max_nodes, n_cta, draft_tokens, trees);
+        if (e != cudaSuccess && gamma * n_cta > ss::kPortableCtas) (void)cudaGetLastError();    // (there is a way out)
+        return e;
+    });
     return err == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }
 

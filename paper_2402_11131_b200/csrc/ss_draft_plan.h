@@ -1,4 +1,4 @@
-// How the next draft cuts its rows into CTAs.  Host code without CUDA, so that the rule can be checked without a GPU.
+// How the next draft cuts its rows into CTAs.  Host code without CUDA, so that the rule and its ways out can be checked without a GPU.
 #pragma once
 
 namespace ss {
@@ -22,6 +22,17 @@ inline int draft_ctas(int batch, int gamma, int vocab, int most) {
     while (vocab / (n * 2) >= kDraftThreads * 4 &&
            (gamma * n * 2 <= kPortableCtas || (batch <= 6 && gamma > 1 && draft_segment_words(vocab, n) > kDraftBatch && gamma * n * 2 <= most))) n *= 2;
     return n;
+}
+
+// launch(CTAs per row), which gives 0 or an error.  More than 8 CTAs cannot be placed on every part of a GPU: then 8 at most take the sequence, whether
+// fits(CTAs) says so beforehand or the launch.
+template <typename Fits, typename Launch>
+inline auto launch_draft(int batch, int gamma, int vocab, Fits&& fits, Launch&& launch) -> decltype(launch(1)) {
+    const int narrow = draft_ctas(batch, gamma, vocab, kPortableCtas);
+    int n = draft_ctas(batch, gamma, vocab, kMaxClusterCtas);
+    if (n != narrow && !fits(gamma * n)) n = narrow;
+    const auto err = launch(n);
+    return err != decltype(err)(0) && n != narrow ? launch(narrow) : err;
 }
 
 }  // namespace ss

@@ -239,3 +239,18 @@ def test_next_draft_cluster_sizes(tmp_path):
              ((1, 2, 65536), 8), ((1, 2, 65540), 16), ((1, 1, 131072), 8), ((1, 1, 131100), 8), ((1, 1, 262144), 8), ((1, 4, 4095), 4), ((1, 1, 37), 1)]
     got = _draft_plan(tmp_path, "\n".join('printf("%%d\\n", %d * ss::draft_ctas(%d, %d, %d, ss::kMaxClusterCtas));' % (c[1], *c) for c, _ in cases))
     assert [int(x) for x in got] == [want for _, want in cases]
+
+
+def test_next_draft_falls_back_to_clusters_that_can_be_placed(tmp_path):
+    """Where the device says that 12 CTAs do not fit, or the launch does, 6 take the sequence; an error of these is an error."""
+    body = """
+    const auto run = [](int vocab, bool fits, int limit) {          // a device that says `fits` and launches up to `limit` CTAs
+        int asked = 0;
+        const int err = ss::launch_draft(1, 3, vocab, [&](int ctas) { asked = ctas; return fits; },
+                                         [&](int n) { std::printf("launch:%d ", 3 * n); return 3 * n <= limit ? 0 : 7; });
+        std::printf("asked:%d error:%d\\n", asked, err);
+    };
+    run(51200, true, 16); run(51200, false, 16); run(51200, true, 8); run(51200, true, 0); run(32000, false, 16); run(32000, true, 0);"""
+    assert _draft_plan(tmp_path, body) == ["launch:12", "asked:12", "error:0", "launch:6", "asked:12", "error:0", "launch:12", "launch:6", "asked:12",
+                                           "error:0", "launch:12", "launch:6", "asked:12", "error:7", "launch:6", "asked:0", "error:0", "launch:6",
+                                           "asked:0", "error:7"]
