@@ -1654,10 +1654,10 @@ static bool make_plan(const ss_attn_params& p, AttnPlan* plan) {
     if (plan->few_rows) {
         few_plan(plan->few_rows);
         plan->n_blocks = few.n_blocks; plan->groups = few.groups; plan->cluster = few.cluster;
-        // no more CTAs than the slab's slots can ask for (a sequence of a batch: twice the mean); one that finds nothing to
-        // do still costs its launch: 128 or 256 CTAs for 32 whole heads of 528 keys 5.0 and 5.7 us
-        const long long most = (p.batch > 1 ? 2 : 1) * (p.kv_total_slots / p.batch) + static_cast<long long>(p.max_nodes) * p.gamma;
-        const long long tiles = (most + kFwKeys - 1) / kFwKeys + 1;
+        // no more CTAs than the slab's slots can ask for (a sequence of a batch: twice the mean), by the kernel's own count of tiles; one that finds
+        // nothing to do still costs its launch: 128 or 256 CTAs for 32 whole heads of 528 keys 5.0 and 5.7 us
+        const long long slots = (p.batch > 1 ? 2 : 1) * (p.kv_total_slots / p.batch), streams = static_cast<long long>(p.max_nodes) * p.gamma;
+        const long long tiles = (slots + kFwKeys - 1) / kFwKeys + (streams + kFwKeys - 1) / kFwKeys;
         const int whole = few_whole(p.head_dim, plan->few_rows);
         // (the kernel rounds down: 4.9 tiles per CTA are not split further.  32 heads, 32 rows of 80 and 12 of 128, 512 keys, with CTAs that find
         // nothing to do 7.82 and 7.02 us, without 7.0 and 6.27)

@@ -316,18 +316,22 @@ def test_attention_with_less_workspace_than_a_further_split_could_use(cuda, orac
         assert_attention_close(oracle, st, st.layer(1 if gamma else 0), dev, 0, heads=(98, 100))
 
 
-@pytest.mark.parametrize("head_dim,T", [(64, 12), (80, 30), (128, 12)])
-@pytest.mark.parametrize("tiles", [7, 9, 16, 19, 20, 39, 41])
-def test_attention_few_rows_at_the_steps_of_the_split(cuda, oracle, head_dim, T, tiles):
+@pytest.mark.parametrize("head_dim,T,whole", [(64, 12, 20), (80, 30, 6), (128, 12, 8)])
+@pytest.mark.parametrize("tiles", [7, 8, 9, 16, 19, 20, 39, 41])
+def test_attention_few_rows_at_the_steps_of_the_split(cuda, oracle, head_dim, T, whole, tiles):
     """Heads of as many tiles of 32 keys as the host's and the kernel's rules change the number of CTAs per head at, the last tile
-    with one key."""
+    with one key, on a slab of as many tiles: every CTA that is launched has tiles."""
     api, DeviceStep = cuda
     cfg = W.custom_config("split", n_layers=2, n_msa_layers=1, prefix_len=32 * (tiles - 1) + 1 - T, n_nodes=T, gamma=1, max_depth=4, n_heads=6,
                           head_dim=head_dim, config_id=960 + tiles)
     st = W.make_step(cfg)
     dev = DeviceStep(st, layers=[0], with_lse=True)
-    for _ in range(2):
-        dev.run_attention()
+    dev.params[0].kv_total_slots = 32 * tiles             # (the step's slab is rounded up to 64 slots)
+    ctas = 1
+    while tiles > whole and ctas < 8 and tiles // ctas > 4:
+        ctas *= 2
+    assert [k["grid"][0] for k in launch_info.kernels(dev.run_attention)] == [6 * ctas]
+    dev.run_attention()
     assert api.ss_status(dev.attn_ws) == 0
     assert_attention_close(oracle, st, st.layer(0), dev, 0, check_lse=True)
 
