@@ -179,21 +179,27 @@ def test_tree_prune_matches_the_oracle(cuda, oracle, name):
 @pytest.mark.parametrize("soft", [False, True])
 @pytest.mark.parametrize("V", [1, 2, 33, 1023, 8191, 8193, 20001])       # one vector, unaligned rows, a batch of loads and one logit more
 def test_row_statistics_at_the_edges_of_a_scan(cuda, V, soft):
-    """Edge probabilities (and entropies) of short, unaligned and peaked rows with -inf and NaN among the logits, against fp64.  A
-    term is off by at most 2 ulp of the exponential and a row's sum by the roundings of its longest chain of additions (20001
-    logits over 256 threads and 4 partial sums, then 10 merges: 30 roundings), 34 * 2^-24 = 2e-6 in all; the entropy's terms
-    carry a factor |x - m| <= 12 for the logits that count.  PROB_RTOL is ten times the former."""
+    """Edge probabilities (and entropies) of short, unaligned and peaked rows with -inf and NaN among the logits, against fp64.  Rows 6
+    and 7 have their mass away from the maximum: one logit above all others by 8, and one in 256 above the others by 5.25 (with
+    others of its thread).  A term is off by at most 2 ulp of the exponential and a row's sum by the roundings of its longest chain of
+    additions (20001 logits over 256 threads and 4 partial sums, then 10 merges: 30 roundings), SUM = 34 * 2^-24 = 2e-6 in all.  A
+    probability's exponent child - (m + log Z) is rounded at the size of its terms, each by half an ulp, log Z by one; the entropy
+    log Z - W / Z has SUM for log Z and twice that for the quotient.  (An exponential without the correction of its argument's rounding is off by
+    3e-7 of such a row's sum, which no bound on fp32 results tells from their own roundings.)"""
     api = cuda
-    B, T = 2, 6
+    B, T = 2, 9
+    SUM, ULP = 34 * 2.0 ** -24, 2.0 ** -23
     rng = np.random.default_rng(77 + V)
-    scale = np.array([1.0, 1.0, 4.0, 30.0, 1.0, 1.0])[None, :, None]
-    lg = (rng.standard_normal((B, T, V)) * scale + np.array([0.0, 300.0, 0.0, 0.0, -80.0, 5.0])[None, :, None]).astype(np.float32)
+    scale = np.array([1.0, 1.0, 4.0, 30.0, 1.0, 1.0, 0.0, 0.0, 1.0])[None, :, None]
+    lg = (rng.standard_normal((B, T, V)) * scale + np.array([0.0, 300.0, 0.0, 0.0, -80.0, 5.0, -8.0, -5.25, 0.0])[None, :, None]).astype(np.float32)
+    lg[:, 6, V // 2] = 0.0
+    lg[:, 7, ::256] = 0.0
     tok = rng.integers(0, V, (B, T)).astype(np.int32)
     if V > 8:                                                            # (not at the children's tokens)
         for t, bad in ((0, np.nan), (4, -np.inf), (5, np.nan)):
             at = np.setdiff1d(rng.integers(0, V, V // 3), tok)
             lg[:, t, at] = bad
-    parent = [-1, 0, 1, 2, 3, 4]
+    parent = list(range(-1, T - 1))
     trees = api.trees_to_device([api.ss_tree_build(parent, 2)] * B)
     edge = torch.zeros((B, T), device="cuda")
     i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")  # noqa: E731
@@ -202,20 +208,24 @@ def test_row_statistics_at_the_edges_of_a_scan(cuda, V, soft):
     m = x.max(-1, keepdims=True)
     e = np.exp(x - m)
     z = e.sum(-1)
+    log_z, lse = np.log(z), m[..., 0] + np.log(z)
     if soft:
         ent = torch.zeros((B, T), device="cuda")
         api.ss_tree_verify_soft(torch.from_numpy(lg).cuda(), _i32(tok), trees, 0.09, 0.3, i32(B), i32(B, api.SS_PATH_STRIDE), i32(B), i32(B), edge, ent, ws)
-        want = np.log(z) - (np.where(e > 0, x - m, 0.0) * e).sum(-1) / z
-        # log z and the mean of x - m may cancel: their sizes bound the error
-        np.testing.assert_allclose(ent.cpu().numpy(), want, rtol=0, atol=PROB_RTOL * (1.0 + np.log(V)))
+        w = -(np.where(e > 0, x - m, 0.0) * e).sum(-1) / z
+        err = np.abs(ent.cpu().numpy() - (log_z + w))
+        assert (err <= SUM + 2 * SUM * w + ULP * (log_z + w)).all(), err
     else:
         api.ss_tree_prune(torch.from_numpy(lg).cuda(), _i32(tok), trees, 0.1, edge, i32(B, T), i32(B, T), i32(B, T), api.empty_trees(B), ws)
     assert api.ss_status(ws) == 0
-    want = np.ones((B, T))
-    for c in range(1, T):
-        want[:, c] = [np.exp(x[b, c - 1, tok[b, c]] - m[b, c - 1, 0]) / z[b, c - 1] for b in range(B)]
-    # (the exponent child - log-sum-exp is rounded at the size of the logits: 300 * 2^-24 = 1.8e-5 in the second row)
-    np.testing.assert_allclose(edge.cpu().numpy(), want, rtol=PROB_RTOL + 4e-5, atol=1e-30)
+    child = np.take_along_axis(x[:, :-1], tok[:, 1:, None].astype(np.int64), -1)[..., 0]
+    log_z, lse, z = log_z[:, :-1], lse[:, :-1], z[:, :-1]
+    want = np.exp(child - m[:, :-1, 0]) / z
+    rel = SUM + 2 * ULP + ULP * log_z + ULP / 2 * (np.abs(lse) + np.abs(child - lse))
+    got = edge.cpu().numpy()
+    assert (got[:, 0] == 1.0).all()
+    err = np.abs(got[:, 1:] - want)
+    assert (err <= rel * want + 1e-30).all(), err / want
 
 
 @pytest.mark.parametrize("call", ["greedy", "soft", "prune"])
