@@ -12,8 +12,7 @@
 // slots [0, L+T) (prefix, then this step's tree nodes, masked by ancestry) and the block's transient
 // stream keys (node-major) are cut into 16-key units and CTA r takes units [U*r/C, U*(r+1)/C), so every
 // CTA of a block streams the same number of bytes.  The CTAs of a pair run in the same wave, so a K/V
-// tile crosses HBM once and is served from L2 to the other row blocks.  A batch (up to 32 sequences, no
-// key split) is dispatched longest prefix first.
+// tile crosses HBM once and is served from L2 to the other row blocks.
 //
 // Inside a CTA of msa_attention_kernel.
 //   threads 0, 96  TMA producers of the K ring and of the V ring (mbarrier complete_tx); swizzle-128B

@@ -8,7 +8,7 @@
 // The pass over a segment runs from registers, eight 16-byte loads per thread in flight.  Everything behind it is short:
 // for one sequence these kernels are chains of latencies, in which most instructions execute once per CTA.  Measured and
 // not kept: the segment staged in shared memory by bulk copies, one pass there for the maximum and one for the rest
-// (1024 rows of 32000 logits: arg-max 35 us, softmax statistics 52 us, against 24 and 31 us).
+// (1024 rows of 32000 logits: arg-max 35 us, softmax statistics 52 us, against 24 and 31 us before anything was asked for ahead).
 //
 // Order of logits.  Entries are ranked by an integer key that is monotone in the IEEE order of fp32 values, with
 // -0 == +0 and every NaN below -inf, and equal keys by ascending index.  Compiled without fast-math: nothing is
@@ -19,8 +19,9 @@
 namespace ss {
 
 // Threads of a scan: 256 with eight 16-byte loads each in flight, four CTAs per SM (64 registers a thread): 128 KB in
-// flight per SM.  Measured for 1024 rows of 32000 logits, arg-max / softmax statistics: 23.6 / 31.2 us; four loads and
-// six CTAs 28.2 / 36.6; 512 threads 25.1 / 36.1; two CTAs per row 27.5 / 39.1 (a CTA costs 4 us besides its loads).
+// flight per SM.  Measured for 1024 rows of 32000 logits, arg-max / softmax statistics, before what is asked for ahead and the packed
+// exponentials (21.6 / 27.2 us now): 23.6 / 31.2; four loads and six CTAs 28.2 / 36.6; 512 threads 25.1 / 36.1; two CTAs per row
+// 27.5 / 39.1 (a CTA costs 4 us besides its loads).
 constexpr int kRowThreads = 256;
 constexpr int kRowVecs = 8;
 constexpr int kRowBlocks = 4;         // CTAs per SM

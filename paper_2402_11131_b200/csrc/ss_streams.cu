@@ -21,12 +21,14 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 
 // Both kernels: a thread owns 8 columns (16 bytes) of the width and walks down the rows, kRowBatch of them at a time, so
 // that no index is divided and a thread has kRowBatch loads and gamma * kRowBatch stores in flight.  Bound by HBM, four
-// fifths of it writes: both together take 15.8 us for 1024 rows of 4096 with four streams (84 MB; 17.0 us without the prefetch
-// before the wait, 21.4 us with one thread per output vector and its index divided into row, stream and column).
+// fifths of it writes: both together take 15.7 us for 1024 rows of 4096 with four streams (84 MB; 17.0 us without the prefetch
+// before the wait, behind a kernel that releases its successor early and with inputs in HBM; 21.4 us with one thread per output vector and its index
+// divided into row, stream and column).
 constexpr int kRowBatch = 2;
 
 // A thread's first rows on their way to L2 (one thread asks for a line of 128 bytes): no data reaches the SM, so it may be asked
-// for before the wait for the previous kernel, whoever writes them.
+// for before the wait for the previous kernel, whoever writes them.  (Without / with it behind a kernel that does not release
+// early 16.9 / 16.2 us; with inputs in L2 13.9 / 14.1.)
 __device__ __forceinline__ void prefetch_rows(const uint4* in, long long first, int by, long long rows, int vec, int c) {
     if (c >= vec || (c & 7) != 0) return;
     #pragma unroll

@@ -5,7 +5,7 @@
 // launch: a cluster per row (see ss_rows.cuh) finds the row's arg-max; the CTA that finishes a sequence's last row
 // reads the T arg-maxes and picks the path from the ancestor words, all nodes at once.  Measured on a B200, before (a grid of
 // 4096-logit chunks, one arrival per chunk, a serial walk) and after: 64 rows of 32000 logits 8.7 and 5.0 us, 1024 such
-// rows 37.3 and 24.1 us; with the prefetch 21.4 (6.1 TB/s).
+// rows 37.3 and 24.1 us; with the prefetch 21.6 (6.1 TB/s).
 #include "ss_rows.cuh"
 
 namespace ss {
