@@ -184,8 +184,8 @@ inline int row_cluster(long long rows, int vocab) {
     return c;
 }
 // kEveryRow on grids of at most half of the slots: at most a batch each for 296 CTAs, 9.7 MB, which little waits for.  64 rows of 32000,
-// arg-max, loads behind the length / beside it and prefetched 5.2 / 4.5 us, 16 of them owned 4.25 / 4.2; 128 rows of 32000 6.8 / 6.1 and, 32
-// owned, 5.45 / 5.45.  On larger grids it costs smaller trees more than it gives full ones: sixteen trees of 16 of 64 nodes, 32000 logits a row
+// arg-max, loads behind the length / beside it and prefetched 5.2 / 4.5 us, 16 of them owned 4.25 / 4.2; 128 rows of 32000 6.8 / 6.1 (in L2
+// 5.05 / 5.4) and, 32 owned, 5.45 / 5.45.  On larger grids it costs smaller trees more than it gives full ones: sixteen trees of 16 of 64 nodes, 32000 logits a row
 // 11.9 us and 9.3 with owned rows only, 8000 logits 8.4 and 5.3.  kOwnedRows where the logits are too many to be in L2 (126 MB), 1024
 // rows of 32000, kOwnedRows / kIfWaiting: 21.1 / 21.6 us, behind a kernel that does not release early 22.0 / 23.5; but 20000 logits (82 MB) that
 // are in L2 10.8 / 9.4.
